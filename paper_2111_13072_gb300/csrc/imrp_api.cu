@@ -96,7 +96,7 @@ struct imrp_ctx {
   StepState* st = nullptr;
   int* derr = nullptr;
   double* dft = nullptr;
-  int64_t dft_cap = 0;
+  int64_t dft_cap = 0;  // doubles
   // radial ion profile (App. D) in place of the uniform background
   double* ion_q = nullptr;    // device copy, units e n_inf R^3
   int64_t ion_n = 0;
@@ -1567,11 +1567,13 @@ extern "C" int imrp_spectrum(imrp_ctx* ctx, int64_t n_freq, double w_max, double
   const int64_t ns = ctx->host_step;
   if (ns < 8) return ctx->fail(IMRP_E_STATE, "spectrum needs at least 8 recorded steps (have %lld)", (long long)ns);
   if (n_freq < 3 || !(w_max > 0)) return ctx->fail(IMRP_E_INVAL, "spectrum: n_freq >= 3 and w_max > 0 required");
-  if (n_freq > ctx->dft_cap) {
+  const int64_t work = dft_work_doubles(ns, n_freq);
+  if (work > ctx->dft_cap) {
     cudaFree(ctx->dft);
     ctx->dft = nullptr;
-    CK(cudaMalloc(&ctx->dft, 4 * n_freq * sizeof(double)));
-    ctx->dft_cap = n_freq;
+    ctx->dft_cap = 0;
+    CK(cudaMalloc(&ctx->dft, work * sizeof(double)));
+    ctx->dft_cap = work;
   }
   const double dt = ctx->p.dt;
   launch_dft(ctx->qhist, ctx->uhist, ns, dt, 0.5 * dt, n_freq, w_max, ctx->dft, ctx->stream);
@@ -1631,15 +1633,14 @@ extern "C" int imrp_fit_damped_sine(const double* q, int64_t ns, double dt, doub
 extern "C" int imrp_admittance(const double* q, const double* u, int64_t ns, double dt, double first_kick,
                                int64_t n_freq, double w_max, double* omega, double* reY, double* imY) {
   if (!q || !u || ns < 8 || n_freq < 3 || !(w_max > 0) || !(dt > 0)) return IMRP_E_INVAL;
-  double *dq = nullptr, *du = nullptr, *dout = nullptr;
-  const size_t bs = size_t(ns) * sizeof(double), bo = size_t(4 * n_freq) * sizeof(double);
-  if (cudaMalloc(&dq, bs) != cudaSuccess || cudaMalloc(&du, bs) != cudaSuccess ||
-      cudaMalloc(&dout, bo) != cudaSuccess) {
-    cudaFree(dq);
-    cudaFree(du);
-    cudaFree(dout);
+  // one buffer: q [ns], u [ns], then the transform's work space
+  double* dbuf = nullptr;
+  if (cudaMalloc(&dbuf, (2 * size_t(ns) + size_t(dft_work_doubles(ns, n_freq))) * sizeof(double)) != cudaSuccess) {
+    cudaGetLastError();
     return IMRP_E_NOMEM;
   }
+  double *dq = dbuf, *du = dbuf + ns, *dout = dbuf + 2 * ns;
+  const size_t bs = size_t(ns) * sizeof(double);
   std::vector<double> h(4 * n_freq);
   cudaError_t e = cudaMemcpy(dq, q, bs, cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMemcpy(du, u, bs, cudaMemcpyHostToDevice);
@@ -1647,10 +1648,8 @@ extern "C" int imrp_admittance(const double* q, const double* u, int64_t ns, dou
     launch_dft(dq, du, ns, dt, first_kick, n_freq, w_max, dout, 0);
     e = cudaGetLastError();
   }
-  if (e == cudaSuccess) e = cudaMemcpy(h.data(), dout, bo, cudaMemcpyDeviceToHost);
-  cudaFree(dq);
-  cudaFree(du);
-  cudaFree(dout);
+  if (e == cudaSuccess) e = cudaMemcpy(h.data(), dout, h.size() * sizeof(double), cudaMemcpyDeviceToHost);
+  cudaFree(dbuf);
   if (e != cudaSuccess) return IMRP_E_CUDA;
   for (int64_t j = 0; j < n_freq; ++j) {
     const double w = double(j + 1) * (w_max / double(n_freq));

@@ -123,9 +123,12 @@ cudaError_t set_sort_attributes();
 void launch_init_step(StepState* st, cudaStream_t s);
 
 // Spectrum sums: Qh[j] = dt sum_n (q_n - q_0) e^{-i w_j t_n},
-// Uh[j] = sum_n kw_n u_n e^{-i w_j t_n}, w_j = (j+1) w_max / nf; out [nf][4].
+// Uh[j] = sum_n kw_n u_n e^{-i w_j t_n}, w_j = (j+1) w_max / nf. work:
+// dft_work_doubles(ns, nf) doubles, of which the first [nf][4] receive the sums
+// (Q re, im, U re, im) and the rest is scratch.
+int64_t dft_work_doubles(int64_t ns, int64_t nf);
 void launch_dft(const double* q, const double* u, int64_t ns, double dt, double first_kick,
-                int64_t nf, double w_max, double* out, cudaStream_t s);
+                int64_t nf, double w_max, double* work, cudaStream_t s);
 
 // ---- per-degree kernels (imrp_inst_*.cu) ------------------------------------
 // SMs of the current device (cached per device; contexts may be created from
