@@ -69,7 +69,10 @@ struct imrp_ctx {
   bool loaded = false, keys_valid = false;
   int nc = 0;
   int64_t ntiles = 0, ngroups = 0;
-  int wpb = 8;
+  int wpb = 8;                 // warps per CTA of the field kernel for the loaded n
+  int wpb_full = 8;            // its choice when the tiles fill the GPU several times
+  int resident[4] = {0};       // resident warps per SM at kFieldWpb[k] warps per CTA
+  bool tuned = false;          // wpb was chosen by the autotuner
   int gseg = 32;  // least groups per segment of the group scan
   // streams / graphs
   cudaStream_t own_stream = nullptr, stream = nullptr;
@@ -154,6 +157,36 @@ double n_tilde_of(const imrp_ctx* c, int64_t n) {
 // Ion super-particles of the immobile uniform background after a load of n.
 double n_ion_of(const imrp_ctx* c, int64_t n) { return c->species ? c->sp_bg : double(n); }
 
+// Warps per CTA of the field kernel for ntiles tiles. When all tiles fit on the
+// GPU at once, the shape that gives the fullest SM the fewest tiles: FP64
+// N = 20000, l_max = 8 takes 0.130 ms with one tile per CTA and 0.183 with 8
+// (79 CTAs on 152 SMs); FP32 N = 1e5, l_max = 16 0.045 with one and 0.050 with
+// 4 (782 CTAs in 760 places). Beyond that the larger CTAs are faster (create).
+constexpr int kFieldWpb[4] = {8, 4, 2, 1};
+int field_wpb(const imrp_ctx* c, int64_t ntiles) {
+  const int64_t sms = sm_count();
+  int best = c->wpb_full;
+  int64_t load = INT64_MAX;
+  for (int q = 0; q < 4; ++q) {
+    const int64_t w = kFieldWpb[q], ctas = (ntiles + w - 1) / w, per = (ctas + sms - 1) / sms * w;
+    if (per <= c->resident[q] && per < load) {
+      best = int(w);
+      load = per;
+    }
+  }
+  return best;
+}
+
+// What depends on the number of particles of a load or restore.
+void set_count(imrp_ctx* c, int64_t n) {
+  c->n = n;
+  c->n_tilde = n_tilde_of(c, n);
+  c->n_ion = n_ion_of(c, n);
+  c->ntiles = (n + 31) / 32;
+  c->ngroups = (c->ntiles + kTilesPerGroup - 1) / kTilesPerGroup;
+  if (!c->tuned) c->wpb = field_wpb(c, c->ntiles);
+}
+
 void free_all(imrp_ctx* c) {
   drop_graphs(c);
   cudaFree(c->state);
@@ -235,6 +268,7 @@ template <class T> MomArgs<T> make_mom_args(imrp_ctx* ctx) {
   ma.rho = T(ctx->r_out);
   ma.rho_inv = T(1.0 / ctx->r_out);
   ma.agg = static_cast<T*>(ctx->agg);
+  ma.parts = mom_parts(sizeof(T), ctx->L, ctx->n, mom_ppt(sizeof(T), ctx->n));
   ma.species = ctx->species;
   ma.n_e = uint32_t(std::min<int64_t>(ctx->sp_ne, int64_t(UINT32_MAX)));
   ma.q_ion = T(ctx->sp_q);
@@ -561,17 +595,17 @@ int imrp_create(const imrp_params* p, imrp_ctx** out) {
   // l_max = 16: 4 warps (20 resident) beat 2 warps (22 resident) by 27%;
   // at l_max = 24: 2 warps (10 resident) beat 4 warps (8 resident) by 9%.
   {
-    int nbw[4] = {0, 0, 0, 0}, best = 0;
-    const int ws[4] = {8, 4, 2, 1};
+    int best = 0;
     for (int q = 0; q < 4; ++q) {
-      const int nb = ctx->prec == 1 ? find_set<float>(ctx->L)->field_blocks_per_sm(ws[q])
-                                    : find_set<double>(ctx->L)->field_blocks_per_sm(ws[q]);
-      nbw[q] = nb * ws[q];
-      best = std::max(best, nbw[q]);
+      const int nb = ctx->prec == 1 ? find_set<float>(ctx->L)->field_blocks_per_sm(kFieldWpb[q])
+                                    : find_set<double>(ctx->L)->field_blocks_per_sm(kFieldWpb[q]);
+      ctx->resident[q] = nb * kFieldWpb[q];
+      best = std::max(best, ctx->resident[q]);
     }
     ctx->wpb = 0;
     for (int q = 0; q < 4 && !ctx->wpb; ++q)
-      if (nbw[q] > 0 && 100 * nbw[q] >= 85 * best) ctx->wpb = ws[q];
+      if (ctx->resident[q] > 0 && 100 * ctx->resident[q] >= 85 * best) ctx->wpb = kFieldWpb[q];
+    ctx->wpb_full = ctx->wpb;
   }
   if (ctx->wpb < 1) { free_all(ctx); delete ctx; return IMRP_E_INVAL; }
   rc = alloc_ctx(ctx);
@@ -704,11 +738,7 @@ int imrp_load_particles(imrp_ctx* ctx, const double* x, const double* v, int64_t
   const bool same_n = ctx->loaded && ctx->n == n && ctx->hist_first == 0;
   int rc = check_err(ctx);
   if (rc) { ctx->loaded = false; return rc; }
-  ctx->n = n;
-  ctx->n_tilde = n_tilde_of(ctx, n);
-  ctx->n_ion = n_ion_of(ctx, n);
-  ctx->ntiles = (n + 31) / 32;
-  ctx->ngroups = (ctx->ntiles + kTilesPerGroup - 1) / kTilesPerGroup;
+  set_count(ctx, n);
   ctx->host_step = 0;
   ctx->hist_first = 0;
   ctx->loaded = true;
@@ -789,11 +819,7 @@ int imrp_load_particles_async(imrp_ctx* ctx, const double* x, const double* v, i
   CK(cudaGetLastError());
   const bool same_n = ctx->loaded && ctx->n == n && ctx->hist_first == 0;
   ctx->cur = 0;
-  ctx->n = n;
-  ctx->n_tilde = n_tilde_of(ctx, n);
-  ctx->n_ion = n_ion_of(ctx, n);
-  ctx->ntiles = (n + 31) / 32;
-  ctx->ngroups = (ctx->ntiles + kTilesPerGroup - 1) / kTilesPerGroup;
+  set_count(ctx, n);
   ctx->host_step = 0;
   ctx->hist_first = 0;
   ctx->loaded = true;
@@ -923,11 +949,7 @@ int imrp_restore(imrp_ctx* ctx, const double* x, const double* v, const uint32_t
   CK(cudaMemcpyAsync(ctx->st, &s0, sizeof(s0), cudaMemcpyHostToDevice, ctx->stream));
   int rc = check_err(ctx);
   if (rc) { ctx->loaded = false; return rc; }
-  ctx->n = n;
-  ctx->n_tilde = n_tilde_of(ctx, n);
-  ctx->n_ion = n_ion_of(ctx, n);
-  ctx->ntiles = (n + 31) / 32;
-  ctx->ngroups = (ctx->ntiles + kTilesPerGroup - 1) / kTilesPerGroup;
+  set_count(ctx, n);
   ctx->host_step = step;
   ctx->hist_first = step;
   ctx->loaded = true;
@@ -1041,6 +1063,7 @@ extern "C" int imrp_autotune(imrp_ctx* ctx, int* wpb_out, int* gseg_out) {
       if (ms < best) { best = ms; best_w = w; }
     }
     ctx->wpb = best_w;
+    ctx->tuned = true;
   }
   // group scan: least groups per segment
   {
@@ -1068,7 +1091,7 @@ struct BatchGroup {
   std::vector<int> members;     // indices into the batch's contexts
   void* dmom = nullptr;         // MomArgs<T>[members]
   void* dfield = nullptr;       // FieldArgs<T>[members] (push mode)
-  int2* dmom_items = nullptr;   // (member, block): first the members of mom_ppt 16, then of 4
+  int2* dmom_items = nullptr;   // (member, item): first the members of mom_ppt 16, then of 4
   int2* dfield_items = nullptr; // (member, first tile of a CTA)
   int nmom = 0, nmom_small = 0, nfield = 0;
 };
@@ -1143,8 +1166,8 @@ template <class T> int fill_group(imrp_batch* b, BatchGroup& g) {
     fa.push_back(make_field_args<T>(ctx, true));
     // the moments' blocks as the context's own launch takes them (bit-identical sums)
     const int ppt = mom_ppt(sizeof(T), ctx->n);
-    const int64_t mblocks = mom_blocks(ctx->n, ppt);
-    for (int64_t q = 0; q < mblocks; ++q) (ppt == 16 ? mi : ms).push_back(make_int2(int(k), int(q)));
+    const int64_t mitems = mom_blocks(ctx->n, ppt) * ma.back().parts;
+    for (int64_t q = 0; q < mitems; ++q) (ppt == 16 ? mi : ms).push_back(make_int2(int(k), int(q)));
     for (int64_t t = 0; t < ctx->ntiles; t += g.wpb) fi.push_back(make_int2(int(k), int(t)));
   }
   g.nmom_small = int(ms.size());

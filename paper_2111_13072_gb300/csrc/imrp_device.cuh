@@ -281,6 +281,7 @@ template <class T> struct MomArgs {
   T rho;       // r_out
   T rho_inv;   // 1 / r_out: regular harmonics use x / r_out so |Rs| <= 1
   T* agg;      // [2 ncomp(L)][ntiles] tile sums, u = 2 e + s (s = 0 Rs, s = 1 Is)
+  int parts;   // column ranges per block (mom_parts)
   // mobile ions (species = 1): particles with id >= n_e have charge q_ion,
   // the others -1; qtile[tile] receives each tile's charge (FP64)
   int species;

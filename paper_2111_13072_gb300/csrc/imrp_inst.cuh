@@ -106,7 +106,7 @@ const PrologueInit g_prologue_init;
 template <class T, int L> void mom_launch(const MomArgs<T>& a, cudaStream_t s) {
   if (a.n <= 0) return;
   const int ppt = mom_ppt(sizeof(T), a.n);
-  const unsigned blocks = unsigned(mom_blocks(a.n, ppt));
+  const unsigned blocks = unsigned(mom_blocks(a.n, ppt) * a.parts);
   if (ppt == kMomPPT)
     k_moments<T, L, kMomPPT><<<blocks, kMomThreads, moments_smem<T, L, kMomPPT>(), s>>>(a);
   else

@@ -146,18 +146,29 @@ inline int sm_count() {
   return c;
 }
 // Particles per thread of the moments kernel for an instance of n particles:
-// 16 (1024 per CTA of 64 threads), or 4 (256 per CTA) for an FP64 instance
-// that would give fewer than two CTAs per SM. FP64 runs at a small fraction
-// of the FP32 rate here, so a small FP64 instance gains from four times the
-// SMs (N = 2e4, l_max = 8: 0.292 -> 0.103 ms); in FP32 the wider reduction
-// over each tile's threads costs more than the SMs bring (N = 1e5, l_max =
-// 16: 0.045 -> 0.068 ms), so FP32 keeps 16.
-inline int mom_ppt(int elem_size, int64_t n) {
-  return (elem_size == 8 && (n + 1023) / 1024 < 2 * sm_count()) ? 4 : 16;
-}
-// CTAs of the moments kernel (64 threads of ppt particles): whole scan groups
-// of 1024 particles, so that every tile the scans read is written
+// 16 (1024 per CTA of 64 threads), or 4 (256 per CTA) for an FP64 instance of
+// fewer than 100 such blocks, whose columns alone (below) would not fill the
+// GPU: FP64 N = 60000, l_max = 12 takes 0.184 ms with 4 and 0.219 with 16;
+// N = 250001, l_max = 16 (245 blocks) 1.19 and 0.96, since with 4 each tile's
+// sums go through a butterfly over 8 threads. FP32 keeps 16 (N = 1e5,
+// l_max = 16: 0.045 -> 0.068 ms with 4).
+inline int mom_ppt(int elem_size, int64_t n) { return (elem_size == 8 && (n + 1023) / 1024 < 100) ? 4 : 16; }
+// CTAs of the moments kernel per column range (64 threads of ppt particles):
+// whole scan groups of 1024 particles, so that every tile the scans read is written
 inline int64_t mom_blocks(int64_t n, int ppt) { return (n + 1023) / 1024 * (16 / ppt); }
+// Column ranges per block of the moments kernel: a small instance has too few
+// blocks for the SMs (N = 1e5: 98 CTAs of two warps), so its columns m are cut
+// into ranges that separate CTAs take (a range first walks its particles'
+// diagonal terms up to its first column). As many ranges as give the stated
+// CTAs per SM: FP32 N = 1e5, l_max = 16: 0.043 ms with one range, 0.0225 with
+// 6 per SM, 0.028 with 8; N = 3e5, l_max = 8: 0.0262, 0.0206, 0.0267; FP64
+// N = 20000, l_max = 8: 0.102 with one, 0.046 with 7 ranges, 0.051 with 9.
+inline int mom_parts(int elem_size, int L, int64_t n, int ppt) {
+  const int per_sm = elem_size == 4 ? 6 : ppt == 4 ? 5 : 8;
+  const int64_t want = int64_t(per_sm) * sm_count() / mom_blocks(n, ppt);
+  const int most = elem_size == 4 ? L + 1 : 3 * (L + 1) / 4;
+  return int(want < 1 ? 1 : want > most ? most : want);
+}
 
 template <class T> struct KernelSet {
   int L;
@@ -168,8 +179,8 @@ template <class T> struct KernelSet {
   int (*field_blocks_per_sm)(int wpb);  // occupancy of the field kernel at wpb warps per CTA
   // Batched launches over several instances of this degree and precision:
   // args[i] in device memory, items[b] = (instance, block) for the moments
-  // (blocks of 64 ppt particles, ppt = mom_ppt of every listed instance) and
-  // (instance, first tile) for the field (CTAs of wpb tiles).
+  // (item = block parts + column range, ppt = mom_ppt of every listed
+  // instance) and (instance, first tile) for the field (CTAs of wpb tiles).
   void (*moments_batch)(const MomArgs<T>* args, const int2* items, int nitems, int ppt, cudaStream_t);
   void (*field_batch)(const FieldArgs<T>* args, const int2* items, int nitems, int wpb, cudaStream_t);
 };

@@ -77,14 +77,15 @@ template <> __device__ __forceinline__ double fma_t<double>(double x, double y, 
 //   Is_l^m(x) = Rs_l^m(x / r_out) * r_out^l / r^(2l+1),
 // the scale advancing by one factor r_out / r^2 per degree. A CTA of 64
 // threads takes 64 PPT particles (2 PPT tiles), PPT particles per thread,
-// 32 / PPT threads per tile.
+// 32 / PPT threads per tile, and all columns or (small instances, mom_parts)
+// one of several ranges of them.
 // At the end of a column the threads of each tile are combined: with two
 // (PPT = 16), one shuffle per Rs/Is pair (the even lane keeps the Rs sum, the
 // odd lane the Is sum); with more, a butterfly over the tile's threads, each
 // then writing its share. Written: agg[u][tile], u = 2 e + s (s = 0 Rs, s = 1 Is).
 constexpr int kMomThreads = 64;
 constexpr int kMomPPT = 16;       // particles per thread (1024 per CTA) when that fills the GPU
-constexpr int kMomPPTSmall = 4;   // particles per thread (256 per CTA) when it would leave SMs idle
+constexpr int kMomPPTSmall = 4;   // particles per thread (256 per CTA) of small FP64 instances (mom_ppt)
 constexpr int kMomBreak = 2;      // steps between the column-end tests
 // particles advanced together (independent recurrence chains): four in FP32
 // (N = 2e6, l_max = 16: 0.174 -> 0.168 ms against two; l_max = 24, N = 4e6:
@@ -98,10 +99,22 @@ __host__ __device__ constexpr size_t moments_smem() {
   return sizeof(T) * 7 * PPT * (kMomThreads + 1);
 }
 
-// Body of the moments kernel for CTA `blk` of the instance whose arguments are
-// `a` (a kernel parameter, or a copy in shared memory for the batched launch).
+// First column of part p when the columns m = 0..L are cut into `parts`
+// contiguous ranges of about equal work (a column's entries and its fixed cost,
+// about two entries' worth).
+__device__ __forceinline__ int mom_part_begin(int L, int parts, int p) {
+  const int total = (L + 1) * (L + 2) / 2 + 2 * (L + 1);
+  const int want = total * p / parts;
+  int m = 0, acc = 0;
+  while (m <= L && acc < want) acc += L - m++ + 3;
+  return m;
+}
+
+// Body of the moments kernel for item `item` (block item / parts of the
+// instance, column range item % parts) of the instance whose arguments are `a`
+// (a kernel parameter, or a copy in shared memory for the batched launch).
 template <class T, int L, int PPT>
-__device__ __forceinline__ void moments_block(const MomArgs<T>& a, int64_t blk, unsigned char* smem_raw) {
+__device__ __forceinline__ void moments_block(const MomArgs<T>& a, int64_t item, unsigned char* smem_raw) {
   constexpr int NT = kMomThreads;  // threads of the CTA
   constexpr int TPT = 32 / PPT;    // threads per tile
   constexpr int S = NT + 1;       // padded row
@@ -115,6 +128,10 @@ __device__ __forceinline__ void moments_block(const MomArgs<T>& a, int64_t blk, 
   const Tables<T>& tb = tab<T>();
   const int th = threadIdx.x;
   const int64_t ntiles = (a.n + 31) >> 5;
+  const int64_t blk = a.parts == 1 ? item : item / a.parts;
+  const int part = int(item - blk * a.parts);
+  const int mlo = part == 0 ? 0 : mom_part_begin(L, a.parts, part);
+  const int mhi = part == a.parts - 1 ? L + 1 : mom_part_begin(L, a.parts, part + 1);
   const int64_t pbase = blk * (NT * PPT);
   const T ri = a.rho_inv;
   constexpr int kMomChains = mom_chains<T, L>() < PPT ? mom_chains<T, L>() : PPT;
@@ -131,15 +148,21 @@ __device__ __forceinline__ void moments_block(const MomArgs<T>& a, int64_t blk, 
     sq[o] = a.rho / r2;
     // the particle's charge seeds its harmonics: -1 for an electron, q_ion
     // for a mobile ion
-    sRr[o] = valid ? ((a.species && a.id[j] >= a.n_e) ? a.q_ion : T(-1)) : T(0);
-    sRi[o] = T(0);
-    ssc[o] = rsqrt_t(r2);
+    T Dr = valid ? ((a.species && a.id[j] >= a.n_e) ? a.q_ion : T(-1)) : T(0), Di = T(0), sc = rsqrt_t(r2);
+    for (int m = 1; m < mlo; ++m) {  // the diagonal up to the column before this part's first
+      const T cx = tb.dg[m] * (X * ri), cy = tb.dg[m] * (Y * ri);
+      const T nr = cx * Dr - cy * Di, ni = cx * Di + cy * Dr;
+      Dr = nr; Di = ni; sc *= a.rho / r2;
+    }
+    sRr[o] = Dr;
+    sRi[o] = Di;
+    ssc[o] = sc;
   }
   __syncthreads();
   const int sub = th % TPT;  // this thread's part of its tile
   const bool odd = (th & 1) != 0;
   const int64_t tile = blk * (NT * PPT / 32) + th / TPT;
-  if (a.species) {
+  if (a.species && part == 0) {
     // the tile's charge (FP64): this thread's particles, then the tile's threads
     double qs = 0.0;
 #pragma unroll
@@ -154,7 +177,7 @@ __device__ __forceinline__ void moments_block(const MomArgs<T>& a, int64_t blk, 
   T* const agg_t = a.agg + tile + (odd ? ts : 0);  // row u = 2 e + odd
 
 #pragma unroll 1
-  for (int m = 0; m <= L; ++m) {
+  for (int m = mlo; m < mhi; ++m) {
     T acc[4 * (L + 1)];  // [j][R re, I re, R im, I im], l = m + j
 #pragma unroll
     for (int k = 0; k < 4 * (L + 1); ++k) acc[k] = T(0);
@@ -271,7 +294,7 @@ __global__ void __launch_bounds__(kMomThreads) k_moments(MomArgs<T> a) {
   moments_block<T, L, PPT>(a, blockIdx.x, smem_raw);
 }
 
-// Batched moments: CTA b takes block items[b].y (of 64 PPT particles) of
+// Batched moments: CTA b takes item items[b].y (block and column range) of
 // instance items[b].x, whose arguments args[items[b].x] are first copied to
 // shared memory.
 template <class T> __device__ __forceinline__ void copy_args(const T* src, T* dst) {

@@ -164,6 +164,7 @@ int run(const imrp_params* p, const double* x, int64_t n, int64_t step, double* 
   ma.rho = T(r_out);
   ma.rho_inv = T(1.0 / r_out);
   ma.agg = static_cast<T*>(P(o.agg));
+  ma.parts = mom_parts(sizeof(T), L, n, mom_ppt(sizeof(T), n));
   ks->moments(ma, s);
   launch_tile_scan<T>(static_cast<T*>(P(o.agg)), static_cast<T*>(P(o.pfx)), static_cast<double*>(P(o.gagg)),
                       ntiles, nc, s);
@@ -227,9 +228,7 @@ int run(const imrp_params* p, const double* x, int64_t n, int64_t step, double* 
     rl *= r_out;
     a.cdrive[l] = canti[l] * 4.0 * kPi * n_tilde;
   }
-  const size_t spw = ks->smem_per_warp;
-  const int wpb = int(spw * 8 <= 227 * 1024 ? 8 : (227 * 1024) / spw);
-  ks->field(a, wpb, s);
+  ks->field(a, 1, s);  // at most 512 tiles: one per CTA spreads them over the SMs
   const T* eo = static_cast<const T*>(P(o.eout));
   const T* cs[3] = {eo, eo + n, eo + 2 * n};
   launch_scatter_by_id<T>(cs, 3, id1, E, n, s);
