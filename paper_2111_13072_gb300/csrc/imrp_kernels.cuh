@@ -110,6 +110,15 @@ __device__ __forceinline__ int mom_part_begin(int L, int parts, int p) {
   return m;
 }
 
+// Diagonal step of the regular harmonics: Rs_m^m = (cx + i cy) Rs_{m-1}^{m-1}. The
+// roundings are written out, so that a column range that starts past m = 0 and
+// one that walks there have the same diagonal bit for bit.
+template <class T> __device__ __forceinline__ void diag_step(T cx, T cy, T& Dr, T& Di) {
+  const T nr = fma_t(cx, Dr, -(cy * Di)), ni = fma_t(cy, Dr, cx * Di);
+  Dr = nr;
+  Di = ni;
+}
+
 // Body of the moments kernel for item `item` (block item / parts of the
 // instance, column range item % parts) of the instance whose arguments are `a`
 // (a kernel parameter, or a copy in shared memory for the batched launch).
@@ -150,9 +159,8 @@ __device__ __forceinline__ void moments_block(const MomArgs<T>& a, int64_t item,
     // for a mobile ion
     T Dr = valid ? ((a.species && a.id[j] >= a.n_e) ? a.q_ion : T(-1)) : T(0), Di = T(0), sc = rsqrt_t(r2);
     for (int m = 1; m < mlo; ++m) {  // the diagonal up to the column before this part's first
-      const T cx = tb.dg[m] * (X * ri), cy = tb.dg[m] * (Y * ri);
-      const T nr = cx * Dr - cy * Di, ni = cx * Di + cy * Dr;
-      Dr = nr; Di = ni; sc *= a.rho / r2;
+      diag_step(tb.dg[m] * (X * ri), tb.dg[m] * (Y * ri), Dr, Di);
+      sc *= a.rho / r2;
     }
     sRr[o] = Dr;
     sRi[o] = Di;
@@ -198,10 +206,9 @@ __device__ __forceinline__ void moments_block(const MomArgs<T>& a, int64_t item,
         Zs[u] = sz[o]; q[u] = sq[o];
         Dr[u] = sRr[o]; Di[u] = sRi[o]; sc[u] = ssc[o];
         if (m > 0) {  // diagonal step: Rs_m^m = dg_m (x + i y) / r_out * Rs_{m-1}^{m-1}
-          const T cx = dg * Xs, cy = dg * Ys;
-          const T nr = cx * Dr[u] - cy * Di[u], ni = cx * Di[u] + cy * Dr[u];
-          Dr[u] = nr; Di[u] = ni; sc[u] *= q[u];
-          sRr[o] = nr; sRi[o] = ni; ssc[o] = sc[u];
+          diag_step(dg * Xs, dg * Ys, Dr[u], Di[u]);
+          sc[u] *= q[u];
+          sRr[o] = Dr[u]; sRi[o] = Di[u]; ssc[o] = sc[u];
         }
         rs2[u] = Xs * Xs + Ys * Ys + Zs[u] * Zs[u];
         P1[u] = T(1); P0[u] = T(0);
