@@ -49,9 +49,16 @@ def sort_launches(n):
 
 
 def step_launches(n):
-    """Kernel launches of one step of one instance: sort, reorder, moments, tile
-    scan, two group-scan kernels, finalize, field."""
+    """Kernel stages of one step of one instance: sort, reorder, moments, tile
+    scan, two group-scan passes, finalize, field."""
     return sort_launches(n) + 7
+
+
+def fused_stages(n):
+    """Stages that ride in another stage's launch: the finalize in the first
+    group-scan kernel, and up to 32 scan groups of 1024 particles the second
+    group-scan pass too."""
+    return 2 if n <= 32 * 1024 else 1
 
 
 def workload_desc(w):
@@ -303,9 +310,9 @@ def ensemble_measure(steps, warmup, autotune=True, n_instances=64, stream=None):
     ntot = sum(w.N for w in ws)
     for s in sims:
         s.close()
-    # per context: sort, reorder, tile scan, two group-scan kernels, finalize;
-    # per degree and precision: one moments and one field launch
-    launches = sum(sort_launches(w.N) + 5 for w in ws) + 2 * len({(w.precision, w.l_max) for w in ws})
+    # per context: all stages but moments and field; per degree and precision:
+    # one moments and one field launch
+    launches = sum(step_launches(w.N) - 2 - fused_stages(w.N) for w in ws) + 2 * len({(w.precision, w.l_max) for w in ws})
     return {"value": ntot * steps / (ms / 1e3), "unit": UNIT, "instances": n_instances,
             "gpu_launches_per_step": launches,
             "particles": ntot, "steps": steps, "ms_per_step": ms / steps, "autotuned": autotune,
@@ -507,7 +514,7 @@ def sub_config(name, steps, warmup, nprof, peak_tflops, stream):
     out = {"workload": workload_desc(w), "value": w.N * steps / (ms / 1e3), "unit": UNIT, "steps": steps,
            "warmup": warmup, "ms_per_step": ms / steps, "dtype": "f32" if w.precision else "f64",
            "stage_ms_per_step": {k: v / nprof for k, v in stages.items()},
-           "gpu_launches": step_launches(w.N) * steps}
+           "gpu_launches": (step_launches(w.N) - fused_stages(w.N)) * steps}
     if w.precision:
         ach = field_flops_per_particle(w.l_max) * w.N / (field_ms / 1e3) / 1e12
         ach24 = 24.0 * K * w.N / (field_ms / 1e3) / 1e12
@@ -733,7 +740,7 @@ def main():
                            "l2": "inputs larger than L2 (per-step working set > 300 MB)",
                            "autotuned": {"warps_per_cta": tuned[0], "groups_per_segment": tuned[1]}},
                 "roofline": roofline, "cpu_baseline": cpu, "e2e": e2e,
-                "gpu_launches": step_launches(N) * args.steps, "clocks": clocks, "fp64_gpu": fp64,
+                "gpu_launches": (step_launches(N) - fused_stages(N)) * args.steps, "clocks": clocks, "fp64_gpu": fp64,
                 "oracle_err": oerr, "configs": subs, "serving": serving, "ensemble": ensemble,
                 "drude": drude}
         print(json.dumps(line), flush=True)

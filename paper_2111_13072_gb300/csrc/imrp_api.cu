@@ -71,7 +71,7 @@ struct imrp_ctx {
   int64_t ntiles = 0, ngroups = 0;
   int wpb = 8;                 // warps per CTA of the field kernel for the loaded n
   int wpb_full = 8;            // its choice when the tiles fill the GPU several times
-  int resident[4] = {0};       // resident warps per SM at kFieldWpb[k] warps per CTA
+  int resident[4] = {0};       // resident warps per SM at 8, 4, 2, 1 warps per CTA
   bool tuned = false;          // wpb was chosen by the autotuner
   int gseg = 32;  // least groups per segment of the group scan
   // streams / graphs
@@ -161,7 +161,7 @@ double n_ion_of(const imrp_ctx* c, int64_t n) { return c->species ? c->sp_bg : d
 // GPU at once, the shape that gives the fullest SM the fewest tiles: FP64
 // N = 20000, l_max = 8 takes 0.130 ms with one tile per CTA and 0.183 with 8
 // (79 CTAs on 152 SMs); FP32 N = 1e5, l_max = 16 0.045 with one and 0.050 with
-// 4 (782 CTAs in 760 places). Beyond that the larger CTAs are faster (create).
+// 4 (782 CTAs in 760 places). Beyond that the shape of create.
 constexpr int kFieldWpb[4] = {8, 4, 2, 1};
 int field_wpb(const imrp_ctx* c, int64_t ntiles) {
   const int64_t sms = sm_count();
@@ -335,35 +335,40 @@ template <class T> FieldArgs<T> make_field_args(imrp_ctx* ctx, bool record) {
   return a;
 }
 
+// Stage boundary k of a timed step: the event, and a full dependency after it.
+void stage_event(LaunchSeq& seq, cudaEvent_t* ev, int k) {
+  if (!ev) return;
+  cudaEventRecord(ev[k], seq.s);
+  seq.unchain();
+}
+
 // The stages of one step (or field evaluation) of a context: radius keys (if
 // stale), sort and reorder; then the moments; then the scans and finalize;
 // then the field. The batch runs the moments and the field of many contexts
 // as one launch each (per degree and precision) between the others.
-template <class T> void enqueue_pre(imrp_ctx* ctx, cudaEvent_t* ev = nullptr, bool shared_gpu = false) {
-  cudaStream_t s = ctx->stream;
+// seq: the launches on the context's stream so far; an event between two
+// stages (ev) breaks the chain.
+template <class T> void enqueue_pre(imrp_ctx* ctx, LaunchSeq& seq, cudaEvent_t* ev = nullptr, bool shared_gpu = false) {
   const int64_t n = ctx->n;
   Part<T>* st = state_of<T>(ctx);
   if (!ctx->keys_valid) {
-    launch_keys<T>(st, ctx->key0, ctx->idx0, n, ctx->r_out, s);
+    launch_keys<T>(st, ctx->key0, ctx->idx0, n, ctx->r_out, seq);
   }
-  if (ev) cudaEventRecord(ev[0], s);
+  stage_event(seq, ev, 0);
   const uint32_t* perm = launch_radix_sort(ctx->key0, ctx->idx0, ctx->key1, ctx->idx1, ctx->hist, n,
-                                           sort_first_byte(ctx->prec), s, shared_gpu);
-  if (ev) cudaEventRecord(ev[1], s);
-  launch_reorder<T>(st, sorted_ptrs<T>(ctx), ctx->srt_id, perm, n, s);
+                                           sort_first_byte(ctx->prec), seq, shared_gpu);
+  stage_event(seq, ev, 1);
+  launch_reorder<T>(st, sorted_ptrs<T>(ctx), ctx->srt_id, perm, n, seq);
 }
 
-template <class T> void enqueue_mid(imrp_ctx* ctx, bool record) {
-  cudaStream_t s = ctx->stream;
+template <class T> void enqueue_mid(imrp_ctx* ctx, LaunchSeq& seq, bool record) {
   if (ctx->species) {
     // the charge inside each particle's radius: a scan of the tiles' charges (FP64)
-    launch_tile_scan<double>(ctx->qtile, ctx->qpfx, ctx->qgagg, ctx->ntiles, 1, s);
+    launch_tile_scan<double>(ctx->qtile, ctx->qpfx, ctx->qgagg, ctx->ntiles, 1, seq);
     launch_group_scan<double>(ctx->qgagg, ctx->qwork, ctx->qticket, ctx->qgbase, ctx->qtot, ctx->qtotd,
-                              ctx->ngroups, 1, ctx->gseg, s);
+                              ctx->ngroups, 1, ctx->gseg, nullptr, seq);
   }
-  launch_tile_scan<T>(static_cast<T*>(ctx->agg), static_cast<T*>(ctx->pfx), ctx->gagg, ctx->ntiles, ctx->nc, s);
-  launch_group_scan<T>(ctx->gagg, ctx->gswork, ctx->gsticket, static_cast<T*>(ctx->gbase),
-                       static_cast<T*>(ctx->tot), ctx->totd, ctx->ngroups, ctx->nc, ctx->gseg, s);
+  launch_tile_scan<T>(static_cast<T*>(ctx->agg), static_cast<T*>(ctx->pfx), ctx->gagg, ctx->ntiles, ctx->nc, seq);
   FinalizeArgs fa;
   fa.st = ctx->st;
   fa.totd = ctx->totd;
@@ -380,29 +385,33 @@ template <class T> void enqueue_mid(imrp_ctx* ctx, bool record) {
   fa.t0 = ctx->t0;
   fa.dt = ctx->p.dt;
   for (int l = 0; l < kTabL; ++l) fa.canti[l] = ctx->canti[l];
-  launch_finalize(fa, s);
+  launch_group_scan<T>(ctx->gagg, ctx->gswork, ctx->gsticket, static_cast<T*>(ctx->gbase),
+                       static_cast<T*>(ctx->tot), ctx->totd, ctx->ngroups, ctx->nc, ctx->gseg, &fa, seq);
 }
 
 // Launches one step (record = 1) or the field evaluation without push (record = 0).
 // ev (optional): IMRP_N_STAGES + 1 events recorded at the stage boundaries.
-template <class T> int enqueue(imrp_ctx* ctx, bool record, cudaEvent_t* ev = nullptr) {
+template <class T> int enqueue(imrp_ctx* ctx, LaunchSeq& seq, bool record, cudaEvent_t* ev = nullptr) {
   const KernelSet<T>* ks = find_set<T>(ctx->L);
-  cudaStream_t s = ctx->stream;
-  enqueue_pre<T>(ctx, ev);
-  if (ev) cudaEventRecord(ev[2], s);
-  ks->moments(make_mom_args<T>(ctx), s);
-  if (ev) cudaEventRecord(ev[3], s);
-  enqueue_mid<T>(ctx, record);
-  if (ev) cudaEventRecord(ev[4], s);
-  ks->field(make_field_args<T>(ctx, record), ctx->wpb, s);
-  if (ev) cudaEventRecord(ev[5], s);
+  enqueue_pre<T>(ctx, seq, ev);
+  stage_event(seq, ev, 2);
+  ks->moments(make_mom_args<T>(ctx), seq);
+  stage_event(seq, ev, 3);
+  enqueue_mid<T>(ctx, seq, record);
+  stage_event(seq, ev, 4);
+  ks->field(make_field_args<T>(ctx, record), ctx->wpb, seq);
+  stage_event(seq, ev, 5);
   // the field kernel wrote fresh keys for the (now sorted) state in push mode
   ctx->keys_valid = record;
   return IMRP_OK;
 }
 
+int enqueue_any(imrp_ctx* ctx, LaunchSeq& seq, bool record, cudaEvent_t* ev = nullptr) {
+  return ctx->prec == 1 ? enqueue<float>(ctx, seq, record, ev) : enqueue<double>(ctx, seq, record, ev);
+}
 int enqueue_any(imrp_ctx* ctx, bool record, cudaEvent_t* ev = nullptr) {
-  return ctx->prec == 1 ? enqueue<float>(ctx, record, ev) : enqueue<double>(ctx, record, ev);
+  LaunchSeq seq(ctx->stream);
+  return enqueue_any(ctx, seq, record, ev);
 }
 
 // Captures `count` steps (1 or 2) of the current configuration into *out.
@@ -411,7 +420,8 @@ int capture_steps(imrp_ctx* ctx, int count, cudaGraphExec_t* out) {
   cudaGraph_t g = nullptr;
   CK(cudaStreamBeginCapture(ctx->stream, cudaStreamCaptureModeThreadLocal));
   int r = 0;
-  for (int k = 0; k < count && !r; ++k) r = enqueue_any(ctx, true);
+  LaunchSeq seq(ctx->stream);
+  for (int k = 0; k < count && !r; ++k) r = enqueue_any(ctx, seq, true);
   cudaError_t ec = cudaStreamEndCapture(ctx->stream, &g);
   if (r) { if (g) cudaGraphDestroy(g); return r; }
   if (ec != cudaSuccess) return ctx->fail(IMRP_E_CUDA, "graph capture: %s", cudaGetErrorString(ec));
@@ -466,7 +476,7 @@ size_t footprint_bytes(int64_t N, int L, int prec) {
   b += size_t(sort_hist_words(N)) * 4;              // histogram
   b += 2 * size_t(tile_stride(ntiles) * nc) * es;   // tile sums and in-group scans
   b += size_t(ngroups * nc) * (es + 8) + size_t(nc) * (es + 8);
-  b += size_t(gs_work_doubles(int(nc))) * 8 + size_t(gs_col_blocks(int(nc))) * 4;
+  b += size_t(gs_work_doubles(int(nc))) * 8 + size_t(gs_tickets(int(nc))) * 4;
   b += 3 * size_t(N) * es + 6 * size_t(N) * 8;      // field output, staging
   b += sizeof(StepState) + sizeof(int);
   return b;
@@ -493,8 +503,8 @@ int alloc_ctx(imrp_ctx* ctx) {
   CK(cudaMalloc(&ctx->gagg, ngroups * nc * sizeof(double)));
   CK(cudaMalloc(&ctx->totd, nc * sizeof(double)));
   CK(cudaMalloc(&ctx->gswork, gs_work_doubles(nc) * sizeof(double)));
-  CK(cudaMalloc(&ctx->gsticket, gs_col_blocks(nc) * sizeof(unsigned)));
-  CK(cudaMemset(ctx->gsticket, 0, gs_col_blocks(nc) * sizeof(unsigned)));
+  CK(cudaMalloc(&ctx->gsticket, gs_tickets(nc) * sizeof(unsigned)));
+  CK(cudaMemset(ctx->gsticket, 0, gs_tickets(nc) * sizeof(unsigned)));
   CK(cudaMalloc(&ctx->eout, 3 * N * es));
   CK(cudaMalloc(&ctx->stage, 6 * N * sizeof(double)));
   CK(cudaMalloc(&ctx->st, sizeof(StepState)));
@@ -588,12 +598,16 @@ int imrp_create(const imrp_params* p, imrp_ctx** out) {
                           : find_set<double>(ctx->L)->init(ctx->device);
   if (rc == 0 && set_sort_attributes() != cudaSuccess) rc = 1;
   if (rc != 0) { free_all(ctx); delete ctx; return IMRP_E_CUDA; }
-  // warps per CTA of the field kernel: the largest of 8, 4, 2, 1 whose
-  // resident warps per SM reach 85% of the best. Larger CTAs keep their warps
-  // at nearby points of the long unrolled body (fewer instruction-cache
-  // misses); more resident warps hide latency. Measured on GB300 at
-  // l_max = 16: 4 warps (20 resident) beat 2 warps (22 resident) by 27%;
-  // at l_max = 24: 2 warps (10 resident) beat 4 warps (8 resident) by 9%.
+  // warps per CTA of the field kernel with many tiles: the largest of 4, 2, 1
+  // (FP64: 2, 1) whose resident warps per SM reach 85% of the best. In FP32
+  // larger CTAs keep their warps at nearby points of the long unrolled body
+  // (fewer instruction-cache misses), more resident warps hide latency:
+  // l_max = 16, N = 2e6: 4 warps (20 resident) beat 2 warps (22 resident) by
+  // 27%; l_max = 24: 2 warps (10 resident) beat 4 warps (8 resident) by 9%; 8
+  // warps lose to 4 everywhere (l_max = 12, N = 7e5: 0.173 against 0.158 ms).
+  // FP64 is bound by its pipe and loses only the uneven ends of large CTAs
+  // (l_max = 16, N = 250001: 2 / 4 / 8 warps 2.49 / 2.54 / 2.68 ms; l_max = 8,
+  // N = 40000: 0.267 / 0.309 / 0.352).
   {
     int best = 0;
     for (int q = 0; q < 4; ++q) {
@@ -603,7 +617,7 @@ int imrp_create(const imrp_params* p, imrp_ctx** out) {
       best = std::max(best, ctx->resident[q]);
     }
     ctx->wpb = 0;
-    for (int q = 0; q < 4 && !ctx->wpb; ++q)
+    for (int q = ctx->prec == 1 ? 1 : 2; q < 4 && !ctx->wpb; ++q)
       if (ctx->resident[q] > 0 && 100 * ctx->resident[q] >= 85 * best) ctx->wpb = kFieldWpb[q];
     ctx->wpb_full = ctx->wpb;
   }
@@ -659,8 +673,8 @@ int imrp_set_species(imrp_ctx* ctx, int64_t n_electrons, double ion_charge, doub
       CK(cudaMalloc(&ctx->qtot, sizeof(double)));
       CK(cudaMalloc(&ctx->qtotd, sizeof(double)));
       CK(cudaMalloc(&ctx->qwork, gs_work_doubles(1) * sizeof(double)));
-      CK(cudaMalloc(&ctx->qticket, gs_col_blocks(1) * sizeof(unsigned)));
-      CK(cudaMemset(ctx->qticket, 0, gs_col_blocks(1) * sizeof(unsigned)));
+      CK(cudaMalloc(&ctx->qticket, gs_tickets(1) * sizeof(unsigned)));
+      CK(cudaMemset(ctx->qticket, 0, gs_tickets(1) * sizeof(unsigned)));
     }
     ctx->species = 1;
     ctx->sp_ne = n_electrons;
@@ -853,18 +867,19 @@ int imrp_step(imrp_ctx* ctx, int64_t n_steps, double* qdiff_out, double* uasy_ou
 int imrp_get_field(imrp_ctx* ctx, double* E) {
   if (!ctx || !E) return IMRP_E_INVAL;
   if (!ctx->loaded) return ctx->fail(IMRP_E_STATE, "get_field before load");
-  int rc = enqueue_any(ctx, false);
+  LaunchSeq seq(ctx->stream);
+  int rc = enqueue_any(ctx, seq, false);
   if (rc) return rc;
   CK(cudaGetLastError());
   const int64_t n = ctx->n;
   if (ctx->prec == 1) {
     const float* e = static_cast<const float*>(ctx->eout);
     const float* cs[3] = {e, e + n, e + 2 * n};
-    launch_scatter_by_id<float>(cs, 3, ctx->srt_id, ctx->stage, n, ctx->stream);
+    launch_scatter_by_id<float>(cs, 3, ctx->srt_id, ctx->stage, n, seq);
   } else {
     const double* e = static_cast<const double*>(ctx->eout);
     const double* cs[3] = {e, e + n, e + 2 * n};
-    launch_scatter_by_id<double>(cs, 3, ctx->srt_id, ctx->stage, n, ctx->stream);
+    launch_scatter_by_id<double>(cs, 3, ctx->srt_id, ctx->stage, n, seq);
   }
   CK(cudaMemcpyAsync(E, ctx->stage, 3 * n * sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));
   return check_err(ctx);
@@ -1015,8 +1030,9 @@ namespace {
 // Radius keys for the current storage order (no step is taken).
 int ensure_keys(imrp_ctx* ctx) {
   if (ctx->keys_valid) return IMRP_OK;
-  if (ctx->prec == 1) launch_keys<float>(state_of<float>(ctx), ctx->key0, ctx->idx0, ctx->n, ctx->r_out, ctx->stream);
-  else launch_keys<double>(state_of<double>(ctx), ctx->key0, ctx->idx0, ctx->n, ctx->r_out, ctx->stream);
+  LaunchSeq seq(ctx->stream);
+  if (ctx->prec == 1) launch_keys<float>(state_of<float>(ctx), ctx->key0, ctx->idx0, ctx->n, ctx->r_out, seq);
+  else launch_keys<double>(state_of<double>(ctx), ctx->key0, ctx->idx0, ctx->n, ctx->r_out, seq);
   CK(cudaGetLastError());
   ctx->keys_valid = true;
   return IMRP_OK;
@@ -1199,7 +1215,7 @@ int build_groups(imrp_batch* b) {
       g = &b->groups.back();
       g->prec = ctx->prec;
       g->L = ctx->L;
-      g->wpb = ctx->wpb;  // the launch shape of the group's first context, unless tuned
+      g->wpb = ctx->tuned ? ctx->wpb : ctx->wpb_full;  // of the group's first context, unless tuned
       for (const int3& t : b->tuned)
         if (t.x == g->prec && t.y == g->L) g->wpb = t.z;
     }
@@ -1221,8 +1237,9 @@ int enqueue_batch_step(imrp_batch* b) {
   for (int i = 0; i < n; ++i) {
     imrp_ctx* ctx = b->c[i];
     cudaStreamWaitEvent(ctx->stream, b->fork, 0);
-    if (ctx->prec == 1) enqueue_pre<float>(ctx, nullptr, true);
-    else enqueue_pre<double>(ctx, nullptr, true);
+    LaunchSeq seq(ctx->stream);
+    if (ctx->prec == 1) enqueue_pre<float>(ctx, seq, nullptr, true);
+    else enqueue_pre<double>(ctx, seq, nullptr, true);
     cudaEventRecord(b->join[i], ctx->stream);
     cudaStreamWaitEvent(b->stream, b->join[i], 0);
   }
@@ -1244,8 +1261,9 @@ int enqueue_batch_step(imrp_batch* b) {
   for (int i = 0; i < n; ++i) {
     imrp_ctx* ctx = b->c[i];
     cudaStreamWaitEvent(ctx->stream, b->fork, 0);
-    if (ctx->prec == 1) enqueue_mid<float>(ctx, true);
-    else enqueue_mid<double>(ctx, true);
+    LaunchSeq seq(ctx->stream);
+    if (ctx->prec == 1) enqueue_mid<float>(ctx, seq, true);
+    else enqueue_mid<double>(ctx, seq, true);
     cudaEventRecord(b->join[i], ctx->stream);
     cudaStreamWaitEvent(b->stream, b->join[i], 0);
   }
@@ -1419,14 +1437,15 @@ extern "C" int imrp_batch_autotune(imrp_batch* b) {
   for (imrp_ctx* ctx : b->c) {
     int rc = ensure_keys(ctx);
     if (rc) return batch_fail(b, ctx, rc);
+    LaunchSeq seq(ctx->stream);
     if (ctx->prec == 1) {
-      enqueue_pre<float>(ctx);
-      find_set<float>(ctx->L)->moments(make_mom_args<float>(ctx), ctx->stream);
-      enqueue_mid<float>(ctx, false);
+      enqueue_pre<float>(ctx, seq);
+      find_set<float>(ctx->L)->moments(make_mom_args<float>(ctx), seq);
+      enqueue_mid<float>(ctx, seq, false);
     } else {
-      enqueue_pre<double>(ctx);
-      find_set<double>(ctx->L)->moments(make_mom_args<double>(ctx), ctx->stream);
-      enqueue_mid<double>(ctx, false);
+      enqueue_pre<double>(ctx, seq);
+      find_set<double>(ctx->L)->moments(make_mom_args<double>(ctx), seq);
+      enqueue_mid<double>(ctx, seq, false);
     }
     ctx->keys_valid = false;
     if (cudaStreamSynchronize(ctx->stream) != cudaSuccess) return batch_fail(b, ctx, IMRP_E_CUDA);

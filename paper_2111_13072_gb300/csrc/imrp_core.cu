@@ -21,6 +21,7 @@ template <int ND>
 __global__ void __launch_bounds__(kSortThreads) k_sort_hist(const uint32_t* __restrict__ keys,
                                                            int64_t n, int shift, int64_t nblk,
                                                            uint32_t* __restrict__ hist) {
+  chain_wait();
   __shared__ uint32_t h[ND];
   for (int d = threadIdx.x; d < ND; d += kSortThreads) h[d] = 0;
   __syncthreads();
@@ -79,6 +80,7 @@ __device__ __forceinline__ uint32_t block_excl_scan(uint32_t v, uint32_t* wsum, 
 // goes to rowtot[d]. One CTA per digit.
 __global__ void __launch_bounds__(kSortThreads) k_sort_rowscan(uint32_t* __restrict__ hist, int64_t nblk,
                                                               uint32_t* __restrict__ rowtot) {
+  chain_wait();
   constexpr int R = 8;  // consecutive entries per thread, loaded together
   __shared__ uint32_t wsum[kSortThreads / 32];
   uint32_t* row = hist + int64_t(blockIdx.x) * nblk;
@@ -136,6 +138,7 @@ __global__ void __launch_bounds__(kSortThreads, ND == 256 ? 7 : 6) k_sort_scatte
     const uint32_t* __restrict__ kin, const uint32_t* __restrict__ vin, uint32_t* __restrict__ kout,
     uint32_t* __restrict__ vout, int64_t n, int shift, int64_t nblk,
     const uint32_t* __restrict__ hist, const uint32_t* __restrict__ rowtot) {
+  chain_wait();
   constexpr int kWarps = kSortThreads / 32;
   constexpr int DPT = ND / kSortThreads;
   static_assert(kSortItems * 32 <= 256 && kSortTile <= 65535, "per-warp counts fit 16 bits");
@@ -379,6 +382,7 @@ template <int NT, int MINB>
 __global__ void __launch_bounds__(NT, MINB) k_bucket_sort(uint32_t* k1, uint32_t* v1, uint32_t* k0, uint32_t* v0,
                                                           const uint32_t* __restrict__ rowtot, int64_t n_single,
                                                           int cap, int g, int nd) {
+  chain_wait();
   extern __shared__ __align__(16) uint32_t sbuf[];
   __shared__ BsShared<NT> sh;
   __shared__ uint32_t s_len[8];
@@ -484,13 +488,13 @@ cudaError_t set_sort_attributes() {
 }
 
 const uint32_t* launch_radix_sort(uint32_t* k0, uint32_t* v0, uint32_t* k1, uint32_t* v1, uint32_t* hist,
-                                  int64_t n, int first_byte, cudaStream_t s, bool shared_gpu) {
+                                  int64_t n, int first_byte, LaunchSeq& seq, bool shared_gpu) {
   if (n <= 1) return v0;
   const int64_t nblk = sort_blocks(n);
   if (first_byte == 0 && n <= kBsSingleN) {
     // one CTA sorts the whole array in shared memory, all four bytes
     const int cap = int((n + 255) / 256 * 256);
-    k_bucket_sort<256, 3><<<1, 256, size_t(16) * cap, s>>>(k1, v1, k0, v0, nullptr, n, cap, 256, 256);
+    seq(k_bucket_sort<256, 3>, 1, 256, size_t(16) * cap, k1, v1, k0, v0, nullptr, n, cap, 256, 256);
     return v0;
   }
   if (first_byte == 0 && n <= kBucketSortMaxN) {
@@ -508,16 +512,16 @@ const uint32_t* launch_radix_sort(uint32_t* k0, uint32_t* v0, uint32_t* k1, uint
     while (shared_gpu && g < nd && int64_t(g) * 2 * n <= int64_t(2048) * nd) g *= 2;
     const int cap = bucket_cap(n, g, nd);
     if (wide) {
-      k_sort_hist<512><<<unsigned(nblk), kSortThreads, 0, s>>>(k0, n, shift, nblk, hist);
-      k_sort_rowscan<<<512, kSortThreads, 0, s>>>(hist, nblk, rowtot);
-      k_sort_scatter<512><<<unsigned(nblk), kSortThreads, 0, s>>>(k0, v0, k1, v1, n, shift, nblk, hist, rowtot);
-      k_bucket_sort<256, 2><<<unsigned(512 / g), 256, size_t(16) * cap, s>>>(k1, v1, k0, v0, rowtot, 0, cap, g,
+      seq(k_sort_hist<512>, unsigned(nblk), kSortThreads, 0, k0, n, shift, nblk, hist);
+      seq(k_sort_rowscan, 512, kSortThreads, 0, hist, nblk, rowtot);
+      seq(k_sort_scatter<512>, unsigned(nblk), kSortThreads, 0, k0, v0, k1, v1, n, shift, nblk, hist, rowtot);
+      seq(k_bucket_sort<256, 2>, unsigned(512 / g), 256, size_t(16) * cap, k1, v1, k0, v0, rowtot, 0, cap, g,
                                                                              512);
     } else {
-      k_sort_hist<256><<<unsigned(nblk), kSortThreads, 0, s>>>(k0, n, shift, nblk, hist);
-      k_sort_rowscan<<<256, kSortThreads, 0, s>>>(hist, nblk, rowtot);
-      k_sort_scatter<256><<<unsigned(nblk), kSortThreads, 0, s>>>(k0, v0, k1, v1, n, shift, nblk, hist, rowtot);
-      k_bucket_sort<256, 3><<<unsigned(256 / g), 256, size_t(16) * cap, s>>>(k1, v1, k0, v0, rowtot, 0, cap, g,
+      seq(k_sort_hist<256>, unsigned(nblk), kSortThreads, 0, k0, n, shift, nblk, hist);
+      seq(k_sort_rowscan, 256, kSortThreads, 0, hist, nblk, rowtot);
+      seq(k_sort_scatter<256>, unsigned(nblk), kSortThreads, 0, k0, v0, k1, v1, n, shift, nblk, hist, rowtot);
+      seq(k_bucket_sort<256, 3>, unsigned(256 / g), 256, size_t(16) * cap, k1, v1, k0, v0, rowtot, 0, cap, g,
                                                                              256);
     }
     return v0;
@@ -526,9 +530,9 @@ const uint32_t* launch_radix_sort(uint32_t* k0, uint32_t* v0, uint32_t* k1, uint
   uint32_t *ki = k0, *vi = v0, *ko = k1, *vo = v1;
   for (int pass = first_byte; pass < 4; ++pass) {
     const int shift = 8 * pass;
-    k_sort_hist<256><<<unsigned(nblk), kSortThreads, 0, s>>>(ki, n, shift, nblk, hist);
-    k_sort_rowscan<<<256, kSortThreads, 0, s>>>(hist, nblk, rowtot);
-    k_sort_scatter<256><<<unsigned(nblk), kSortThreads, 0, s>>>(ki, vi, ko, vo, n, shift, nblk, hist, rowtot);
+    seq(k_sort_hist<256>, unsigned(nblk), kSortThreads, 0, ki, n, shift, nblk, hist);
+    seq(k_sort_rowscan, 256, kSortThreads, 0, hist, nblk, rowtot);
+    seq(k_sort_scatter<256>, unsigned(nblk), kSortThreads, 0, ki, vi, ko, vo, n, shift, nblk, hist, rowtot);
     uint32_t* tk = ki; ki = ko; ko = tk;
     uint32_t* tv = vi; vi = vo; vo = tv;
   }
@@ -546,6 +550,7 @@ template <class T> struct SoA { T* d[6]; uint32_t* id; };
 template <class T>
 __global__ void k_reorder(const Part<T>* __restrict__ src, SoA<T> dst, const uint32_t* __restrict__ perm,
                           int64_t n) {
+  chain_wait();
   const int64_t j = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   if (j >= n) return;
   const Part<T> p = src[perm[j]];
@@ -556,11 +561,11 @@ __global__ void k_reorder(const Part<T>* __restrict__ src, SoA<T> dst, const uin
 
 template <class T>
 void launch_reorder(const Part<T>* src, T* const* dst, uint32_t* id_dst, const uint32_t* perm, int64_t n,
-                    cudaStream_t s) {
+                    LaunchSeq& seq) {
   SoA<T> d;
   for (int c = 0; c < 6; ++c) d.d[c] = dst[c];
   d.id = id_dst;
-  k_reorder<T><<<unsigned((n + 255) / 256), 256, 0, s>>>(src, d, perm, n);
+  seq(k_reorder<T>, unsigned((n + 255) / 256), 256, 0, src, d, perm, n);
 }
 
 // Radius keys of the state in its storage order (after a load or a field
@@ -568,6 +573,7 @@ void launch_reorder(const Part<T>* src, T* const* dst, uint32_t* id_dst, const u
 template <class T>
 __global__ void k_keys(const Part<T>* __restrict__ st, uint32_t* __restrict__ key, uint32_t* __restrict__ kidx,
                        int64_t n, RadiusKey rk) {
+  chain_wait();
   const int64_t j = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   if (j >= n) return;
   const Part<T> p = st[j];
@@ -576,8 +582,8 @@ __global__ void k_keys(const Part<T>* __restrict__ st, uint32_t* __restrict__ ke
 }
 
 template <class T>
-void launch_keys(const Part<T>* st, uint32_t* key, uint32_t* kidx, int64_t n, double r_out, cudaStream_t s) {
-  k_keys<T><<<unsigned((n + 255) / 256), 256, 0, s>>>(st, key, kidx, n, make_radius_key(r_out));
+void launch_keys(const Part<T>* st, uint32_t* key, uint32_t* kidx, int64_t n, double r_out, LaunchSeq& seq) {
+  seq(k_keys<T>, unsigned((n + 255) / 256), 256, 0, st, key, kidx, n, make_radius_key(r_out));
 }
 
 // FP64 -> FP32 rounding to nearest, ties to even (IEEE 754 binary64 ->
@@ -713,6 +719,7 @@ template <class T> struct Ptr6 { const T* d[6]; };
 template <class T>
 __global__ void k_scatter_by_id(Ptr6<T> p, int nc, const uint32_t* __restrict__ id,
                                 double* __restrict__ out, int64_t n) {
+  chain_wait();
   const int64_t j = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   if (j >= n) return;
   const int64_t k = id[j];
@@ -721,10 +728,10 @@ __global__ void k_scatter_by_id(Ptr6<T> p, int nc, const uint32_t* __restrict__ 
 
 template <class T>
 void launch_scatter_by_id(const T* const* comps, int ncomp, const uint32_t* id, double* out, int64_t n,
-                          cudaStream_t s) {
+                          LaunchSeq& seq) {
   Ptr6<T> p;
   for (int c = 0; c < ncomp; ++c) p.d[c] = comps[c];
-  k_scatter_by_id<T><<<unsigned((n + 255) / 256), 256, 0, s>>>(p, ncomp, id, out, n);
+  seq(k_scatter_by_id<T>, unsigned((n + 255) / 256), 256, 0, p, ncomp, id, out, n);
 }
 
 // The state in id order: x[id][3] and v[id][3], FP64.
@@ -800,6 +807,7 @@ constexpr int kTsTiles = 128;  // tiles per CTA
 template <class T>
 __global__ void __launch_bounds__(256) k_tile_scan(const T* __restrict__ agg, T* __restrict__ pfx,
                                                    double* __restrict__ gagg, int64_t tw, int64_t ts, int nc) {
+  chain_wait();
   using V4 = typename Vec4<T>::type;
   using C = CSum<T>;
   __shared__ T buf[kTsRows][kTsTiles + 1];  // [row][tile], padded: the transposed reads hit distinct banks
@@ -866,38 +874,80 @@ __global__ void __launch_bounds__(256) k_tile_scan(const T* __restrict__ agg, T*
 }
 
 template <class T>
-void launch_tile_scan(const T* agg, T* pfx, double* gagg, int64_t ntiles, int nc, cudaStream_t s) {
+void launch_tile_scan(const T* agg, T* pfx, double* gagg, int64_t ntiles, int nc, LaunchSeq& seq) {
   const int64_t tw = tiles_whole(ntiles), ts = tile_stride(ntiles);
   const dim3 grid(unsigned((tw + kTsTiles - 1) / kTsTiles), unsigned((nc + kTsRows - 1) / kTsRows));
-  if (tw > 0) k_tile_scan<T><<<grid, 256, 0, s>>>(agg, pfx, gagg, tw, ts, nc);
+  if (tw > 0) seq(k_tile_scan<T>, grid, 256, 0, agg, pfx, gagg, tw, ts, nc);
 }
 
 // ============================================================================
 // Group scan. Input: the FP64 totals gagg[g][u] of the scan groups (written
-// by the moments kernel). Output: gbase[g][u] = the sum over the earlier
-// groups (Rs components, u even) or over the later groups (Is components, u
-// odd), each summed in its own direction, and the totals tot / totd.
+// by the tile scan). Output: gbase[g][u] = the sum over the earlier groups (Rs
+// components, u even) or over the later groups (Is components, u odd), each
+// summed in its own direction, and the totals tot / totd.
 // The groups are cut into nseg segments of G groups (G a multiple of 8);
 // CTA (column block b, segment s) handles components 32 b + lane with its 8
 // warps splitting the segment. k_group_sums forms the warp and segment sums;
 // the last CTA of a column block to finish (an atomic ticket, no waiting)
 // scans the segment sums of that block in a fixed order, so the result is
 // the same whichever CTA finishes last. k_group_bases then walks each warp's
-// groups once more and writes the bases.
+// groups once more and writes the bases. With one segment (up to kGsOne
+// groups) k_group_sums writes the bases itself.
+// The CTA that completes the last column block (a second ticket) runs the
+// step's finalize, which needs the totals alone.
 // Work space w (FP64): [nseg][8][nc] warp sums, then [nseg][nc] segment sums,
 // then [nseg][nc] segment bases.
 // ============================================================================
+
+// Finalize: u_asy(t_n), the kick weight, and Q_diff(t_n) = -(1/n~) sum over odd
+// l of c_l' b^P_l * (sum_i q_i Is_l^0(x_i)) (Sec. 4; Is_l^0 = P_l(cos t)/r^{l+1}).
+// By one thread.
+__device__ __forceinline__ void finalize_step(const FinalizeArgs& a) {
+  StepState* st = a.st;
+  const int64_t n = st->next;
+  const double t = double(n) * a.dt;
+  double u = 0.0;
+  if (a.drive_kind == 0) {
+    const double z = (t - a.t0) / a.sigma;
+    u = a.v_hat * exp(-0.5 * z * z);
+  } else if (a.drive_kind == 1) {
+    u = n == 0 ? a.v_hat : 0.0;
+  }
+  st->step = n;
+  st->u = u;
+  st->kick = st->sync ? 0.5 * a.dt : a.dt;
+  // electrons absorbed at the probe since the last fold (wall_rule 2) join Q_S
+  // (charge -1 each) before the field of this step is evaluated
+  st->qs_acc -= double(st->nabs_step);
+  st->nabs_total += st->nabs_step;
+  st->nabs_step = 0;
+  if (a.record) {
+    double q = 0.0;
+    for (int l = 1; l <= a.L; l += 2) q += a.canti[l] * __ldcg(a.totd + 2 * (l - 1) + 1);
+    q *= -a.inv_ntilde;
+    const int64_t h = n - a.first;
+    if (h >= 0 && h < a.cap) {
+      a.qhist[h] = q;
+      a.uhist[h] = u;
+    }
+    st->next = n + 1;
+    st->sync = 0;
+  }
+}
+
 template <class T>
 __global__ void __launch_bounds__(kGsWarps * 32) k_group_sums(const double* __restrict__ gagg,
                                                               double* __restrict__ w, unsigned* __restrict__ ticket,
-                                                              T* __restrict__ tot, double* __restrict__ totd,
-                                                              int64_t ngroups, int nc, int64_t G, int nseg) {
+                                                              T* __restrict__ gbase, T* __restrict__ tot, double* totd,
+                                                              int64_t ngroups, int nc, int64_t G, int nseg,
+                                                              FinalizeArgs fin) {
+  chain_wait();
   __shared__ double ws[kGsWarps][32];
   __shared__ double sst[kGsMaxSeg][32];  // the segment sums of this column block (last CTA)
   __shared__ bool last;
   const unsigned lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int c = blockIdx.x * 32 + lane;
-  const bool okc = c < nc;
+  const bool okc = c < nc, suffix = (c & 1) != 0;
   const int seg = blockIdx.y;
   double* wsum = w;
   double* ssum = w + int64_t(kGsMaxSeg) * kGsWarps * nc;
@@ -909,44 +959,77 @@ __global__ void __launch_bounds__(kGsWarps * 32) k_group_sums(const double* __re
   if (okc) {
 #pragma unroll 4
     for (int64_t g = g0; g < g1; ++g) run += gagg[g * nc + c];
-    wsum[(int64_t(seg) * kGsWarps + warp) * nc + c] = run;
+    if (nseg > 1) wsum[(int64_t(seg) * kGsWarps + warp) * nc + c] = run;
   }
   ws[warp][lane] = run;
   __syncthreads();
-  if (warp == 0 && okc) {
-    double sum = 0.0;
+  if (nseg == 1) {
+    double base = 0.0, all = 0.0;
 #pragma unroll
-    for (int k = 0; k < kGsWarps; ++k) sum += ws[k][lane];
-    ssum[int64_t(seg) * nc + c] = sum;
-  }
-  __threadfence();
-  __syncthreads();
-  if (threadIdx.x == 0) last = atomicAdd(&ticket[blockIdx.x], 1u) == unsigned(nseg - 1);
-  __syncthreads();
-  if (!last) return;
-  __threadfence();
-  // all warps stage the segment sums (independent loads in flight together),
-  // then warp 0 scans them from shared memory in a fixed order
-  for (int k = int(warp); k < nseg; k += kGsWarps) sst[k][lane] = okc ? __ldcg(ssum + int64_t(k) * nc + c) : 0.0;
-  __syncthreads();
-  if (warp == 0 && okc) {
-    double all = 0.0;
-    const bool suffix = (c & 1) != 0;
-    for (int k = 0; k < nseg; ++k) {
-      const int s2 = suffix ? nseg - 1 - k : k;
-      sbase[int64_t(s2) * nc + c] = all;
-      all += sst[s2][lane];
+    for (int k = 0; k < kGsWarps; ++k) {
+      const double v = ws[suffix ? kGsWarps - 1 - k : k][lane];
+      if (suffix ? kGsWarps - 1 - k > int(warp) : k < int(warp)) base += v;
+      all += v;
     }
-    tot[c] = T(all);
-    totd[c] = all;
+    if (okc) {
+#pragma unroll 4
+      for (int64_t k = 0; k < g1 - g0; ++k) {
+        const int64_t g = suffix ? g1 - 1 - k : g0 + k;
+        gbase[g * nc + c] = T(base);
+        base += gagg[g * nc + c];
+      }
+      if (warp == 0) {
+        tot[c] = T(all);
+        totd[c] = all;
+      }
+    }
+  } else {
+    if (warp == 0 && okc) {
+      double sum = 0.0;
+#pragma unroll
+      for (int k = 0; k < kGsWarps; ++k) sum += ws[k][lane];
+      ssum[int64_t(seg) * nc + c] = sum;
+    }
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicAdd(&ticket[blockIdx.x], 1u) == unsigned(nseg - 1);
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    // all warps stage the segment sums (independent loads in flight together),
+    // then warp 0 scans them from shared memory in a fixed order
+    for (int k = int(warp); k < nseg; k += kGsWarps) sst[k][lane] = okc ? __ldcg(ssum + int64_t(k) * nc + c) : 0.0;
+    __syncthreads();
+    if (warp == 0 && okc) {
+      double all = 0.0;
+      for (int k = 0; k < nseg; ++k) {
+        const int s2 = suffix ? nseg - 1 - k : k;
+        sbase[int64_t(s2) * nc + c] = all;
+        all += sst[s2][lane];
+      }
+      tot[c] = T(all);
+      totd[c] = all;
+    }
+    if (threadIdx.x == 0) ticket[blockIdx.x] = 0u;  // ready for the next step
   }
-  if (threadIdx.x == 0) ticket[blockIdx.x] = 0u;  // ready for the next step
+  if (!fin.st) return;
+  // the totals of this column block are written (by warp 0): the last block finalizes
+  if (warp == 0) {
+    __threadfence();
+    __syncwarp();
+    if (lane == 0 && atomicAdd(&ticket[gridDim.x], 1u) == gridDim.x - 1) {
+      __threadfence();
+      ticket[gridDim.x] = 0u;
+      finalize_step(fin);
+    }
+  }
 }
 
 template <class T>
 __global__ void __launch_bounds__(kGsWarps * 32) k_group_bases(const double* __restrict__ gagg,
                                                                const double* __restrict__ w, T* __restrict__ gbase,
                                                                int64_t ngroups, int nc, int64_t G) {
+  chain_wait();
   const unsigned lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int c = blockIdx.x * 32 + lane;
   if (c >= nc) return;  // no barrier below
@@ -971,54 +1054,15 @@ __global__ void __launch_bounds__(kGsWarps * 32) k_group_bases(const double* __r
 
 template <class T>
 void launch_group_scan(const double* gagg, double* work, unsigned* ticket, T* gbase, T* tot, double* totd,
-                       int64_t ngroups, int nc, int gseg, cudaStream_t s) {
+                       int64_t ngroups, int nc, int gseg, const FinalizeArgs* fin, LaunchSeq& seq) {
   if (ngroups <= 0) return;
   const int64_t G = gs_seg_len(ngroups, gseg);
   const int nseg = int(gs_nseg(ngroups, gseg));
-  dim3 grid(unsigned(gs_col_blocks(nc)), unsigned(nseg));
-  k_group_sums<T><<<grid, kGsWarps * 32, 0, s>>>(gagg, work, ticket, tot, totd, ngroups, nc, G, nseg);
-  k_group_bases<T><<<grid, kGsWarps * 32, 0, s>>>(gagg, work, gbase, ngroups, nc, G);
+  const dim3 grid(unsigned(gs_col_blocks(nc)), unsigned(nseg));
+  seq(k_group_sums<T>, grid, kGsWarps * 32, 0, gagg, work, ticket, gbase, tot, totd, ngroups, nc, G, nseg,
+      fin ? *fin : FinalizeArgs{});
+  if (nseg > 1) seq(k_group_bases<T>, grid, kGsWarps * 32, 0, gagg, work, gbase, ngroups, nc, G);
 }
-
-// ============================================================================
-// Finalize: u_asy(t_n), the kick weight, and Q_diff(t_n) = -(1/n~) sum over odd
-// l of c_l' b^P_l * (sum_i q_i Is_l^0(x_i)) (Sec. 4; Is_l^0 = P_l(cos t)/r^{l+1}).
-// ============================================================================
-__global__ void k_finalize(FinalizeArgs a) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  StepState* st = a.st;
-  const int64_t n = st->next;
-  const double t = double(n) * a.dt;
-  double u = 0.0;
-  if (a.drive_kind == 0) {
-    const double z = (t - a.t0) / a.sigma;
-    u = a.v_hat * exp(-0.5 * z * z);
-  } else if (a.drive_kind == 1) {
-    u = n == 0 ? a.v_hat : 0.0;
-  }
-  st->step = n;
-  st->u = u;
-  st->kick = st->sync ? 0.5 * a.dt : a.dt;
-  // electrons absorbed at the probe since the last fold (wall_rule 2) join Q_S
-  // (charge -1 each) before the field of this step is evaluated
-  st->qs_acc -= double(st->nabs_step);
-  st->nabs_total += st->nabs_step;
-  st->nabs_step = 0;
-  if (a.record) {
-    double q = 0.0;
-    for (int l = 1; l <= a.L; l += 2) q += a.canti[l] * a.totd[2 * (l - 1) + 1];
-    q *= -a.inv_ntilde;
-    const int64_t h = n - a.first;
-    if (h >= 0 && h < a.cap) {
-      a.qhist[h] = q;
-      a.uhist[h] = u;
-    }
-    st->next = n + 1;
-    st->sync = 0;
-  }
-}
-
-void launch_finalize(const FinalizeArgs& a, cudaStream_t s) { k_finalize<<<1, 32, 0, s>>>(a); }
 
 // Step state after a load: step 0, nothing recorded, the first kick is a half kick.
 __global__ void k_init_step(StepState* st) {
@@ -1197,7 +1241,6 @@ cudaError_t preload_core_kernels() {
                        reinterpret_cast<const void*>(&k_sort_scatter<512>),
                        reinterpret_cast<const void*>(&k_bucket_sort<256, 3>),
                        reinterpret_cast<const void*>(&k_bucket_sort<256, 2>),
-                       reinterpret_cast<const void*>(&k_finalize),
                        reinterpret_cast<const void*>(&k_init_step)};
   for (const void* f : fns) {
     const cudaError_t e = cudaFuncGetAttributes(&fa, f);
@@ -1210,18 +1253,18 @@ cudaError_t preload_core_kernels() {
 // explicit instantiations
 #define IMRP_INST_CORE(T)                                                                          \
   template void launch_reorder<T>(const Part<T>*, T* const*, uint32_t*, const uint32_t*, int64_t,  \
-                                  cudaStream_t);                                                   \
-  template void launch_keys<T>(const Part<T>*, uint32_t*, uint32_t*, int64_t, double, cudaStream_t); \
+                                  LaunchSeq&);                                                     \
+  template void launch_keys<T>(const Part<T>*, uint32_t*, uint32_t*, int64_t, double, LaunchSeq&); \
   template void launch_load<T>(const double*, const double*, const uint32_t*, Part<T>*, uint32_t*, \
                                uint32_t*, int64_t, double, int*, cudaStream_t);                    \
   template void launch_state_dump<T>(const Part<T>*, double*, double*, uint32_t*, int64_t,         \
                                      cudaStream_t);                                                \
   template void launch_scatter_by_id<T>(const T* const*, int, const uint32_t*, double*, int64_t,   \
-                                        cudaStream_t);                                             \
+                                        LaunchSeq&);                                               \
   template void launch_state_out<T>(const Part<T>*, double*, double*, int64_t, cudaStream_t);     \
-  template void launch_tile_scan<T>(const T*, T*, double*, int64_t, int, cudaStream_t);                \
+  template void launch_tile_scan<T>(const T*, T*, double*, int64_t, int, LaunchSeq&);                \
   template void launch_group_scan<T>(const double*, double*, unsigned*, T*, T*, double*, int64_t, int, \
-                                     int, cudaStream_t);
+                                     int, const FinalizeArgs*, LaunchSeq&);
 IMRP_INST_CORE(float)
 IMRP_INST_CORE(double)
 

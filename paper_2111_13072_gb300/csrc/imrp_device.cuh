@@ -152,6 +152,18 @@ template <class T> struct Tables {
 
 __device__ __forceinline__ unsigned lane_id() { return threadIdx.x & 31u; }
 
+// First statement of every kernel of a step. A step is a chain of short
+// kernels, each reading what the one before wrote; launched with programmatic
+// stream serialisation, a kernel is brought up while its predecessor drains and
+// waits here until the predecessor has completed with its writes visible (a
+// no-op without that attribute). Since every kernel waits before it touches
+// memory, a kernel that passes here has all earlier kernels of the chain behind
+// it. No kernel triggers its successor early: CTAs that come up while the
+// predecessor is still spread over the SMs are placed unevenly, and the field
+// and moments kernels of one wave then run longer (triggering at the start:
+// FP64 N = 20000, l_max 8, step 0.209 -> 0.222 ms; N = 7e5, l_max 12, 0.306 -> 0.323).
+__device__ __forceinline__ void chain_wait() { cudaGridDependencySynchronize(); }
+
 // Transpose reduction of 32 registers over the warp: on return lane i holds
 // sum over all lanes of v[i]. 31 shuffles instead of 32 x 5.
 template <class T>
@@ -247,7 +259,11 @@ __host__ __device__ constexpr int64_t tile_stride(int64_t ntiles) { return tiles
 // kGsWarps warps (32 components per CTA, one per lane).
 constexpr int kGsWarps = 8;
 constexpr int kGsMaxSeg = 64;
+// Up to kGsOne groups (4 per warp) one CTA per 32 components does it all: the
+// sums, the bases and no second kernel.
+constexpr int64_t kGsOne = 32;
 __host__ __device__ inline int64_t gs_seg_len(int64_t ngroups, int gseg) {
+  if (ngroups <= kGsOne) return (ngroups + kGsWarps - 1) / kGsWarps * kGsWarps;
   int64_t G = (ngroups + kGsMaxSeg - 1) / kGsMaxSeg;
   if (G < gseg) G = gseg;
   return (G + kGsWarps - 1) / kGsWarps * kGsWarps;
@@ -256,6 +272,8 @@ __host__ __device__ inline int64_t gs_nseg(int64_t ngroups, int gseg) {
   const int64_t G = gs_seg_len(ngroups, gseg);
   return ngroups > 0 ? (ngroups + G - 1) / G : 0;
 }
+// tickets of the group scan: one per column block, one for the finalize
+__host__ __device__ constexpr int gs_tickets(int nc) { return (nc + 31) / 32 + 1; }
 // FP64 work space of the group scan for nc components: per segment the
 // kGsWarps warp sums, the segment sum and the segment's base.
 __host__ __device__ constexpr int64_t gs_work_doubles(int nc) { return int64_t(kGsMaxSeg) * (kGsWarps + 2) * nc; }

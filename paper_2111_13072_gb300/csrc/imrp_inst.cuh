@@ -103,21 +103,21 @@ const PrologueInit g_prologue_init;
 // CTAs of 64 threads, mom_ppt particles per thread, covering whole scan groups
 // of 1024 particles (every tile the scans read is written; past the particles
 // the sums are zero)
-template <class T, int L> void mom_launch(const MomArgs<T>& a, cudaStream_t s) {
+template <class T, int L> void mom_launch(const MomArgs<T>& a, LaunchSeq& seq) {
   if (a.n <= 0) return;
   const int ppt = mom_ppt(sizeof(T), a.n);
   const unsigned blocks = unsigned(mom_blocks(a.n, ppt) * a.parts);
   if (ppt == kMomPPT)
-    k_moments<T, L, kMomPPT><<<blocks, kMomThreads, moments_smem<T, L, kMomPPT>(), s>>>(a);
+    seq(k_moments<T, L, kMomPPT>, blocks, kMomThreads, moments_smem<T, L, kMomPPT>(), a);
   else
-    k_moments<T, L, kMomPPTSmall><<<blocks, kMomThreads, moments_smem<T, L, kMomPPTSmall>(), s>>>(a);
+    seq(k_moments<T, L, kMomPPTSmall>, blocks, kMomThreads, moments_smem<T, L, kMomPPTSmall>(), a);
 }
 
-template <class T, int L> void field_launch(const FieldArgs<T>& a, int wpb, cudaStream_t s) {
+template <class T, int L> void field_launch(const FieldArgs<T>& a, int wpb, LaunchSeq& seq) {
   const int64_t ntiles = (a.n + 31) / 32;
   const int64_t blocks = (ntiles + wpb - 1) / wpb;
   const size_t smem = size_t(wpb) * field_smem_per_warp<T>(L);
-  if (blocks > 0) k_field<T, L><<<unsigned(blocks), wpb * 32, smem, s>>>(a);
+  if (blocks > 0) seq(k_field<T, L>, unsigned(blocks), unsigned(wpb * 32), smem, a);
 }
 
 template <class T, int L>

@@ -39,6 +39,36 @@ inline double coef_canti(int l, double d, double eps) {
   return (l % 2 == 1) ? coef_cprime((l + 1) / 2) * coef_bP(l, d, eps) : 0.0;
 }
 
+// ---- launches ---------------------------------------------------------------
+// A sequence of dependent kernel launches on one stream. A launch whose
+// predecessor on the stream is a kernel of the same sequence gets the
+// programmatic serialisation attribute (all these kernels begin with
+// chain_wait); the first one, and the first after an event or another
+// operation (unchain), a full dependency. Step, full dependencies -> chained (us,
+// captured graphs): N = 3001, l_max 8: 53.4 -> 51.4; N = 1e5, l_max 16: 97.5 ->
+// 94.8; N = 3e5, l_max 8: 108.2 -> 105.0.
+struct LaunchSeq {
+  cudaStream_t s;
+  bool chained = false;
+  explicit LaunchSeq(cudaStream_t stream) : s(stream) {}
+  void unchain() { chained = false; }
+  template <class... P, class... A>
+  void operator()(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, A&&... args) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = chained ? 1 : 0;
+    cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);  // errors: cudaGetLastError of the caller
+    chained = true;
+  }
+};
+
 // ---- radix sort (imrp_core.cu) ---------------------------------------------
 constexpr int kSortThreads = 256;
 constexpr int kSortItems = 8;
@@ -58,17 +88,16 @@ constexpr int64_t sort_hist_words(int64_t n) { return 512 * sort_blocks(n) + 512
 // so even radii that FP32 arithmetic cannot tell apart are ordered exactly.
 inline int sort_first_byte(int) { return 0; }
 const uint32_t* launch_radix_sort(uint32_t* k0, uint32_t* v0, uint32_t* k1, uint32_t* v1, uint32_t* hist,
-                                  int64_t n, int first_byte, cudaStream_t s,
-                                  bool shared_gpu = false);
+                                  int64_t n, int first_byte, LaunchSeq& seq, bool shared_gpu = false);
 
 // ---- state movement and keys (imrp_core.cu) ---------------------------------
 // The state is an array of Part<T> records in the order of the last push (or
 // load); each step gathers it into radius order as component arrays.
 template <class T>
 void launch_reorder(const Part<T>* src, T* const* dst, uint32_t* id_dst, const uint32_t* perm, int64_t n,
-                    cudaStream_t s);
+                    LaunchSeq& seq);
 template <class T>
-void launch_keys(const Part<T>* st, uint32_t* key, uint32_t* kidx, int64_t n, double r_out, cudaStream_t s);
+void launch_keys(const Part<T>* st, uint32_t* key, uint32_t* kidx, int64_t n, double r_out, LaunchSeq& seq);
 template <class T>
 void launch_load(const double* x /* [n][3] */, const double* v /* [n][3] */, const uint32_t* ids /* or null */,
                  Part<T>* st, uint32_t* key, uint32_t* kidx, int64_t n, double r_out, int* err, cudaStream_t s);
@@ -78,7 +107,7 @@ void launch_state_dump(const Part<T>* st, double* x, double* v, uint32_t* id, in
 // out[id[j]][c] = comp_c[j] for c < ncomp
 template <class T>
 void launch_scatter_by_id(const T* const* comps, int ncomp, const uint32_t* id, double* out,
-                          int64_t n, cudaStream_t s);
+                          int64_t n, LaunchSeq& seq);
 // the state in id order: x[n][3], v[n][3] (FP64)
 template <class T>
 void launch_state_out(const Part<T>* st, double* x, double* v, int64_t n, cudaStream_t s);
@@ -88,15 +117,7 @@ void launch_state_out(const Part<T>* st, double* x, double* v, int64_t n, cudaSt
 // pfx[tile][u] (tile-major: one tile's nc carries contiguous), group totals
 // into gagg[g][u] (FP64)
 template <class T>
-void launch_tile_scan(const T* agg, T* pfx, double* gagg, int64_t ntiles, int nc, cudaStream_t s);
-// group scan over gagg:
-// gseg: least number of groups per segment (16, 32 or 64; chosen by the
-// autotuner). work: gs_work_doubles(nc) doubles; ticket: gs_col_blocks(nc)
-// counters, zero before the first call (each call leaves them zero).
-template <class T>
-void launch_group_scan(const double* gagg, double* work, unsigned* ticket, T* gbase, T* tot, double* totd,
-                       int64_t ngroups, int nc, int gseg, cudaStream_t s);
-
+void launch_tile_scan(const T* agg, T* pfx, double* gagg, int64_t ntiles, int nc, LaunchSeq& seq);
 struct FinalizeArgs {
   StepState* st;
   const double* totd;
@@ -111,7 +132,15 @@ struct FinalizeArgs {
   double v_hat, sigma, t0, dt;
   double canti[kTabL];
 };
-void launch_finalize(const FinalizeArgs& a, cudaStream_t s);
+// group scan over gagg:
+// gseg: least number of groups per segment (16, 32 or 64; chosen by the
+// autotuner). work: gs_work_doubles(nc) doubles; ticket: gs_tickets(nc)
+// counters, zero before the first call (each call leaves them zero). fin (or
+// null): the step's finalize (drive, kick weight, Q_diff tally), run once the
+// totals are complete.
+template <class T>
+void launch_group_scan(const double* gagg, double* work, unsigned* ticket, T* gbase, T* tot, double* totd,
+                       int64_t ngroups, int nc, int gseg, const FinalizeArgs* fin, LaunchSeq& seq);
 // Loads the device code of every degree-independent kernel of both precisions
 // (CUDA loads modules lazily, at a kernel's first launch or query, and the
 // load reserves device memory): the allocation-free entry point calls it at
@@ -162,18 +191,18 @@ inline int64_t mom_blocks(int64_t n, int ppt) { return (n + 1023) / 1024 * (16 /
 // diagonal terms up to its first column). As many ranges as give the stated
 // CTAs per SM: FP32 N = 1e5, l_max = 16: 0.043 ms with one range, 0.0225 with
 // 6 per SM, 0.028 with 8; N = 3e5, l_max = 8: 0.0262, 0.0206, 0.0267; FP64
-// N = 20000, l_max = 8: 0.102 with one, 0.046 with 7 ranges, 0.051 with 9.
+// N = 20000, l_max = 8: 0.102 with one, 0.046 with 7 ranges, 0.051 with 9 (0.055
+// with 6, where a short last range unbalances them).
 inline int mom_parts(int elem_size, int L, int64_t n, int ppt) {
-  const int per_sm = elem_size == 4 ? 6 : ppt == 4 ? 5 : 8;
+  const int per_sm = elem_size == 4 ? 6 : ppt == 4 ? 4 : 8;
   const int64_t want = int64_t(per_sm) * sm_count() / mom_blocks(n, ppt);
-  const int most = elem_size == 4 ? L + 1 : 3 * (L + 1) / 4;
-  return int(want < 1 ? 1 : want > most ? most : want);
+  return int(want < 1 ? 1 : want > L + 1 ? L + 1 : want);
 }
 
 template <class T> struct KernelSet {
   int L;
-  void (*moments)(const MomArgs<T>&, cudaStream_t);
-  void (*field)(const FieldArgs<T>&, int wpb, cudaStream_t);
+  void (*moments)(const MomArgs<T>&, LaunchSeq&);
+  void (*field)(const FieldArgs<T>&, int wpb, LaunchSeq&);
   int (*init)(int device);  // tables + attributes, once per device
   size_t smem_per_warp;
   int (*field_blocks_per_sm)(int wpb);  // occupancy of the field kernel at wpb warps per CTA

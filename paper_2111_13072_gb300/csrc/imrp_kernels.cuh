@@ -298,6 +298,7 @@ __device__ __forceinline__ void moments_block(const MomArgs<T>& a, int64_t item,
 template <class T, int L, int PPT>
 __global__ void __launch_bounds__(kMomThreads) k_moments(MomArgs<T> a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  chain_wait();
   moments_block<T, L, PPT>(a, blockIdx.x, smem_raw);
 }
 
@@ -1043,6 +1044,7 @@ __host__ __device__ constexpr int field_min_blocks() { return sizeof(T) == 4 ? 3
 template <class T, int L>
 __global__ void __launch_bounds__(256, field_min_blocks<T>()) k_field(FieldArgs<T> a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  chain_wait();
   const int warp = threadIdx.x >> 5, wpb = blockDim.x >> 5;
   // tiles in decreasing order: the particle rows written last (still in L2) first
   field_tile<T, L>(a, smem_raw, warp, wpb, int64_t(gridDim.x - 1 - blockIdx.x) * wpb + warp);

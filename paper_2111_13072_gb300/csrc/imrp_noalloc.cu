@@ -47,7 +47,7 @@ constexpr Layout layout(int64_t n, int L, size_t es) {
   o.tot = at; at += align256(size_t(nc) * es);
   o.totd = at; at += align256(size_t(nc) * 8);
   o.gswork = at; at += align256(size_t(gs_work_doubles(int(nc))) * 8);
-  o.gsticket = at; at += align256(size_t(gs_col_blocks(int(nc))) * 4);
+  o.gsticket = at; at += align256(size_t(gs_tickets(int(nc))) * 4);
   o.eout = at; at += align256(size_t(3 * n) * es);
   o.step = at; at += align256(sizeof(StepState));
   o.err = at; at += align256(sizeof(int));
@@ -83,6 +83,7 @@ constexpr double kEps0 = 8.8541878128e-12;
 // outside 1 < r < r_out or non-finite.
 template <class T>
 __global__ void k_na_load(const double* __restrict__ x, Part<T>* st, int64_t n, double r_out, int* err) {
+  chain_wait();
   const int64_t j = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   if (j >= n) return;
   const double a = x[3 * j], b = x[3 * j + 1], c = x[3 * j + 2];
@@ -100,6 +101,7 @@ __global__ void k_na_load(const double* __restrict__ x, Part<T>* st, int64_t n, 
 // state, the error flag and the group scan's tickets (the scratch keeps the
 // previous call's contents, and another n or degree lays it out differently).
 __global__ void k_na_init(StepState* st, int64_t step, int* err, unsigned* ticket, int nticket) {
+  chain_wait();
   st->step = step;
   st->next = step;
   st->u = 0.0;
@@ -151,12 +153,13 @@ int run(const imrp_params* p, const double* x, int64_t n, int64_t step, double* 
   uint32_t* idx0 = static_cast<uint32_t*>(P(o.idx0));
   StepState* st = static_cast<StepState*>(P(o.step));
   int* err = static_cast<int*>(P(o.err));
-  k_na_init<<<1, 1, 0, s>>>(st, step, err, static_cast<unsigned*>(P(o.gsticket)), gs_col_blocks(nc));
-  k_na_load<T><<<unsigned((n + 255) / 256), 256, 0, s>>>(x, st0, n, r_out, err);
-  launch_keys<T>(st0, key0, idx0, n, r_out, s);
+  LaunchSeq seq(s);
+  seq(k_na_init, 1, 1, 0, st, step, err, static_cast<unsigned*>(P(o.gsticket)), gs_tickets(nc));
+  seq(k_na_load<T>, unsigned((n + 255) / 256), 256, 0, x, st0, n, r_out, err);
+  launch_keys<T>(st0, key0, idx0, n, r_out, seq);
   const uint32_t* perm = launch_radix_sort(key0, idx0, static_cast<uint32_t*>(P(o.key1)), static_cast<uint32_t*>(P(o.idx1)),
-                    static_cast<uint32_t*>(P(o.hist)), n, sort_first_byte(sizeof(T) == 4 ? 1 : 0), s);
-  launch_reorder<T>(st0, st1, id1, perm, n, s);
+                    static_cast<uint32_t*>(P(o.hist)), n, sort_first_byte(sizeof(T) == 4 ? 1 : 0), seq);
+  launch_reorder<T>(st0, st1, id1, perm, n, seq);
   MomArgs<T> ma;
   memset(&ma, 0, sizeof(ma));  // all electrons (species = 0)
   ma.x = st1[0]; ma.y = st1[1]; ma.z = st1[2];
@@ -165,12 +168,9 @@ int run(const imrp_params* p, const double* x, int64_t n, int64_t step, double* 
   ma.rho_inv = T(1.0 / r_out);
   ma.agg = static_cast<T*>(P(o.agg));
   ma.parts = mom_parts(sizeof(T), L, n, mom_ppt(sizeof(T), n));
-  ks->moments(ma, s);
+  ks->moments(ma, seq);
   launch_tile_scan<T>(static_cast<T*>(P(o.agg)), static_cast<T*>(P(o.pfx)), static_cast<double*>(P(o.gagg)),
-                      ntiles, nc, s);
-  launch_group_scan<T>(static_cast<double*>(P(o.gagg)), static_cast<double*>(P(o.gswork)),
-                       static_cast<unsigned*>(P(o.gsticket)), static_cast<T*>(P(o.gbase)),
-                       static_cast<T*>(P(o.tot)), static_cast<double*>(P(o.totd)), ngroups, nc, 32, s);
+                      ntiles, nc, seq);
   double canti[kTabL] = {0}, f[kTabL] = {0};
   for (int l = 1; l <= L; ++l) {
     f[l] = coef_f(l, d, p->eps_D);
@@ -189,7 +189,9 @@ int run(const imrp_params* p, const double* x, int64_t n, int64_t step, double* 
   fa.t0 = p->t0_wpe > 0 ? p->t0_wpe : 4.0 * p->width_wpe;
   fa.dt = p->dt;
   for (int l = 0; l < kTabL; ++l) fa.canti[l] = canti[l];
-  launch_finalize(fa, s);
+  launch_group_scan<T>(static_cast<double*>(P(o.gagg)), static_cast<double*>(P(o.gswork)),
+                       static_cast<unsigned*>(P(o.gsticket)), static_cast<T*>(P(o.gbase)),
+                       static_cast<T*>(P(o.tot)), static_cast<double*>(P(o.totd)), ngroups, nc, 32, &fa, seq);
   FieldArgs<T> a;
   memset(&a, 0, sizeof(a));
   a.x = st1[0]; a.y = st1[1]; a.z = st1[2]; a.vx = st1[3]; a.vy = st1[4]; a.vz = st1[5];
@@ -228,10 +230,10 @@ int run(const imrp_params* p, const double* x, int64_t n, int64_t step, double* 
     rl *= r_out;
     a.cdrive[l] = canti[l] * 4.0 * kPi * n_tilde;
   }
-  ks->field(a, 1, s);  // at most 512 tiles: one per CTA spreads them over the SMs
+  ks->field(a, 1, seq);  // at most 512 tiles: one per CTA spreads them over the SMs
   const T* eo = static_cast<const T*>(P(o.eout));
   const T* cs[3] = {eo, eo + n, eo + 2 * n};
-  launch_scatter_by_id<T>(cs, 3, id1, E, n, s);
+  launch_scatter_by_id<T>(cs, 3, id1, E, n, seq);
   if (cudaGetLastError() != cudaSuccess) return IMRP_E_CUDA;
   int h = 0;
   if (cudaMemcpyAsync(&h, err, sizeof(int), cudaMemcpyDeviceToHost, s) != cudaSuccess) return IMRP_E_CUDA;
