@@ -332,6 +332,7 @@ template <class T> FieldArgs<T> make_field_args(imrp_ctx* ctx, bool record) {
     rl *= ctx->r_out;
     a.cdrive[l] = ctx->canti[l] * 4.0 * kPi * ctx->n_tilde;
   }
+  derive_field_args(a);
   return a;
 }
 
@@ -384,7 +385,10 @@ template <class T> void enqueue_mid(imrp_ctx* ctx, LaunchSeq& seq, bool record) 
   fa.sigma = ctx->p.width_wpe;
   fa.t0 = ctx->t0;
   fa.dt = ctx->p.dt;
-  for (int l = 0; l < kTabL; ++l) fa.canti[l] = ctx->canti[l];
+  for (int l = 0; l < kTabL; ++l) {
+    fa.canti[l] = ctx->canti[l];
+    fa.cdrive[l] = ctx->canti[l] * 4.0 * kPi * ctx->n_tilde;
+  }
   launch_group_scan<T>(ctx->gagg, ctx->gswork, ctx->gsticket, static_cast<T*>(ctx->gbase),
                        static_cast<T*>(ctx->tot), ctx->totd, ctx->ngroups, ctx->nc, ctx->gseg, &fa, seq);
 }

@@ -899,12 +899,15 @@ void launch_tile_scan(const T* agg, T* pfx, double* gagg, int64_t ntiles, int nc
 // then [nseg][nc] segment bases.
 // ============================================================================
 
-// Finalize: u_asy(t_n), the kick weight, and Q_diff(t_n) = -(1/n~) sum over odd
+// Finalize: u_asy(t_n) and its products with the drive coefficients, the kick
+// weight, and Q_diff(t_n) = -(1/n~) sum over odd
 // l of c_l' b^P_l * (sum_i q_i Is_l^0(x_i)) (Sec. 4; Is_l^0 = P_l(cos t)/r^{l+1}).
-// By one thread.
-__device__ __forceinline__ void finalize_step(const FinalizeArgs& a) {
+// By one warp (the per-degree products and loads one per lane).
+__device__ __forceinline__ void finalize_step(const FinalizeArgs& a, int lane) {
+  static_assert(kTabL <= 32, "one degree per lane");
   StepState* st = a.st;
   const int64_t n = st->next;
+  const int32_t sync = st->sync, nabs = st->nabs_step;
   const double t = double(n) * a.dt;
   double u = 0.0;
   if (a.drive_kind == 0) {
@@ -913,18 +916,23 @@ __device__ __forceinline__ void finalize_step(const FinalizeArgs& a) {
   } else if (a.drive_kind == 1) {
     u = n == 0 ? a.v_hat : 0.0;
   }
+  if (lane < kTabL) st->drive_f[lane] = float(u * a.cdrive[lane]);
+  const double is0 = (lane & 1) && lane <= a.L ? __ldcg(a.totd + 2 * (lane - 1) + 1) : 0.0;  // l = lane
+  double q = 0.0;
+  for (int l = 1; l <= a.L; l += 2) q += a.canti[l] * __shfl_sync(0xffffffffu, is0, l);
+  q *= -a.inv_ntilde;
+  if (lane != 0) return;
   st->step = n;
   st->u = u;
-  st->kick = st->sync ? 0.5 * a.dt : a.dt;
+  const double kick = sync ? 0.5 * a.dt : a.dt;
+  st->kick = kick;
+  st->kick_f = float(kick);
   // electrons absorbed at the probe since the last fold (wall_rule 2) join Q_S
   // (charge -1 each) before the field of this step is evaluated
-  st->qs_acc -= double(st->nabs_step);
-  st->nabs_total += st->nabs_step;
+  st->qs_acc -= double(nabs);
+  st->nabs_total += nabs;
   st->nabs_step = 0;
   if (a.record) {
-    double q = 0.0;
-    for (int l = 1; l <= a.L; l += 2) q += a.canti[l] * __ldcg(a.totd + 2 * (l - 1) + 1);
-    q *= -a.inv_ntilde;
     const int64_t h = n - a.first;
     if (h >= 0 && h < a.cap) {
       a.qhist[h] = q;
@@ -1017,10 +1025,12 @@ __global__ void __launch_bounds__(kGsWarps * 32) k_group_sums(const double* __re
   if (warp == 0) {
     __threadfence();
     __syncwarp();
-    if (lane == 0 && atomicAdd(&ticket[gridDim.x], 1u) == gridDim.x - 1) {
+    unsigned t = 0;
+    if (lane == 0) t = atomicAdd(&ticket[gridDim.x], 1u);
+    if (__shfl_sync(0xffffffffu, t, 0) == gridDim.x - 1) {
       __threadfence();
-      ticket[gridDim.x] = 0u;
-      finalize_step(fin);
+      if (lane == 0) ticket[gridDim.x] = 0u;
+      finalize_step(fin, int(lane));
     }
   }
 }

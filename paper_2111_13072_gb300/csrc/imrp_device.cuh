@@ -49,12 +49,17 @@ __host__ __device__ constexpr int comp_idx(int L, int l, int m, int part) {
   return m == 0 ? (l - 1) : col_off(L, m) + 2 * (l - m) + part;
 }
 
-// Per-step scalars written by the finalize kernel and read by the field kernel.
+// Per-step scalars written by the finalize and read by the field kernel. The
+// FP32 values are formed once here: FP64 operations, conversions included, run
+// at 1/64 of the FP32 rate on this part and would otherwise be repeated by every
+// thread of the field kernel (they bound it at low degrees).
 struct StepState {
   int64_t step;     // absolute index of the step being taken (since the last load)
   int64_t next;     // index of the next step to record
   double u;         // u_asy(t_step)
   double kick;      // kick weight of this step (dt, or dt/2 right after a load)
+  float kick_f;     // the same, rounded
+  float drive_f[kTabL];  // u * cdrive[l], rounded (the FP32 field kernel's drive per degree)
   int32_t sync;     // 1: velocities synchronous with x (next kick is dt/2)
   int32_t nabs_step;  // electrons absorbed at the probe in the step in progress (wall_rule 2)
   double qs_acc;      // surface charge they brought since the load (super-particle charges),
@@ -340,6 +345,9 @@ template <class T> struct FieldArgs {
   int L;              // degree (equals the template L)
   T rho, rho_inv;     // r_out and 1 / r_out
   double pf;          // 1 / (4 pi n~)
+  T pf_t, mpf, mpfr;  // T(pf), T(-pf), T(-pf) / r_out
+  T self_pf;          // T(self-image sign times pf)
+  int self_sign;      // self-image term: -1 taken off, 1 added, 0 none
   double ion_coef;    // n_ion / (r_out^3 - 1) (uniform ions, used when ion_q is null)
   const double* ion_q;  // radial ion profile (App. D): ion charge inside r_k = 1 + k h, units e n_inf R^3
   double ion_inv_h;   // 1 / h
@@ -347,6 +355,7 @@ template <class T> struct FieldArgs {
   int ion_n;          // nodes of ion_q (>= 2 when ion_q is set)
   double q_s;         // surface charge of the parameters (the absorbed charge st->qs_acc adds to it)
   double r_out2;      // r_out^2
+  T near_hi;          // T(r_out^2 (1 - 1e-5)): beyond it the exact wall test
   RadiusKey rk;       // the radius key of the next step's sort
   T dt;
   T r_out;

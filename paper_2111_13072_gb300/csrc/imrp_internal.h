@@ -131,7 +131,19 @@ struct FinalizeArgs {
   double inv_ntilde;
   double v_hat, sigma, t0, dt;
   double canti[kTabL];
+  double cdrive[kTabL];  // 4 pi n~ canti (FieldArgs::cdrive)
 };
+// The derived scalars of a FieldArgs whose pf, rho_inv, r_out2, self_image and
+// img_in_tile are set.
+template <class T> inline void derive_field_args(FieldArgs<T>& a) {
+  a.pf_t = T(a.pf);
+  a.mpf = T(-a.pf);
+  a.mpfr = T(-a.pf) * a.rho_inv;
+  // the image moments include the particle itself, or (img_in_tile) leave its tile out
+  a.self_sign = a.img_in_tile ? (a.self_image ? 1 : 0) : (a.self_image ? 0 : -1);
+  a.self_pf = T(a.self_sign * a.pf);
+  a.near_hi = T(a.r_out2 * (1.0 - 1e-5));
+}
 // group scan over gagg:
 // gseg: least number of groups per segment (16, 32 or 64; chosen by the
 // autotuner). work: gs_work_doubles(nc) doubles; ticket: gs_tickets(nc)

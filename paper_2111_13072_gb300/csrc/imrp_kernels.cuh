@@ -337,6 +337,12 @@ __host__ __device__ constexpr double leg_g(int l) { return double(l) * l / (4.0 
 __host__ __device__ constexpr double leg_eps(int l) { return l == 0 ? 1.0 : double(2 * l - 1) * leg_c(l - 1); }
 __host__ __device__ constexpr double leg_r(int l) { return leg_eps(l - 1) / leg_eps(l + 1); }
 
+// u_asy(t_n) cdrive[l] and the kick weight of the step, in T.
+__device__ __forceinline__ float drive_of(const FieldArgs<float>& a, int l) { return a.st->drive_f[l]; }
+__device__ __forceinline__ double drive_of(const FieldArgs<double>& a, int l) { return a.st->u * a.cdrive[l]; }
+__device__ __forceinline__ float kick_of(const FieldArgs<float>& a) { return a.st->kick_f; }
+__device__ __forceinline__ double kick_of(const FieldArgs<double>& a) { return a.st->kick; }
+
 // One warp per tile. Phase 1 forms the tile's expansion coefficients, phase 2
 // their gradients (ladder identities) in shared memory, phase 3 evaluates the
 // far field of all other tiles, the near field of the pairs inside the tile,
@@ -362,8 +368,6 @@ __device__ __forceinline__ void field_tile(const FieldArgs<T>& a, unsigned char*
   T* sc = reinterpret_cast<T*>(reinterpret_cast<V2*>(reinterpret_cast<V4*>(smem_raw) + size_t(wpb) * CH) +
                                size_t(wpb) * CH) + size_t(warp) * (NC + 2);
   const int64_t g = tile / kTilesPerGroup;
-  const double u_drive = a.st->u;
-  const T kick = T(a.st->kick);
   const double q_s = a.q_s + a.st->qs_acc;  // with the charge absorbed at the probe so far
   const bool img_in_tile = img_in_tile_for<T>(0) && a.img_in_tile;  // FP32 contexts only
 
@@ -382,7 +386,7 @@ __device__ __forceinline__ void field_tile(const FieldArgs<T>& a, unsigned char*
   // with the gradient's scale -pf (and 1/r_out for Rs) applied, and the zero slot.
   // The loop has a fixed trip count and is unrolled, so that all loads of the
   // scan carries are in flight at once.
-  const T mpf = T(-a.pf), mpfr = T(-a.pf) * a.rho_inv;
+  const T mpf = a.mpf, mpfr = a.mpfr;
   if (lane == 0) { sc[NC] = T(0); sc[NC + 1] = T(0); }
   {
     const V2* pt = reinterpret_cast<const V2*>(a.pfx + tile * NC);  // [tile][u]: (A, B) pairs
@@ -404,7 +408,7 @@ __device__ __forceinline__ void field_tile(const FieldArgs<T>& a, unsigned char*
         // other tiles when the own tile's image pairs are summed directly
         const T W = img_in_tile ? a.tot[2 * e + 1] - at[(2 * e + 1) * ts] : a.tot[2 * e + 1];
         T cI = rl * A - a.f[l] * W;
-        if ((cr >> 8) & 1) cI += T(u_drive * a.cdrive[l]);
+        if ((cr >> 8) & 1) cI += drive_of(a, l);
         T cR = rl * B;
         if (a.m0_only && ((cr >> 9) & 1)) { cI = T(0); cR = T(0); }
         sc[2 * e] = cI * mpf;
@@ -846,7 +850,7 @@ __device__ __forceinline__ void field_tile(const FieldArgs<T>& a, unsigned char*
       Nx += ir * Gx; Ny += ir * Gy; Nz += ir * Gz;
     }
     // E = -pf sum_i q_i grad phi (N holds the sum weighted by -q_i)
-    const T pfT = T(a.pf);
+    const T pfT = a.pf_t;
     Ex += pfT * Nx; Ey += pfT * Ny; Ez += pfT * Nz;
   }
 
@@ -890,12 +894,12 @@ __device__ __forceinline__ void field_tile(const FieldArgs<T>& a, unsigned char*
       }
       qmob = a.qgbase[g] + a.qpfx[tile] + (incl - qc);
     } else {
-      qmob = -double(j);  // j electrons inside
+      qmob = -double(int32_t(j));  // j electrons inside (j < N <= 2^31)
     }
     const double qin = qion + (q_s + qmob);
-    const T er = T(qin) * (T(a.pf) * ir2 * ir);  // multiplies x (gives r^ / r^2)
+    const T er = T(qin) * (a.pf_t * ir2 * ir);  // multiplies x (gives r^ / r^2)
     Ex += er * X; Ey += er * Y; Ez += er * Z;
-    const int self_sign = img_in_tile ? (a.self_image ? 1 : 0) : (a.self_image ? 0 : -1);
+    const int self_sign = a.self_sign;
     if (self_sign != 0 && a.m0_only) {
       // own image with the m = 0 kernel: pf sum_l f_l r^{-(2l+3)} [(l+1) P_l^2 r^ - P_l P_l' (z^ - u r^)]
       const T u = Z * ir;
@@ -912,7 +916,7 @@ __device__ __forceinline__ void field_tile(const FieldArgs<T>& a, unsigned char*
         hr += a.f[l] * T(l + 1) * P * P * rp;
         ha += a.f[l] * P * D * rp;
       }
-      const T pfT = T(self_sign * a.pf) * qneg;
+      const T pfT = a.self_pf * qneg;
       // r^ = x / r, z^ - u r^ = (0, 0, 1) - u x / r
       Ex += pfT * (hr * X * ir + ha * u * X * ir);
       Ey += pfT * (hr * Y * ir + ha * u * Y * ir);
@@ -922,7 +926,7 @@ __device__ __forceinline__ void field_tile(const FieldArgs<T>& a, unsigned char*
       T h = T(0);
 #pragma unroll
       for (int l = L; l >= 1; --l) h = h * ir2 + a.f[l] * T(l + 1);
-      const T es = T(self_sign * a.pf) * qneg * h * ir2 * ir2 * ir2;  // r^{-(2l+3)} r^ = ir2^{l-1} ir2^3 x
+      const T es = a.self_pf * qneg * h * ir2 * ir2 * ir2;  // r^{-(2l+3)} r^ = ir2^{l-1} ir2^3 x
       Ex += es * X; Ey += es * Y; Ez += es * Z;
     }
   }
@@ -937,6 +941,7 @@ __device__ __forceinline__ void field_tile(const FieldArgs<T>& a, unsigned char*
   }
   if (!valid) return;
 
+  const T kick = kick_of(a);
   // ---- leapfrog: v += kick (q/m) E (q/m = -1 for an electron); x += dt v
   if (is_ion) {
     const T kq = kick * a.qm_ion;
@@ -952,7 +957,7 @@ __device__ __forceinline__ void field_tile(const FieldArgs<T>& a, unsigned char*
     bool hit = false;
     {
       const T rt = X * X + Y * Y + Z * Z;
-      const bool near_wall = rt < T(1.0 + 1e-5) || rt > T(a.r_out2 * (1.0 - 1e-5));
+      const bool near_wall = rt < T(1.0 + 1e-5) || rt > a.near_hi;
       if (near_wall) {  // the exact test in FP64 only near a wall
         const double xd = double(X), yd = double(Y), zd = double(Z);
         rr = xd * xd + yd * yd + zd * zd;  // exact for FP32 positions

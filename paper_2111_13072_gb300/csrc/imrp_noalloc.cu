@@ -188,7 +188,10 @@ int run(const imrp_params* p, const double* x, int64_t n, int64_t step, double* 
   fa.sigma = p->width_wpe;
   fa.t0 = p->t0_wpe > 0 ? p->t0_wpe : 4.0 * p->width_wpe;
   fa.dt = p->dt;
-  for (int l = 0; l < kTabL; ++l) fa.canti[l] = canti[l];
+  for (int l = 0; l < kTabL; ++l) {
+    fa.canti[l] = canti[l];
+    fa.cdrive[l] = canti[l] * 4.0 * kPi * n_tilde;
+  }
   launch_group_scan<T>(static_cast<double*>(P(o.gagg)), static_cast<double*>(P(o.gswork)),
                        static_cast<unsigned*>(P(o.gsticket)), static_cast<T*>(P(o.gbase)),
                        static_cast<T*>(P(o.tot)), static_cast<double*>(P(o.totd)), ngroups, nc, 32, &fa, seq);
@@ -230,6 +233,7 @@ int run(const imrp_params* p, const double* x, int64_t n, int64_t step, double* 
     rl *= r_out;
     a.cdrive[l] = canti[l] * 4.0 * kPi * n_tilde;
   }
+  derive_field_args(a);
   ks->field(a, 1, seq);  // at most 512 tiles: one per CTA spreads them over the SMs
   const T* eo = static_cast<const T*>(P(o.eout));
   const T* cs[3] = {eo, eo + n, eo + 2 * n};
