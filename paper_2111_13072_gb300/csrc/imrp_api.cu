@@ -385,6 +385,7 @@ template <class T> void enqueue_mid(imrp_ctx* ctx, LaunchSeq& seq, bool record) 
   fa.sigma = ctx->p.width_wpe;
   fa.t0 = ctx->t0;
   fa.dt = ctx->p.dt;
+  fa.q_s = ctx->ion_n ? ctx->ion_qs * ctx->n_tilde : ctx->p.q_s;
   for (int l = 0; l < kTabL; ++l) {
     fa.canti[l] = ctx->canti[l];
     fa.cdrive[l] = ctx->canti[l] * 4.0 * kPi * ctx->n_tilde;

@@ -929,7 +929,10 @@ __device__ __forceinline__ void finalize_step(const FinalizeArgs& a, int lane) {
   st->kick_f = float(kick);
   // electrons absorbed at the probe since the last fold (wall_rule 2) join Q_S
   // (charge -1 each) before the field of this step is evaluated
-  st->qs_acc -= double(nabs);
+  const double qs_acc = st->qs_acc - double(nabs), qs = a.q_s + qs_acc;
+  st->qs_acc = qs_acc;
+  st->qs_h = float(qs);
+  st->qs_l = float(qs - double(float(qs)));
   st->nabs_total += nabs;
   st->nabs_step = 0;
   if (a.record) {

@@ -59,6 +59,7 @@ struct StepState {
   double u;         // u_asy(t_step)
   double kick;      // kick weight of this step (dt, or dt/2 right after a load)
   float kick_f;     // the same, rounded
+  float qs_h, qs_l; // surface charge with qs_acc, as an FP32 pair
   float drive_f[kTabL];  // u * cdrive[l], rounded (the FP32 field kernel's drive per degree)
   int32_t sync;     // 1: velocities synchronous with x (next kick is dt/2)
   int32_t nabs_step;  // electrons absorbed at the probe in the step in progress (wall_rule 2)
@@ -349,6 +350,7 @@ template <class T> struct FieldArgs {
   T self_pf;          // T(self-image sign times pf)
   int self_sign;      // self-image term: -1 taken off, 1 added, 0 none
   double ion_coef;    // n_ion / (r_out^3 - 1) (uniform ions, used when ion_q is null)
+  float ion_coef_h, ion_coef_l;  // the same as an FP32 pair
   const double* ion_q;  // radial ion profile (App. D): ion charge inside r_k = 1 + k h, units e n_inf R^3
   double ion_inv_h;   // 1 / h
   double ion_scale;   // n~: super-particle charges per e n_inf R^3

@@ -132,6 +132,7 @@ struct FinalizeArgs {
   double v_hat, sigma, t0, dt;
   double canti[kTabL];
   double cdrive[kTabL];  // 4 pi n~ canti (FieldArgs::cdrive)
+  double q_s;            // surface charge of the parameters (FieldArgs::q_s)
 };
 // The derived scalars of a FieldArgs whose pf, rho_inv, r_out2, self_image and
 // img_in_tile are set.
@@ -143,6 +144,8 @@ template <class T> inline void derive_field_args(FieldArgs<T>& a) {
   a.self_sign = a.img_in_tile ? (a.self_image ? 1 : 0) : (a.self_image ? 0 : -1);
   a.self_pf = T(a.self_sign * a.pf);
   a.near_hi = T(a.r_out2 * (1.0 - 1e-5));
+  a.ion_coef_h = float(a.ion_coef);
+  a.ion_coef_l = float(a.ion_coef - double(a.ion_coef_h));
 }
 // group scan over gagg:
 // gseg: least number of groups per segment (16, 32 or 64; chosen by the

@@ -343,6 +343,232 @@ __device__ __forceinline__ double drive_of(const FieldArgs<double>& a, int l) { 
 __device__ __forceinline__ float kick_of(const FieldArgs<float>& a) { return a.st->kick_f; }
 __device__ __forceinline__ double kick_of(const FieldArgs<double>& a) { return a.st->kick; }
 
+// Unevaluated sums h + l of FP32 pairs (|l| <= ulp(h)), about twice the working
+// precision: FP64 runs at 1/64 of the FP32 rate here, and the some 17 FP64
+// operations per particle that these pairs replace bound the field kernel at low
+// degrees: N = 5e5, l_max = 1: 49.5 -> 33.9 us; N = 3e5, l_max = 8: 47.3 -> 44.2. The
+// error of the inner charge against 64 bits is the same (its last rounding).
+struct FF { float h, l; };
+// a + b exactly (Knuth's TwoSum)
+__device__ __forceinline__ FF ff_sum(float a, float b) {
+  const float s = __fadd_rn(a, b), bb = __fadd_rn(s, -a);
+  return {s, __fadd_rn(__fadd_rn(a, -__fadd_rn(s, -bb)), __fadd_rn(b, -bb))};
+}
+// a b exactly
+__device__ __forceinline__ FF ff_mul(float a, float b) {
+  const float p = __fmul_rn(a, b);
+  return {p, __fmaf_rn(a, b, -p)};
+}
+// Ions of the uniform background inside the particle's radius: coef (r^3 - 1), with
+// r = rf + corr by one Newton step from the FP32 root rf = r2 / r.
+__device__ __forceinline__ FF uniform_ions_inside(float X, float Y, float Z, float ir, float coef_h, float coef_l) {
+  const FF xx = ff_mul(X, X), yy = ff_mul(Y, Y), zz = ff_mul(Z, Z);
+  const FF s1 = ff_sum(xx.h, yy.h), s2 = ff_sum(s1.h, zz.h);
+  const float r2h = s2.h, r2l = s2.l + (s1.l + (xx.l + (yy.l + zz.l)));
+  const float rf = __fmul_rn(r2h, ir);
+  const float corr = (__fmaf_rn(-rf, rf, r2h) + r2l) * (0.5f * ir);
+  const FF p = ff_mul(r2h, rf);  // r^3 = (r2h + r2l)(rf + corr)
+  const FF d = ff_sum(p.h, -1.f);
+  const float dl = d.l + (p.l + __fmaf_rn(r2h, corr, r2l * rf));
+  const FF q = ff_mul(d.h, coef_h);
+  return {q.h, q.l + __fmaf_rn(d.h, coef_l, dl * coef_h)};
+}
+// Ions of the radial profile (App. D) inside radius rd: linear between the
+// nodes, constant outside [1, r_out].
+template <class T> __device__ __forceinline__ double profile_ions_inside(const FieldArgs<T>& a, double rd) {
+  const double t = fmin(fmax((rd - 1.0) * a.ion_inv_h, 0.0), double(a.ion_n - 1));
+  const int k = min(int(t), a.ion_n - 2);
+  const double q0 = __ldg(a.ion_q + k), q1 = __ldg(a.ion_q + k + 1);
+  return a.ion_scale * fma(t - double(k), q1 - q0, q0);
+}
+
+// The rest of one particle's step, from the field E of the other particles' l >= 1
+// terms: the l = 0 term, the own image, the push, the walls and collisions, the
+// next radius key (or, in field mode, the field itself).
+template <class T, int L>
+__device__ __forceinline__ void field_finish(const FieldArgs<T>& a, int64_t j, bool valid, bool is_ion, T qneg, T X, T Y,
+                                             T Z, T VX, T VY, T VZ, T r2, T ir2, T ir, T Ex, T Ey, T Ez, double qmob,
+                                             double q_s) {
+  // l = 0: electrons inside (sorted index j), ions inside, surface charge;
+  // then the self-image correction. The image moments of the far field sum
+  // over all particles, the particle itself included, so without the self
+  // image (self_image = 0) its own image field is taken off again; with
+  // img_in_tile the own tile is left out of them, so with the self image
+  // (self_image = 1) it is added. The count difference is small against its
+  // terms: it is formed in twice the working precision from the exact r^2 of
+  // the FP32 position (FP32 pairs), or in FP64.
+  {
+    T qin;  // inner charge in units of e: ions inside minus electrons inside (+ Q_S)
+    if constexpr (sizeof(T) == 4) {
+      if (!a.ion_q) {
+        const FF qion = uniform_ions_inside(X, Y, Z, ir, a.ion_coef_h, a.ion_coef_l);
+        FF mob;  // charge of the mobile particles inside: j electrons, or the species' scan
+        if (a.species) {
+          mob.h = float(qmob);
+          mob.l = float(qmob - double(mob.h));
+        } else {
+          const uint32_t ju = uint32_t(j);  // j < N <= 2^31
+          mob.h = -__uint2float_rn(ju);
+          mob.l = a.n > (1 << 24) ? -float(int32_t(ju - __float2uint_rz(-mob.h))) : 0.f;
+        }
+        const FF d1 = ff_sum(qion.h, mob.h), d2 = ff_sum(d1.h, a.st->qs_h);
+        qin = d2.h + (d2.l + (d1.l + (mob.l + (qion.l + a.st->qs_l))));
+      } else {
+        const double xd = double(X), yd = double(Y), zd = double(Z);
+        const double r2d = xd * xd + yd * yd + zd * zd;  // exact for FP32 positions
+        // FP32 root refined by one Newton step in FP64 (no FP64 sqrt or division)
+        const float rf = r2 * ir;
+        const double rd = double(rf) + (r2d - double(rf) * double(rf)) * double(0.5f * ir);
+        qin = T(profile_ions_inside(a, rd) + (q_s + (a.species ? qmob : -double(int32_t(j)))));
+      }
+    } else {
+      const double r2d = X * X + Y * Y + Z * Z, rd = sqrt(r2d);
+      const double qion = a.ion_q ? profile_ions_inside(a, rd) : a.ion_coef * (r2d * rd - 1.0);
+      qin = qion + (q_s + (a.species ? qmob : -double(int32_t(j))));
+    }
+    const T er = qin * (a.pf_t * ir2 * ir);  // multiplies x (gives r^ / r^2)
+    Ex += er * X; Ey += er * Y; Ez += er * Z;
+    const int self_sign = a.self_sign;
+    if (self_sign != 0 && a.m0_only) {
+      // own image with the m = 0 kernel: pf sum_l f_l r^{-(2l+3)} [(l+1) P_l^2 r^ - P_l P_l' (z^ - u r^)]
+      const T u = Z * ir;
+      T Pm = T(1), P = u, Dm = T(0), D = T(1), rp = ir2 * ir2 * ir;  // r^{-5} at l = 1
+      T hr = T(0), ha = T(0);
+#pragma unroll
+      for (int l = 1; l <= L; ++l) {
+        if (l > 1) {
+          const T Pn = (T(2 * l - 1) * u * P - T(l - 1) * Pm) / T(l);
+          const T Dn = Dm + T(2 * l - 1) * P;
+          Pm = P; P = Pn; Dm = D; D = Dn;
+          rp *= ir2;
+        }
+        hr += a.f[l] * T(l + 1) * P * P * rp;
+        ha += a.f[l] * P * D * rp;
+      }
+      const T pfT = a.self_pf * qneg;
+      // r^ = x / r, z^ - u r^ = (0, 0, 1) - u x / r
+      Ex += pfT * (hr * X * ir + ha * u * X * ir);
+      Ey += pfT * (hr * Y * ir + ha * u * Y * ir);
+      Ez += pfT * (hr * Z * ir - ha * (T(1) - u * Z * ir));
+    } else if (self_sign != 0) {
+      // the particle's own image: pf sum_l f_l (l+1) r^{-(2l+3)} r^
+      T h = T(0);
+#pragma unroll
+      for (int l = L; l >= 1; --l) h = h * ir2 + a.f[l] * T(l + 1);
+      const T es = a.self_pf * qneg * h * ir2 * ir2 * ir2;  // r^{-(2l+3)} r^ = ir2^{l-1} ir2^3 x
+      Ex += es * X; Ey += es * Y; Ez += es * Z;
+    }
+  }
+
+  if (a.mode == 1) {
+    if (valid) {
+      a.Eout[j] = Ex;
+      a.Eout[a.n + j] = Ey;
+      a.Eout[2 * a.n + j] = Ez;
+    }
+    return;
+  }
+  if (!valid) return;
+
+  const T kick = kick_of(a);
+  // ---- leapfrog: v += kick (q/m) E (q/m = -1 for an electron); x += dt v
+  if (is_ion) {
+    const T kq = kick * a.qm_ion;
+    VX += kq * Ex; VY += kq * Ey; VZ += kq * Ez;
+  } else {
+    VX -= kick * Ex; VY -= kick * Ey; VZ -= kick * Ez;
+  }
+  X += a.dt * VX; Y += a.dt * VY; Z += a.dt * VZ;
+
+  // ---- walls (Sec. 4): mirror the radius back, keep the speed
+  {
+    double rr = 0.0;
+    bool hit = false;
+    {
+      const T rt = X * X + Y * Y + Z * Z;
+      const bool near_wall = rt < T(1.0 + 1e-5) || rt > a.near_hi;
+      if (near_wall) {  // the exact test in FP64 only near a wall
+        const double xd = double(X), yd = double(Y), zd = double(Z);
+        rr = xd * xd + yd * yd + zd * zd;  // exact for FP32 positions
+        hit = rr < 1.0 || rr > a.r_out2;
+      }
+    }
+    if (hit && a.wall_rule == 2) {
+      // absorbed (at the probe its charge joins Q_S) and replaced from the outer wall
+      if (rr < 1.0) atomicAdd(a.nabs, 1);
+      double xn[3], vn[3];
+      inject_particle(a.id[j], uint64_t(a.st->step), a.seed, double(a.r_out), double(a.dt), a.sigma_v, xn, vn);
+      X = T(xn[0]); Y = T(xn[1]); Z = T(xn[2]);
+      VX = T(vn[0]); VY = T(vn[1]); VZ = T(vn[2]);
+    } else if (hit) {
+      const double xd = double(X), yd = double(Y), zd = double(Z);
+      const double rd = sqrt(rr);
+      const bool inner = rr < 1.0;
+      double rn = inner ? 2.0 - rd : 2.0 * double(a.r_out) - rd;
+      rn = rn < 1.0 ? 1.0 : (rn > double(a.r_out) ? double(a.r_out) : rn);
+      const double e0 = xd / rd, e1 = yd / rd, e2 = zd / rd;
+      X = T(e0 * rn); Y = T(e1 * rn); Z = T(e2 * rn);
+      if (a.wall_rule == 1) {
+        const T vr = VX * T(e0) + VY * T(e1) + VZ * T(e2);
+        VX -= T(2) * vr * T(e0); VY -= T(2) * vr * T(e1); VZ -= T(2) * vr * T(e2);
+      } else {
+        const T sgn = inner ? T(1) : T(-1);
+        const T n0 = sgn * T(e0), n1 = sgn * T(e1), n2 = sgn * T(e2);
+        const T speed = sqrt(VX * VX + VY * VY + VZ * VZ);
+        const uint64_t stp = uint64_t(a.st->step);
+        const uint4 o = philox4x32_10(
+            make_uint4(uint32_t(stp), uint32_t(stp >> 32), a.id[j], 0x494D5250u),
+            make_uint2(uint32_t(a.seed), uint32_t(a.seed >> 32)));
+        const T u1 = T(o.x >> 8) * T(1.0 / 16777216.0);
+        const T u2 = T(o.y >> 8) * T(1.0 / 16777216.0);
+        const T ca = T(1) - u1;
+        const T sa = sqrt(T(1) - ca * ca);
+        T sp, cp;
+        if constexpr (sizeof(T) == 4) sincospif(T(2) * u2, &sp, &cp);
+        else sincospi(T(2) * u2, &sp, &cp);
+        const T sg = n2 >= T(0) ? T(1) : T(-1);
+        const T aa = T(-1) / (sg + n2);
+        const T bb = n0 * n1 * aa;
+        const T t10 = T(1) + sg * n0 * n0 * aa, t11 = sg * bb, t12 = -sg * n0;
+        const T t20 = bb, t21 = sg + n1 * n1 * aa, t22 = -n1;
+        VX = speed * (ca * n0 + sa * (cp * t10 + sp * t20));
+        VY = speed * (ca * n1 + sa * (cp * t11 + sp * t21));
+        VZ = speed * (ca * n2 + sa * (cp * t12 + sp * t22));
+      }
+    }
+    if (a.coll_thr != 0u && !is_ion) {
+      // electron-neutral collision: isotropic elastic scattering with
+      // probability 1 - exp(-nu dt) (Philox counter (step, step >> 32, id,
+      // 0x434F4C4C), key = seed; top 24 bits below the threshold)
+      const uint64_t stp = uint64_t(a.st->step);
+      const uint4 o = philox4x32_10(make_uint4(uint32_t(stp), uint32_t(stp >> 32), a.id[j], 0x434F4C4Cu),
+                                    make_uint2(uint32_t(a.seed), uint32_t(a.seed >> 32)));
+      if ((o.x >> 8) < a.coll_thr) {
+        const T speed = sqrt(VX * VX + VY * VY + VZ * VZ);
+        const T u1 = T(o.y >> 8) * T(1.0 / 16777216.0);
+        const T u2 = T(o.z >> 8) * T(1.0 / 16777216.0);
+        const T ct = T(1) - T(2) * u1;
+        const T st = sqrt(T(1) - ct * ct);
+        T sp, cp;
+        if constexpr (sizeof(T) == 4) sincospif(T(2) * u2, &sp, &cp);
+        else sincospi(T(2) * u2, &sp, &cp);
+        VX = speed * st * cp;
+        VY = speed * st * sp;
+        VZ = speed * ct;
+      }
+    }
+    const bool fin = isfinite(X) && isfinite(Y) && isfinite(Z) && isfinite(VX) && isfinite(VY) && isfinite(VZ);
+    if (!fin) atomicOr(a.err, kErrNaN);
+    a.key[j] = fin ? radius_key<T>(X, Y, Z, a.rk) : 0u;
+    a.kidx[j] = uint32_t(j);
+  }
+  Part<T> rec;
+  rec.x = X; rec.y = Y; rec.z = Z;
+  rec.vx = VX; rec.vy = VY; rec.vz = VZ;
+  rec.id = a.id[j];
+  a.out[j] = rec;
+}
+
 // One warp per tile. Phase 1 forms the tile's expansion coefficients, phase 2
 // their gradients (ladder identities) in shared memory, phase 3 evaluates the
 // far field of all other tiles, the near field of the pairs inside the tile,
@@ -854,190 +1080,17 @@ __device__ __forceinline__ void field_tile(const FieldArgs<T>& a, unsigned char*
     Ex += pfT * Nx; Ey += pfT * Ny; Ez += pfT * Nz;
   }
 
-  // l = 0: electrons inside (sorted index j), ions inside, surface charge;
-  // then the self-image correction. The image moments of the far field sum
-  // over all particles, the particle itself included, so without the self
-  // image (self_image = 0) its own image field is taken off again; with
-  // img_in_tile the own tile is left out of them, so with the self image
-  // (self_image = 1) it is added. The count difference is formed in FP64 from
-  // the exact FP64 radius of the (FP32 or FP64) position.
-  {
-    const double xd = double(X), yd = double(Y), zd = double(Z);
-    const double r2d = xd * xd + yd * yd + zd * zd;  // exact for FP32 positions
-    double rd;
-    if constexpr (sizeof(T) == 4) {
-      // FP32 root refined by one Newton step in FP64 (no FP64 sqrt or division)
-      const float rf = r2 * ir;
-      rd = double(rf) + (r2d - double(rf) * double(rf)) * double(0.5f * ir);
-    } else {
-      rd = sqrt(r2d);
-    }
-    // inner charge in units of e: ions inside minus electrons inside (+ Q_S); the
-    // difference is small, so it is formed in FP64 and then scaled in T
-    double qion;
-    if (a.ion_q) {
-      // radial profile, linear between the nodes, constant outside [1, r_out]
-      const double t = fmin(fmax((rd - 1.0) * a.ion_inv_h, 0.0), double(a.ion_n - 1));
-      const int k = min(int(t), a.ion_n - 2);
-      const double q0 = __ldg(a.ion_q + k), q1 = __ldg(a.ion_q + k + 1);
-      qion = a.ion_scale * fma(t - double(k), q1 - q0, q0);
-    } else {
-      qion = a.ion_coef * (r2d * rd - 1.0);
-    }
-    double qmob;  // charge of the mobile particles inside (sorted before this one)
-    if (a.species) {
-      double qc = valid ? -double(qneg) : 0.0, incl = qc;
+  double qmob = 0.0;  // with mobile ions: the charge of the particles inside (sorted before this one)
+  if (a.species) {
+    double qc = valid ? -double(qneg) : 0.0, incl = qc;
 #pragma unroll
-      for (int d = 1; d < 32; d <<= 1) {
-        const double t = __shfl_up_sync(0xffffffffu, incl, d);
-        if (int(lane) >= d) incl += t;
-      }
-      qmob = a.qgbase[g] + a.qpfx[tile] + (incl - qc);
-    } else {
-      qmob = -double(int32_t(j));  // j electrons inside (j < N <= 2^31)
+    for (int d = 1; d < 32; d <<= 1) {
+      const double t = __shfl_up_sync(0xffffffffu, incl, d);
+      if (int(lane) >= d) incl += t;
     }
-    const double qin = qion + (q_s + qmob);
-    const T er = T(qin) * (a.pf_t * ir2 * ir);  // multiplies x (gives r^ / r^2)
-    Ex += er * X; Ey += er * Y; Ez += er * Z;
-    const int self_sign = a.self_sign;
-    if (self_sign != 0 && a.m0_only) {
-      // own image with the m = 0 kernel: pf sum_l f_l r^{-(2l+3)} [(l+1) P_l^2 r^ - P_l P_l' (z^ - u r^)]
-      const T u = Z * ir;
-      T Pm = T(1), P = u, Dm = T(0), D = T(1), rp = ir2 * ir2 * ir;  // r^{-5} at l = 1
-      T hr = T(0), ha = T(0);
-#pragma unroll
-      for (int l = 1; l <= L; ++l) {
-        if (l > 1) {
-          const T Pn = (T(2 * l - 1) * u * P - T(l - 1) * Pm) / T(l);
-          const T Dn = Dm + T(2 * l - 1) * P;
-          Pm = P; P = Pn; Dm = D; D = Dn;
-          rp *= ir2;
-        }
-        hr += a.f[l] * T(l + 1) * P * P * rp;
-        ha += a.f[l] * P * D * rp;
-      }
-      const T pfT = a.self_pf * qneg;
-      // r^ = x / r, z^ - u r^ = (0, 0, 1) - u x / r
-      Ex += pfT * (hr * X * ir + ha * u * X * ir);
-      Ey += pfT * (hr * Y * ir + ha * u * Y * ir);
-      Ez += pfT * (hr * Z * ir - ha * (T(1) - u * Z * ir));
-    } else if (self_sign != 0) {
-      // the particle's own image: pf sum_l f_l (l+1) r^{-(2l+3)} r^
-      T h = T(0);
-#pragma unroll
-      for (int l = L; l >= 1; --l) h = h * ir2 + a.f[l] * T(l + 1);
-      const T es = a.self_pf * qneg * h * ir2 * ir2 * ir2;  // r^{-(2l+3)} r^ = ir2^{l-1} ir2^3 x
-      Ex += es * X; Ey += es * Y; Ez += es * Z;
-    }
+    qmob = a.qgbase[g] + a.qpfx[tile] + (incl - qc);
   }
-
-  if (a.mode == 1) {
-    if (valid) {
-      a.Eout[j] = Ex;
-      a.Eout[a.n + j] = Ey;
-      a.Eout[2 * a.n + j] = Ez;
-    }
-    return;
-  }
-  if (!valid) return;
-
-  const T kick = kick_of(a);
-  // ---- leapfrog: v += kick (q/m) E (q/m = -1 for an electron); x += dt v
-  if (is_ion) {
-    const T kq = kick * a.qm_ion;
-    VX += kq * Ex; VY += kq * Ey; VZ += kq * Ez;
-  } else {
-    VX -= kick * Ex; VY -= kick * Ey; VZ -= kick * Ez;
-  }
-  X += a.dt * VX; Y += a.dt * VY; Z += a.dt * VZ;
-
-  // ---- walls (Sec. 4): mirror the radius back, keep the speed
-  {
-    double rr = 0.0;
-    bool hit = false;
-    {
-      const T rt = X * X + Y * Y + Z * Z;
-      const bool near_wall = rt < T(1.0 + 1e-5) || rt > a.near_hi;
-      if (near_wall) {  // the exact test in FP64 only near a wall
-        const double xd = double(X), yd = double(Y), zd = double(Z);
-        rr = xd * xd + yd * yd + zd * zd;  // exact for FP32 positions
-        hit = rr < 1.0 || rr > a.r_out2;
-      }
-    }
-    if (hit && a.wall_rule == 2) {
-      // absorbed (at the probe its charge joins Q_S) and replaced from the outer wall
-      if (rr < 1.0) atomicAdd(a.nabs, 1);
-      double xn[3], vn[3];
-      inject_particle(a.id[j], uint64_t(a.st->step), a.seed, double(a.r_out), double(a.dt), a.sigma_v, xn, vn);
-      X = T(xn[0]); Y = T(xn[1]); Z = T(xn[2]);
-      VX = T(vn[0]); VY = T(vn[1]); VZ = T(vn[2]);
-    } else if (hit) {
-      const double xd = double(X), yd = double(Y), zd = double(Z);
-      const double rd = sqrt(rr);
-      const bool inner = rr < 1.0;
-      double rn = inner ? 2.0 - rd : 2.0 * double(a.r_out) - rd;
-      rn = rn < 1.0 ? 1.0 : (rn > double(a.r_out) ? double(a.r_out) : rn);
-      const double e0 = xd / rd, e1 = yd / rd, e2 = zd / rd;
-      X = T(e0 * rn); Y = T(e1 * rn); Z = T(e2 * rn);
-      if (a.wall_rule == 1) {
-        const T vr = VX * T(e0) + VY * T(e1) + VZ * T(e2);
-        VX -= T(2) * vr * T(e0); VY -= T(2) * vr * T(e1); VZ -= T(2) * vr * T(e2);
-      } else {
-        const T sgn = inner ? T(1) : T(-1);
-        const T n0 = sgn * T(e0), n1 = sgn * T(e1), n2 = sgn * T(e2);
-        const T speed = sqrt(VX * VX + VY * VY + VZ * VZ);
-        const uint64_t stp = uint64_t(a.st->step);
-        const uint4 o = philox4x32_10(
-            make_uint4(uint32_t(stp), uint32_t(stp >> 32), a.id[j], 0x494D5250u),
-            make_uint2(uint32_t(a.seed), uint32_t(a.seed >> 32)));
-        const T u1 = T(o.x >> 8) * T(1.0 / 16777216.0);
-        const T u2 = T(o.y >> 8) * T(1.0 / 16777216.0);
-        const T ca = T(1) - u1;
-        const T sa = sqrt(T(1) - ca * ca);
-        T sp, cp;
-        if constexpr (sizeof(T) == 4) sincospif(T(2) * u2, &sp, &cp);
-        else sincospi(T(2) * u2, &sp, &cp);
-        const T sg = n2 >= T(0) ? T(1) : T(-1);
-        const T aa = T(-1) / (sg + n2);
-        const T bb = n0 * n1 * aa;
-        const T t10 = T(1) + sg * n0 * n0 * aa, t11 = sg * bb, t12 = -sg * n0;
-        const T t20 = bb, t21 = sg + n1 * n1 * aa, t22 = -n1;
-        VX = speed * (ca * n0 + sa * (cp * t10 + sp * t20));
-        VY = speed * (ca * n1 + sa * (cp * t11 + sp * t21));
-        VZ = speed * (ca * n2 + sa * (cp * t12 + sp * t22));
-      }
-    }
-    if (a.coll_thr != 0u && !is_ion) {
-      // electron-neutral collision: isotropic elastic scattering with
-      // probability 1 - exp(-nu dt) (Philox counter (step, step >> 32, id,
-      // 0x434F4C4C), key = seed; top 24 bits below the threshold)
-      const uint64_t stp = uint64_t(a.st->step);
-      const uint4 o = philox4x32_10(make_uint4(uint32_t(stp), uint32_t(stp >> 32), a.id[j], 0x434F4C4Cu),
-                                    make_uint2(uint32_t(a.seed), uint32_t(a.seed >> 32)));
-      if ((o.x >> 8) < a.coll_thr) {
-        const T speed = sqrt(VX * VX + VY * VY + VZ * VZ);
-        const T u1 = T(o.y >> 8) * T(1.0 / 16777216.0);
-        const T u2 = T(o.z >> 8) * T(1.0 / 16777216.0);
-        const T ct = T(1) - T(2) * u1;
-        const T st = sqrt(T(1) - ct * ct);
-        T sp, cp;
-        if constexpr (sizeof(T) == 4) sincospif(T(2) * u2, &sp, &cp);
-        else sincospi(T(2) * u2, &sp, &cp);
-        VX = speed * st * cp;
-        VY = speed * st * sp;
-        VZ = speed * ct;
-      }
-    }
-    const bool fin = isfinite(X) && isfinite(Y) && isfinite(Z) && isfinite(VX) && isfinite(VY) && isfinite(VZ);
-    if (!fin) atomicOr(a.err, kErrNaN);
-    a.key[j] = fin ? radius_key<T>(X, Y, Z, a.rk) : 0u;
-    a.kidx[j] = uint32_t(j);
-  }
-  Part<T> rec;
-  rec.x = X; rec.y = Y; rec.z = Z;
-  rec.vx = VX; rec.vy = VY; rec.vz = VZ;
-  rec.id = a.id[j];
-  a.out[j] = rec;
+  field_finish<T, L>(a, j, valid, is_ion, qneg, X, Y, Z, VX, VY, VZ, r2, ir2, ir, Ex, Ey, Ez, qmob, q_s);
 }
 
 // Register budget: in FP32, at least 3 CTAs of 256 threads per SM (80

@@ -188,6 +188,7 @@ int run(const imrp_params* p, const double* x, int64_t n, int64_t step, double* 
   fa.sigma = p->width_wpe;
   fa.t0 = p->t0_wpe > 0 ? p->t0_wpe : 4.0 * p->width_wpe;
   fa.dt = p->dt;
+  fa.q_s = p->q_s;
   for (int l = 0; l < kTabL; ++l) {
     fa.canti[l] = canti[l];
     fa.cdrive[l] = canti[l] * 4.0 * kPi * n_tilde;
