@@ -163,7 +163,11 @@ double n_ion_of(const imrp_ctx* c, int64_t n) { return c->species ? c->sp_bg : d
 // (79 CTAs on 152 SMs); FP32 N = 1e5, l_max = 16 0.045 with one and 0.050 with
 // 4 (782 CTAs in 760 places). Beyond that the shape of create.
 constexpr int kFieldWpb[4] = {8, 4, 2, 1};
+bool uses_pairs(const imrp_ctx* c, int64_t n) {
+  return c->prec == 1 ? field_pair_rule<float>(c->L, n, c->p.m0_only) : field_pair_rule<double>(c->L, n, c->p.m0_only);
+}
 int field_wpb(const imrp_ctx* c, int64_t ntiles) {
+  if (uses_pairs(c, c->n)) return kPairWarps;
   const int64_t sms = sm_count();
   int best = c->wpb_full;
   int64_t load = INT64_MAX;
@@ -1076,7 +1080,7 @@ extern "C" int imrp_autotune(imrp_ctx* ctx, int* wpb_out, int* gseg_out) {
     for (int w : {8, 4, 2, 1}) {
       const int nb = ctx->prec == 1 ? find_set<float>(ctx->L)->field_blocks_per_sm(w)
                                     : find_set<double>(ctx->L)->field_blocks_per_sm(w);
-      if (nb < 1) continue;
+      if (nb < 1 || (uses_pairs(ctx, ctx->n) && w > kPairMaxWarps)) continue;
       ctx->wpb = w;
       float ms = 0.f;
       int rc = time_stage(ctx, 4, reps, &ms);
@@ -1113,8 +1117,9 @@ struct BatchGroup {
   void* dmom = nullptr;         // MomArgs<T>[members]
   void* dfield = nullptr;       // FieldArgs<T>[members] (push mode)
   int2* dmom_items = nullptr;   // (member, item): first the members of mom_ppt 16, then of 4
-  int2* dfield_items = nullptr; // (member, first tile of a CTA)
-  int nmom = 0, nmom_small = 0, nfield = 0;
+  int2* dfield_items = nullptr; // (member, first tile of a CTA); the members of field_pair_rule:
+                                // (member, first pair of tiles), after the others
+  int nmom = 0, nmom_small = 0, nfield = 0, npair = 0;
 };
 
 struct imrp_batch {
@@ -1180,7 +1185,7 @@ void free_groups(imrp_batch* b) {
 template <class T> int fill_group(imrp_batch* b, BatchGroup& g) {
   std::vector<MomArgs<T>> ma;
   std::vector<FieldArgs<T>> fa;
-  std::vector<int2> mi, ms, fi;
+  std::vector<int2> mi, ms, fi, pi;
   for (size_t k = 0; k < g.members.size(); ++k) {
     imrp_ctx* ctx = b->c[g.members[k]];
     ma.push_back(make_mom_args<T>(ctx));
@@ -1189,12 +1194,17 @@ template <class T> int fill_group(imrp_batch* b, BatchGroup& g) {
     const int ppt = mom_ppt(sizeof(T), ctx->n);
     const int64_t mitems = mom_blocks(ctx->n, ppt) * ma.back().parts;
     for (int64_t q = 0; q < mitems; ++q) (ppt == 16 ? mi : ms).push_back(make_int2(int(k), int(q)));
-    for (int64_t t = 0; t < ctx->ntiles; t += g.wpb) fi.push_back(make_int2(int(k), int(t)));
+    if (uses_pairs(ctx, ctx->n))
+      for (int64_t t = 0; t < (ctx->ntiles + 1) / 2; t += kPairWarps) pi.push_back(make_int2(int(k), int(t)));
+    else
+      for (int64_t t = 0; t < ctx->ntiles; t += g.wpb) fi.push_back(make_int2(int(k), int(t)));
   }
   g.nmom_small = int(ms.size());
   mi.insert(mi.end(), ms.begin(), ms.end());
   g.nmom = int(mi.size());
   g.nfield = int(fi.size());
+  g.npair = int(pi.size());
+  fi.insert(fi.end(), pi.begin(), pi.end());
   if (cudaMalloc(&g.dmom, ma.size() * sizeof(MomArgs<T>)) != cudaSuccess ||
       cudaMalloc(&g.dfield, fa.size() * sizeof(FieldArgs<T>)) != cudaSuccess ||
       cudaMalloc(&g.dmom_items, mi.size() * sizeof(int2)) != cudaSuccess ||
@@ -1273,12 +1283,15 @@ int enqueue_batch_step(imrp_batch* b) {
     cudaStreamWaitEvent(b->stream, b->join[i], 0);
   }
   for (auto& g : b->groups) {
-    if (g.prec == 1)
-      find_set<float>(g.L)->field_batch(static_cast<const FieldArgs<float>*>(g.dfield), g.dfield_items, g.nfield,
-                                        g.wpb, b->stream);
-    else
-      find_set<double>(g.L)->field_batch(static_cast<const FieldArgs<double>*>(g.dfield), g.dfield_items,
-                                         g.nfield, g.wpb, b->stream);
+    if (g.prec == 1) {
+      const KernelSet<float>* ks = find_set<float>(g.L);
+      const FieldArgs<float>* fa = static_cast<const FieldArgs<float>*>(g.dfield);
+      ks->field_batch(fa, g.dfield_items, g.nfield, g.wpb, b->stream);
+      ks->pair_batch(fa, g.dfield_items + g.nfield, g.npair, b->stream);
+    } else {
+      find_set<double>(g.L)->field_batch(static_cast<const FieldArgs<double>*>(g.dfield), g.dfield_items, g.nfield,
+                                         g.wpb, b->stream);
+    }
   }
   for (imrp_ctx* ctx : b->c) ctx->keys_valid = true;  // the field kernels wrote the next keys
   return IMRP_OK;
@@ -1399,8 +1412,11 @@ template <class T> int time_group_field(imrp_batch* b, const BatchGroup& g, int 
   for (size_t k = 0; k < g.members.size(); ++k) {
     imrp_ctx* ctx = b->c[g.members[k]];
     fa.push_back(make_field_args<T>(ctx, false));
+    if (uses_pairs(ctx, ctx->n)) continue;  // their launch has one shape
     for (int64_t t = 0; t < ctx->ntiles; t += wpb) fi.push_back(make_int2(int(k), int(t)));
   }
+  *ms = 0.f;
+  if (fi.empty()) return IMRP_OK;
   void* dfa = nullptr;
   int2* dfi = nullptr;
   int rc = IMRP_OK;

@@ -395,6 +395,18 @@ __host__ __device__ constexpr int img_in_tile_for(int64_t n) {
   return sizeof(T) == 4 && n <= kImgInTileMaxN ? 1 : 0;
 }
 
+// Whether an instance's field runs in the pair kernel (field_pair): FP32, degree 12
+// and up, enough tiles to fill the GPU several times (smaller instances keep the
+// kernel of one tile per warp, which has twice the warps), all m. A rule of n, so
+// that an instance computes the same alone and in a batch.
+constexpr int64_t kPairMinN = int64_t(1) << 19;
+constexpr int kPairMinL = 12;
+constexpr int kPairWarps = 2, kPairMaxWarps = 4;  // warps per CTA: default, at most
+template <class T> __host__ __device__ constexpr bool pair_degree(int L) { return sizeof(T) == 4 && L >= kPairMinL; }
+template <class T> __host__ __device__ constexpr bool field_pair_rule(int L, int64_t n, int m0_only) {
+  return pair_degree<T>(L) && n >= kPairMinN && !m0_only;
+}
+
 // Column chunks of the far field: chunk q of the multipole (Is) part covers
 // columns [chunkI(L, q), chunkI(L, q + 1)), greedily filled to at most kChunk
 // gradient entries; likewise for the local (Rs) part.

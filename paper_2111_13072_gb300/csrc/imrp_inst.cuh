@@ -36,6 +36,9 @@ template <class T> void fill_tables(Tables<T>& t) {
 // Host copies of the prologue tables, computed when the library is loaded
 // (fixed-size arrays: no allocation), uploaded once per device by unit_init.
 EntryRec h_ent[kEntTotal];
+PairSrc h_psrc[kRecTotal];
+float4 h_pfac[2][kRecTotal];
+float2 h_an2[kTabL * kTabL];
 uint16_t h_comp[kCompTotal];
 
 void fill_prologue_tables() {
@@ -93,7 +96,30 @@ void fill_prologue_tables() {
       for (int Lp = (M > 1 ? M : 1); Lp <= L + 1; ++Lp) h_ent[eo + idxI(L, Lp, M)] = record(true, Lp, M);
     for (int M = 0; M <= L - 1; ++M)
       for (int Lp = M; Lp <= L - 1; ++Lp) h_ent[eo + nI(L) + idxR(L, Lp, M)] = record(false, Lp, M);
+    // the pair kernel's records: the same entries, sources as complex coefficients
+    const int zero = 2 * pair_run(L);
+    for (int M = 0; M <= L + 1; ++M)
+      for (int Lp = M; Lp <= L + 1; ++Lp) {
+        const int k = rec_off(L) + offP(L, M) + Lp - M;
+        PairSrc src{};
+        for (int s = 0; s < 2; ++s) {
+          const bool have = s == 0 ? Lp >= 1 : (M <= L - 1 && Lp <= L - 1);
+          const EntryRec e = !have ? EntryRec{} : s == 0 ? h_ent[eo + idxI(L, Lp, M)] : h_ent[eo + nI(L) + idxR(L, Lp, M)];
+          const int lq = s == 0 ? Lp - 1 : Lp + 1, ms[3] = {M - 1, M + 1, M};
+          for (int q = 0; q < 3; ++q) {
+            const int am = ms[q] < 0 ? -ms[q] : ms[q];
+            src.i[3 * s + q] = int16_t(have && lq >= 1 && lq <= L && am <= lq ? pair_pos(L, lq, am, s) : zero);
+          }
+          h_pfac[s][k] = make_float4(e.s1r, e.s1i, e.s2, e.sz);
+        }
+        h_psrc[k] = src;
+      }
   }
+  for (int m = 0; m < kTabL; ++m)
+    for (int l = m; l < kTabL; ++l) {
+      const float an = float(m < l ? rec_a(l, m) * rec_nu(l - 1, m) / rec_nu(l, m) : 0.0);
+      h_an2[m * kTabL + l - m] = make_float2(an, an);
+    }
 }
 struct PrologueInit {
   PrologueInit() { fill_prologue_tables(); }
@@ -116,6 +142,14 @@ template <class T, int L> void mom_launch(const MomArgs<T>& a, LaunchSeq& seq) {
 template <class T, int L> void field_launch(const FieldArgs<T>& a, int wpb, LaunchSeq& seq) {
   const int64_t ntiles = (a.n + 31) / 32;
   const int64_t blocks = (ntiles + wpb - 1) / wpb;
+  if constexpr (pair_degree<T>(L)) {
+    if (field_pair_rule<T>(L, a.n, a.m0_only)) {
+      if (wpb > kPairMaxWarps) wpb = kPairMaxWarps;
+      const int64_t pairs = (ntiles + 1) / 2;
+      seq(k_field_pair<L>, unsigned((pairs + wpb - 1) / wpb), unsigned(wpb * 32), wpb * pair_smem_per_warp(L), a);
+      return;
+    }
+  }
   const size_t smem = size_t(wpb) * field_smem_per_warp<T>(L);
   if (blocks > 0) seq(k_field<T, L>, unsigned(blocks), unsigned(wpb * 32), smem, a);
 }
@@ -134,6 +168,14 @@ template <class T, int L>
 void field_batch_launch(const FieldArgs<T>* args, const int2* items, int nitems, int wpb, cudaStream_t s) {
   const size_t smem = size_t(wpb) * field_smem_per_warp<T>(L);
   if (nitems > 0) k_field_batch<T, L><<<unsigned(nitems), wpb * 32, smem, s>>>(args, items);
+}
+
+template <class T, int L>
+void pair_batch_launch(const FieldArgs<T>* args, const int2* items, int nitems, cudaStream_t s) {
+  if constexpr (pair_degree<T>(L)) {
+    if (nitems > 0)
+      k_field_pair_batch<L><<<unsigned(nitems), kPairWarps * 32, kPairWarps * pair_smem_per_warp(L), s>>>(args, items);
+  }
 }
 
 template <class T, int L> int field_occ(int wpb) {
@@ -160,6 +202,14 @@ template <class T, int L> cudaError_t set_attr() {
   const int fmax = int(8 * field_smem_per_warp<T>(L) > 227 * 1024 ? 227 * 1024 : 8 * field_smem_per_warp<T>(L));
   e = cudaFuncSetAttribute(k_field<T, L>, cudaFuncAttributeMaxDynamicSharedMemorySize, fmax);
   if (e != cudaSuccess) return e;
+  if constexpr (pair_degree<T>(L)) {
+    e = cudaFuncSetAttribute(k_field_pair<L>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             int(kPairMaxWarps * pair_smem_per_warp(L)));
+    if (e != cudaSuccess) return e;
+    e = cudaFuncSetAttribute(k_field_pair_batch<L>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             int(kPairWarps * pair_smem_per_warp(L)));
+    if (e != cudaSuccess) return e;
+  }
   // the batched kernel also holds one instance's arguments in static shared memory
   const int bmax = int(227 * 1024 - sizeof(FieldArgs<T>));
   return cudaFuncSetAttribute(k_field_batch<T, L>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -188,6 +238,12 @@ template <class T, int L> cudaError_t set_attr() {
     if (e != cudaSuccess) return int(e);                                                     \
     e = cudaMemcpyToSymbol(g_comp, h_comp, sizeof(h_comp));                                  \
     if (e != cudaSuccess) return int(e);                                                     \
+    if (sizeof(T) == 4) {                                                                    \
+      e = cudaMemcpyToSymbol(g_psrc, h_psrc, sizeof(h_psrc));                                \
+      if (e == cudaSuccess) e = cudaMemcpyToSymbol(g_pfac, h_pfac, sizeof(h_pfac));          \
+      if (e == cudaSuccess) e = cudaMemcpyToSymbol(c_an2, h_an2, sizeof(h_an2));             \
+      if (e != cudaSuccess) return int(e);                                                   \
+    }                                                                                        \
     cudaError_t es[] = {set_attr<T, Ls>()...};                                               \
     for (cudaError_t x : es)                                                                 \
       if (x != cudaSuccess) return int(x);                                                   \
@@ -198,7 +254,7 @@ template <class T, int L> cudaError_t set_attr() {
     KernelSet<T> ks[] = {KernelSet<T>{Ls, &mom_launch<T, Ls>, &field_launch<T, Ls>,         \
                                       &unit_init<Ls...>, field_smem_per_warp<T>(Ls),        \
                                       &field_occ<T, Ls>, &mom_batch_launch<T, Ls>,          \
-                                      &field_batch_launch<T, Ls>}...};                      \
+                                      &field_batch_launch<T, Ls>, &pair_batch_launch<T, Ls>}...};                      \
     for (auto& k : ks) v.push_back(k);                                                       \
   }                                                                                          \
   }                                                                                          \

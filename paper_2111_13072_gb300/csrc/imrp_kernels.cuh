@@ -4,6 +4,8 @@
 // recurrence tables in constant memory.
 #pragma once
 
+#include <type_traits>
+
 #include "imrp_device.cuh"
 
 namespace imrp {
@@ -55,6 +57,33 @@ __host__ __device__ constexpr int comp_tab_off(int L) {
 }
 constexpr int kEntTotal = ent_off(24) + nI(24) + nR(24);
 constexpr int kCompTotal = comp_tab_off(24) + ncomp(24);
+// Recurrence coefficients an_lm of the field's pair kernel, twice each (one
+// instruction advances two recurrences), by columns: [m][l - m].
+static __constant__ float2 c_an2[kTabL * kTabL];
+// Record offP(L, m) + l - m of the pair kernel (columns m, degrees l = m..L + 1): the
+// sources (complex coefficients at pair_pos: c1, c2, c0 of the multipole entry (l, m),
+// then of the local one) and the factors (s1r, s1i, s2, sz) of the two entries, as in
+// EntryRec; factors 0 where a part has no such entry. Arrays of 16-byte parts, so
+// that a warp's loads are contiguous.
+struct __align__(16) PairSrc { int16_t i[8]; };
+__host__ __device__ constexpr int pair_run(int L) { return L + L * (L + 1) / 2; }
+__host__ __device__ constexpr int pair_pos(int L, int l, int m, int s) {
+  return s * pair_run(L) + (m == 0 ? l - 1 : L + (m - 1) * (L + 1) - (m - 1) * m / 2 + l - m);
+}
+__host__ __device__ constexpr int nP(int L) { return nI(L) + 1; }
+__host__ __device__ constexpr int offP(int L, int m) { return m == 0 ? 0 : offI(L, m) + 1; }
+__host__ __device__ constexpr int rec_off(int L) {
+  int o = 0;
+  for (int i = 0; i < kNumDegrees; ++i) {
+    const int d = degree_at(i);
+    if (d == L) return o;
+    o += nP(d);
+  }
+  return -1;
+}
+constexpr int kRecTotal = rec_off(24) + nP(24);
+static __device__ PairSrc g_psrc[kRecTotal];
+static __device__ float4 g_pfac[2][kRecTotal];  // multipole, local
 static __device__ EntryRec g_ent[kEntTotal];
 static __device__ uint16_t g_comp[kCompTotal];  // per component: l | (drive << 8) | (m > 0) << 9
 
@@ -388,7 +417,7 @@ template <class T> __device__ __forceinline__ double profile_ions_inside(const F
 template <class T, int L>
 __device__ __forceinline__ void field_finish(const FieldArgs<T>& a, int64_t j, bool valid, bool is_ion, T qneg, T X, T Y,
                                              T Z, T VX, T VY, T VZ, T r2, T ir2, T ir, T Ex, T Ey, T Ez, double qmob,
-                                             double q_s) {
+                                             double q_s, const uint32_t* id) {
   // l = 0: electrons inside (sorted index j), ions inside, surface charge;
   // then the self-image correction. The image moments of the far field sum
   // over all particles, the particle itself included, so without the self
@@ -497,7 +526,7 @@ __device__ __forceinline__ void field_finish(const FieldArgs<T>& a, int64_t j, b
       // absorbed (at the probe its charge joins Q_S) and replaced from the outer wall
       if (rr < 1.0) atomicAdd(a.nabs, 1);
       double xn[3], vn[3];
-      inject_particle(a.id[j], uint64_t(a.st->step), a.seed, double(a.r_out), double(a.dt), a.sigma_v, xn, vn);
+      inject_particle(*id, uint64_t(a.st->step), a.seed, double(a.r_out), double(a.dt), a.sigma_v, xn, vn);
       X = T(xn[0]); Y = T(xn[1]); Z = T(xn[2]);
       VX = T(vn[0]); VY = T(vn[1]); VZ = T(vn[2]);
     } else if (hit) {
@@ -517,7 +546,7 @@ __device__ __forceinline__ void field_finish(const FieldArgs<T>& a, int64_t j, b
         const T speed = sqrt(VX * VX + VY * VY + VZ * VZ);
         const uint64_t stp = uint64_t(a.st->step);
         const uint4 o = philox4x32_10(
-            make_uint4(uint32_t(stp), uint32_t(stp >> 32), a.id[j], 0x494D5250u),
+            make_uint4(uint32_t(stp), uint32_t(stp >> 32), *id, 0x494D5250u),
             make_uint2(uint32_t(a.seed), uint32_t(a.seed >> 32)));
         const T u1 = T(o.x >> 8) * T(1.0 / 16777216.0);
         const T u2 = T(o.y >> 8) * T(1.0 / 16777216.0);
@@ -541,7 +570,7 @@ __device__ __forceinline__ void field_finish(const FieldArgs<T>& a, int64_t j, b
       // probability 1 - exp(-nu dt) (Philox counter (step, step >> 32, id,
       // 0x434F4C4C), key = seed; top 24 bits below the threshold)
       const uint64_t stp = uint64_t(a.st->step);
-      const uint4 o = philox4x32_10(make_uint4(uint32_t(stp), uint32_t(stp >> 32), a.id[j], 0x434F4C4Cu),
+      const uint4 o = philox4x32_10(make_uint4(uint32_t(stp), uint32_t(stp >> 32), *id, 0x434F4C4Cu),
                                     make_uint2(uint32_t(a.seed), uint32_t(a.seed >> 32)));
       if ((o.x >> 8) < a.coll_thr) {
         const T speed = sqrt(VX * VX + VY * VY + VZ * VZ);
@@ -565,7 +594,7 @@ __device__ __forceinline__ void field_finish(const FieldArgs<T>& a, int64_t j, b
   Part<T> rec;
   rec.x = X; rec.y = Y; rec.z = Z;
   rec.vx = VX; rec.vy = VY; rec.vz = VZ;
-  rec.id = a.id[j];
+  rec.id = *id;
   a.out[j] = rec;
 }
 
@@ -1090,7 +1119,523 @@ __device__ __forceinline__ void field_tile(const FieldArgs<T>& a, unsigned char*
     }
     qmob = a.qgbase[g] + a.qpfx[tile] + (incl - qc);
   }
-  field_finish<T, L>(a, j, valid, is_ion, qneg, X, Y, Z, VX, VY, VZ, r2, ir2, ir, Ex, Ey, Ez, qmob, q_s);
+  field_finish<T, L>(a, j, valid, is_ion, qneg, X, Y, Z, VX, VY, VZ, r2, ir2, ir, Ex, Ey, Ez, qmob, q_s, a.id + j);
+}
+
+// ----------------------------------------------------------------------------
+// Field kernel of large FP32 instances of degree 12 and up (field_pair_rule): one
+// warp per pair of tiles, half a warp per tile, two particles per lane (a: positions
+// 0..15 of the tile, b: 16..31). field_tile is bound by issue slots (77 % busy, FMA
+// pipe 52 %) and shared-memory wavefronts (58 %). Here the far field advances the
+// multipole and the local harmonic of an (l, m) in one instruction (their recurrence
+// shares its coefficients, their gradient factors lie side by side), one load serves
+// two particles, and the near field takes two pairs per instruction: 5670 instructions
+// per tile against 8370, FMA pipe 61 %, issue 60 % (ncu, N = 1e6, l_max = 16). The near
+// field runs first, while the scan carries, velocities and ids are copied to shared
+// memory. Field ms, field_tile -> this: l_max = 16, N = 2e6: 0.535 -> 0.470; l_max = 24,
+// N = 4e6: 2.376 -> 1.843; l_max = 12, N = 7e5: 0.153 -> 0.128; l_max = 8, N = 2e6: 0.227 ->
+// 0.224, l_max = 4: 0.145 -> 0.150 (not instantiated below 12).
+// ----------------------------------------------------------------------------
+// Two FP32 values advanced by one instruction.
+__device__ __forceinline__ float2 f2(float x, float y) { return make_float2(x, y); }
+__device__ __forceinline__ float2 f2(float x) { return make_float2(x, x); }
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 neg2(float2 a) { return f2(-a.x, -a.y); }
+__device__ __forceinline__ float2 sel2(bool p, float2 a, float2 b) { return f2(p ? a.x : b.x, p ? a.y : b.y); }
+
+// Constants of pair_sums, twice each: leg_c(l), l leg_c(l), -leg_g(l + 1).
+struct __align__(16) LegRec { float2 c, lc, g, pad; };
+struct LegTab { LegRec r[kTabL]; };
+constexpr LegTab leg_tab() {
+  LegTab t{};
+  for (int l = 0; l < kTabL; ++l) {
+    const float c = float(leg_c(l)), lc = float(l * leg_c(l)), g = float(-leg_g(l + 1));
+    if (l == 0) { t.r[l] = LegRec{float2{0.f, 0.f}, float2{0.f, 0.f}, float2{g, g}, float2{0.f, 0.f}}; continue; }
+    t.r[l] = LegRec{float2{c, c}, float2{lc, lc}, float2{g, g}, float2{0.f, 0.f}};
+  }
+  return t;
+}
+static __constant__ LegTab c_leg = leg_tab();
+
+// The pair sums at (x1, y2) = (s u, s^2), s = r_inner / r_outer, u the cosine
+// between the two: S0 = sum_{l=1..L} s^l P_l(u), S1 = sum l s^l P_l(u),
+// S2 = sum s^(l-1) P'_l(u), by Clenshaw's backward recurrence for the monic
+// polynomials q_l = s^l P_l / c_l (leg_g, leg_c) and its derivative in x1:
+// 7 operations per degree (the forward recurrences of q_l and P'_l and three
+// sums take 8), the same rounding error. Two sets of two pairs at once.
+template <int L>
+__device__ __forceinline__ void pair_sums(const float2 (&x1)[2], const float2 (&y2)[2], float2 (&S0)[2],
+                                          float2 (&S1)[2], float2 (&S2)[2]) {
+  float2 b2[2], d2[2], e2[2];
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    S0[k] = f2(float(leg_c(L)));
+    S1[k] = f2(float(L * leg_c(L)));
+    S2[k] = b2[k] = d2[k] = e2[k] = f2(0.f);
+  }
+  constexpr int kUnr = L == 12 ? 12 : 8;  // l_max = 12: 0.128 ms with 12, 0.133 with 8 (N = 7e5)
+#pragma unroll kUnr
+  for (int l = L - 1; l >= 0; --l) {
+    const LegRec r = c_leg.r[l];  // c = lc = 0 at l = 0
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      const float2 G = mul2(r.g, y2[k]);
+      const float2 nb = fma2(x1[k], S0[k], fma2(G, b2[k], r.c)), nd = fma2(x1[k], S1[k], fma2(G, d2[k], r.lc)),
+                   ne = fma2(x1[k], S2[k], fma2(G, e2[k], S0[k]));
+      b2[k] = S0[k]; S0[k] = nb;
+      d2[k] = S1[k]; S1[k] = nd;
+      e2[k] = S2[k]; S2[k] = ne;
+    }
+  }
+}
+
+// Records of a tile built at once, in chunks of whole columns of at most this many:
+// enough warps stay resident (l_max = 16 at N = 2e6, field ms: 96 gives 0.470 with 14
+// warps per SM, 128 0.515, 80 0.479 with one chunk more).
+constexpr int kPairCap = 96;
+__host__ __device__ constexpr int pair_cap(int L) { return kPairCap < nP(L) ? kPairCap : nP(L); }
+__host__ __device__ constexpr int pair_chunk(int L, int q) {  // first column of chunk q
+  int m = 0;
+  for (int c = 0; c < q && m <= L + 1; ++c) {
+    int acc = 0;
+    while (m <= L + 1 && acc + L + 2 - m <= pair_cap(L)) acc += L + 2 - m++;
+  }
+  return m;
+}
+__host__ __device__ constexpr int pair_nchunk(int L) {
+  int q = 0;
+  while (pair_chunk(L, q) <= L + 1) ++q;
+  return q;
+}
+__host__ __device__ constexpr int pair_most(int L) {  // records of the largest chunk
+  int most = 0;
+  for (int q = 0; q < pair_nchunk(L); ++q) {
+    const int n = offP(L, pair_chunk(L, q + 1)) - offP(L, pair_chunk(L, q));
+    most = n > most ? n : most;
+  }
+  return most;
+}
+// float4s of a tile's records (three each), so that the two tiles start half a
+// bank row apart (the two halves of a warp read different addresses at once).
+__host__ __device__ constexpr int pair_stride(int L) { return (3 * pair_most(L) + 3) / 8 * 8 + 4; }
+// The near field's particle data of the two tiles (over the entries, which are
+// done with by then): 16 records of 12 + 12 + 8 floats per tile.
+constexpr int kPairNear = 2 * 16 * 32 * 4;
+// Words of one tile's complex coefficients and their zero slot (first its row of
+// scan carries), and of the staged velocities, ids and positions of the two tiles.
+__host__ __device__ constexpr int pair_row(int L) { return (4 * pair_run(L) + 2 + 3) / 4 * 4; }
+constexpr int kPairVel = 7 * 64;
+__host__ __device__ constexpr size_t pair_smem_per_warp(int L) {
+  const size_t ent = size_t(2) * 16 * pair_stride(L);
+  return (ent > size_t(kPairNear) ? ent : size_t(kPairNear)) + size_t(4) * (2 * pair_row(L) + kPairVel);
+}
+// Asynchronous copies of 4, 8 or 16 bytes from global to shared memory.
+template <int B> __device__ __forceinline__ void copy_async(void* dst, const void* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(uint32_t(__cvta_generic_to_shared(dst))), "l"(src),
+               "n"(B)
+               : "memory");
+}
+__device__ __forceinline__ void copy_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+template <int L>
+__device__ __forceinline__ void field_pair(const FieldArgs<float>& a, unsigned char* smem_raw, int warp, int64_t pr) {
+  constexpr int NC = 2 * ncomp(L), SR = pair_stride(L);
+  const Tables<float>& tb = tab<float>();
+  const int lane = int(lane_id()), h = lane >> 4, i = lane & 15;
+  const int64_t ntiles = (a.n + 31) >> 5;
+  if (2 * pr >= ntiles) return;  // warp-uniform; no block-wide barrier below
+  unsigned char* const base = smem_raw + size_t(warp) * pair_smem_per_warp(L);
+  float4* const rec0 = reinterpret_cast<float4*>(base);
+  constexpr int SCW = pair_row(L);
+  float* const sc0 = reinterpret_cast<float*>(base + pair_smem_per_warp(L)) - (2 * SCW + kPairVel);
+  float* const vel = sc0 + 2 * SCW;  // [vx, vy, vz, id, x, y, z][64]
+  const int64_t g = 2 * pr / kTilesPerGroup;  // both tiles lie in one group
+  const int64_t tile = 2 * pr + h;
+  const double q_s = a.q_s + a.st->qs_acc;
+
+  int64_t j[2];
+  bool valid[2];
+  float X[2], Y[2], Z[2];
+#pragma unroll
+  for (int p = 0; p < 2; ++p) {
+    j[p] = tile * 32 + 16 * p + i;
+    valid[p] = j[p] < a.n;
+    X[p] = valid[p] ? a.x[j[p]] : a.r_out;  // empty places count as outermost (weight 0)
+    Y[p] = valid[p] ? a.y[j[p]] : 0.f;
+    Z[p] = valid[p] ? a.z[j[p]] : 0.f;
+  }
+
+  // the scan carries of both tiles, the velocities and ids: copied to shared memory
+  // while the near field computes
+  {
+    constexpr int B = NC % 4 == 0 ? 16 : 8, PER = NC * 4 / B;  // pieces of a row
+    const char* src = reinterpret_cast<const char*>(a.pfx + 2 * pr * NC);
+    char* const dst = reinterpret_cast<char*>(sc0);
+#pragma unroll
+    for (int k = 0; k < 2 * PER; k += 32) {
+      const int c = k + lane;
+      if (c < 2 * PER) copy_async<B>(dst + (c >= PER ? c - PER : c) * B + (c >= PER ? SCW * 4 : 0), src + c * B);
+    }
+#pragma unroll
+    for (int p = 0; p < 2; ++p) {
+      const int o = 32 * h + 16 * p + i;
+      vel[256 + o] = X[p]; vel[320 + o] = Y[p]; vel[384 + o] = Z[p];
+      if (valid[p]) {
+        copy_async<4>(vel + o, a.vx + j[p]);
+        copy_async<4>(vel + 64 + o, a.vy + j[p]);
+        copy_async<4>(vel + 128 + o, a.vz + j[p]);
+        copy_async<4>(vel + 192 + o, a.id + j[p]);
+      }
+    }
+  }
+
+  float r2[2], ir[2];
+  float2 E[2][3];  // the field: near field and multipole part, local part
+#pragma unroll
+  for (int p = 0; p < 2; ++p) {
+    r2[p] = X[p] * X[p] + Y[p] * Y[p] + Z[p] * Z[p];
+    ir[p] = rsqrtf(r2[p]);
+  }
+
+  // near field: the pairs inside each tile. Lane i of a tile holds a_i and b_i
+  // (a inner, b outer); in round t it takes (a_i, b_{i+t}) with (a_i, b_{i+t+8}), and
+  // (a_i, a_{i+t+1}) with (b_i, b_{i+t+1}), two pairs per instruction. The other
+  // end's factors go back to their lane, which applies them to the sender's
+  // direction.
+  float qneg[2];
+  bool is_ion[2];
+#pragma unroll
+  for (int p = 0; p < 2; ++p) {
+    is_ion[p] = a.species && valid[p] && a.id[j[p]] >= a.n_e;
+    qneg[p] = valid[p] ? (is_ion[p] ? -a.q_ion : 1.f) : 0.f;
+  }
+  {
+    float* const nb = reinterpret_cast<float*>(base) + h * (16 * 32);
+    float4* const PB = reinterpret_cast<float4*>(nb);            // [16][3]: (b_j, b_{j+8}) x, y, z, r, 1/r, w
+    float4* const PA = reinterpret_cast<float4*>(nb + 16 * 12);  // [16][3]: (a_j, b_j)
+    float4* const PC = reinterpret_cast<float4*>(nb + 16 * 24);  // [16][2]: (a_j, a_{j+8}) x, y, z
+    const float2 ux = f2(X[0] * ir[0], X[1] * ir[1]), uy = f2(Y[0] * ir[0], Y[1] * ir[1]),
+                 uz = f2(Z[0] * ir[0], Z[1] * ir[1]), rk = f2(r2[0] * ir[0], r2[1] * ir[1]);
+    {
+      PA[3 * i] = make_float4(ux.x, ux.y, uy.x, uy.y);
+      PA[3 * i + 1] = make_float4(uz.x, uz.y, rk.x, rk.y);
+      PA[3 * i + 2] = make_float4(ir[0], ir[1], qneg[0], qneg[1]);
+      const int i8 = (i + 8) & 15;
+      float* const pb = nb;
+      float* const pc = nb + 16 * 24;
+      pb[12 * i + 0] = ux.y; pb[12 * i + 2] = uy.y; pb[12 * i + 4] = uz.y;
+      pb[12 * i + 6] = rk.y; pb[12 * i + 8] = ir[1]; pb[12 * i + 10] = qneg[1];
+      pb[12 * i8 + 1] = ux.y; pb[12 * i8 + 3] = uy.y; pb[12 * i8 + 5] = uz.y;
+      pb[12 * i8 + 7] = rk.y; pb[12 * i8 + 9] = ir[1]; pb[12 * i8 + 11] = qneg[1];
+      pc[8 * i + 0] = ux.x; pc[8 * i + 2] = uy.x; pc[8 * i + 4] = uz.x;
+      pc[8 * i8 + 1] = ux.x; pc[8 * i8 + 3] = uy.x; pc[8 * i8 + 5] = uz.x;
+    }
+    __syncwarp();
+    const float2 irab = f2(ir[0], ir[1]), w = f2(qneg[0], qneg[1]);
+    // sums of -q grad phi: along the own direction (al) and the rest; of a (halves
+    // of the rounds), of b (halves) and of (a, b)
+    float2 aN[4] = {f2(0.f), f2(0.f), f2(0.f), f2(0.f)}, bN[4] = {f2(0.f), f2(0.f), f2(0.f), f2(0.f)},
+           cN[4] = {f2(0.f), f2(0.f), f2(0.f), f2(0.f)};
+    constexpr unsigned M = 0xffffffffu;
+#pragma unroll 1
+    for (int t = 0; t < 8; ++t) {
+      // set 0: (a_i, b_{i+t}), (a_i, b_{i+t+8}), a the inner end; set 1:
+      // (a_i, a_{i+t+1}), (b_i, b_{i+t+1})
+      const int js0 = (i + t) & 15, js1 = (i + t + 1) & 15;
+      const bool me_inner = i < js1;
+      const float4 q0 = PB[3 * js0], q1 = PB[3 * js0 + 1], q2 = PB[3 * js0 + 2];
+      const float4 o0 = PA[3 * js1], o1 = PA[3 * js1 + 1], o2 = PA[3 * js1 + 2];
+      const float2 px[2] = {f2(q0.x, q0.y), f2(o0.x, o0.y)}, py[2] = {f2(q0.z, q0.w), f2(o0.z, o0.w)},
+                   pz[2] = {f2(q1.x, q1.y), f2(o1.x, o1.y)}, pir[2] = {f2(q2.x, q2.y), f2(o2.x, o2.y)},
+                   pw[2] = {f2(q2.z, q2.w), f2(o2.z, o2.w)};
+      const float2 u[2] = {fma2(f2(ux.x), px[0], fma2(f2(uy.x), py[0], mul2(f2(uz.x), pz[0]))),
+                           fma2(ux, px[1], fma2(uy, py[1], mul2(uz, pz[1])))};
+      const float2 iro1 = sel2(me_inner, pir[1], irab);
+      const float2 sr[2] = {mul2(f2(rk.x), pir[0]), mul2(sel2(me_inner, rk, f2(o1.z, o1.w)), iro1)};
+      float2 S0[2], S1[2], S2[2];
+      {
+        const float2 x1[2] = {mul2(sr[0], u[0]), mul2(sr[1], u[1])}, y2[2] = {mul2(sr[0], sr[0]), mul2(sr[1], sr[1])};
+        pair_sums<L>(x1, y2, S0, S1, S2);
+      }
+      // gradient of phi = sum_l r_i^l / r_o^{l+1} P_l(u): at the inner end
+      // (S1 - u S') gab e_i + S' gab e_o, at the outer end -(S0 + S1 + u S') go2 e_o +
+      // S' go2 e_i, with S' = s S2, gab = 1 / (r_i r_o), go2 = 1 / r_o^2
+      float2 cin[2], cout[2], Sp[2];
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        Sp[k] = mul2(S2[k], sr[k]);
+        cin[k] = fma2(neg2(u[k]), Sp[k], S1[k]);
+        cout[k] = neg2(fma2(u[k], Sp[k], add2(S0[k], S1[k])));
+      }
+      {
+        const float2 gi = mul2(mul2(f2(ir[0]), pir[0]), pw[0]), go = mul2(mul2(pir[0], pir[0]), f2(qneg[0]));
+        const float2 be = mul2(Sp[0], gi);
+        aN[0] = fma2(be, px[0], aN[0]); aN[1] = fma2(be, py[0], aN[1]); aN[2] = fma2(be, pz[0], aN[2]);
+        aN[3] = fma2(cin[0], gi, aN[3]);
+        // to b_{i+t}, b_{i+t+8}; here from a_{i-t}, a_{i-t-8}
+        const float2 ao = mul2(cout[0], go), bo = mul2(Sp[0], go);
+        const int s1 = (i - t) & 15, s2 = (i - t + 8) & 15;
+        const float2 ra = f2(__shfl_sync(M, ao.x, s1, 16), __shfl_sync(M, ao.y, s2, 16));
+        const float2 rb = f2(__shfl_sync(M, bo.x, s1, 16), __shfl_sync(M, bo.y, s2, 16));
+        const float4 c0 = PC[2 * s1];
+        const float2 cz = *reinterpret_cast<const float2*>(&PC[2 * s1 + 1]);
+        bN[0] = fma2(rb, f2(c0.x, c0.y), bN[0]); bN[1] = fma2(rb, f2(c0.z, c0.w), bN[1]);
+        bN[2] = fma2(rb, cz, bN[2]);
+        bN[3] = add2(ra, bN[3]);
+      }
+      {
+        const float2 gab = mul2(irab, pir[1]), go2 = mul2(iro1, iro1);
+        const float2 gm = mul2(sel2(me_inner, gab, go2), pw[1]);  // at my end, with the partner's weight
+        const float2 be = mul2(Sp[1], gm);
+        cN[0] = fma2(be, px[1], cN[0]); cN[1] = fma2(be, py[1], cN[1]); cN[2] = fma2(be, pz[1], cN[2]);
+        cN[3] = fma2(sel2(me_inner, cin[1], cout[1]), gm, cN[3]);
+        if (t < 7) {  // (at t = 7 both lanes of a pair took it)
+          const float2 gp = mul2(sel2(me_inner, go2, gab), w);
+          const float2 ao = mul2(sel2(me_inner, cout[1], cin[1]), gp), bo = mul2(Sp[1], gp);
+          const int s1 = (i - t - 1) & 15;
+          const float2 ra = f2(__shfl_sync(M, ao.x, s1, 16), __shfl_sync(M, ao.y, s1, 16));
+          const float2 rb = f2(__shfl_sync(M, bo.x, s1, 16), __shfl_sync(M, bo.y, s1, 16));
+          const float4 c0 = PA[3 * s1];
+          const float2 cz = *reinterpret_cast<const float2*>(&PA[3 * s1 + 1]);
+          cN[0] = fma2(rb, f2(c0.x, c0.y), cN[0]); cN[1] = fma2(rb, f2(c0.z, c0.w), cN[1]);
+          cN[2] = fma2(rb, cz, cN[2]);
+          cN[3] = add2(ra, cN[3]);
+        }
+      }
+    }
+    const float pf = a.pf_t;
+    const float ala = cN[3].x + (aN[3].x + aN[3].y), alb = cN[3].y + (bN[3].x + bN[3].y);
+    E[0][0] = f2(pf * (cN[0].x + (aN[0].x + aN[0].y) + ala * ux.x), 0.f);
+    E[0][1] = f2(pf * (cN[1].x + (aN[1].x + aN[1].y) + ala * uy.x), 0.f);
+    E[0][2] = f2(pf * (cN[2].x + (aN[2].x + aN[2].y) + ala * uz.x), 0.f);
+    E[1][0] = f2(pf * (cN[0].y + (bN[0].x + bN[0].y) + alb * ux.y), 0.f);
+    E[1][1] = f2(pf * (cN[1].y + (bN[1].x + bN[1].y) + alb * uy.y), 0.f);
+    E[1][2] = f2(pf * (cN[2].y + (bN[2].x + bN[2].y) + alb * uz.y), 0.f);
+  }
+
+  // phase 1: the tiles' expansion coefficients (as in field_tile), in place of the
+  // copied carries. Component e goes to word e + L (2 e for m = 0) of its run of complex
+  // coefficients: a warp's stores, and the gathers of phase 2 for consecutive l, are
+  // free of bank conflicts.
+  copy_wait();
+  __syncwarp();
+  {
+    const float2* gb = reinterpret_cast<const float2*>(a.gbase + g * NC);
+    const uint16_t* ctab = g_comp + comp_tab_off(L);
+    const float mpf = a.mpf, mpfr = a.mpfr;
+    constexpr int NIT = (NC / 2 + 31) / 32;
+    float2 v[2][NIT];
+#pragma unroll
+    for (int it = 0; it < NIT; ++it) {
+      const int e = lane + 32 * it;
+      if (e < NC / 2) {
+        const uint16_t cr = ctab[e];
+        const int l = cr & 0xff;
+        const float rl = a.rhol[l];
+        const float2 gv = gb[e];
+        float im = a.f[l] * a.tot[2 * e + 1];
+        if ((cr >> 8) & 1) im -= drive_of(a, l);
+#pragma unroll
+        for (int t = 0; t < 2; ++t) {
+          const float2 c = *reinterpret_cast<const float2*>(sc0 + t * SCW + 2 * e);
+          v[t][it] = f2((rl * (gv.x + c.x) - im) * mpf, rl * (gv.y + c.y) * mpfr);
+        }
+      }
+    }
+    __syncwarp();
+#pragma unroll
+    for (int it = 0; it < NIT; ++it) {
+      const int e = lane + 32 * it;
+      if (e < NC / 2) {
+        const int o = e < L ? 2 * e : e + L;
+#pragma unroll
+        for (int t = 0; t < 2; ++t) {
+          sc0[t * SCW + o] = v[t][it].x;
+          sc0[t * SCW + 2 * pair_run(L) + o] = v[t][it].y;
+          if (e < L) sc0[t * SCW + o + 1] = sc0[t * SCW + 2 * pair_run(L) + o + 1] = 0.f;
+        }
+      }
+    }
+    if (lane < 4) sc0[(lane >> 1) * SCW + 4 * pair_run(L) + (lane & 1)] = 0.f;
+  }
+  __syncwarp();
+
+  // phase 2: the records k0 .. k1 - 1 of both tiles: per (l, m) the gradient's
+  // factors of the multipole and of the local harmonic side by side,
+  // (x, y, z of the real part), (x, y, z of the imaginary part)
+  auto build = [&](int k0, int k1) {
+    __syncwarp();
+    constexpr int NB = (pair_most(L) + 31) / 32;
+#pragma unroll 1
+    for (int it = 0; it < NB; ++it) {
+      const int k = k0 + lane + 32 * it;
+      if (k < k1) {
+        const PairSrc src = g_psrc[rec_off(L) + k];
+        const float4 fac[2] = {g_pfac[0][rec_off(L) + k], g_pfac[1][rec_off(L) + k]};
+#pragma unroll
+        for (int t = 0; t < 2; ++t) {
+          const float2* sc = reinterpret_cast<const float2*>(sc0 + t * SCW);
+          float v[2][6];
+#pragma unroll
+          for (int s = 0; s < 2; ++s) {
+            const float2 c1 = sc[src.i[3 * s]], c2 = sc[src.i[3 * s + 1]], c0 = sc[src.i[3 * s + 2]];
+            const float s1r = fac[s].x, s1i = fac[s].y, s2 = fac[s].z, sz = fac[s].w;
+            v[s][0] = s1r * c1.x + s2 * c2.x;
+            v[s][1] = s2 * c2.y - s1i * c1.y;
+            v[s][2] = sz * c0.x;
+            v[s][3] = s1i * c1.y + s2 * c2.y;
+            v[s][4] = s1r * c1.x - s2 * c2.x;
+            v[s][5] = sz * c0.y;
+          }
+          float4* o = rec0 + t * SR + 3 * (k - k0);
+          o[0] = make_float4(v[0][0], v[1][0], v[0][1], v[1][1]);
+          o[1] = make_float4(v[0][2], v[1][2], v[0][3], v[1][3]);
+          o[2] = make_float4(v[0][4], v[1][4], v[0][5], v[1][5]);
+        }
+      }
+    }
+    __syncwarp();
+  };
+  const float4* const rec = rec0 + h * SR;
+
+  // phase 3: the far field. Multipole and local harmonics share the recurrence's
+  // coefficients, so one instruction advances both (first half: Is(x), second:
+  // Rs(x / r_out), whose factors past its degrees are zero): column m is
+  // (dr + i di) times the real p_l with p_{l+1} = an zz p_l - ww p_{l-1}, and the six
+  // sums over l of a column are multiplied by its diagonal once.
+  {
+    float2 zz[2], ww[2], cx[2], cy[2], dr[2], di[2];
+#pragma unroll
+    for (int p = 0; p < 2; ++p) {
+      const float ri = a.rho_inv, ir2 = 1.f / r2[p];
+      zz[p] = f2(Z[p] * ir2, Z[p] * ri);
+      ww[p] = f2(-ir2, -(r2[p] * ri * ri));
+      cx[p] = f2(X[p] * ir2, X[p] * ri);
+      cy[p] = f2(Y[p] * ir2, Y[p] * ri);
+      dr[p] = f2(ir[p], 1.f);
+      di[p] = f2(0.f);
+    }
+#pragma unroll
+    for (int q = 0; q < pair_nchunk(L); ++q) {
+      const int m0 = pair_chunk(L, q), m1 = pair_chunk(L, q + 1), k0 = offP(L, m0);
+      build(k0, offP(L, m1));
+      if (m0 == 0) {  // the real column m = 0
+        float2 p1[2] = {dr[0], dr[1]}, p0[2] = {f2(0.f), f2(0.f)};
+        auto add = [&](int l) {
+          const float4 r0 = rec[3 * l];
+          const float2 rz = *reinterpret_cast<const float2*>(&rec[3 * l + 1]);
+#pragma unroll
+          for (int p = 0; p < 2; ++p) {
+            E[p][0] = fma2(f2(r0.x, r0.y), p1[p], E[p][0]);
+            E[p][1] = fma2(f2(r0.z, r0.w), p1[p], E[p][1]);
+            E[p][2] = fma2(rz, p1[p], E[p][2]);
+          }
+        };
+        add(0);
+#pragma unroll 2
+        for (int l = 1; l <= L + 1; ++l) {  // (unrolled whole, its products fill the registers)
+          const float2 c = c_an2[l];
+#pragma unroll
+          for (int p = 0; p < 2; ++p) {
+            const float2 pn = fma2(mul2(c, zz[p]), p1[p], mul2(ww[p], p0[p]));
+            p0[p] = p1[p]; p1[p] = pn;
+          }
+          add(l);
+        }
+      }
+#pragma unroll 1
+      for (int m = m0 > 1 ? m0 : 1; m < m1; ++m) {
+        const float2 dg = f2(tb.dg[m]);
+        const float4* rc = rec + 3 * (offP(L, m) - k0);
+        const float2* an = c_an2 + m * kTabL;
+        float2 p1[2], p0[2], S[2][3], T[2][3];
+        {
+          const float4 r0 = rc[0], r1 = rc[1], r2_ = rc[2];
+#pragma unroll
+          for (int p = 0; p < 2; ++p) {
+            const float2 ex = mul2(dg, cx[p]), ey = mul2(dg, cy[p]);
+            const float2 nr = fma2(ex, dr[p], neg2(mul2(ey, di[p]))), ni = fma2(ex, di[p], mul2(ey, dr[p]));
+            dr[p] = nr; di[p] = ni;
+            p1[p] = f2(1.f); p0[p] = f2(0.f);
+            S[p][0] = f2(r0.x, r0.y); S[p][1] = f2(r0.z, r0.w); S[p][2] = f2(r1.x, r1.y);
+            T[p][0] = f2(r1.z, r1.w); T[p][1] = f2(r2_.x, r2_.y); T[p][2] = f2(r2_.z, r2_.w);
+          }
+        }
+#pragma unroll 4
+        for (int jj = 1; jj <= L + 1 - m; ++jj) {
+          const float2 c = an[jj];
+          const float4 r0 = rc[3 * jj], r1 = rc[3 * jj + 1], r2_ = rc[3 * jj + 2];
+#pragma unroll
+          for (int p = 0; p < 2; ++p) {
+            const float2 pn = fma2(mul2(c, zz[p]), p1[p], mul2(ww[p], p0[p]));
+            p0[p] = p1[p]; p1[p] = pn;
+            S[p][0] = fma2(f2(r0.x, r0.y), pn, S[p][0]);
+            S[p][1] = fma2(f2(r0.z, r0.w), pn, S[p][1]);
+            S[p][2] = fma2(f2(r1.x, r1.y), pn, S[p][2]);
+            T[p][0] = fma2(f2(r1.z, r1.w), pn, T[p][0]);
+            T[p][1] = fma2(f2(r2_.x, r2_.y), pn, T[p][1]);
+            T[p][2] = fma2(f2(r2_.z, r2_.w), pn, T[p][2]);
+          }
+        }
+#pragma unroll
+        for (int p = 0; p < 2; ++p)
+#pragma unroll
+          for (int k = 0; k < 3; ++k) E[p][k] = fma2(dr[p], S[p][k], fma2(di[p], T[p][k], E[p][k]));
+      }
+    }
+  }
+
+  double qmob[2] = {0.0, 0.0};
+  if (a.species) {
+    const double qa = -double(qneg[0]), qb = -double(qneg[1]);  // 0 in an empty place
+    double ia = qa, ib = qb;
+#pragma unroll
+    for (int d = 1; d < 16; d <<= 1) {
+      const double ta = __shfl_up_sync(0xffffffffu, ia, d, 16), tb2 = __shfl_up_sync(0xffffffffu, ib, d, 16);
+      if (i >= d) { ia += ta; ib += tb2; }
+    }
+    const double before = a.qgbase[g] + (valid[0] ? a.qpfx[tile] : 0.0);
+    qmob[0] = before + (ia - qa);
+    qmob[1] = before + __shfl_sync(0xffffffffu, ia, 15, 16) + (ib - qb);
+  }
+#pragma unroll
+  for (int p = 0; p < 2; ++p) {
+    // the particle again (kept in shared memory meanwhile)
+    const int o = 32 * h + 16 * p + i;
+    const int64_t jp = tile * 32 + 16 * p + i;
+    const bool ok = jp < a.n;
+    const float x = vel[256 + o], y = vel[320 + o], z = vel[384 + o];
+    const uint32_t* id = reinterpret_cast<const uint32_t*>(vel + 192 + o);
+    const bool ion = a.species && ok && *id >= a.n_e;
+    const float rr = x * x + y * y + z * z;
+    field_finish<float, L>(a, jp, ok, ion, ok ? (ion ? -a.q_ion : 1.f) : 0.f, x, y, z, vel[o], vel[64 + o], vel[128 + o],
+                           rr, 1.f / rr, rsqrtf(rr), E[p][0].x + E[p][0].y, E[p][1].x + E[p][1].y,
+                           E[p][2].x + E[p][2].y, qmob[p], q_s, id);
+  }
+}
+
+// 128 registers (4 CTAs of 128 threads): with 96 the near field spills and the
+// kernel is slower (l_max = 16: 0.553 against 0.470 ms).
+template <int L>
+__global__ void __launch_bounds__(kPairMaxWarps * 32, 4) k_field_pair(FieldArgs<float> a) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  chain_wait();
+  const int warp = threadIdx.x >> 5, wpb = blockDim.x >> 5;
+  field_pair<L>(a, smem_raw, warp, int64_t(gridDim.x - 1 - blockIdx.x) * wpb + warp);
+}
+
+// Batched: CTA b takes the pairs of tiles from items[b].y on of instance items[b].x.
+template <int L>
+__global__ void __launch_bounds__(kPairMaxWarps * 32, 4) k_field_pair_batch(const FieldArgs<float>* __restrict__ args,
+                                                                          const int2* __restrict__ items) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ FieldArgs<float> sa;
+  const int2 it = items[blockIdx.x];
+  copy_args(args + it.x, &sa);
+  __syncthreads();
+  field_pair<L>(sa, smem_raw, threadIdx.x >> 5, int64_t(it.y) + (threadIdx.x >> 5));
 }
 
 // Register budget: in FP32, at least 3 CTAs of 256 threads per SM (80
