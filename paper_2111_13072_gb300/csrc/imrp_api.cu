@@ -52,6 +52,14 @@ uint32_t coll_threshold(double nu, double dt) {
 
 }  // namespace
 
+// Samples of a series staged at once on the way to the caller.
+constexpr int64_t kHostSamples = 2048;
+struct HostBlock {
+  volatile int err;
+  int pad[15];
+  double samples[2 * kHostSamples];
+};
+
 struct imrp_ctx {
   imrp_params p{};
   std::string err;
@@ -97,7 +105,11 @@ struct imrp_ctx {
   cudaEvent_t ev_copied[2] = {nullptr, nullptr}, ev_free[2] = {nullptr, nullptr};
   int next_stage = 0;
   StepState* st = nullptr;
-  int* derr = nullptr;
+  // one page-locked mapped block per context: the error flags, which the kernels
+  // write through derr (only when there is an error), and a staging area for the
+  // recorded samples; so a synchronising call copies nothing to learn that all is well
+  HostBlock* host = nullptr;
+  int* derr = nullptr;        // device address of host->err
   double* dft = nullptr;
   int64_t dft_cap = 0;  // doubles
   // radial ion profile (App. D) in place of the uniform background
@@ -199,8 +211,8 @@ void free_all(imrp_ctx* c) {
   cudaFree(c->srt_id);
   c->srt_id = nullptr;
   void* ps[] = {c->key0, c->idx0, c->key1, c->idx1, c->hist, c->agg, c->pfx, c->gbase, c->tot,
-                c->eout, c->gagg, c->totd, c->gswork, c->gsticket, c->qhist, c->uhist, c->stage, c->st,
-                c->derr, c->dft};
+                c->eout, c->gagg, c->totd, c->gswork, c->gsticket, c->qhist, c->stage, c->st,
+                c->dft};
   for (void* p : ps) cudaFree(p);
   cudaFree(c->ion_q);
   c->ion_q = nullptr;
@@ -216,6 +228,8 @@ void free_all(imrp_ctx* c) {
   c->gagg = c->totd = c->gswork = c->qhist = c->uhist = c->stage = c->dft = nullptr;
   c->gsticket = nullptr;
   c->st = nullptr;
+  if (c->host) cudaFreeHost(c->host);
+  c->host = nullptr;
   c->derr = nullptr;
   for (int k = 0; k < 2; ++k) {
     cudaFree(c->astage[k]);
@@ -230,12 +244,12 @@ void free_all(imrp_ctx* c) {
   c->own_stream = nullptr;
 }
 
+// Waits for the context's stream and takes its error flags.
 int check_err(imrp_ctx* ctx) {
-  int h = 0;
-  CK(cudaMemcpyAsync(&h, ctx->derr, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
   CK(cudaStreamSynchronize(ctx->stream));
+  const int h = ctx->host->err;
   if (h) {
-    CK(cudaMemsetAsync(ctx->derr, 0, sizeof(int), ctx->stream));
+    ctx->host->err = 0;
     if (h & kErrNaN) return ctx->fail(IMRP_E_NAN, "non-finite value in the particle state");
     if (h & kErrRange) return ctx->fail(IMRP_E_INVAL, "a particle lies outside 1 < r < r_out");
   }
@@ -245,16 +259,15 @@ int check_err(imrp_ctx* ctx) {
 int grow_history(imrp_ctx* ctx, int64_t need) {
   if (need <= ctx->hcap) return IMRP_OK;
   int64_t ncap = std::max<int64_t>(need, std::max<int64_t>(2 * ctx->hcap, 4096));
-  double *q = nullptr, *u = nullptr;
-  CK(cudaMalloc(&q, ncap * sizeof(double)));
-  CK(cudaMalloc(&u, ncap * sizeof(double)));
+  double* q = nullptr;  // Q_diff [ncap], then u_asy [ncap]
+  CK(cudaMalloc(&q, 2 * ncap * sizeof(double)));
+  double* u = q + ncap;
   if (ctx->hcap) {
     CK(cudaMemcpyAsync(q, ctx->qhist, ctx->hcap * sizeof(double), cudaMemcpyDeviceToDevice, ctx->stream));
     CK(cudaMemcpyAsync(u, ctx->uhist, ctx->hcap * sizeof(double), cudaMemcpyDeviceToDevice, ctx->stream));
     CK(cudaStreamSynchronize(ctx->stream));
   }
   cudaFree(ctx->qhist);
-  cudaFree(ctx->uhist);
   ctx->qhist = q;
   ctx->uhist = u;
   ctx->hcap = ncap;
@@ -487,7 +500,7 @@ size_t footprint_bytes(int64_t N, int L, int prec) {
   b += size_t(ngroups * nc) * (es + 8) + size_t(nc) * (es + 8);
   b += size_t(gs_work_doubles(int(nc))) * 8 + size_t(gs_tickets(int(nc))) * 4;
   b += 3 * size_t(N) * es + 6 * size_t(N) * 8;      // field output, staging
-  b += sizeof(StepState) + sizeof(int);
+  b += sizeof(StepState);
   return b;
 }
 
@@ -517,8 +530,9 @@ int alloc_ctx(imrp_ctx* ctx) {
   CK(cudaMalloc(&ctx->eout, 3 * N * es));
   CK(cudaMalloc(&ctx->stage, 6 * N * sizeof(double)));
   CK(cudaMalloc(&ctx->st, sizeof(StepState)));
-  CK(cudaMalloc(&ctx->derr, sizeof(int)));
-  CK(cudaMemset(ctx->derr, 0, sizeof(int)));
+  CK(cudaHostAlloc(&ctx->host, sizeof(HostBlock), cudaHostAllocMapped | cudaHostAllocPortable));
+  ctx->host->err = 0;
+  CK(cudaHostGetDevicePointer(&ctx->derr, ctx->host, 0));
   return IMRP_OK;
 }
 
@@ -805,6 +819,17 @@ int imrp_get_qdiff(imrp_ctx* ctx, int64_t first, int64_t count, double* qd, doub
                      (long long)ctx->host_step);
   if (count == 0) return IMRP_OK;
   const int64_t h = first - ctx->hist_first;
+  if (count <= kHostSamples && (qd || ua)) {
+    // both series in one copy through the page-locked block: two copies to pageable
+    // memory and one of the error flag took 37 us a call, this and the wait 17
+    double* s = ctx->host->samples;
+    CK(cudaMemcpy2DAsync(s, count * sizeof(double), ctx->qhist + h, ctx->hcap * sizeof(double), count * sizeof(double),
+                         2, cudaMemcpyDeviceToHost, ctx->stream));
+    const int rc = check_err(ctx);
+    if (qd) memcpy(qd, s, count * sizeof(double));
+    if (ua) memcpy(ua, s + count, count * sizeof(double));
+    return rc;
+  }
   if (qd) CK(cudaMemcpyAsync(qd, ctx->qhist + h, count * sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));
   if (ua) CK(cudaMemcpyAsync(ua, ctx->uhist + h, count * sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));
   return check_err(ctx);

@@ -24,7 +24,7 @@ constexpr size_t align256(size_t b) { return (b + 255) & ~size_t(255); }
 // Byte layout of the scratch for n particles, degree L, element size es.
 struct Layout {
   size_t part, st[6], id, key0, idx0, key1, idx1, hist, agg, pfx, gagg, gbase, tot, totd, gswork, gsticket, eout,
-      step, err, total;
+      step, total;
 };
 constexpr Layout layout(int64_t n, int L, size_t es) {
   Layout o{};
@@ -50,7 +50,6 @@ constexpr Layout layout(int64_t n, int L, size_t es) {
   o.gsticket = at; at += align256(size_t(gs_tickets(int(nc))) * 4);
   o.eout = at; at += align256(size_t(3 * n) * es);
   o.step = at; at += align256(sizeof(StepState));
-  o.err = at; at += align256(sizeof(int));
   o.total = at;
   return o;
 }
@@ -62,6 +61,10 @@ static __device__ __align__(256) unsigned char g_scratch[kScratchBytes];
 
 std::mutex g_mu;
 void* g_addr[64] = {nullptr};  // device address of g_scratch, per device
+// error flag per device, in page-locked mapped memory (written by the kernels
+// only when there is an error; a call reads it after its wait, without a copy)
+volatile int* g_err[64] = {nullptr};
+int* g_derr[64] = {nullptr};
 // The table of per-degree kernels is built when the library is loaded, so
 // that the entry point itself never allocates (not even host memory).
 std::vector<KernelSet<float>> g_f;
@@ -98,9 +101,9 @@ __global__ void k_na_load(const double* __restrict__ x, Part<T>* st, int64_t n, 
 }
 
 // Per-call set-up of what must start at zero or at the given step: the step
-// state, the error flag and the group scan's tickets (the scratch keeps the
+// state and the group scan's tickets (the scratch keeps the
 // previous call's contents, and another n or degree lays it out differently).
-__global__ void k_na_init(StepState* st, int64_t step, int* err, unsigned* ticket, int nticket) {
+__global__ void k_na_init(StepState* st, int64_t step, unsigned* ticket, int nticket) {
   chain_wait();
   st->step = step;
   st->next = step;
@@ -110,7 +113,6 @@ __global__ void k_na_init(StepState* st, int64_t step, int* err, unsigned* ticke
   st->nabs_step = 0;
   st->qs_acc = 0.0;
   st->nabs_total = 0;
-  *err = 0;
   for (int k = 0; k < nticket; ++k) ticket[k] = 0u;
 }
 
@@ -152,9 +154,10 @@ int run(const imrp_params* p, const double* x, int64_t n, int64_t step, double* 
   uint32_t* key0 = static_cast<uint32_t*>(P(o.key0));
   uint32_t* idx0 = static_cast<uint32_t*>(P(o.idx0));
   StepState* st = static_cast<StepState*>(P(o.step));
-  int* err = static_cast<int*>(P(o.err));
+  int* err = g_derr[dev];
+  *g_err[dev] = 0;
   LaunchSeq seq(s);
-  seq(k_na_init, 1, 1, 0, st, step, err, static_cast<unsigned*>(P(o.gsticket)), gs_tickets(nc));
+  seq(k_na_init, 1, 1, 0, st, step, static_cast<unsigned*>(P(o.gsticket)), gs_tickets(nc));
   seq(k_na_load<T>, unsigned((n + 255) / 256), 256, 0, x, st0, n, r_out, err);
   launch_keys<T>(st0, key0, idx0, n, r_out, seq);
   const uint32_t* perm = launch_radix_sort(key0, idx0, static_cast<uint32_t*>(P(o.key1)), static_cast<uint32_t*>(P(o.idx1)),
@@ -240,9 +243,8 @@ int run(const imrp_params* p, const double* x, int64_t n, int64_t step, double* 
   const T* cs[3] = {eo, eo + n, eo + 2 * n};
   launch_scatter_by_id<T>(cs, 3, id1, E, n, seq);
   if (cudaGetLastError() != cudaSuccess) return IMRP_E_CUDA;
-  int h = 0;
-  if (cudaMemcpyAsync(&h, err, sizeof(int), cudaMemcpyDeviceToHost, s) != cudaSuccess) return IMRP_E_CUDA;
   if (cudaStreamSynchronize(s) != cudaSuccess) return IMRP_E_CUDA;
+  const int h = *g_err[dev];
   if (h & kErrNaN) return IMRP_E_NAN;
   if (h & kErrRange) return IMRP_E_INVAL;
   return IMRP_OK;
@@ -279,6 +281,15 @@ extern "C" int imrp_field_noalloc(const imrp_params* p, const double* x_dev, int
         if (k.L <= kMaxL && k.init(dev) != 0) return IMRP_E_CUDA;
       void* ptr = nullptr;
       if (cudaGetSymbolAddress(&ptr, g_scratch) != cudaSuccess || !ptr) return IMRP_E_CUDA;
+      int *he = nullptr, *de = nullptr;
+      if (cudaHostAlloc(&he, sizeof(int), cudaHostAllocMapped | cudaHostAllocPortable) != cudaSuccess)
+        return IMRP_E_CUDA;
+      if (cudaHostGetDevicePointer(&de, he, 0) != cudaSuccess) {
+        cudaFreeHost(he);
+        return IMRP_E_CUDA;
+      }
+      g_err[dev] = he;
+      g_derr[dev] = de;
       g_addr[dev] = ptr;
     }
     base = static_cast<unsigned char*>(g_addr[dev]);
