@@ -923,9 +923,10 @@ int imrp_get_particles(imrp_ctx* ctx, double* x, double* v) {
   if (!ctx) return IMRP_E_INVAL;
   if (!ctx->loaded) return ctx->fail(IMRP_E_STATE, "get_particles before load");
   const int64_t n = ctx->n;
-  // positions to stage[0, 3n) and velocities to stage[3n, 6n), each [n][3] in id order
-  if (ctx->prec == 1) launch_state_out<float>(state_of<float>(ctx), ctx->stage, ctx->stage + 3 * n, n, ctx->stream);
-  else launch_state_out<double>(state_of<double>(ctx), ctx->stage, ctx->stage + 3 * n, n, ctx->stream);
+  // positions to stage[0, 3n) and velocities to stage[3n, 6n), each [n][3] in id
+  // order (key1 is free between steps)
+  if (ctx->prec == 1) launch_state_out<float>(state_of<float>(ctx), ctx->stage, ctx->stage + 3 * n, ctx->key1, n, ctx->stream);
+  else launch_state_out<double>(state_of<double>(ctx), ctx->stage, ctx->stage + 3 * n, ctx->key1, n, ctx->stream);
   if (x) CK(cudaMemcpyAsync(x, ctx->stage, 3 * n * sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));
   if (v) CK(cudaMemcpyAsync(v, ctx->stage + 3 * n, 3 * n * sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));
   return check_err(ctx);

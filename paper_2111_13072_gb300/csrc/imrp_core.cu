@@ -734,7 +734,14 @@ void launch_scatter_by_id(const T* const* comps, int ncomp, const uint32_t* id, 
   seq(k_scatter_by_id<T>, unsigned((n + 255) / 256), 256, 0, p, ncomp, id, out, n);
 }
 
-// The state in id order: x[id][3] and v[id][3], FP64.
+// The state in id order: x[id][3] and v[id][3], FP64. Up to kGatherMinN particles
+// each record is scattered to its id's place; beyond, where the outputs (48 bytes
+// per particle) leave L2 and every scattered 24-byte piece costs two sectors read and
+// written, the inverse order is written first (4 bytes per particle) and each id's
+// record gathered, one sector, so that the outputs are written in order: N = 1.6e7:
+// 1.94 -> 0.60 ms, N = 2e6: 0.147 -> 0.065, N = 5e5: 0.028 -> 0.021 (N = 3e5: 0.014
+// against 0.016).
+constexpr int64_t kGatherMinN = 393216;
 template <class T>
 __global__ void k_state_out(const Part<T>* __restrict__ st, double* __restrict__ x, double* __restrict__ v,
                             int64_t n) {
@@ -745,10 +752,32 @@ __global__ void k_state_out(const Part<T>* __restrict__ st, double* __restrict__
   x[3 * k] = p.x; x[3 * k + 1] = p.y; x[3 * k + 2] = p.z;
   v[3 * k] = p.vx; v[3 * k + 1] = p.vy; v[3 * k + 2] = p.vz;
 }
+template <class T>
+__global__ void k_inverse_ids(const Part<T>* __restrict__ st, uint32_t* __restrict__ inv, int64_t n) {
+  const int64_t j = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+  if (j < n) inv[st[j].id] = uint32_t(j);
+}
+template <class T>
+__global__ void k_state_gather(const Part<T>* __restrict__ st, const uint32_t* __restrict__ inv,
+                               double* __restrict__ x, double* __restrict__ v, int64_t n) {
+  chain_wait();
+  const int64_t k = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+  if (k >= n) return;
+  const Part<T> p = st[inv[k]];
+  x[3 * k] = p.x; x[3 * k + 1] = p.y; x[3 * k + 2] = p.z;
+  v[3 * k] = p.vx; v[3 * k + 1] = p.vy; v[3 * k + 2] = p.vz;
+}
 
 template <class T>
-void launch_state_out(const Part<T>* st, double* x, double* v, int64_t n, cudaStream_t s) {
-  k_state_out<T><<<unsigned((n + 255) / 256), 256, 0, s>>>(st, x, v, n);
+void launch_state_out(const Part<T>* st, double* x, double* v, uint32_t* inv, int64_t n, cudaStream_t s) {
+  LaunchSeq seq(s);
+  const unsigned blocks = unsigned((n + 255) / 256);
+  if (n < kGatherMinN) {
+    seq(k_state_out<T>, blocks, 256, 0, st, x, v, n);
+  } else {
+    seq(k_inverse_ids<T>, blocks, 256, 0, st, inv, n);
+    seq(k_state_gather<T>, blocks, 256, 0, st, static_cast<const uint32_t*>(inv), x, v, n);
+  }
 }
 
 // ============================================================================
@@ -1274,7 +1303,7 @@ cudaError_t preload_core_kernels() {
                                      cudaStream_t);                                                \
   template void launch_scatter_by_id<T>(const T* const*, int, const uint32_t*, double*, int64_t,   \
                                         LaunchSeq&);                                               \
-  template void launch_state_out<T>(const Part<T>*, double*, double*, int64_t, cudaStream_t);     \
+  template void launch_state_out<T>(const Part<T>*, double*, double*, uint32_t*, int64_t, cudaStream_t); \
   template void launch_tile_scan<T>(const T*, T*, double*, int64_t, int, LaunchSeq&);                \
   template void launch_group_scan<T>(const double*, double*, unsigned*, T*, T*, double*, int64_t, int, \
                                      int, const FinalizeArgs*, LaunchSeq&);

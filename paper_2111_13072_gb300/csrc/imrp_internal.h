@@ -108,9 +108,9 @@ void launch_state_dump(const Part<T>* st, double* x, double* v, uint32_t* id, in
 template <class T>
 void launch_scatter_by_id(const T* const* comps, int ncomp, const uint32_t* id, double* out,
                           int64_t n, LaunchSeq& seq);
-// the state in id order: x[n][3], v[n][3] (FP64)
+// the state in id order: x[n][3], v[n][3] (FP64); inv: scratch of n words
 template <class T>
-void launch_state_out(const Part<T>* st, double* x, double* v, int64_t n, cudaStream_t s);
+void launch_state_out(const Part<T>* st, double* x, double* v, uint32_t* inv, int64_t n, cudaStream_t s);
 
 // ---- scans (imrp_core.cu) ---------------------------------------------------
 // in-group scans of agg[u][tile] (row stride tile_stride(ntiles)) into

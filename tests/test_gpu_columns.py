@@ -57,3 +57,18 @@ def test_reloads_of_other_sizes(imrp, prec):
                 fresh.step(3)
                 for a, b in zip(got, fresh.particles()):
                     np.testing.assert_array_equal(a, b)
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+@pytest.mark.parametrize("n", [1, 257, 393215, 393216, 500001])
+def test_read_back_in_id_order(imrp, prec, n):
+    """imrp_get_particles (scattering small states, gathering large ones) against the checkpoint's
+    storage order and ids, exactly, after steps that permuted the storage."""
+    x, v = workload_state(W, N=n)
+    with imrp.Sim(imrp.params_from_workload(W, N=n, precision=prec, l_max=1)) as sim:
+        sim.load(x, v)
+        sim.step(2)
+        xs, vs = sim.particles()
+        xc, vc, ids, _ = sim.checkpoint()
+    np.testing.assert_array_equal(xs[ids], xc)
+    np.testing.assert_array_equal(vs[ids], vc)
