@@ -135,7 +135,7 @@ template <class T, int L> void mom_launch(const MomArgs<T>& a, LaunchSeq& seq) {
   const unsigned blocks = unsigned(mom_blocks(a.n, ppt) * a.parts);
   if (ppt == kMomPPT)
     seq(k_moments<T, L, kMomPPT>, blocks, kMomThreads, moments_smem<T, L, kMomPPT>(), a);
-  else
+  else if constexpr (sizeof(T) == 8)
     seq(k_moments<T, L, kMomPPTSmall>, blocks, kMomThreads, moments_smem<T, L, kMomPPTSmall>(), a);
 }
 
@@ -159,7 +159,7 @@ void mom_batch_launch(const MomArgs<T>* args, const int2* items, int nitems, int
   if (nitems <= 0) return;
   if (ppt == kMomPPT)
     k_moments_batch<T, L, kMomPPT><<<unsigned(nitems), kMomThreads, moments_smem<T, L, kMomPPT>(), s>>>(args, items);
-  else
+  else if constexpr (sizeof(T) == 8)
     k_moments_batch<T, L, kMomPPTSmall>
         <<<unsigned(nitems), kMomThreads, moments_smem<T, L, kMomPPTSmall>(), s>>>(args, items);
 }
@@ -190,15 +190,17 @@ template <class T, int L> cudaError_t set_attr() {
   cudaError_t e = cudaFuncSetAttribute(k_moments<T, L, kMomPPT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        int(moments_smem<T, L, kMomPPT>()));
   if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(k_moments<T, L, kMomPPTSmall>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           int(moments_smem<T, L, kMomPPTSmall>()));
-  if (e != cudaSuccess) return e;
   e = cudaFuncSetAttribute(k_moments_batch<T, L, kMomPPT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            int(moments_smem<T, L, kMomPPT>()));
   if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(k_moments_batch<T, L, kMomPPTSmall>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           int(moments_smem<T, L, kMomPPTSmall>()));
-  if (e != cudaSuccess) return e;
+  if constexpr (sizeof(T) == 8) {
+    e = cudaFuncSetAttribute(k_moments<T, L, kMomPPTSmall>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             int(moments_smem<T, L, kMomPPTSmall>()));
+    if (e != cudaSuccess) return e;
+    e = cudaFuncSetAttribute(k_moments_batch<T, L, kMomPPTSmall>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             int(moments_smem<T, L, kMomPPTSmall>()));
+    if (e != cudaSuccess) return e;
+  }
   const int fmax = int(8 * field_smem_per_warp<T>(L) > 227 * 1024 ? 227 * 1024 : 8 * field_smem_per_warp<T>(L));
   e = cudaFuncSetAttribute(k_field<T, L>, cudaFuncAttributeMaxDynamicSharedMemorySize, fmax);
   if (e != cudaSuccess) return e;

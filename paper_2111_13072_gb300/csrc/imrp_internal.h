@@ -192,10 +192,10 @@ inline int sm_count() {
 // Particles per thread of the moments kernel for an instance of n particles:
 // 16 (1024 per CTA of 64 threads), or 4 (256 per CTA) for an FP64 instance of
 // fewer than 100 such blocks, whose columns alone (below) would not fill the
-// GPU: FP64 N = 60000, l_max = 12 takes 0.184 ms with 4 and 0.219 with 16;
+// GPU: FP64 N = 60000, l_max = 12 took 0.184 ms with 4 and 0.219 with 16;
 // N = 250001, l_max = 16 (245 blocks) 1.19 and 0.96, since with 4 each tile's
-// sums go through a butterfly over 8 threads. FP32 keeps 16 (N = 1e5,
-// l_max = 16: 0.045 -> 0.068 ms with 4).
+// sums go over 8 threads. FP32 keeps 16 (N = 1e5, l_max = 16: 0.045 -> 0.068 ms
+// with 4).
 inline int mom_ppt(int elem_size, int64_t n) { return (elem_size == 8 && (n + 1023) / 1024 < 100) ? 4 : 16; }
 // CTAs of the moments kernel per column range (64 threads of ppt particles):
 // whole scan groups of 1024 particles, so that every tile the scans read is written
@@ -206,8 +206,7 @@ inline int64_t mom_blocks(int64_t n, int ppt) { return (n + 1023) / 1024 * (16 /
 // diagonal terms up to its first column). As many ranges as give the stated
 // CTAs per SM: FP32 N = 1e5, l_max = 16: 0.043 ms with one range, 0.0225 with
 // 6 per SM, 0.028 with 8; N = 3e5, l_max = 8: 0.0262, 0.0206, 0.0267; FP64
-// N = 20000, l_max = 8: 0.102 with one, 0.046 with 7 ranges, 0.051 with 9 (0.055
-// with 6, where a short last range unbalances them).
+// N = 20000, l_max = 8: 0.102 with one, 0.039 with 7 ranges (4 CTAs per SM), 0.043 with 9.
 inline int mom_parts(int elem_size, int L, int64_t n, int ppt) {
   const int per_sm = elem_size == 4 ? 6 : ppt == 4 ? 4 : 8;
   const int64_t want = int64_t(per_sm) * sm_count() / mom_blocks(n, ppt);

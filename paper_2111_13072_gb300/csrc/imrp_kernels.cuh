@@ -110,7 +110,7 @@ template <> __device__ __forceinline__ double fma_t<double>(double x, double y, 
 // one of several ranges of them.
 // At the end of a column the threads of each tile are combined: with two
 // (PPT = 16), one shuffle per Rs/Is pair (the even lane keeps the Rs sum, the
-// odd lane the Is sum); with more, a butterfly over the tile's threads, each
+// odd lane the Is sum); with more, by halving over the tile's threads, each
 // then writing its share. Written: agg[u][tile], u = 2 e + s (s = 0 Rs, s = 1 Is).
 constexpr int kMomThreads = 64;
 constexpr int kMomPPT = 16;       // particles per thread (1024 per CTA) when that fills the GPU
@@ -182,14 +182,19 @@ __device__ __forceinline__ void moments_block(const MomArgs<T>& a, int64_t item,
     const T X = valid ? a.x[j] : T(1), Y = valid ? a.y[j] : T(0), Z = valid ? a.z[j] : T(0);
     const int o = (k % PPT) * S + k / PPT;
     const T r2 = X * X + Y * Y + Z * Z;
+    // FP64: from the reciprocal root, which is needed anyway (a division costs some 20
+    // FP64 operations, and every column range stages its particles)
+    T ir = rsqrt_t(r2), q;
+    if constexpr (sizeof(T) == 8) q = a.rho * (ir * ir);
+    else q = a.rho / r2;
     sx[o] = X * ri; sy[o] = Y * ri; sz[o] = Z * ri;
-    sq[o] = a.rho / r2;
+    sq[o] = q;
     // the particle's charge seeds its harmonics: -1 for an electron, q_ion
     // for a mobile ion
-    T Dr = valid ? ((a.species && a.id[j] >= a.n_e) ? a.q_ion : T(-1)) : T(0), Di = T(0), sc = rsqrt_t(r2);
+    T Dr = valid ? ((a.species && a.id[j] >= a.n_e) ? a.q_ion : T(-1)) : T(0), Di = T(0), sc = ir;
     for (int m = 1; m < mlo; ++m) {  // the diagonal up to the column before this part's first
       diag_step(tb.dg[m] * (X * ri), tb.dg[m] * (Y * ri), Dr, Di);
-      sc *= a.rho / r2;
+      sc *= q;
     }
     sRr[o] = Dr;
     sRi[o] = Di;
@@ -291,33 +296,36 @@ __device__ __forceinline__ void moments_block(const MomArgs<T>& a, int64_t item,
         }
       }
     } else {
-      // sums over the tile's threads (butterfly), then value 2 p + s of the
-      // column goes out from the thread with sub = (2 p + s) % TPT
+      // sums over the tile's threads, TPT values at a time by halving (each step a thread
+      // keeps half of its values and adds its partner's share of them), so that value k of a
+      // run of TPT ends on the thread sub = k
       T* const agg_c = a.agg + tile;
-      if (m == 0) {
+      const int nv = m == 0 ? 2 * L : 4 * (L - m + 1);  // values of the column, (Rs, Is) pairs
+      constexpr int NV = 4 * L;
 #pragma unroll
-        for (int p = 0; p < L; ++p) {
+      for (int v0 = 0; v0 < NV; v0 += TPT) {
+        if (v0 >= nv) break;
+        T v[TPT];
 #pragma unroll
-          for (int sp = 0; sp < 2; ++sp) {
-            T v = acc[4 * (p + 1) + sp];
+        for (int k = 0; k < TPT; ++k) {
+          // m = 0: value 2 p + s is acc[4 (p + 1) + s] (no imaginary part); else acc[2 p + s]
+          const int i0 = 4 * ((v0 + k) / 2 + 1) + (v0 + k) % 2, i1 = v0 + k;
+          const T x0 = i0 < 4 * (L + 1) ? acc[i0 < 4 * (L + 1) ? i0 : 0] : T(0);
+          v[k] = m == 0 ? x0 : acc[i1];
+        }
 #pragma unroll
-            for (int d = 1; d < TPT; d <<= 1) v += __shfl_xor_sync(0xffffffffu, v, d);
-            if ((2 * p + sp) % TPT == sub) agg_c[(2 * (e0 + p) + sp) * ts] = v * tb.nu[(p + 1) * kTabL];
+        for (int d = TPT / 2; d >= 1; d >>= 1) {
+          const bool up = (sub & d) != 0;
+#pragma unroll
+          for (int k = 0; k < d; ++k) {
+            const T send = up ? v[k] : v[k + d], keep = up ? v[k + d] : v[k];
+            v[k] = keep + __shfl_xor_sync(0xffffffffu, send, d);
           }
         }
-      } else {
-        const int np = 2 * (L - m + 1);
-#pragma unroll
-        for (int p = 0; p < 2 * L; ++p) {
-          if (p >= np) break;
-#pragma unroll
-          for (int sp = 0; sp < 2; ++sp) {
-            T v = acc[2 * p + sp];
-#pragma unroll
-            for (int d = 1; d < TPT; d <<= 1) v += __shfl_xor_sync(0xffffffffu, v, d);
-            if ((2 * p + sp) % TPT == sub)
-              agg_c[(2 * (e0 + p) + sp) * ts] = v * tb.nu[(m + (p >> 1)) * kTabL + m];
-          }
+        const int val = v0 + sub;
+        if (val < nv) {
+          const int l = m == 0 ? val / 2 + 1 : m + val / 4;
+          agg_c[(2 * e0 + val) * ts] = v[0] * tb.nu[l * kTabL + m];
         }
       }
     }
