@@ -170,14 +170,13 @@ double n_tilde_of(const imrp_ctx* c, int64_t n) {
 double n_ion_of(const imrp_ctx* c, int64_t n) { return c->species ? c->sp_bg : double(n); }
 
 // Warps per CTA of the field kernel for ntiles tiles. When all tiles fit on the
-// GPU at once, the shape that gives the fullest SM the fewest tiles: FP64
-// N = 20000, l_max = 8 takes 0.130 ms with one tile per CTA and 0.183 with 8
-// (79 CTAs on 152 SMs); FP32 N = 1e5, l_max = 16 0.045 with one and 0.050 with
-// 4 (782 CTAs in 760 places). Beyond that the shape of create.
+// GPU at once, the shape that gives the fullest SM the fewest tiles: FP32 N = 1e5,
+// l_max = 16 0.045 ms with one tile per CTA and 0.050 with 4 (782 CTAs in 760 places).
+// Beyond that the shape of create. (The FP64 kernel of four warps per tile has one
+// shape; with m0_only FP64 runs one tile per warp too.)
 constexpr int kFieldWpb[4] = {8, 4, 2, 1};
-bool uses_pairs(const imrp_ctx* c, int64_t n) {
-  return c->prec == 1 ? field_pair_rule<float>(c->L, n, c->p.m0_only) : field_pair_rule<double>(c->L, n, c->p.m0_only);
-}
+bool uses_pairs(const imrp_ctx* c, int64_t n) { return c->prec == 1 && field_pair_rule<float>(c->L, n, c->p.m0_only); }
+bool uses_team(const imrp_ctx* c) { return c->prec == 0 && field_team_rule<double>(c->p.m0_only); }
 int field_wpb(const imrp_ctx* c, int64_t ntiles) {
   if (uses_pairs(c, c->n)) return kPairWarps;
   const int64_t sms = sm_count();
@@ -628,9 +627,9 @@ int imrp_create(const imrp_params* p, imrp_ctx** out) {
   // l_max = 16, N = 2e6: 4 warps (20 resident) beat 2 warps (22 resident) by
   // 27%; l_max = 24: 2 warps (10 resident) beat 4 warps (8 resident) by 9%; 8
   // warps lose to 4 everywhere (l_max = 12, N = 7e5: 0.173 against 0.158 ms).
-  // FP64 is bound by its pipe and loses only the uneven ends of large CTAs
-  // (l_max = 16, N = 250001: 2 / 4 / 8 warps 2.49 / 2.54 / 2.68 ms; l_max = 8,
-  // N = 40000: 0.267 / 0.309 / 0.352).
+  // FP64 (here with m0_only alone) is bound by its pipe and loses only the uneven
+  // ends of large CTAs (all m, l_max = 8, N = 40000: 2 / 4 / 8 warps 0.267 / 0.309 /
+  // 0.352 ms).
   {
     int best = 0;
     for (int q = 0; q < 4; ++q) {
@@ -1143,9 +1142,9 @@ struct BatchGroup {
   void* dmom = nullptr;         // MomArgs<T>[members]
   void* dfield = nullptr;       // FieldArgs<T>[members] (push mode)
   int2* dmom_items = nullptr;   // (member, item): first the members of mom_ppt 16, then of 4
-  int2* dfield_items = nullptr; // (member, first tile of a CTA); the members of field_pair_rule:
-                                // (member, first pair of tiles), after the others
-  int nmom = 0, nmom_small = 0, nfield = 0, npair = 0;
+  int2* dfield_items = nullptr; // (member, first tile of a CTA); after them the members of
+                                // field_pair_rule (member, first pair of tiles) or field_team_rule (member, tile)
+  int nmom = 0, nmom_small = 0, nfield = 0, nalt = 0;
 };
 
 struct imrp_batch {
@@ -1222,6 +1221,8 @@ template <class T> int fill_group(imrp_batch* b, BatchGroup& g) {
     for (int64_t q = 0; q < mitems; ++q) (ppt == 16 ? mi : ms).push_back(make_int2(int(k), int(q)));
     if (uses_pairs(ctx, ctx->n))
       for (int64_t t = 0; t < (ctx->ntiles + 1) / 2; t += kPairWarps) pi.push_back(make_int2(int(k), int(t)));
+    else if (uses_team(ctx))
+      for (int64_t t = 0; t < ctx->ntiles; ++t) pi.push_back(make_int2(int(k), int(t)));
     else
       for (int64_t t = 0; t < ctx->ntiles; t += g.wpb) fi.push_back(make_int2(int(k), int(t)));
   }
@@ -1229,7 +1230,7 @@ template <class T> int fill_group(imrp_batch* b, BatchGroup& g) {
   mi.insert(mi.end(), ms.begin(), ms.end());
   g.nmom = int(mi.size());
   g.nfield = int(fi.size());
-  g.npair = int(pi.size());
+  g.nalt = int(pi.size());
   fi.insert(fi.end(), pi.begin(), pi.end());
   if (cudaMalloc(&g.dmom, ma.size() * sizeof(MomArgs<T>)) != cudaSuccess ||
       cudaMalloc(&g.dfield, fa.size() * sizeof(FieldArgs<T>)) != cudaSuccess ||
@@ -1313,10 +1314,12 @@ int enqueue_batch_step(imrp_batch* b) {
       const KernelSet<float>* ks = find_set<float>(g.L);
       const FieldArgs<float>* fa = static_cast<const FieldArgs<float>*>(g.dfield);
       ks->field_batch(fa, g.dfield_items, g.nfield, g.wpb, b->stream);
-      ks->pair_batch(fa, g.dfield_items + g.nfield, g.npair, b->stream);
+      ks->alt_batch(fa, g.dfield_items + g.nfield, g.nalt, b->stream);
     } else {
-      find_set<double>(g.L)->field_batch(static_cast<const FieldArgs<double>*>(g.dfield), g.dfield_items, g.nfield,
-                                         g.wpb, b->stream);
+      const KernelSet<double>* ks = find_set<double>(g.L);
+      const FieldArgs<double>* fa = static_cast<const FieldArgs<double>*>(g.dfield);
+      ks->field_batch(fa, g.dfield_items, g.nfield, g.wpb, b->stream);
+      ks->alt_batch(fa, g.dfield_items + g.nfield, g.nalt, b->stream);
     }
   }
   for (imrp_ctx* ctx : b->c) ctx->keys_valid = true;  // the field kernels wrote the next keys
@@ -1438,7 +1441,7 @@ template <class T> int time_group_field(imrp_batch* b, const BatchGroup& g, int 
   for (size_t k = 0; k < g.members.size(); ++k) {
     imrp_ctx* ctx = b->c[g.members[k]];
     fa.push_back(make_field_args<T>(ctx, false));
-    if (uses_pairs(ctx, ctx->n)) continue;  // their launch has one shape
+    if (uses_pairs(ctx, ctx->n) || uses_team(ctx)) continue;  // their launch has one shape
     for (int64_t t = 0; t < ctx->ntiles; t += wpb) fi.push_back(make_int2(int(k), int(t)));
   }
   *ms = 0.f;

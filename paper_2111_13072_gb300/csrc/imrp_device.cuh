@@ -407,6 +407,10 @@ template <class T> __host__ __device__ constexpr bool field_pair_rule(int L, int
   return pair_degree<T>(L) && n >= kPairMinN && !m0_only;
 }
 
+// Whether an instance's field runs in the FP64 kernel of four warps per tile
+// (field_team): all FP64 instances with all m.
+template <class T> __host__ __device__ constexpr bool field_team_rule(int m0_only) { return sizeof(T) == 8 && !m0_only; }
+
 // Column chunks of the far field: chunk q of the multipole (Is) part covers
 // columns [chunkI(L, q), chunkI(L, q + 1)), greedily filled to at most kChunk
 // gradient entries; likewise for the local (Rs) part.

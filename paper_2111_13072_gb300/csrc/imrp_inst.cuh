@@ -38,6 +38,7 @@ template <class T> void fill_tables(Tables<T>& t) {
 EntryRec h_ent[kEntTotal];
 PairSrc h_psrc[kRecTotal];
 float4 h_pfac[2][kRecTotal];
+TeamFac h_tfac[2][kRecTotal];
 float2 h_an2[kTabL * kTabL];
 uint16_t h_comp[kCompTotal];
 
@@ -111,6 +112,9 @@ void fill_prologue_tables() {
             src.i[3 * s + q] = int16_t(have && lq >= 1 && lq <= L && am <= lq ? pair_pos(L, lq, am, s) : zero);
           }
           h_pfac[s][k] = make_float4(e.s1r, e.s1i, e.s2, e.sz);
+          double dg = 1.0;
+          for (int q = 1; q <= M; ++q) dg *= -sqrt((2.0 * q - 1.0) / (2.0 * q));
+          h_tfac[s][k] = TeamFac{dg * e.s1r, dg * e.s1i, dg * e.s2, dg * e.sz};
         }
         h_psrc[k] = src;
       }
@@ -150,6 +154,12 @@ template <class T, int L> void field_launch(const FieldArgs<T>& a, int wpb, Laun
       return;
     }
   }
+  if constexpr (sizeof(T) == 8) {
+    if (field_team_rule<T>(a.m0_only)) {
+      if (ntiles > 0) seq(k_field_team<L>, unsigned(ntiles), kTeam * 32, team_smem(L), a);
+      return;
+    }
+  }
   const size_t smem = size_t(wpb) * field_smem_per_warp<T>(L);
   if (blocks > 0) seq(k_field<T, L>, unsigned(blocks), unsigned(wpb * 32), smem, a);
 }
@@ -171,10 +181,13 @@ void field_batch_launch(const FieldArgs<T>* args, const int2* items, int nitems,
 }
 
 template <class T, int L>
-void pair_batch_launch(const FieldArgs<T>* args, const int2* items, int nitems, cudaStream_t s) {
+void alt_batch_launch(const FieldArgs<T>* args, const int2* items, int nitems, cudaStream_t s) {
   if constexpr (pair_degree<T>(L)) {
     if (nitems > 0)
       k_field_pair_batch<L><<<unsigned(nitems), kPairWarps * 32, kPairWarps * pair_smem_per_warp(L), s>>>(args, items);
+  }
+  if constexpr (sizeof(T) == 8) {
+    if (nitems > 0) k_field_team_batch<L><<<unsigned(nitems), kTeam * 32, team_smem(L), s>>>(args, items);
   }
 }
 
@@ -212,6 +225,12 @@ template <class T, int L> cudaError_t set_attr() {
                              int(kPairWarps * pair_smem_per_warp(L)));
     if (e != cudaSuccess) return e;
   }
+  if constexpr (sizeof(T) == 8) {
+    e = cudaFuncSetAttribute(k_field_team<L>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(team_smem(L)));
+    if (e != cudaSuccess) return e;
+    e = cudaFuncSetAttribute(k_field_team_batch<L>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(team_smem(L)));
+    if (e != cudaSuccess) return e;
+  }
   // the batched kernel also holds one instance's arguments in static shared memory
   const int bmax = int(227 * 1024 - sizeof(FieldArgs<T>));
   return cudaFuncSetAttribute(k_field_batch<T, L>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -240,9 +259,13 @@ template <class T, int L> cudaError_t set_attr() {
     if (e != cudaSuccess) return int(e);                                                     \
     e = cudaMemcpyToSymbol(g_comp, h_comp, sizeof(h_comp));                                  \
     if (e != cudaSuccess) return int(e);                                                     \
-    if (sizeof(T) == 4) {                                                                    \
-      e = cudaMemcpyToSymbol(g_psrc, h_psrc, sizeof(h_psrc));                                \
-      if (e == cudaSuccess) e = cudaMemcpyToSymbol(g_pfac, h_pfac, sizeof(h_pfac));          \
+    e = cudaMemcpyToSymbol(g_psrc, h_psrc, sizeof(h_psrc));                                  \
+    if (e != cudaSuccess) return int(e);                                                     \
+    if (sizeof(T) == 8) {                                                                    \
+      e = cudaMemcpyToSymbol(g_tfac, h_tfac, sizeof(h_tfac));                                \
+      if (e != cudaSuccess) return int(e);                                                   \
+    } else {                                                                                 \
+      e = cudaMemcpyToSymbol(g_pfac, h_pfac, sizeof(h_pfac));                                \
       if (e == cudaSuccess) e = cudaMemcpyToSymbol(c_an2, h_an2, sizeof(h_an2));             \
       if (e != cudaSuccess) return int(e);                                                   \
     }                                                                                        \
@@ -256,7 +279,7 @@ template <class T, int L> cudaError_t set_attr() {
     KernelSet<T> ks[] = {KernelSet<T>{Ls, &mom_launch<T, Ls>, &field_launch<T, Ls>,         \
                                       &unit_init<Ls...>, field_smem_per_warp<T>(Ls),        \
                                       &field_occ<T, Ls>, &mom_batch_launch<T, Ls>,          \
-                                      &field_batch_launch<T, Ls>, &pair_batch_launch<T, Ls>}...};                      \
+                                      &field_batch_launch<T, Ls>, &alt_batch_launch<T, Ls>}...};                      \
     for (auto& k : ks) v.push_back(k);                                                       \
   }                                                                                          \
   }                                                                                          \

@@ -226,8 +226,9 @@ template <class T> struct KernelSet {
   // instance) and (instance, first tile) for the field (CTAs of wpb tiles).
   void (*moments_batch)(const MomArgs<T>* args, const int2* items, int nitems, int ppt, cudaStream_t);
   void (*field_batch)(const FieldArgs<T>* args, const int2* items, int nitems, int wpb, cudaStream_t);
-  // the same for instances of field_pair_rule: (instance, first pair of tiles), kPairWarps pairs per CTA
-  void (*pair_batch)(const FieldArgs<T>* args, const int2* items, int nitems, cudaStream_t);
+  // the same for instances of field_pair_rule: (instance, first pair of tiles), kPairWarps pairs
+  // per CTA; or of field_team_rule: (instance, tile)
+  void (*alt_batch)(const FieldArgs<T>* args, const int2* items, int nitems, cudaStream_t);
 };
 void register_all(std::vector<KernelSet<float>>& f, std::vector<KernelSet<double>>& d);
 

@@ -84,6 +84,9 @@ __host__ __device__ constexpr int rec_off(int L) {
 constexpr int kRecTotal = rec_off(24) + nP(24);
 static __device__ PairSrc g_psrc[kRecTotal];
 static __device__ float4 g_pfac[2][kRecTotal];  // multipole, local
+// the same factors for the FP64 kernel, times the diagonal's constants up to column m
+struct __align__(16) TeamFac { double s1r, s1i, s2, sz; };
+static __device__ TeamFac g_tfac[2][kRecTotal];
 static __device__ EntryRec g_ent[kEntTotal];
 static __device__ uint16_t g_comp[kCompTotal];  // per component: l | (drive << 8) | (m > 0) << 9
 
@@ -1644,6 +1647,236 @@ __global__ void __launch_bounds__(kPairMaxWarps * 32, 4) k_field_pair_batch(cons
   copy_args(args + it.x, &sa);
   __syncthreads();
   field_pair<L>(sa, smem_raw, threadIdx.x >> 5, int64_t(it.y) + (threadIdx.x >> 5));
+}
+
+// ----------------------------------------------------------------------------
+// Field kernel of FP64 instances: one CTA of four warps per tile. FP64 runs at 1/64
+// of the FP32 rate (half a lane per clock and scheduler), so the operation count is
+// what bounds it, and a tile held by one warp keeps three of an SM's four FP64 pipes
+// idle when there are few tiles. Warp w takes every fourth column of the far field
+// and every fourth round of the near field; the partial fields are added in a fixed
+// order. Operations per particle at l_max = 16: 2600 far + 2200 near (field_tile: 3300
+// + 2900): multipole and local part share the angular recurrence and the diagonal
+// (powers of r from a table in shared memory, whose pipe is idle), the pair sums run
+// by Clenshaw's recurrence. Field ms, field_tile (its best CTA size) -> this: l_max = 8,
+// N = 3001: 0.092 -> 0.038, N = 20000: 0.130 -> 0.115 (5 tiles on the fullest SM, 4.1 on
+// average), N = 40000: 0.266 -> 0.194; l_max = 12, N = 60000: 0.486 -> 0.415; l_max = 16,
+// N = 250001: 2.49 -> 2.28; l_max = 2, N = 1e6: 1.79 -> 1.54.
+// ----------------------------------------------------------------------------
+constexpr int kTeam = 4;
+__host__ __device__ constexpr size_t team_smem(int L) {
+  return sizeof(double) * (size_t(12) * nP(L) + 32 * (2 * L + 2) + 32 * 6 + kTeam * 3 * 32 + 2 * (2 * pair_run(L) + 1));
+}
+
+// The pair sums of pair_sums, for one pair in FP64.
+template <int L>
+__device__ __forceinline__ void pair_sums_f64(double x1, double y2, double& S0, double& S1, double& S2) {
+  double b1 = leg_c(L), b2 = 0.0, d1 = L * leg_c(L), d2 = 0.0, e1 = 0.0, e2 = 0.0;
+#pragma unroll
+  for (int l = L - 1; l >= 0; --l) {
+    const double G = -leg_g(l + 1) * y2;
+    double nb = l > 0 ? leg_c(l) : 0.0, nd = l > 0 ? l * leg_c(l) : 0.0, ne = b1;
+    if (l < L - 1) {
+      nb = l > 0 ? fma(G, b2, nb) : G * b2;
+      nd = l > 0 ? fma(G, d2, nd) : G * d2;
+      if (l < L - 2) ne = fma(G, e2, ne);
+      ne = fma(x1, e1, ne);
+    }
+    nb = l == 0 && L == 1 ? x1 * b1 : fma(x1, b1, nb);
+    nd = l == 0 && L == 1 ? x1 * d1 : fma(x1, d1, nd);
+    b2 = b1; b1 = nb; d2 = d1; d1 = nd; e2 = e1; e1 = ne;
+  }
+  S0 = b1; S1 = d1; S2 = e1;
+}
+
+template <int L>
+__device__ __forceinline__ void field_team(const FieldArgs<double>& a, unsigned char* smem_raw, int64_t tile) {
+  constexpr int NC = 2 * ncomp(L), NP = nP(L), RUN = pair_run(L);
+  const Tables<double>& tb = tab<double>();
+  const int lane = int(lane_id()), warp = threadIdx.x >> 5;
+  double* const rec = reinterpret_cast<double*>(smem_raw);       // [NP][12]
+  double* const uI = rec + 12 * NP;                              // [L + 2][32]: r^-(l+1)
+  double* const uR = uI + 32 * (L + 2);                          // [L][32]: (r / r_out)^l
+  double2* const pd = reinterpret_cast<double2*>(uR + 32 * L);   // [32][3]: (ex, ey), (ez, r), (1/r, -q)
+  double* const part = reinterpret_cast<double*>(pd + 32 * 3);   // [kTeam][3][32]
+  double2* const sc = reinterpret_cast<double2*>(part + kTeam * 3 * 32);
+  const int64_t g = tile / kTilesPerGroup;
+  const int64_t j = tile * 32 + lane;
+  const bool valid = j < a.n;
+  // warp 0 prepares the particles and the powers of r (once per tile: a reciprocal
+  // root alone is some 20 FP64 operations), the others form the coefficients
+  if (warp == 0) {
+    const double X = valid ? a.x[j] : a.r_out, Y = valid ? a.y[j] : 0.0, Z = valid ? a.z[j] : 0.0;
+    const double r2 = X * X + Y * Y + Z * Z, ir = rsqrt(r2), rk = r2 * ir;
+    pd[3 * lane] = make_double2(X * ir, Y * ir);
+    pd[3 * lane + 1] = make_double2(Z * ir, rk);
+    pd[3 * lane + 2] = make_double2(ir, valid ? (a.species && a.id[j] >= a.n_e ? -a.q_ion : 1.0) : 0.0);
+    const double q = rk * a.rho_inv;
+    double u = ir, w = 1.0;
+#pragma unroll 2
+    for (int l = 0; l <= L + 1; ++l) {
+      uI[32 * l + lane] = u;
+      u *= ir;
+      if (l < L) uR[32 * l + lane] = w;
+      w *= q;
+    }
+  } else {
+    // phase 1: the tile's expansion coefficients (as in field_tile)
+    const double2* pt = reinterpret_cast<const double2*>(a.pfx + tile * NC);
+    const double2* gb = reinterpret_cast<const double2*>(a.gbase + g * NC);
+    const uint16_t* ctab = g_comp + comp_tab_off(L);
+    double* const s0 = reinterpret_cast<double*>(sc);
+    for (int e = threadIdx.x - 32; e < NC / 2; e += (kTeam - 1) * 32) {
+      const uint16_t cr = ctab[e];
+      const int l = cr & 0xff;
+      const double rl = a.rhol[l];
+      const double2 ab = pt[e], gv = gb[e];
+      double cI = rl * (gv.x + ab.x) - a.f[l] * a.tot[2 * e + 1];
+      if ((cr >> 8) & 1) cI += drive_of(a, l);
+      const int o = e < L ? 2 * e : e + L;
+      s0[o] = cI * a.mpf;
+      s0[2 * RUN + o] = rl * (gv.y + ab.y) * a.mpfr;
+      if (e < L) s0[o + 1] = s0[2 * RUN + o + 1] = 0.0;
+    }
+    if (threadIdx.x == 32) sc[2 * RUN] = make_double2(0.0, 0.0);
+  }
+  __syncthreads();
+  const double2 d0 = pd[3 * lane], d1 = pd[3 * lane + 1], d2 = pd[3 * lane + 2];
+  const double ex = d0.x, ey = d0.y, ez = d1.x, rk = d1.y, ir = d2.x, qneg = d2.y;
+  // phase 2: the gradient factors per (l, m): real x, y, z, imaginary x, y, z of the
+  // multipole and of the local entry
+  for (int k = threadIdx.x; k < NP; k += kTeam * 32) {
+    const PairSrc src = g_psrc[rec_off(L) + k];
+#pragma unroll
+    for (int s = 0; s < 2; ++s) {
+      const TeamFac f = g_tfac[s][rec_off(L) + k];
+      const double2 c1 = sc[src.i[3 * s]], c2 = sc[src.i[3 * s + 1]], c0 = sc[src.i[3 * s + 2]];
+      double2* o = reinterpret_cast<double2*>(rec + 12 * k + 6 * s);
+      o[0] = make_double2(f.s1r * c1.x + f.s2 * c2.x, f.s2 * c2.y - f.s1i * c1.y);
+      o[1] = make_double2(f.sz * c0.x, f.s1i * c1.y + f.s2 * c2.y);
+      o[2] = make_double2(f.s1r * c1.x - f.s2 * c2.x, f.sz * c0.y);
+    }
+  }
+  // near field: rounds s = warp + 1, warp + 5, ... of the ring of 32 (as field_tile's,
+  // with the factors of field_pair); round 16 is taken by both lanes of a pair
+  double Nx = 0.0, Ny = 0.0, Nz = 0.0, Na = 0.0;
+#pragma unroll 1
+  for (int s = warp + 1; s <= 16; s += kTeam) {
+    const int src = (lane + s) & 31;
+    const bool me_inner = lane < src;
+    const double2 p0 = pd[3 * src], p1 = pd[3 * src + 1], p2 = pd[3 * src + 2];
+    const double u = ex * p0.x + ey * p0.y + ez * p1.x;
+    const double iro = me_inner ? p2.x : ir, sr = (me_inner ? rk : p1.y) * iro;
+    double S0, S1, S2;
+    pair_sums_f64<L>(sr * u, sr * sr, S0, S1, S2);
+    const double Sp = S2 * sr, uS = u * Sp;
+    const double cin = S1 - uS, cout = -(S0 + S1 + uS);
+    const double gab = ir * p2.x, go2 = iro * iro;
+    const double gm = (me_inner ? gab : go2) * p2.y, be = Sp * gm;
+    Nx = fma(be, p0.x, Nx); Ny = fma(be, p0.y, Ny); Nz = fma(be, p1.x, Nz);
+    Na = fma(me_inner ? cin : cout, gm, Na);
+    if (s < 16) {
+      const double gp = (me_inner ? go2 : gab) * qneg;
+      const double ao = (me_inner ? cout : cin) * gp, bo = Sp * gp;
+      const int from = (lane - s) & 31;
+      const double ra = __shfl_sync(0xffffffffu, ao, from), rb = __shfl_sync(0xffffffffu, bo, from);
+      const double2 c0 = pd[3 * from], c1 = pd[3 * from + 1];
+      Nx = fma(rb, c0.x, Nx); Ny = fma(rb, c0.y, Ny); Nz = fma(rb, c1.x, Nz);
+      Na += ra;
+    }
+  }
+  double Ex = a.pf_t * (Nx + Na * ex), Ey = a.pf_t * (Ny + Na * ey), Ez = a.pf_t * (Nz + Na * ez);
+  __syncthreads();
+  // phase 3: far-field columns m = warp, warp + 4, ...: (ex + i ey)^m times the sums over
+  // l of the real p_l, p_{l+1} = an cos(t) p_l - p_{l-1}, with both parts' factors and powers
+  {
+    double dr = 1.0, di = 0.0;
+    for (int k = 0; k < warp; ++k) {
+      const double t = dr * ex - di * ey;
+      di = dr * ey + di * ex;
+      dr = t;
+    }
+    const double q2r = ex * ex - ey * ey, q2i = 2.0 * ex * ey;
+    const double q4r = q2r * q2r - q2i * q2i, q4i = 2.0 * q2r * q2i;
+#pragma unroll 1
+    for (int m = warp; m <= L + 1; m += kTeam) {
+      double p1 = 1.0, p0 = 0.0;
+      double Sx = 0.0, Sy = 0.0, Sz = 0.0, Tx = 0.0, Ty = 0.0, Tz = 0.0;
+      const double2* rc = reinterpret_cast<const double2*>(rec + 12 * offP(L, m));
+      auto step = [&](int l) {
+        if (l > m) {
+          const double pn = fma(tb.an[l * kTabL + m] * ez, p1, -p0);
+          p0 = p1; p1 = pn;
+        }
+      };
+      auto add = [&](const double2* c, double p) {
+        const double2 c0 = c[0], c1 = c[1];
+        Sx = fma(c0.x, p, Sx); Sy = fma(c0.y, p, Sy); Sz = fma(c1.x, p, Sz);
+        if (m > 0) {
+          const double2 c2 = c[2];
+          Tx = fma(c1.y, p, Tx); Ty = fma(c2.x, p, Ty); Tz = fma(c2.y, p, Tz);
+        }
+      };
+      int l = m;
+#pragma unroll 2
+      for (; l <= L - 1; ++l, rc += 6) {
+        step(l);
+        add(rc, p1 * uI[32 * l + lane]);
+        add(rc + 3, p1 * uR[32 * l + lane]);
+      }
+      for (; l <= L + 1; ++l, rc += 6) {
+        step(l);
+        add(rc, p1 * uI[32 * l + lane]);
+      }
+      Ex = fma(dr, Sx, fma(di, Tx, Ex)); Ey = fma(dr, Sy, fma(di, Ty, Ey)); Ez = fma(dr, Sz, fma(di, Tz, Ez));
+      const double t = dr * q4r - di * q4i;
+      di = dr * q4i + di * q4r;
+      dr = t;
+    }
+  }
+  part[96 * warp + lane] = Ex;
+  part[96 * warp + 32 + lane] = Ey;
+  part[96 * warp + 64 + lane] = Ez;
+  __syncthreads();
+  if (warp != kTeam - 1) return;  // the warp with the shortest columns goes on
+  Ex = Ey = Ez = 0.0;
+#pragma unroll
+  for (int w = 0; w < kTeam; ++w) {
+    Ex += part[96 * w + lane]; Ey += part[96 * w + 32 + lane]; Ez += part[96 * w + 64 + lane];
+  }
+  double qmob = 0.0;
+  if (a.species) {
+    const double qc = -qneg;
+    double incl = qc;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const double t = __shfl_up_sync(0xffffffffu, incl, d);
+      if (lane >= d) incl += t;
+    }
+    qmob = a.qgbase[g] + a.qpfx[tile] + (incl - qc);
+  }
+  const bool push = a.mode == 0 && valid;
+  const double VX = push ? a.vx[j] : 0.0, VY = push ? a.vy[j] : 0.0, VZ = push ? a.vz[j] : 0.0;
+  const double X = valid ? a.x[j] : a.r_out, Y = valid ? a.y[j] : 0.0, Z = valid ? a.z[j] : 0.0;
+  field_finish<double, L>(a, j, valid, valid && qneg != 1.0, qneg, X, Y, Z, VX, VY, VZ, rk * rk, ir * ir, ir, Ex, Ey, Ez, qmob,
+                          a.q_s + a.st->qs_acc, a.id + j);
+}
+
+template <int L>
+__global__ void __launch_bounds__(kTeam * 32) k_field_team(FieldArgs<double> a) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  chain_wait();
+  field_team<L>(a, smem_raw, int64_t(gridDim.x) - 1 - blockIdx.x);
+}
+template <int L>
+__global__ void __launch_bounds__(kTeam * 32) k_field_team_batch(const FieldArgs<double>* __restrict__ args,
+                                                               const int2* __restrict__ items) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ FieldArgs<double> sa;
+  const int2 it = items[blockIdx.x];
+  copy_args(args + it.x, &sa);
+  __syncthreads();
+  field_team<L>(sa, smem_raw, it.y);
 }
 
 // Register budget: in FP32, at least 3 CTAs of 256 threads per SM (80
