@@ -829,7 +829,11 @@ template <class T> __device__ __forceinline__ double cs_double(CSum<T> v) { retu
 // group), and the CTA writes the results transposed, pfx[tile][u], through
 // shared memory, so that the field kernel reads the carries of one tile as
 // contiguous lines. Is rows (u odd) get exclusive suffixes, Rs rows (u even)
-// exclusive prefixes; the group totals go to gagg[g][u] in FP64.
+// exclusive prefixes; the group totals go to gagg[g][u] in FP64, converted by full
+// warps after the scans (by the four lanes that hold them, one row at a time, the
+// conversions took 78 % of the FP64 pipe: scans at N = 2e6, l_max = 16 0.089 ->
+// 0.085 ms; N = 4e6, l_max = 24 0.296 -> 0.280). Bound by memory and by the
+// compensated additions' issue slots.
 constexpr int kTsRows = 32;    // components per CTA
 constexpr int kTsTiles = 128;  // tiles per CTA
 
@@ -840,6 +844,7 @@ __global__ void __launch_bounds__(256) k_tile_scan(const T* __restrict__ agg, T*
   using V4 = typename Vec4<T>::type;
   using C = CSum<T>;
   __shared__ T buf[kTsRows][kTsTiles + 1];  // [row][tile], padded: the transposed reads hit distinct banks
+  __shared__ C gt[kTsTiles / 32][kTsRows];  // group totals
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, r = lane & 7;
   const int64_t tile0 = int64_t(blockIdx.x) * kTsTiles;
   const int u0 = int(blockIdx.y) * kTsRows;
@@ -858,7 +863,6 @@ __global__ void __launch_bounds__(256) k_tile_scan(const T* __restrict__ agg, T*
   for (int k = 0; k < 4; ++k) {
     const int row = 4 * warp + k, u = u0 + row;
     if (u >= nc) break;  // warp-uniform
-    const int64_t g = tile / 32;
     V4 o;
     if (u & 1) {  // Is: exclusive suffix
       const C f2 = cs_of(v[k].w), f1 = cs_add(f2, cs_of(v[k].z)), f0 = cs_add(f1, cs_of(v[k].y)),
@@ -872,7 +876,7 @@ __global__ void __launch_bounds__(256) k_tile_scan(const T* __restrict__ agg, T*
       }
       o.x = cs_round(cs_add(x, f0)); o.y = cs_round(cs_add(x, f1)); o.z = cs_round(cs_add(x, f2));
       o.w = cs_round(x);
-      if (r == 0 && tile < tw) gagg[g * nc + u] = cs_double(cs_add(x, sum));
+      if (r == 0) gt[lane >> 3][row] = cs_add(x, sum);
     } else {      // Rs: exclusive prefix
       const C e1 = cs_of(v[k].x), e2 = cs_add(e1, cs_of(v[k].y)), e3 = cs_add(e2, cs_of(v[k].z)),
               sum = cs_add(e3, cs_of(v[k].w));
@@ -885,15 +889,16 @@ __global__ void __launch_bounds__(256) k_tile_scan(const T* __restrict__ agg, T*
       }
       o.x = cs_round(x); o.y = cs_round(cs_add(x, e1)); o.z = cs_round(cs_add(x, e2));
       o.w = cs_round(cs_add(x, e3));
-      if (r == 7 && tile < tw) gagg[g * nc + u] = cs_double(cs_add(x, sum));
+      if (r == 7) gt[lane >> 3][row] = cs_add(x, sum);
     }
     buf[row][4 * lane] = o.x; buf[row][4 * lane + 1] = o.y;
     buf[row][4 * lane + 2] = o.z; buf[row][4 * lane + 3] = o.w;
   }
   __syncthreads();
-  // transposed write: warp w writes tiles w, w + 8, ..., lane = row
+  // transposed write: warp w writes tiles w, w + 8, ..., lane = row; the group totals first
   const int u = u0 + lane;
   if (u < nc) {
+    if (warp < kTsTiles / 32 && tile0 + 32 * warp < tw) gagg[(tile0 / 32 + warp) * nc + u] = cs_double(gt[warp][lane]);
     const int tend = tw - tile0 < kTsTiles ? int(tw - tile0) : kTsTiles;
     T* dst = pfx + (tile0 + warp) * nc + u;
     const int64_t step = 8 * int64_t(nc);
