@@ -33,7 +33,7 @@ sys.path.insert(0, ROOT)
 
 METRIC = "particle-steps/s at N=2e6,l_max=16 (mixed vs FP64); served spectra p50/p99"
 UNIT = "particle-steps/s"
-BUCKET_SORT_SINGLE_N = 3072  # the library sorts up to this many keys in 1 launch,
+BUCKET_SORT_SINGLE_N = 4096  # the library sorts up to this many keys in 1 launch,
 BUCKET_SORT_MAX_N = 2250000  # up to this many in 4, more in 12
 
 

@@ -371,29 +371,47 @@ __device__ __forceinline__ void count_low_byte(const uint32_t* keys, int64_t len
   }
 }
 
-// cap: the largest segment sorted in shared memory (dynamic shared memory of
-// 16 cap bytes: two key and two value buffers). With rowtot (nd digit totals
-// of the first pass), CTA c sorts the top-digit buckets g c .. g c + g - 1 of
-// k1/v1 into k0/v0: by bytes 0..2 when g = 1, by all four bytes when a CTA
-// takes several buckets (small instances: fewer, fuller CTAs). Without rowtot
-// (one CTA, n_single <= cap), the whole array k0/v0 by all four bytes, in
-// place. MINB: resident CTAs per SM asked of the register allocation.
+// Sort of one segment (the whole array, or g consecutive top-digit buckets) in one CTA.
+// The keys of a segment spread over its range like the density over r^2, so a second digit of
+// sb bits with about one key per value leaves almost nothing to sort: the CTA counts the
+// digits (shared atomics), scans the counts, places (key, slot in the segment) by digit in any
+// order, and each placed key finds its rank among the few of its digit by comparing (key, slot):
+// the permutation of a stable sort, whatever the order of the atomics. Against three byte passes
+// (bucket_pass), each of which ranks 32 keys by eight ballots and waits at five barriers a chunk.
+// A digit of more than kBsMaxRun keys (ties, narrow shells) or a segment of more than cap keys
+// sends the segment through those passes: by the bytes below its top bits, in shared memory when
+// 16 bytes a key fit, else through L2.
+// src (keys, slots) -> dst_v: the source slots in key order. src and dst are both scratch then.
+// Bound by the latency of the shared atomics and of the loads from L2; 512 threads rather than
+// 256 keep more of them in flight. Sort ms, byte passes -> this: N = 3001 0.0256 -> 0.0101,
+// 20000 0.0203 -> 0.0165, 5e5 0.040 -> 0.0236, 2e6 0.111 -> 0.091 (this kernel 0.067 -> 0.037).
+// tb: leading key bits the same in all of the segment; sb <= 32 - tb, 2^sb >= NT.
+constexpr int kBsMaxRun = 128;
+constexpr int kBsThreads = 512, kBsPerSM = 3;  // CTA of a segment, resident per SM
+constexpr int kBsOneThreads = 1024;  // the one CTA of a small array
+static_assert(kBsThreads >= 256 && kBsOneThreads >= 256, "256 threads add up the bucket sizes");
+constexpr size_t kBsRankBytes = 6;  // shared memory per key: key and slot (cap < 2^16)
+
 template <int NT, int MINB>
-__global__ void __launch_bounds__(NT, MINB) k_bucket_sort(uint32_t* k1, uint32_t* v1, uint32_t* k0, uint32_t* v0,
-                                                          const uint32_t* __restrict__ rowtot, int64_t n_single,
-                                                          int cap, int g, int nd) {
+__global__ void __launch_bounds__(NT, MINB) k_bucket_sort(uint32_t* src_k, uint32_t* src_v, uint32_t* dst_k,
+                                                          uint32_t* dst_v, const uint32_t* __restrict__ rowtot,
+                                                          int64_t n_single, int cap, int g, int nd, int tb, int sb,
+                                                          unsigned dyn) {
   chain_wait();
   extern __shared__ __align__(16) uint32_t sbuf[];
-  __shared__ BsShared<NT> sh;
-  __shared__ uint32_t s_len[8];
-  __shared__ int64_t s_start, s_n;
+  __shared__ uint32_t s_pre[8], s_len[8], s_w[NT / 32];
   const unsigned t = threadIdx.x, lane = t & 31, warp = t >> 5;
-  const unsigned b0 = blockIdx.x * unsigned(g), b1 = b0 + unsigned(g);
+  uint32_t* const cnt = sbuf;                                   // [2^sb]
+  uint32_t* const ks = cnt + (1 << sb);                         // [cap]
+  uint16_t* const ps = reinterpret_cast<uint16_t*>(ks + cap);   // [cap]
   // segment start and length: the sizes of the buckets before it and in it
   // (thread t < 256 adds the digits nd / 256 t .. nd / 256 (t + 1) - 1)
-  if (t < 256) {
-    uint32_t v = 0u, w = 0u;
-    if (rowtot) {
+  int64_t start = 0, len = n_single;
+  for (int k = t; k < 1 << sb; k += NT) cnt[k] = 0u;
+  if (rowtot) {
+    const unsigned b0 = blockIdx.x * unsigned(g), b1 = b0 + unsigned(g);
+    if (t < 256) {
+      uint32_t v = 0u, w = 0u;
       const unsigned per = unsigned(nd) / 256u;
       for (unsigned k = 0; k < per; ++k) {
         const unsigned d = per * t + k;
@@ -401,62 +419,127 @@ __global__ void __launch_bounds__(NT, MINB) k_bucket_sort(uint32_t* k1, uint32_t
         if (d < b0) v += c;
         else if (d < b1) w += c;
       }
-    }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      v += __shfl_down_sync(0xffffffffu, v, o);
-      w += __shfl_down_sync(0xffffffffu, w, o);
+      for (int o = 16; o > 0; o >>= 1) {
+        v += __shfl_down_sync(0xffffffffu, v, o);
+        w += __shfl_down_sync(0xffffffffu, w, o);
+      }
+      if (lane == 0) {
+        s_pre[warp] = v;
+        s_len[warp] = w;
+      }
     }
-    if (lane == 0) {
-      sh.wsum[warp] = v;
-      s_len[warp] = w;
-    }
-    sh.cnt[0][t] = 0u;
-  }
-  __syncthreads();
-  if (t == 0) {
-    int64_t a = 0, m = 0;
+    __syncthreads();
+    len = 0;
+#pragma unroll
     for (int k = 0; k < 8; ++k) {
-      a += sh.wsum[k];
-      m += s_len[k];
+      start += s_pre[k];
+      len += s_len[k];
     }
-    s_start = a;
-    s_n = m;
+  } else {
+    __syncthreads();
   }
-  __syncthreads();
-  const bool single = rowtot == nullptr;
-  const int64_t start = s_start;
-  const int64_t len = single ? n_single : s_n;
   if (len == 0) return;  // uniform over the CTA
-  const bool all4 = single || g > 1;  // the segment spans several top digits
-  uint32_t *sk = single ? k0 : k1 + start, *sv = single ? v0 : v1 + start;
-  uint32_t *gk0 = k0 + start, *gv0 = v0 + start, *gk1 = k1 + start, *gv1 = v1 + start;
+  const uint32_t* const sk = src_k + start;
+  const uint32_t* const sv = src_v + start;
+  bool fits = len <= cap;
+  if (fits) {
+    const int n = int(len), shift = 32 - sb;
+    constexpr int U = 4;  // loads in flight per thread
+    for (int i0 = 0; i0 < n; i0 += NT * U) {
+      uint32_t k[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) k[u] = i0 + u * NT + int(t) < n ? sk[i0 + u * NT + t] : 0u;
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (i0 + u * NT + int(t) < n) atomicAdd(&cnt[(k[u] << tb) >> shift], 1u);
+    }
+    __syncthreads();
+    // exclusive scan of the counts, each thread 2^sb / NT of them
+    const int per = (1 << sb) / NT;
+    uint32_t* const mine = cnt + per * t;
+    uint32_t sum = 0, big = 0;
+    for (int k = 0; k < per; ++k) {
+      const uint32_t c = mine[k];
+      sum += c;
+      big = c > big ? c : big;
+    }
+    fits = !__syncthreads_or(big > unsigned(kBsMaxRun));
+    if (fits) {
+      uint32_t inc = sum;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t x = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= unsigned(o)) inc += x;
+      }
+      if (lane == 31) s_w[warp] = inc;
+      __syncthreads();
+      uint32_t off = inc - sum;
+      for (unsigned w = 0; w < warp; ++w) off += s_w[w];
+      for (int k = 0; k < per; ++k) {
+        const uint32_t c = mine[k];
+        mine[k] = off;
+        off += c;
+      }
+      __syncthreads();
+      for (int i0 = 0; i0 < n; i0 += NT * U) {
+        uint32_t k[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) k[u] = i0 + u * NT + int(t) < n ? sk[i0 + u * NT + t] : 0u;
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const int i = i0 + u * NT + int(t);
+          if (i < n) {
+            const uint32_t p = atomicAdd(&cnt[(k[u] << tb) >> shift], 1u);
+            ks[p] = k[u];
+            ps[p] = uint16_t(i);
+          }
+        }
+      }
+      __syncthreads();
+      // cnt[s] is now the end of digit s
+      uint32_t* const out = dst_v + start;
+      for (int p = t; p < n; p += NT) {
+        const uint32_t key = ks[p], slot = ps[p], s = (key << tb) >> shift;
+        const uint32_t b = s ? cnt[s - 1] : 0u, e = cnt[s];
+        uint32_t r = b;
+        for (uint32_t q = b; q < e; ++q) {
+          const uint32_t kq = ks[q];
+          r += kq < key || (kq == key && ps[q] < slot) ? 1u : 0u;
+        }
+        out[r] = sv[slot];
+      }
+      return;
+    }
+  }
+  // stable byte passes over the bits that differ
+  __syncthreads();  // the counts have been read
+  BsShared<NT>& sh = *reinterpret_cast<BsShared<NT>*>(sbuf);
+  uint32_t* const bufs = sbuf + (sizeof(BsShared<NT>) + 3) / 4;
+  if (t < 256) sh.cnt[0][t] = 0u;
+  __syncthreads();
+  uint32_t *ak = src_k + start, *av = src_v + start, *dk = dst_k + start, *dv = dst_v + start;
   count_low_byte<NT>(sk, len, sh.cnt[0]);
   __syncthreads();
-  if (len <= cap) {
-    // first pass from global memory, the middle ones in shared memory, the
-    // last into global memory
-    uint32_t *ka = sbuf, *va = sbuf + cap, *kb = sbuf + 2 * cap, *vb = sbuf + 3 * cap;
-    bucket_pass<NT>(sk, sv, ka, va, int(len), 0, sh.cnt[0], sh.cnt[1], sh);
-    bucket_pass<NT>(ka, va, kb, vb, int(len), 8, sh.cnt[1], sh.cnt[0], sh);
+  const bool all4 = tb < 8;  // the segment spans several top bytes
+  if (size_t(16) * size_t(len) + sizeof(BsShared<NT>) + 4 <= dyn) {
+    const int n = int(len);
+    uint32_t *ka = bufs, *va = bufs + n, *kb = bufs + 2 * n, *vb = bufs + 3 * n;
+    bucket_pass<NT>(ak, av, ka, va, n, 0, sh.cnt[0], sh.cnt[1], sh);
+    bucket_pass<NT>(ka, va, kb, vb, n, 8, sh.cnt[1], sh.cnt[0], sh);
     if (all4) {
-      bucket_pass<NT>(kb, vb, ka, va, int(len), 16, sh.cnt[0], sh.cnt[1], sh);
-      bucket_pass<NT>(ka, va, gk0, gv0, int(len), 24, sh.cnt[1], nullptr, sh);
+      bucket_pass<NT>(kb, vb, ka, va, n, 16, sh.cnt[0], sh.cnt[1], sh);
+      bucket_pass<NT>(ka, va, dk, dv, n, 24, sh.cnt[1], nullptr, sh);
     } else {
-      bucket_pass<NT>(kb, vb, gk0, gv0, int(len), 16, sh.cnt[0], nullptr, sh);
+      bucket_pass<NT>(kb, vb, dk, dv, n, 16, sh.cnt[0], nullptr, sh);
     }
-  } else {  // a segment (never the single array) larger than cap: through L2
-    bucket_pass<NT>(gk1, gv1, gk0, gv0, int(len), 0, sh.cnt[0], sh.cnt[1], sh);
-    bucket_pass<NT>(gk0, gv0, gk1, gv1, int(len), 8, sh.cnt[1], sh.cnt[0], sh);
+  } else {
+    bucket_pass<NT>(ak, av, dk, dv, int(len), 0, sh.cnt[0], sh.cnt[1], sh);
+    bucket_pass<NT>(dk, dv, ak, av, int(len), 8, sh.cnt[1], sh.cnt[0], sh);
+    bucket_pass<NT>(ak, av, dk, dv, int(len), 16, sh.cnt[0], all4 ? sh.cnt[1] : nullptr, sh);
     if (all4) {
-      bucket_pass<NT>(gk1, gv1, gk0, gv0, int(len), 16, sh.cnt[0], sh.cnt[1], sh);
-      bucket_pass<NT>(gk0, gv0, gk1, gv1, int(len), 24, sh.cnt[1], nullptr, sh);
-      for (int64_t i = t; i < len; i += NT) {
-        gk0[i] = gk1[i];
-        gv0[i] = gv1[i];
-      }
-    } else {
-      bucket_pass<NT>(gk1, gv1, gk0, gv0, int(len), 16, sh.cnt[0], nullptr, sh);
+      bucket_pass<NT>(dk, dv, ak, av, int(len), 24, sh.cnt[1], nullptr, sh);
+      for (int64_t i = t; i < len; i += NT) dv[i] = av[i];
     }
   }
 }
@@ -467,24 +550,36 @@ __global__ void __launch_bounds__(NT, MINB) k_bucket_sort(uint32_t* k1, uint32_t
 // saved passes (N = 4e6: 0.256 ms against 0.222 for the four global passes;
 // N = 1.6e7: 0.91 against 0.74 ms, both with the 8-bit first pass).
 constexpr int64_t kBucketSortMaxN = 2250000;
-constexpr int kBsCapMax = 13312;  // 208 KB of buckets beside the static shared memory
+constexpr int kBsCapMax = 13312;  // keys (and 2^13 counts in all of the 227 KB: 112 KB)
+constexpr int kBsBitsMax = 13;
 constexpr int64_t kBsSmallN = 1 << 19;  // up to here an 8-bit first pass (256 buckets), beyond a 9-bit one (512)
-constexpr int64_t kBsSingleN = 3072;     // up to here, one CTA sorts everything (N = 1000: 13 us)
-// shared-memory capacity for segments of g of nd buckets: three times the mean
-// segment with 256 buckets; 1.5 times with 512 (at N = 2e6 two CTAs per SM of
-// 101 KB, 94 KB of them buckets; a larger bucket goes through L2)
+constexpr int64_t kBsSingleN = 4096;     // up to here, one CTA sorts everything (0.011 ms; at 6000 keys 0.0145 against 0.015)
+// Shared-memory capacity for segments of g of nd buckets: three times the mean segment with 256
+// buckets; 1.5 times with 512. Larger segments go through L2.
 inline int bucket_cap(int64_t n, int g, int nd) {
   const int64_t mean = int64_t(g) * n / nd;
   int64_t c = ((nd == 256 ? 3 * mean : mean + mean / 2) + 255) / 256 * 256;
   if (c < 2048) c = 2048;
   return int(c < kBsCapMax ? c : kBsCapMax);
 }
+// Bits of the second digit for segments of `mean` keys: about one key per value
+inline int bucket_bits(int64_t mean, int threads) {
+  int sb = 0;
+  while ((1 << sb) < threads || ((int64_t(1) << sb) < mean && sb < kBsBitsMax)) ++sb;
+  return sb;
+}
+template <int NT> inline size_t bucket_smem(int cap, int sb) {
+  const size_t rank = (size_t(4) << sb) + kBsRankBytes * size_t(cap), pass = sizeof(BsShared<NT>) + 16;
+  return rank > pass ? rank : pass;
+}
 
 cudaError_t set_sort_attributes() {
-  const cudaError_t e = cudaFuncSetAttribute(k_bucket_sort<256, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             16 * kBsCapMax);
+  const int most = int(bucket_smem<kBsOneThreads>(kBsCapMax, kBsBitsMax));
+  const cudaError_t e = cudaFuncSetAttribute(k_bucket_sort<kBsOneThreads, 1>,
+                                             cudaFuncAttributeMaxDynamicSharedMemorySize, most);
   if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(k_bucket_sort<256, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, 16 * kBsCapMax);
+  return cudaFuncSetAttribute(k_bucket_sort<kBsThreads, kBsPerSM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              most);
 }
 
 const uint32_t* launch_radix_sort(uint32_t* k0, uint32_t* v0, uint32_t* k1, uint32_t* v1, uint32_t* hist,
@@ -492,38 +587,38 @@ const uint32_t* launch_radix_sort(uint32_t* k0, uint32_t* v0, uint32_t* k1, uint
   if (n <= 1) return v0;
   const int64_t nblk = sort_blocks(n);
   if (first_byte == 0 && n <= kBsSingleN) {
-    // one CTA sorts the whole array in shared memory, all four bytes
-    const int cap = int((n + 255) / 256 * 256);
-    seq(k_bucket_sort<256, 3>, 1, 256, size_t(16) * cap, k1, v1, k0, v0, nullptr, n, cap, 256, 256);
-    return v0;
+    const int cap = int((n + 255) / 256 * 256), sb = bucket_bits(n, kBsOneThreads);
+    const size_t smem = bucket_smem<kBsOneThreads>(cap, sb);
+    seq(k_bucket_sort<kBsOneThreads, 1>, 1, kBsOneThreads, smem, k0, v0, k1, v1, nullptr, n, cap, 1, 0, 0, sb,
+        unsigned(smem));
+    return v1;
   }
   if (first_byte == 0 && n <= kBucketSortMaxN) {
     // the top digit over the whole array into nd contiguous buckets (k0 -> k1),
     // then the bits below it per bucket (into k0): 256 buckets (the top byte)
     // up to kBsSmallN keys, 512 (the top 9 bits, buckets of ~3900 keys at
-    // N = 2e6, two CTAs per SM) beyond. Alone on the GPU, one CTA per bucket
+    // N = 2e6) beyond. Alone on the GPU, one CTA per bucket
     // (the most parallel); sharing it (a batch), a small instance takes
-    // segments of several buckets, about 2048 keys per CTA (fewer CTAs, all
-    // four bytes each): the same permutation either way
+    // segments of several buckets, about 2048 keys per CTA (fewer CTAs): the same
+    // permutation either way
     const bool wide = n > kBsSmallN;
     const int nd = wide ? 512 : 256, shift = wide ? 23 : 24;
     uint32_t* rowtot = hist + int64_t(nd) * nblk;
-    int g = 1;
-    while (shared_gpu && g < nd && int64_t(g) * 2 * n <= int64_t(2048) * nd) g *= 2;
-    const int cap = bucket_cap(n, g, nd);
+    int g = 1, tb = wide ? 9 : 8;
+    while (shared_gpu && g < nd && int64_t(g) * 2 * n <= int64_t(2048) * nd) g *= 2, --tb;
+    const int cap = bucket_cap(n, g, nd), sb = bucket_bits(int64_t(g) * n / nd, kBsThreads);
+    const size_t smem = bucket_smem<kBsThreads>(cap, sb);
     if (wide) {
       seq(k_sort_hist<512>, unsigned(nblk), kSortThreads, 0, k0, n, shift, nblk, hist);
       seq(k_sort_rowscan, 512, kSortThreads, 0, hist, nblk, rowtot);
       seq(k_sort_scatter<512>, unsigned(nblk), kSortThreads, 0, k0, v0, k1, v1, n, shift, nblk, hist, rowtot);
-      seq(k_bucket_sort<256, 2>, unsigned(512 / g), 256, size_t(16) * cap, k1, v1, k0, v0, rowtot, 0, cap, g,
-                                                                             512);
     } else {
       seq(k_sort_hist<256>, unsigned(nblk), kSortThreads, 0, k0, n, shift, nblk, hist);
       seq(k_sort_rowscan, 256, kSortThreads, 0, hist, nblk, rowtot);
       seq(k_sort_scatter<256>, unsigned(nblk), kSortThreads, 0, k0, v0, k1, v1, n, shift, nblk, hist, rowtot);
-      seq(k_bucket_sort<256, 3>, unsigned(256 / g), 256, size_t(16) * cap, k1, v1, k0, v0, rowtot, 0, cap, g,
-                                                                             256);
     }
+    seq(k_bucket_sort<kBsThreads, kBsPerSM>, unsigned(nd / g), kBsThreads, smem, k1, v1, k0, v0, rowtot, 0, cap, g, nd,
+        tb, sb, unsigned(smem));
     return v0;
   }
   uint32_t* rowtot = hist + 256 * nblk;
@@ -1286,8 +1381,8 @@ cudaError_t preload_core_kernels() {
                        reinterpret_cast<const void*>(&k_sort_rowscan),
                        reinterpret_cast<const void*>(&k_sort_scatter<256>),
                        reinterpret_cast<const void*>(&k_sort_scatter<512>),
-                       reinterpret_cast<const void*>(&k_bucket_sort<256, 3>),
-                       reinterpret_cast<const void*>(&k_bucket_sort<256, 2>),
+                       reinterpret_cast<const void*>(&k_bucket_sort<kBsOneThreads, 1>),
+                       reinterpret_cast<const void*>(&k_bucket_sort<kBsThreads, kBsPerSM>),
                        reinterpret_cast<const void*>(&k_init_step)};
   for (const void* f : fns) {
     const cudaError_t e = cudaFuncGetAttributes(&fa, f);
