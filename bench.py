@@ -33,14 +33,14 @@ sys.path.insert(0, ROOT)
 
 METRIC = "particle-steps/s at N=2e6,l_max=16 (mixed vs FP64); served spectra p50/p99"
 UNIT = "particle-steps/s"
-BUCKET_SORT_SINGLE_N = 4096  # the library sorts up to this many keys in 1 launch,
-BUCKET_SORT_MAX_N = 2250000  # up to this many in 4, more in 12
+BUCKET_SORT_SINGLE_N = 4096   # the library sorts up to this many keys in 1 launch,
+BUCKET_SORT_MAX_N = 24000000  # up to this many in 4 stages, more in 12
 
 
 def sort_launches(n):
-    """Kernel launches of one radius sort of n keys: one CTA for all of a small
-    array; up to BUCKET_SORT_MAX_N keys the top-byte pass (histogram, row scan,
-    scatter) and the per-bucket kernel; four such passes (12 launches) beyond."""
+    """Kernel stages of one sort of n keys: one CTA for all of a small array; up to
+    BUCKET_SORT_MAX_N keys the top-digit pass (counts, their scan, spread) and the
+    per-bucket kernel; four byte passes of three kernels (12 launches) beyond."""
     if n <= 1:
         return 0
     if n <= BUCKET_SORT_SINGLE_N:
@@ -56,9 +56,13 @@ def step_launches(n):
 
 def fused_stages(n):
     """Stages that ride in another stage's launch: the finalize in the first
-    group-scan kernel, and up to 32 scan groups of 1024 particles the second
-    group-scan pass too."""
-    return 2 if n <= 32 * 1024 else 1
+    group-scan kernel; up to 32 scan groups of 1024 particles the second
+    group-scan pass too; the reorder in the bucket sort, and the scan of the
+    digit counts in the counting kernel."""
+    fused = 2 if n <= 32 * 1024 else 1
+    if 1 < n <= BUCKET_SORT_MAX_N:
+        fused += 1 if n <= BUCKET_SORT_SINGLE_N else 2
+    return fused
 
 
 def workload_desc(w):

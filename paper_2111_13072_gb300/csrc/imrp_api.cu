@@ -92,7 +92,8 @@ struct imrp_ctx {
   void* srt[6] = {nullptr};   // x, y, z, vx, vy, vz in radius order (rebuilt every step)
   uint32_t* srt_id = nullptr; // their ids
   int cur = 0;                // stays 0: one state buffer (checked by the captured graphs)
-  uint32_t *key0 = nullptr, *idx0 = nullptr, *key1 = nullptr, *idx1 = nullptr, *hist = nullptr;
+  uint32_t *key0 = nullptr, *idx0 = nullptr, *key1 = nullptr, *idx1 = nullptr;
+  void* sort_scratch = nullptr;
   void *agg = nullptr, *pfx = nullptr, *gbase = nullptr, *tot = nullptr, *eout = nullptr;
   double *gagg = nullptr, *totd = nullptr, *gswork = nullptr;
   unsigned* gsticket = nullptr;
@@ -209,7 +210,7 @@ void free_all(imrp_ctx* c) {
   for (int k = 0; k < 6; ++k) { cudaFree(c->srt[k]); c->srt[k] = nullptr; }
   cudaFree(c->srt_id);
   c->srt_id = nullptr;
-  void* ps[] = {c->key0, c->idx0, c->key1, c->idx1, c->hist, c->agg, c->pfx, c->gbase, c->tot,
+  void* ps[] = {c->key0, c->idx0, c->key1, c->idx1, c->sort_scratch, c->agg, c->pfx, c->gbase, c->tot,
                 c->eout, c->gagg, c->totd, c->gswork, c->gsticket, c->qhist, c->stage, c->st,
                 c->dft};
   for (void* p : ps) cudaFree(p);
@@ -222,7 +223,8 @@ void free_all(imrp_ctx* c) {
     c->qticket = nullptr;
   }
   c->ion_n = c->ion_cap = 0;
-  c->key0 = c->idx0 = c->key1 = c->idx1 = c->hist = nullptr;
+  c->key0 = c->idx0 = c->key1 = c->idx1 = nullptr;
+  c->sort_scratch = nullptr;
   c->agg = c->pfx = c->gbase = c->tot = c->eout = nullptr;
   c->gagg = c->totd = c->gswork = c->qhist = c->uhist = c->stage = c->dft = nullptr;
   c->gsticket = nullptr;
@@ -372,10 +374,11 @@ template <class T> void enqueue_pre(imrp_ctx* ctx, LaunchSeq& seq, cudaEvent_t* 
     launch_keys<T>(st, ctx->key0, ctx->idx0, n, ctx->r_out, seq);
   }
   stage_event(seq, ev, 0);
-  const uint32_t* perm = launch_radix_sort(ctx->key0, ctx->idx0, ctx->key1, ctx->idx1, ctx->hist, n,
-                                           sort_first_byte(ctx->prec), seq, shared_gpu);
+  const uint32_t* perm =
+      launch_radix_sort<T>(ctx->key0, ctx->idx0, ctx->key1, ctx->idx1, ctx->sort_scratch, n, sort_first_byte(ctx->prec),
+                           st, sorted_ptrs<T>(ctx), ctx->srt_id, seq, shared_gpu);
   stage_event(seq, ev, 1);
-  launch_reorder<T>(st, sorted_ptrs<T>(ctx), ctx->srt_id, perm, n, seq);
+  if (perm) launch_reorder<T>(st, sorted_ptrs<T>(ctx), ctx->srt_id, perm, n, seq);
 }
 
 template <class T> void enqueue_mid(imrp_ctx* ctx, LaunchSeq& seq, bool record) {
@@ -494,7 +497,7 @@ size_t footprint_bytes(int64_t N, int L, int prec) {
   b += N * (es == 4 ? sizeof(Part<float>) : sizeof(Part<double>));  // state records
   b += 6 * N * es + N * 4;                          // radius-ordered copy + ids
   b += 4 * size_t(N) * 4;                           // keys and slots
-  b += size_t(sort_hist_words(N)) * 4;              // histogram
+  b += sort_scratch_bytes(N);                       // digit counts
   b += 2 * size_t(tile_stride(ntiles) * nc) * es;   // tile sums and in-group scans
   b += size_t(ngroups * nc) * (es + 8) + size_t(nc) * (es + 8);
   b += size_t(gs_work_doubles(int(nc))) * 8 + size_t(gs_tickets(int(nc))) * 4;
@@ -516,7 +519,8 @@ int alloc_ctx(imrp_ctx* ctx) {
   CK(cudaMalloc(&ctx->idx0, N * sizeof(uint32_t)));
   CK(cudaMalloc(&ctx->key1, N * sizeof(uint32_t)));
   CK(cudaMalloc(&ctx->idx1, N * sizeof(uint32_t)));
-  CK(cudaMalloc(&ctx->hist, size_t(sort_hist_words(N)) * sizeof(uint32_t)));
+  CK(cudaMalloc(&ctx->sort_scratch, sort_scratch_bytes(N)));
+  CK(cudaMemset(ctx->sort_scratch, 0, sizeof(SortState)));
   CK(cudaMalloc(&ctx->agg, tile_stride(ntiles) * nc * es));
   CK(cudaMalloc(&ctx->pfx, tile_stride(ntiles) * nc * es));
   CK(cudaMalloc(&ctx->gbase, ngroups * nc * es));

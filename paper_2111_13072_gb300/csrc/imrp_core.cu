@@ -10,18 +10,17 @@
 namespace imrp {
 
 // ============================================================================
-// Radix sort: stable LSD passes of 8-bit digits, and a wide first pass of
-// 9-bit digits for the bucket sort of large arrays. Each CTA owns
-// kSortTile = 2048 consecutive keys in a striped layout (item i of thread t is
-// key base + i*256 + t), which keeps the slot order (item, warp, lane) equal
-// to the key order, so the local ranks below are stable. ND: digits of the
-// pass (256 or 512); hist holds ND rows of nblk block counts.
+// Global passes (arrays too large for the bucket sort below): a stable LSD radix
+// sort of 8-bit digits. Each CTA owns kSortTile = 2048 consecutive keys in a
+// striped layout (item i of thread t is key base + i*256 + t), which keeps the
+// slot order (item, warp, lane) equal to the key order, so the local ranks below
+// are stable; hist holds 256 rows of nblk block counts.
 // ============================================================================
-template <int ND>
 __global__ void __launch_bounds__(kSortThreads) k_sort_hist(const uint32_t* __restrict__ keys,
                                                            int64_t n, int shift, int64_t nblk,
                                                            uint32_t* __restrict__ hist) {
   chain_wait();
+  constexpr int ND = 256;
   __shared__ uint32_t h[ND];
   for (int d = threadIdx.x; d < ND; d += kSortThreads) h[d] = 0;
   __syncthreads();
@@ -128,19 +127,16 @@ __device__ __forceinline__ unsigned digit_peers(unsigned d, bool ok) {
 // The block's keys and slots are staged in shared memory in that order, so
 // that consecutive threads write consecutive positions of each digit's run
 // in the output (coalesced even when the digits are uniformly spread). Thread
-// t owns the digits DPT t .. DPT t + DPT - 1 in the per-digit steps. With 256
-// digits about 22 KB of shared memory and at most 36 registers per thread (7
-// blocks per SM, so all blocks of N = 2e6 keys are resident at once); with
-// 512 digits about 29 KB. Ranking by __match_any_sync: the keys of a warp
-// arrive nearly sorted, so few distinct top digits (faster here than ballots).
-template <int ND>
-__global__ void __launch_bounds__(kSortThreads, ND == 256 ? 7 : 6) k_sort_scatter(
+// t owns digit t in the per-digit steps. About 22 KB of shared memory and at most
+// 36 registers per thread (7 blocks per SM). Ranking by __match_any_sync (faster
+// here than ballots).
+__global__ void __launch_bounds__(kSortThreads, 7) k_sort_scatter(
     const uint32_t* __restrict__ kin, const uint32_t* __restrict__ vin, uint32_t* __restrict__ kout,
     uint32_t* __restrict__ vout, int64_t n, int shift, int64_t nblk,
     const uint32_t* __restrict__ hist, const uint32_t* __restrict__ rowtot) {
   chain_wait();
   constexpr int kWarps = kSortThreads / 32;
-  constexpr int DPT = ND / kSortThreads;
+  constexpr int ND = 256, DPT = ND / kSortThreads;
   static_assert(kSortItems * 32 <= 256 && kSortTile <= 65535, "per-warp counts fit 16 bits");
   __shared__ __align__(16) uint16_t whist[kWarps][ND];
   __shared__ __align__(16) uint32_t sk[kSortTile];
@@ -243,46 +239,33 @@ __global__ void __launch_bounds__(kSortThreads, ND == 256 ? 7 : 6) k_sort_scatte
   }
 }
 
-// Sort of one top-digit bucket by the key bits below the digit, in one CTA.
-// The first pass of the sort (on the top byte, or on the top 9 bits, over the
-// whole array) leaves the keys of bucket b contiguous and in their input
-// order; this CTA then runs three stable LSD passes over its bucket, bytes 0,
-// 1, 2 (with a 9-bit top digit the top bit of byte 2 is the same for the
-// whole bucket), which need no global synchronisation: in shared memory when
-// the bucket fits (the first pass reads the bucket from global memory, the
-// last writes it back), else between the two global key/value buffers (in L2;
-// the CTA alone touches that range). A pass: the scan of the byte's digit
-// counts, then the bucket in chunks of NT * kBsItems keys in order; each warp
-// ranks its 256 keys (item i of lane l is chunk slot 256 w + 32 i + l) against
-// its running digit counts, the warps' counts are scanned per digit, and each
-// key goes to (digit start) + (keys of that digit in earlier chunks and warps)
-// + (its rank in its warp): stable. A warp whose part of the chunk holds no
-// keys, and items past the end, skip the ranking. The peers of a key in its
-// warp come from one ballot per digit bit (the low bytes are spread evenly
-// over the digits, where that is faster than __match_any_sync). The next
-// byte's counts are gathered as keys are placed. The result is the
-// permutation of a stable LSD sort on all four bytes.
-constexpr int kBsItems = 8;
+// Stable byte pass of one CTA over a bucket in global memory (in L2; the CTA alone touches
+// that range): the scan of the byte's digit counts, then the bucket in chunks of NT * kBsItems
+// keys in order; each warp ranks its keys (item i of lane l is slot 32 i + l of its part of the
+// chunk) against its running digit counts, the warps' counts are scanned per digit, and each
+// key goes to (digit start) + (keys of that digit in earlier chunks and warps) + (its rank in
+// its warp). A warp whose part of the chunk holds no keys, and items past the end, skip the
+// ranking. The peers of a key in its warp come from one ballot per digit bit.
+constexpr int kBsItems = 4;
 
 template <int NT> struct BsShared {
-  uint32_t cnt[2][256];              // digit counts of this pass's byte and of the next
+  uint32_t cnt[256];                 // digit counts of this pass's byte
   uint32_t dst[256];                 // output place of the next key of digit d
   uint16_t whist[NT / 32][256];      // per-warp counts, then the counts of earlier warps
   uint32_t wsum[8];
 };
 
 // One pass over len (< 2^31) keys (slots 0 .. len-1 of ki/vi into ko/vo), digit =
-// byte at `shift`; cnt: this byte's counts; cnx (or null): zeroed here, then
-// the counts of the byte at shift + 8.
-template <int NT, class K>
-__device__ __forceinline__ void bucket_pass(const K* ki, const K* vi, K* ko, K* vo, int len, int shift,
-                                            const uint32_t* cnt, uint32_t* cnx, BsShared<NT>& sh) {
+// byte at `shift`, whose counts are in sh.cnt.
+template <int NT>
+__device__ __forceinline__ void bucket_pass(const uint32_t* ki, const uint32_t* vi, uint32_t* ko, uint32_t* vo, int len,
+                                            int shift, BsShared<NT>& sh) {
   constexpr int kWarps = NT / 32, kChunk = NT * kBsItems;
   const unsigned t = threadIdx.x, lane = t & 31, warp = t >> 5;
   const unsigned lt = (1u << lane) - 1u;
   uint32_t c = 0, s1 = 0;
   if (t < 256) {
-    c = cnt[t];
+    c = sh.cnt[t];
     s1 = c;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -290,7 +273,6 @@ __device__ __forceinline__ void bucket_pass(const K* ki, const K* vi, K* ko, K* 
       if (lane >= unsigned(o)) s1 += x;
     }
     if (lane == 31) sh.wsum[warp] = s1;
-    if (cnx) cnx[t] = 0u;
   }
   __syncthreads();
   if (t < 256) {
@@ -345,7 +327,6 @@ __device__ __forceinline__ void bucket_pass(const K* ki, const K* vi, K* ko, K* 
           const uint32_t g = sh.dst[d] + sh.whist[warp][d] + ((wrank[i / 2] >> (16 * (i % 2))) & 0xffffu);
           ko[g] = key[i];
           vo[g] = val[i];
-          if (cnx) atomicAdd(&cnx[(key[i] >> (shift + 8)) & 255u], 1u);
         }
       }
     }
@@ -355,9 +336,9 @@ __device__ __forceinline__ void bucket_pass(const K* ki, const K* vi, K* ko, K* 
   __syncthreads();  // this pass's writes are visible to the CTA's next pass
 }
 
-// Counts of the low byte of keys[0 .. len) into cnt (loads in flight together).
+// Counts of the byte at `shift` of keys[0 .. len) into cnt (loads in flight together).
 template <int NT>
-__device__ __forceinline__ void count_low_byte(const uint32_t* keys, int64_t len, uint32_t* cnt) {
+__device__ __forceinline__ void count_byte(const uint32_t* keys, int64_t len, int shift, uint32_t* cnt) {
   for (int64_t i0 = 0; i0 < len; i0 += int64_t(NT) * kBsItems) {
     uint32_t k[kBsItems];
 #pragma unroll
@@ -367,105 +348,231 @@ __device__ __forceinline__ void count_low_byte(const uint32_t* keys, int64_t len
     }
 #pragma unroll
     for (int i = 0; i < kBsItems; ++i)
-      if (i0 + int64_t(i) * NT + threadIdx.x < len) atomicAdd(&cnt[k[i] & 255u], 1u);
+      if (i0 + int64_t(i) * NT + threadIdx.x < len) atomicAdd(&cnt[(k[i] >> shift) & 255u], 1u);
   }
 }
 
-// Sort of one segment (the whole array, or g consecutive top-digit buckets) in one CTA.
-// The keys of a segment spread over its range like the density over r^2, so a second digit of
-// sb bits with about one key per value leaves almost nothing to sort: the CTA counts the
-// digits (shared atomics), scans the counts, places (key, slot in the segment) by digit in any
-// order, and each placed key finds its rank among the few of its digit by comparing (key, slot):
-// the permutation of a stable sort, whatever the order of the atomics. Against three byte passes
-// (bucket_pass), each of which ranks 32 keys by eight ballots and waits at five barriers a chunk.
-// A digit of more than kBsMaxRun keys (ties, narrow shells) or a segment of more than cap keys
-// sends the segment through those passes: by the bytes below its top bits, in shared memory when
-// 16 bytes a key fit, else through L2.
-// src (keys, slots) -> dst_v: the source slots in key order. src and dst are both scratch then.
-// Bound by the latency of the shared atomics and of the loads from L2; 512 threads rather than
-// 256 keep more of them in flight. Sort ms, byte passes -> this: N = 3001 0.0256 -> 0.0101,
-// 20000 0.0203 -> 0.0165, 5e5 0.040 -> 0.0236, 2e6 0.111 -> 0.091 (this kernel 0.067 -> 0.037).
-// tb: leading key bits the same in all of the segment; sb <= 32 - tb, 2^sb >= NT.
-constexpr int kBsMaxRun = 128;
-constexpr int kBsThreads = 512, kBsPerSM = 3;  // CTA of a segment, resident per SM
-constexpr int kBsOneThreads = 1024;  // the one CTA of a small array
-static_assert(kBsThreads >= 256 && kBsOneThreads >= 256, "256 threads add up the bucket sizes");
-constexpr size_t kBsRankBytes = 6;  // shared memory per key: key and slot (cap < 2^16)
+// ---- bucket sort: top digit over the whole array, then each bucket in one CTA ----
+// First pass: the keys' top digit (log2 nd bits, nd <= kSortDigits) over the whole array, in
+// two kernels. k_sort_count adds up the digits (per CTA in shared memory, then one atomic per
+// digit that occurs), and its last CTA to finish (an atomic ticket, no waiting) turns the totals
+// into the buckets' starts; k_sort_spread reserves each digit's keys of a CTA with one atomic on
+// the bucket's cursor and writes them there, in any order: the order within a bucket is settled
+// by the comparisons of k_bucket_sort, so the result does not depend on the order of the atomics.
+// In its scratch (SortState) the totals and the ticket are zero between sorts.
+// The stable pass (histogram matrix, row scan, ranked scatter; it serves the four global passes of
+// very large arrays) took 7 + 6 + 20 us at N = 2e6; these two take 10 + 16, bound by latency.
+constexpr int kSpreadThreads = 512;
+constexpr int kSpreadItems = 8;
+constexpr int kSpreadTile = kSpreadThreads * kSpreadItems;  // keys per CTA
 
-template <int NT, int MINB>
-__global__ void __launch_bounds__(NT, MINB) k_bucket_sort(uint32_t* src_k, uint32_t* src_v, uint32_t* dst_k,
-                                                          uint32_t* dst_v, const uint32_t* __restrict__ rowtot,
-                                                          int64_t n_single, int cap, int g, int nd, int tb, int sb,
-                                                          unsigned dyn) {
+__global__ void __launch_bounds__(kSpreadThreads) k_sort_count(const uint32_t* __restrict__ keys, int64_t n, int shift,
+                                                               int nd, SortState* st) {
   chain_wait();
   extern __shared__ __align__(16) uint32_t sbuf[];
-  __shared__ uint32_t s_pre[8], s_len[8], s_w[NT / 32];
+  __shared__ uint32_t s_w[kSpreadThreads / 32];
+  __shared__ bool last;
+  uint32_t* const cnt = sbuf;  // [nd]
   const unsigned t = threadIdx.x, lane = t & 31, warp = t >> 5;
-  uint32_t* const cnt = sbuf;                                   // [2^sb]
-  uint32_t* const ks = cnt + (1 << sb);                         // [cap]
-  uint16_t* const ps = reinterpret_cast<uint16_t*>(ks + cap);   // [cap]
-  // segment start and length: the sizes of the buckets before it and in it
-  // (thread t < 256 adds the digits nd / 256 t .. nd / 256 (t + 1) - 1)
-  int64_t start = 0, len = n_single;
-  for (int k = t; k < 1 << sb; k += NT) cnt[k] = 0u;
-  if (rowtot) {
-    const unsigned b0 = blockIdx.x * unsigned(g), b1 = b0 + unsigned(g);
-    if (t < 256) {
-      uint32_t v = 0u, w = 0u;
-      const unsigned per = unsigned(nd) / 256u;
-      for (unsigned k = 0; k < per; ++k) {
-        const unsigned d = per * t + k;
-        const uint32_t c = rowtot[d];
-        if (d < b0) v += c;
-        else if (d < b1) w += c;
-      }
+  for (int d = t; d < nd; d += kSpreadThreads) cnt[d] = 0u;
+  const int64_t base = int64_t(blockIdx.x) * kSpreadTile;
+  uint32_t k[kSpreadItems];
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        v += __shfl_down_sync(0xffffffffu, v, o);
-        w += __shfl_down_sync(0xffffffffu, w, o);
-      }
-      if (lane == 0) {
-        s_pre[warp] = v;
-        s_len[warp] = w;
-      }
-    }
-    __syncthreads();
-    len = 0;
+  for (int i = 0; i < kSpreadItems; ++i) {
+    const int64_t o = base + i * kSpreadThreads + int64_t(t);
+    k[i] = o < n ? keys[o] : 0u;
+  }
+  __syncthreads();
 #pragma unroll
-    for (int k = 0; k < 8; ++k) {
-      start += s_pre[k];
-      len += s_len[k];
+  for (int i = 0; i < kSpreadItems; ++i) {
+    const bool ok = base + i * kSpreadThreads + int64_t(t) < n;
+    const unsigned d = k[i] >> shift, d0 = __shfl_sync(0xffffffffu, d, 0);
+    if (__all_sync(0xffffffffu, ok && d == d0)) {  // 32 keys of one digit (nearly sorted input): one atomic
+      if (lane == 0) atomicAdd(&cnt[d0], 32u);
+    } else if (ok) {
+      atomicAdd(&cnt[d], 1u);
     }
-  } else {
-    __syncthreads();
+  }
+  __syncthreads();
+  for (int d = t; d < nd; d += kSpreadThreads)
+    if (cnt[d]) atomicAdd(&st->tot[d], cnt[d]);
+  __threadfence();
+  __syncthreads();
+  if (t == 0) last = atomicAdd(&st->ticket, 1u) == gridDim.x - 1;
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  // starts of the buckets: exclusive scan of the totals, which go back to zero
+  const int per = (nd + kSpreadThreads - 1) / kSpreadThreads;
+  uint32_t sum = 0;
+  for (int i = 0; i < per; ++i) {
+    const int d = per * int(t) + i;
+    if (d < nd) {
+      const uint32_t c = __ldcg(&st->tot[d]);
+      cnt[d] = c;
+      st->tot[d] = 0u;
+      sum += c;
+    }
+  }
+  uint32_t inc = sum;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t x = __shfl_up_sync(0xffffffffu, inc, o);
+    if (lane >= unsigned(o)) inc += x;
+  }
+  if (lane == 31) s_w[warp] = inc;
+  __syncthreads();
+  uint32_t off = inc - sum;
+  for (unsigned w = 0; w < warp; ++w) off += s_w[w];
+  for (int i = 0; i < per; ++i) {
+    const int d = per * int(t) + i;
+    if (d < nd) {
+      st->cur[d] = off;
+      off += cnt[d];
+    }
+  }
+  if (t == 0) st->ticket = 0u;
+}
+
+__global__ void __launch_bounds__(kSpreadThreads) k_sort_spread(const uint32_t* __restrict__ keys, int64_t n, int shift,
+                                                                int nd, SortState* st, uint32_t* __restrict__ kout,
+                                                                uint32_t* __restrict__ vout) {
+  chain_wait();
+  extern __shared__ __align__(16) uint32_t sbuf[];
+  uint32_t* const cnt = sbuf;  // [nd]: counts, then the place of the CTA's first key of the digit
+  const unsigned t = threadIdx.x, lane = t & 31;
+  for (int d = t; d < nd; d += kSpreadThreads) cnt[d] = 0u;
+  const int64_t base = int64_t(blockIdx.x) * kSpreadTile;
+  uint32_t k[kSpreadItems], r[kSpreadItems];
+#pragma unroll
+  for (int i = 0; i < kSpreadItems; ++i) {
+    const int64_t o = base + i * kSpreadThreads + int64_t(t);
+    k[i] = o < n ? keys[o] : 0u;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < kSpreadItems; ++i) {
+    const bool ok = base + i * kSpreadThreads + int64_t(t) < n;
+    const unsigned d = k[i] >> shift, d0 = __shfl_sync(0xffffffffu, d, 0);
+    r[i] = 0u;
+    if (__all_sync(0xffffffffu, ok && d == d0)) {
+      if (lane == 0) r[i] = atomicAdd(&cnt[d0], 32u);
+      r[i] = __shfl_sync(0xffffffffu, r[i], 0) + lane;
+    } else if (ok) {
+      r[i] = atomicAdd(&cnt[d], 1u);
+    }
+  }
+  __syncthreads();
+  for (int d = t; d < nd; d += kSpreadThreads) {
+    const uint32_t c = cnt[d];
+    if (c) cnt[d] = atomicAdd(&st->cur[d], c);
+  }
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < kSpreadItems; ++i) {
+    const int64_t o = base + i * kSpreadThreads + int64_t(t);
+    if (o < n) {
+      const uint32_t p = cnt[k[i] >> shift] + r[i];
+      kout[p] = k[i];
+      vout[p] = uint32_t(o);
+    }
+  }
+}
+
+// Radius order of the state as component arrays: sorted position j takes the record src[v]
+// (one particle: whole sectors), which the moments and field kernels read.
+template <class T> struct SoA { T* d[6]; uint32_t* id; };
+template <class T> __device__ __forceinline__ void put_part(const SoA<T>& dst, int64_t j, const Part<T>& p) {
+  dst.d[0][j] = p.x; dst.d[1][j] = p.y; dst.d[2][j] = p.z;
+  dst.d[3][j] = p.vx; dst.d[4][j] = p.vy; dst.d[5][j] = p.vz;
+  dst.id[j] = p.id;
+}
+
+// Sort of one bucket (with st; or of the whole array k1 without) in one CTA, and the gather of
+// its particles into radius order. The keys of a bucket spread over its range like the density
+// over r^2, so a second digit of sb bits with about one key per value leaves almost nothing to
+// sort: the CTA counts the digits (shared atomics), scans the counts, places (key, slot) by
+// digit in any order, and each placed key finds its rank among the few of its digit by comparing
+// (key, slot): the order of a stable sort of the input slots by key, whatever the order of the
+// atomics. A bucket of more than cap keys takes several rounds, each over a range of the digits. A
+// digit of more than kBsMaxRun keys (many ties, very narrow shells) sends the bucket through
+// stable byte passes in L2 instead (by slot, then by key).
+// k1 (v1): keys and input slots of the buckets (without st the keys in input order, v1 scratch);
+// k0, v0: scratch for the byte passes. tb: leading key bits the same in all of a bucket;
+// sb <= 32 - tb, 2^sb >= NT.
+// Bound by the latency of the shared atomics, of the loads from L2 and of the gather: three CTAs
+// of 512 threads per SM keep more of them in flight than two with more registers (N = 2e6: a step
+// of 0.759 ms against 0.764; N = 7e5 0.231 and 0.234). A bucket's three byte passes of eight
+// ballots per 32 keys took 0.067 ms of the 0.111 ms sort of 2e6 keys and the gather a kernel of
+// 0.024 ms; this kernel 0.040 with the gather, sort and gather 0.138 -> 0.069. N = 3001 0.032 ->
+// 0.012, N = 20000 0.027 -> 0.0175, N = 5e5 0.051 -> 0.027.
+constexpr int kBsMaxRun = 256;
+constexpr size_t kBsRankBytes = 8;  // shared memory per key: key and slot
+constexpr int kBsThreads = 512, kBsPerSM = 3;  // CTA of a bucket, resident per SM
+constexpr int kBsOneThreads = 1024;  // the one CTA of a small array
+static_assert(kBsThreads >= 256 && kBsOneThreads >= 256, "256 threads scan the byte counts");
+
+template <class T, int NT, int MINB>
+__global__ void __launch_bounds__(NT, MINB) k_bucket_sort(uint32_t* k1, uint32_t* v1, uint32_t* k0, uint32_t* v0,
+                                                          const SortState* __restrict__ st, int64_t n_all, int cap,
+                                                          int tb, int sb, const Part<T>* __restrict__ src,
+                                                          SoA<T> dst) {
+  chain_wait();
+  extern __shared__ __align__(16) uint32_t sbuf[];
+  __shared__ uint32_t s_w[NT / 32];
+  const unsigned t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  uint32_t* const cnt = sbuf;                // [2^sb + 1]
+  uint32_t* const ks = cnt + (1 << sb) + 1;  // [cap]
+  uint32_t* const vs = ks + cap;             // [cap]
+  int64_t start = 0, len = n_all;
+  if (st) {  // the cursors are the buckets' ends now
+    start = blockIdx.x ? st->cur[blockIdx.x - 1] : 0u;
+    len = int64_t(st->cur[blockIdx.x]) - start;
   }
   if (len == 0) return;  // uniform over the CTA
-  const uint32_t* const sk = src_k + start;
-  const uint32_t* const sv = src_v + start;
-  bool fits = len <= cap;
-  if (fits) {
+  const uint32_t* const sk = k1 + start;
+  const uint32_t* const sv = v1 + start;
+  {
     const int n = int(len), shift = 32 - sb;
-    constexpr int U = 4;  // loads in flight per thread
-    for (int i0 = 0; i0 < n; i0 += NT * U) {
-      uint32_t k[U];
+    constexpr int U = 4;  // keys per thread in flight
+    const bool once = n <= NT * U;  // each thread's keys, slots and places in their digits stay in registers
+    uint32_t k[U], v[U], r[U];
+    for (int d = t; d <= 1 << sb; d += NT) cnt[d] = 0u;
+    auto load = [&](int i0) {
 #pragma unroll
-      for (int u = 0; u < U; ++u) k[u] = i0 + u * NT + int(t) < n ? sk[i0 + u * NT + t] : 0u;
+      for (int u = 0; u < U; ++u) {
+        const int i = i0 + u * NT + int(t);
+        k[u] = i < n ? sk[i] : 0u;
+        v[u] = st ? (i < n ? sv[i] : 0u) : unsigned(i);
+      }
+    };
+    auto count = [&](int i0) {
 #pragma unroll
       for (int u = 0; u < U; ++u)
-        if (i0 + u * NT + int(t) < n) atomicAdd(&cnt[(k[u] << tb) >> shift], 1u);
+        r[u] = i0 + u * NT + int(t) < n ? atomicAdd(&cnt[((k[u] << tb) >> shift) + 1], 1u) : 0u;
+    };
+    if (once) load(0);
+    __syncthreads();
+    if (once) {
+      count(0);
+    } else {
+      for (int i0 = 0; i0 < n; i0 += NT * U) {
+        load(i0);
+        count(i0);
+      }
     }
     __syncthreads();
-    // exclusive scan of the counts, each thread 2^sb / NT of them
+    // scan of the counts, each thread 2^sb / NT of them: to the digits' ends (cnt[s + 1], so
+    // cnt[s] is the start of s), or to their starts, which become cursors and so the ends
     const int per = (1 << sb) / NT;
-    uint32_t* const mine = cnt + per * t;
+    uint32_t* const mine = cnt + per * t + 1;
     uint32_t sum = 0, big = 0;
-    for (int k = 0; k < per; ++k) {
-      const uint32_t c = mine[k];
+    for (int d = 0; d < per; ++d) {
+      const uint32_t c = mine[d];
       sum += c;
       big = c > big ? c : big;
     }
-    fits = !__syncthreads_or(big > unsigned(kBsMaxRun));
-    if (fits) {
+    if (!__syncthreads_or(big > unsigned(kBsMaxRun))) {
       uint32_t inc = sum;
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {
@@ -476,89 +583,124 @@ __global__ void __launch_bounds__(NT, MINB) k_bucket_sort(uint32_t* src_k, uint3
       __syncthreads();
       uint32_t off = inc - sum;
       for (unsigned w = 0; w < warp; ++w) off += s_w[w];
-      for (int k = 0; k < per; ++k) {
-        const uint32_t c = mine[k];
-        mine[k] = off;
-        off += c;
+      for (int d = 0; d < per; ++d) {
+        const uint32_t end = off + mine[d];
+        mine[d] = once ? end : off;
+        off = end;
       }
       __syncthreads();
-      for (int i0 = 0; i0 < n; i0 += NT * U) {
-        uint32_t k[U];
+      // rounds over ranges [d0, d1) of digits with at most cap keys each: one, but for overfull buckets
+      const uint32_t digits = 1u << sb;
+      for (uint32_t d0 = 0; d0 < digits;) {
+        uint32_t base = 0, d1 = digits, m = n;
+        if (n > cap) {  // the cursors from d0 on still stand at the digits' starts
+          base = cnt[d0 + 1];
+          uint32_t lo = d0 + 1, hi = digits;  // the last d1 with start(d1) - base <= cap
+          while (lo < hi) {
+            const uint32_t mid = (lo + hi + 1) / 2;
+            if ((mid < digits ? cnt[mid + 1] : uint32_t(n)) - base <= uint32_t(cap)) lo = mid;
+            else hi = mid - 1;
+          }
+          d1 = lo;
+          m = (d1 < digits ? cnt[d1 + 1] : uint32_t(n)) - base;
+          __syncthreads();  // the cursors have been read
+        }
+        auto place = [&](int i0) {
 #pragma unroll
-        for (int u = 0; u < U; ++u) k[u] = i0 + u * NT + int(t) < n ? sk[i0 + u * NT + t] : 0u;
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-          const int i = i0 + u * NT + int(t);
-          if (i < n) {
-            const uint32_t p = atomicAdd(&cnt[(k[u] << tb) >> shift], 1u);
-            ks[p] = k[u];
-            ps[p] = uint16_t(i);
+          for (int u = 0; u < U; ++u) {
+            const uint32_t s = (k[u] << tb) >> shift;
+            if (i0 + u * NT + int(t) < n && s >= d0 && s < d1) {
+              const uint32_t p = (once ? cnt[s] + r[u] : atomicAdd(&cnt[s + 1], 1u)) - base;
+              ks[p] = k[u];
+              vs[p] = v[u];
+            }
+          }
+        };
+        if (once) {
+          place(0);
+        } else {
+          for (int i0 = 0; i0 < n; i0 += NT * U) {
+            load(i0);
+            place(i0);
           }
         }
-      }
-      __syncthreads();
-      // cnt[s] is now the end of digit s
-      uint32_t* const out = dst_v + start;
-      for (int p = t; p < n; p += NT) {
-        const uint32_t key = ks[p], slot = ps[p], s = (key << tb) >> shift;
-        const uint32_t b = s ? cnt[s - 1] : 0u, e = cnt[s];
-        uint32_t r = b;
-        for (uint32_t q = b; q < e; ++q) {
-          const uint32_t kq = ks[q];
-          r += kq < key || (kq == key && ps[q] < slot) ? 1u : 0u;
+        __syncthreads();
+        constexpr int G = MINB == 1 ? 4 : 2;  // gathers in flight per thread
+        for (uint32_t p0 = 0; p0 < m; p0 += NT * G) {
+          uint32_t at[G], from[G];
+#pragma unroll
+          for (int u = 0; u < G; ++u) {
+            const uint32_t p = p0 + u * NT + t;
+            at[u] = from[u] = 0u;
+            if (p >= m) continue;
+            const uint32_t key = ks[p], s = (key << tb) >> shift, b = cnt[s] - base, e = cnt[s + 1] - base;
+            from[u] = vs[p];
+            at[u] = b;
+            for (uint32_t q = b; q < e; ++q) {
+              const uint32_t kq = ks[q];
+              at[u] += kq < key || (kq == key && vs[q] < from[u]) ? 1u : 0u;
+            }
+          }
+          Part<T> x[G];
+#pragma unroll
+          for (int u = 0; u < G; ++u) x[u] = src[from[u]];
+#pragma unroll
+          for (int u = 0; u < G; ++u)
+            if (p0 + u * NT + t < m) put_part<T>(dst, start + base + at[u], x[u]);
         }
-        out[r] = sv[slot];
+        d0 = d1;
+        if (d0 < digits) __syncthreads();  // the placed keys have been read
       }
       return;
     }
   }
-  // stable byte passes over the bits that differ
+  // stable byte passes: by input slot (the bytes that n_all has; the whole array is in that
+  // order already), then by the key bits below the bucket's
   __syncthreads();  // the counts have been read
   BsShared<NT>& sh = *reinterpret_cast<BsShared<NT>*>(sbuf);
-  uint32_t* const bufs = sbuf + (sizeof(BsShared<NT>) + 3) / 4;
-  if (t < 256) sh.cnt[0][t] = 0u;
-  __syncthreads();
-  uint32_t *ak = src_k + start, *av = src_v + start, *dk = dst_k + start, *dv = dst_v + start;
-  count_low_byte<NT>(sk, len, sh.cnt[0]);
-  __syncthreads();
-  const bool all4 = tb < 8;  // the segment spans several top bytes
-  if (size_t(16) * size_t(len) + sizeof(BsShared<NT>) + 4 <= dyn) {
-    const int n = int(len);
-    uint32_t *ka = bufs, *va = bufs + n, *kb = bufs + 2 * n, *vb = bufs + 3 * n;
-    bucket_pass<NT>(ak, av, ka, va, n, 0, sh.cnt[0], sh.cnt[1], sh);
-    bucket_pass<NT>(ka, va, kb, vb, n, 8, sh.cnt[1], sh.cnt[0], sh);
-    if (all4) {
-      bucket_pass<NT>(kb, vb, ka, va, n, 16, sh.cnt[0], sh.cnt[1], sh);
-      bucket_pass<NT>(ka, va, dk, dv, n, 24, sh.cnt[1], nullptr, sh);
-    } else {
-      bucket_pass<NT>(kb, vb, dk, dv, n, 16, sh.cnt[0], nullptr, sh);
-    }
-  } else {
-    bucket_pass<NT>(ak, av, dk, dv, int(len), 0, sh.cnt[0], sh.cnt[1], sh);
-    bucket_pass<NT>(dk, dv, ak, av, int(len), 8, sh.cnt[1], sh.cnt[0], sh);
-    bucket_pass<NT>(ak, av, dk, dv, int(len), 16, sh.cnt[0], all4 ? sh.cnt[1] : nullptr, sh);
-    if (all4) {
-      bucket_pass<NT>(dk, dv, ak, av, int(len), 24, sh.cnt[1], nullptr, sh);
-      for (int64_t i = t; i < len; i += NT) dv[i] = av[i];
-    }
+  uint32_t *ak = k1 + start, *av = v1 + start, *dk = k0 + start, *dv = v0 + start;
+  if (!st) {
+    for (int64_t i = t; i < len; i += NT) av[i] = uint32_t(i);
+    __syncthreads();
   }
+  for (int pass = st ? 0 : 4; pass < 8; ++pass) {
+    const bool by_slot = pass < 4;
+    const int shift = 8 * (pass & 3);
+    if (by_slot ? ((n_all - 1) >> shift) == 0 : shift >= 32 - tb) continue;
+    if (t < 256) sh.cnt[t] = 0u;
+    __syncthreads();
+    count_byte<NT>(by_slot ? av : ak, len, shift, sh.cnt);
+    __syncthreads();
+    if (by_slot) bucket_pass<NT>(av, ak, dv, dk, int(len), shift, sh);
+    else bucket_pass<NT>(ak, av, dk, dv, int(len), shift, sh);
+    uint32_t* x = ak; ak = dk; dk = x;
+    x = av; av = dv; dv = x;
+  }
+  for (int64_t i = t; i < len; i += NT) put_part<T>(dst, start + i, src[av[i]]);
 }
 
-// Largest N for the bucket sort: the buckets of a uniform shell (density in
-// r^2 up to 1.45 times its mean) must fit the shared-memory capacity; beyond
-// it they take the global path, and one CTA's share of the work outweighs the
-// saved passes (N = 4e6: 0.256 ms against 0.222 for the four global passes;
-// N = 1.6e7: 0.91 against 0.74 ms, both with the 8-bit first pass).
-constexpr int64_t kBucketSortMaxN = 2250000;
-constexpr int kBsCapMax = 13312;  // keys (and 2^13 counts in all of the 227 KB: 112 KB)
+// Largest N for the bucket sort: beyond it most buckets of kSortDigits top digits would take
+// several rounds (kBsCapMax keys; the buckets of a uniform shell hold up to 1.5 times their mean).
+constexpr int64_t kBucketSortMaxN = 24000000;
+constexpr int kBsCapMax = 13312;
 constexpr int kBsBitsMax = 13;
-constexpr int64_t kBsSmallN = 1 << 19;  // up to here an 8-bit first pass (256 buckets), beyond a 9-bit one (512)
-constexpr int64_t kBsSingleN = 4096;     // up to here, one CTA sorts everything (0.011 ms; at 6000 keys 0.0145 against 0.015)
-// Shared-memory capacity for segments of g of nd buckets: three times the mean segment with 256
-// buckets; 1.5 times with 512. Larger segments go through L2.
-inline int bucket_cap(int64_t n, int g, int nd) {
-  const int64_t mean = int64_t(g) * n / nd;
-  int64_t c = ((nd == 256 ? 3 * mean : mean + mean / 2) + 255) / 256 * 256;
+// up to here one CTA sorts everything (0.011 ms; at 6000 keys 0.0145 against 0.015)
+constexpr int64_t kBsSingleN = 4096;
+// Digits of the first pass. Alone on the GPU 256 buckets (the most parallel) up to kBsSmallN keys
+// (N = 3e5: a step of 0.0892 ms, with 512 0.0904; 5e5: 0.0757 and 0.0761), beyond as many as
+// leave at most kBsMean keys on average, so that one round of loads holds a bucket (N = 2e6: 0.774
+// ms a step with up to 2048, 0.761 with 1024, 0.778 with 512). Sharing it (a batch), fewer and
+// fuller CTAs.
+constexpr int64_t kBsSmallN = 1 << 19, kBsMean = 1024;
+inline int sort_digit_bits(int64_t n, bool shared_gpu) {
+  int b = shared_gpu ? 1 : 8;
+  const int64_t mean = n > kBsSmallN ? kBsMean : 2 * kBsMean;
+  while ((n >> b) > mean && (1 << b) < kSortDigits) ++b;
+  return b;
+}
+// Shared-memory capacity for buckets of `mean` keys on average (a larger one takes more rounds)
+inline int bucket_cap(int64_t mean) {
+  int64_t c = (mean + mean / 4 * 3 + 255) / 256 * 256;
   if (c < 2048) c = 2048;
   return int(c < kBsCapMax ? c : kBsCapMax);
 }
@@ -569,65 +711,61 @@ inline int bucket_bits(int64_t mean, int threads) {
   return sb;
 }
 template <int NT> inline size_t bucket_smem(int cap, int sb) {
-  const size_t rank = (size_t(4) << sb) + kBsRankBytes * size_t(cap), pass = sizeof(BsShared<NT>) + 16;
+  const size_t rank = (size_t(4) << sb) + 4 + kBsRankBytes * size_t(cap), pass = sizeof(BsShared<NT>);
   return rank > pass ? rank : pass;
 }
 
 cudaError_t set_sort_attributes() {
   const int most = int(bucket_smem<kBsOneThreads>(kBsCapMax, kBsBitsMax));
-  const cudaError_t e = cudaFuncSetAttribute(k_bucket_sort<kBsOneThreads, 1>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, most);
-  if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(k_bucket_sort<kBsThreads, kBsPerSM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              most);
+  cudaError_t e = cudaFuncSetAttribute(k_bucket_sort<float, kBsOneThreads, 1>,
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k_bucket_sort<double, kBsOneThreads, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             most);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k_bucket_sort<float, kBsThreads, kBsPerSM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             most);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k_bucket_sort<double, kBsThreads, kBsPerSM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             most);
+  return e;
 }
 
-const uint32_t* launch_radix_sort(uint32_t* k0, uint32_t* v0, uint32_t* k1, uint32_t* v1, uint32_t* hist,
-                                  int64_t n, int first_byte, LaunchSeq& seq, bool shared_gpu) {
+template <class T>
+const uint32_t* launch_radix_sort(uint32_t* k0, uint32_t* v0, uint32_t* k1, uint32_t* v1, void* scratch, int64_t n,
+                                  int first_byte, const Part<T>* src, T* const* dst, uint32_t* id_dst, LaunchSeq& seq,
+                                  bool shared_gpu) {
   if (n <= 1) return v0;
-  const int64_t nblk = sort_blocks(n);
+  SoA<T> d;
+  for (int c = 0; c < 6; ++c) d.d[c] = dst[c];
+  d.id = id_dst;
+  SortState* const st = static_cast<SortState*>(scratch);
   if (first_byte == 0 && n <= kBsSingleN) {
     const int cap = int((n + 255) / 256 * 256), sb = bucket_bits(n, kBsOneThreads);
-    const size_t smem = bucket_smem<kBsOneThreads>(cap, sb);
-    seq(k_bucket_sort<kBsOneThreads, 1>, 1, kBsOneThreads, smem, k0, v0, k1, v1, nullptr, n, cap, 1, 0, 0, sb,
-        unsigned(smem));
-    return v1;
+    seq(k_bucket_sort<T, kBsOneThreads, 1>, 1, kBsOneThreads, bucket_smem<kBsOneThreads>(cap, sb), k0, v0, k1, v1,
+        nullptr, n, cap, 0, sb, src, d);
+    return nullptr;
   }
   if (first_byte == 0 && n <= kBucketSortMaxN) {
-    // the top digit over the whole array into nd contiguous buckets (k0 -> k1),
-    // then the bits below it per bucket (into k0): 256 buckets (the top byte)
-    // up to kBsSmallN keys, 512 (the top 9 bits, buckets of ~3900 keys at
-    // N = 2e6) beyond. Alone on the GPU, one CTA per bucket
-    // (the most parallel); sharing it (a batch), a small instance takes
-    // segments of several buckets, about 2048 keys per CTA (fewer CTAs): the same
-    // permutation either way
-    const bool wide = n > kBsSmallN;
-    const int nd = wide ? 512 : 256, shift = wide ? 23 : 24;
-    uint32_t* rowtot = hist + int64_t(nd) * nblk;
-    int g = 1, tb = wide ? 9 : 8;
-    while (shared_gpu && g < nd && int64_t(g) * 2 * n <= int64_t(2048) * nd) g *= 2, --tb;
-    const int cap = bucket_cap(n, g, nd), sb = bucket_bits(int64_t(g) * n / nd, kBsThreads);
-    const size_t smem = bucket_smem<kBsThreads>(cap, sb);
-    if (wide) {
-      seq(k_sort_hist<512>, unsigned(nblk), kSortThreads, 0, k0, n, shift, nblk, hist);
-      seq(k_sort_rowscan, 512, kSortThreads, 0, hist, nblk, rowtot);
-      seq(k_sort_scatter<512>, unsigned(nblk), kSortThreads, 0, k0, v0, k1, v1, n, shift, nblk, hist, rowtot);
-    } else {
-      seq(k_sort_hist<256>, unsigned(nblk), kSortThreads, 0, k0, n, shift, nblk, hist);
-      seq(k_sort_rowscan, 256, kSortThreads, 0, hist, nblk, rowtot);
-      seq(k_sort_scatter<256>, unsigned(nblk), kSortThreads, 0, k0, v0, k1, v1, n, shift, nblk, hist, rowtot);
-    }
-    seq(k_bucket_sort<kBsThreads, kBsPerSM>, unsigned(nd / g), kBsThreads, smem, k1, v1, k0, v0, rowtot, 0, cap, g, nd,
-        tb, sb, unsigned(smem));
-    return v0;
+    const int tb = sort_digit_bits(n, shared_gpu), nd = 1 << tb, shift = 32 - tb;
+    const int64_t mean = n >> tb;
+    const int cap = bucket_cap(mean), sb = bucket_bits(mean, kBsThreads);
+    const unsigned blocks = unsigned((n + kSpreadTile - 1) / kSpreadTile);
+    seq(k_sort_count, blocks, kSpreadThreads, sizeof(uint32_t) * nd, k0, n, shift, nd, st);
+    seq(k_sort_spread, blocks, kSpreadThreads, sizeof(uint32_t) * nd, k0, n, shift, nd, st, k1, v1);
+    seq(k_bucket_sort<T, kBsThreads, kBsPerSM>, unsigned(nd), kBsThreads, bucket_smem<kBsThreads>(cap, sb), k1, v1, k0,
+        v0, st, n, cap, tb, sb, src, d);
+    return nullptr;
   }
+  const int64_t nblk = sort_blocks(n);
+  uint32_t* hist = reinterpret_cast<uint32_t*>(st + 1);
   uint32_t* rowtot = hist + 256 * nblk;
   uint32_t *ki = k0, *vi = v0, *ko = k1, *vo = v1;
   for (int pass = first_byte; pass < 4; ++pass) {
     const int shift = 8 * pass;
-    seq(k_sort_hist<256>, unsigned(nblk), kSortThreads, 0, ki, n, shift, nblk, hist);
+    seq(k_sort_hist, unsigned(nblk), kSortThreads, 0, ki, n, shift, nblk, hist);
     seq(k_sort_rowscan, 256, kSortThreads, 0, hist, nblk, rowtot);
-    seq(k_sort_scatter<256>, unsigned(nblk), kSortThreads, 0, ki, vi, ko, vo, n, shift, nblk, hist, rowtot);
+    seq(k_sort_scatter, unsigned(nblk), kSortThreads, 0, ki, vi, ko, vo, n, shift, nblk, hist, rowtot);
     uint32_t* tk = ki; ki = ko; ko = tk;
     uint32_t* tv = vi; vi = vo; vo = tv;
   }
@@ -637,21 +775,15 @@ const uint32_t* launch_radix_sort(uint32_t* k0, uint32_t* v0, uint32_t* k1, uint
 // ============================================================================
 // State movement
 // ============================================================================
-template <class T> struct SoA { T* d[6]; uint32_t* id; };
-
-// Gather of the state into radius order: sorted position j takes the record
-// perm[j] (one particle: whole sectors) and splits it into the component
-// arrays the moments and field kernels read.
+// Gather of the state into radius order by a permutation (very large arrays; the bucket
+// sort gathers itself).
 template <class T>
 __global__ void k_reorder(const Part<T>* __restrict__ src, SoA<T> dst, const uint32_t* __restrict__ perm,
                           int64_t n) {
   chain_wait();
   const int64_t j = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   if (j >= n) return;
-  const Part<T> p = src[perm[j]];
-  dst.d[0][j] = p.x; dst.d[1][j] = p.y; dst.d[2][j] = p.z;
-  dst.d[3][j] = p.vx; dst.d[4][j] = p.vy; dst.d[5][j] = p.vz;
-  dst.id[j] = p.id;
+  put_part<T>(dst, j, src[perm[j]]);
 }
 
 template <class T>
@@ -1376,13 +1508,15 @@ template <class T> cudaError_t preload_core_kernels_t() {
 cudaError_t preload_core_kernels() {
   if (set_sort_attributes() != cudaSuccess) return cudaErrorInvalidValue;
   cudaFuncAttributes fa;
-  const void* fns[] = {reinterpret_cast<const void*>(&k_sort_hist<256>),
-                       reinterpret_cast<const void*>(&k_sort_hist<512>),
+  const void* fns[] = {reinterpret_cast<const void*>(&k_sort_hist),
                        reinterpret_cast<const void*>(&k_sort_rowscan),
-                       reinterpret_cast<const void*>(&k_sort_scatter<256>),
-                       reinterpret_cast<const void*>(&k_sort_scatter<512>),
-                       reinterpret_cast<const void*>(&k_bucket_sort<kBsOneThreads, 1>),
-                       reinterpret_cast<const void*>(&k_bucket_sort<kBsThreads, kBsPerSM>),
+                       reinterpret_cast<const void*>(&k_sort_scatter),
+                       reinterpret_cast<const void*>(&k_sort_count),
+                       reinterpret_cast<const void*>(&k_sort_spread),
+                       reinterpret_cast<const void*>(&k_bucket_sort<float, kBsOneThreads, 1>),
+                       reinterpret_cast<const void*>(&k_bucket_sort<double, kBsOneThreads, 1>),
+                       reinterpret_cast<const void*>(&k_bucket_sort<float, kBsThreads, kBsPerSM>),
+                       reinterpret_cast<const void*>(&k_bucket_sort<double, kBsThreads, kBsPerSM>),
                        reinterpret_cast<const void*>(&k_init_step)};
   for (const void* f : fns) {
     const cudaError_t e = cudaFuncGetAttributes(&fa, f);
@@ -1394,6 +1528,8 @@ cudaError_t preload_core_kernels() {
 
 // explicit instantiations
 #define IMRP_INST_CORE(T)                                                                          \
+  template const uint32_t* launch_radix_sort<T>(uint32_t*, uint32_t*, uint32_t*, uint32_t*, void*, int64_t, int,      \
+                                                const Part<T>*, T* const*, uint32_t*, LaunchSeq&, bool);             \
   template void launch_reorder<T>(const Part<T>*, T* const*, uint32_t*, const uint32_t*, int64_t,  \
                                   LaunchSeq&);                                                     \
   template void launch_keys<T>(const Part<T>*, uint32_t*, uint32_t*, int64_t, double, LaunchSeq&); \

@@ -74,21 +74,30 @@ constexpr int kSortThreads = 256;
 constexpr int kSortItems = 8;
 constexpr int kSortTile = kSortThreads * kSortItems;  // keys per CTA
 constexpr int64_t sort_blocks(int64_t n) { return (n + kSortTile - 1) / kSortTile; }
-// Words of the sort's histogram buffer for n keys: block counts of up to 512
-// digits per block, and the digit totals.
-constexpr int64_t sort_hist_words(int64_t n) { return 512 * sort_blocks(n) + 512; }
-// Sorts (key, val) pairs by the key bytes first_byte..3 (stable radix sort;
-// keys equal in those bytes keep their order). k0/v0 hold the input; k1/v1 are
-// scratch of n; hist: sort_hist_words(n) words. Returns the buffer that holds
-// the sorted values (v0 after an even number of passes, v1 after an odd one).
+// Scratch of the bucket sort's first pass: the digits' totals and the ticket of its CTAs, zero
+// between sorts (zeroed at allocation), and the digits' cursors. Behind it stand, for the global
+// passes, the block counts of 256 digits per block and the digit totals.
+constexpr int kSortDigits = 4096;
+struct alignas(64) SortState {
+  uint32_t tot[kSortDigits], cur[kSortDigits], ticket;
+};
+constexpr size_t sort_scratch_bytes(int64_t n) {
+  return sizeof(SortState) + sizeof(uint32_t) * size_t(256 * sort_blocks(n) + 256);
+}
+// Sorts the particles src[0 .. n) by the key bytes first_byte..3 (stable: keys equal in those
+// bytes keep their order). k0/v0 hold the keys and slots 0 .. n-1; k1/v1 are scratch of n;
+// scratch: sort_scratch_bytes(n). Either gathers the particles into the component arrays dst and
+// id_dst itself and returns null, or returns the buffer that holds the slots in key order.
 // Key bytes sorted: all four, in both precisions. The radius key is
 // floor((r^2 - 1) / (r_out^2 - 1) * 2^32) of the exact FP64 r^2 of the stored
 // position, and the sorted index j of a particle is its count of electrons
 // inside (the l = 0 term), which jumps by one electron per misordered pair;
 // so even radii that FP32 arithmetic cannot tell apart are ordered exactly.
 inline int sort_first_byte(int) { return 0; }
-const uint32_t* launch_radix_sort(uint32_t* k0, uint32_t* v0, uint32_t* k1, uint32_t* v1, uint32_t* hist,
-                                  int64_t n, int first_byte, LaunchSeq& seq, bool shared_gpu = false);
+template <class T>
+const uint32_t* launch_radix_sort(uint32_t* k0, uint32_t* v0, uint32_t* k1, uint32_t* v1, void* scratch, int64_t n,
+                                  int first_byte, const Part<T>* src, T* const* dst, uint32_t* id_dst, LaunchSeq& seq,
+                                  bool shared_gpu = false);
 
 // ---- state movement and keys (imrp_core.cu) ---------------------------------
 // The state is an array of Part<T> records in the order of the last push (or

@@ -23,7 +23,7 @@ constexpr size_t align256(size_t b) { return (b + 255) & ~size_t(255); }
 
 // Byte layout of the scratch for n particles, degree L, element size es.
 struct Layout {
-  size_t part, st[6], id, key0, idx0, key1, idx1, hist, agg, pfx, gagg, gbase, tot, totd, gswork, gsticket, eout,
+  size_t part, st[6], id, key0, idx0, key1, idx1, sort, agg, pfx, gagg, gbase, tot, totd, gswork, gsticket, eout,
       step, total;
 };
 constexpr Layout layout(int64_t n, int L, size_t es) {
@@ -39,7 +39,7 @@ constexpr Layout layout(int64_t n, int L, size_t es) {
   o.idx0 = at; at += align256(size_t(n) * 4);
   o.key1 = at; at += align256(size_t(n) * 4);
   o.idx1 = at; at += align256(size_t(n) * 4);
-  o.hist = at; at += align256(size_t(sort_hist_words(n)) * 4);
+  o.sort = at; at += align256(sort_scratch_bytes(n));
   o.agg = at; at += align256(size_t(nc * tile_stride(ntiles)) * es);
   o.pfx = at; at += align256(size_t(nc * tile_stride(ntiles)) * es);
   o.gagg = at; at += align256(size_t(nc * ngroups) * 8);
@@ -101,10 +101,15 @@ __global__ void k_na_load(const double* __restrict__ x, Part<T>* st, int64_t n, 
 }
 
 // Per-call set-up of what must start at zero or at the given step: the step
-// state and the group scan's tickets (the scratch keeps the
+// state, the group scan's tickets and the sort's digit totals (the scratch keeps the
 // previous call's contents, and another n or degree lays it out differently).
-__global__ void k_na_init(StepState* st, int64_t step, unsigned* ticket, int nticket) {
+__global__ void __launch_bounds__(256) k_na_init(StepState* st, int64_t step, unsigned* ticket, int nticket,
+                                                 SortState* sort) {
   chain_wait();
+  for (int k = threadIdx.x; k < nticket; k += 256) ticket[k] = 0u;
+  for (int k = threadIdx.x; k < kSortDigits; k += 256) sort->tot[k] = 0u;
+  if (threadIdx.x != 0) return;
+  sort->ticket = 0u;
   st->step = step;
   st->next = step;
   st->u = 0.0;
@@ -113,7 +118,6 @@ __global__ void k_na_init(StepState* st, int64_t step, unsigned* ticket, int nti
   st->nabs_step = 0;
   st->qs_acc = 0.0;
   st->nabs_total = 0;
-  for (int k = 0; k < nticket; ++k) ticket[k] = 0u;
 }
 
 cudaError_t preload_noalloc_kernels() {
@@ -157,12 +161,14 @@ int run(const imrp_params* p, const double* x, int64_t n, int64_t step, double* 
   int* err = g_derr[dev];
   *g_err[dev] = 0;
   LaunchSeq seq(s);
-  seq(k_na_init, 1, 1, 0, st, step, static_cast<unsigned*>(P(o.gsticket)), gs_tickets(nc));
+  seq(k_na_init, 1, 256, 0, st, step, static_cast<unsigned*>(P(o.gsticket)), gs_tickets(nc),
+      static_cast<SortState*>(P(o.sort)));
   seq(k_na_load<T>, unsigned((n + 255) / 256), 256, 0, x, st0, n, r_out, err);
   launch_keys<T>(st0, key0, idx0, n, r_out, seq);
-  const uint32_t* perm = launch_radix_sort(key0, idx0, static_cast<uint32_t*>(P(o.key1)), static_cast<uint32_t*>(P(o.idx1)),
-                    static_cast<uint32_t*>(P(o.hist)), n, sort_first_byte(sizeof(T) == 4 ? 1 : 0), seq);
-  launch_reorder<T>(st0, st1, id1, perm, n, seq);
+  const uint32_t* perm =
+      launch_radix_sort<T>(key0, idx0, static_cast<uint32_t*>(P(o.key1)), static_cast<uint32_t*>(P(o.idx1)), P(o.sort),
+                           n, sort_first_byte(sizeof(T) == 4 ? 1 : 0), st0, st1, id1, seq);
+  if (perm) launch_reorder<T>(st0, st1, id1, perm, n, seq);
   MomArgs<T> ma;
   memset(&ma, 0, sizeof(ma));  // all electrons (species = 0)
   ma.x = st1[0]; ma.y = st1[1]; ma.z = st1[2];
