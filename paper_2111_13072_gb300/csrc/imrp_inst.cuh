@@ -161,6 +161,12 @@ template <class T, int L> void field_launch(const FieldArgs<T>& a, int wpb, Laun
     }
   }
   const size_t smem = size_t(wpb) * field_smem_per_warp<T>(L);
+  if constexpr (sizeof(T) == 4) {
+    if (a.img_in_tile) {
+      if (blocks > 0) seq(k_field_small<L>, unsigned(blocks), unsigned(wpb * 32), smem, a);
+      return;
+    }
+  }
   if (blocks > 0) seq(k_field<T, L>, unsigned(blocks), unsigned(wpb * 32), smem, a);
 }
 
@@ -217,6 +223,10 @@ template <class T, int L> cudaError_t set_attr() {
   const int fmax = int(8 * field_smem_per_warp<T>(L) > 227 * 1024 ? 227 * 1024 : 8 * field_smem_per_warp<T>(L));
   e = cudaFuncSetAttribute(k_field<T, L>, cudaFuncAttributeMaxDynamicSharedMemorySize, fmax);
   if (e != cudaSuccess) return e;
+  if constexpr (sizeof(T) == 4) {
+    e = cudaFuncSetAttribute(k_field_small<L>, cudaFuncAttributeMaxDynamicSharedMemorySize, fmax);
+    if (e != cudaSuccess) return e;
+  }
   if constexpr (pair_degree<T>(L)) {
     e = cudaFuncSetAttribute(k_field_pair<L>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              int(kPairMaxWarps * pair_smem_per_warp(L)));
