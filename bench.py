@@ -55,11 +55,11 @@ def step_launches(n):
 
 
 def fused_stages(n):
-    """Stages that ride in another stage's launch: the finalize in the first
-    group-scan kernel; up to 32 scan groups of 1024 particles the second
-    group-scan pass too; the reorder in the bucket sort, and the scan of the
-    digit counts in the counting kernel."""
-    fused = 2 if n <= 32 * 1024 else 1
+    """Stages that ride in another stage's launch: the finalize in a group-scan
+    kernel; up to 320 scan groups of 1024 particles the two group-scan passes in
+    one; the reorder in the bucket sort, and the scan of the digit counts in the
+    counting kernel."""
+    fused = 2 if n <= 320 * 1024 else 1
     if 1 < n <= BUCKET_SORT_MAX_N:
         fused += 1 if n <= BUCKET_SORT_SINGLE_N else 2
     return fused

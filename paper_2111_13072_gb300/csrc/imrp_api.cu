@@ -384,11 +384,9 @@ template <class T> void enqueue_pre(imrp_ctx* ctx, LaunchSeq& seq, cudaEvent_t* 
 template <class T> void enqueue_mid(imrp_ctx* ctx, LaunchSeq& seq, bool record) {
   if (ctx->species) {
     // the charge inside each particle's radius: a scan of the tiles' charges (FP64)
-    launch_tile_scan<double>(ctx->qtile, ctx->qpfx, ctx->qgagg, ctx->ntiles, 1, seq);
-    launch_group_scan<double>(ctx->qgagg, ctx->qwork, ctx->qticket, ctx->qgbase, ctx->qtot, ctx->qtotd,
-                              ctx->ngroups, 1, ctx->gseg, nullptr, seq);
+    launch_scans<double>(ctx->qtile, ctx->qpfx, ctx->qgagg, ctx->qwork, ctx->qticket, ctx->qgbase, ctx->qtot,
+                         ctx->qtotd, ctx->ntiles, 1, ctx->gseg, nullptr, seq);
   }
-  launch_tile_scan<T>(static_cast<T*>(ctx->agg), static_cast<T*>(ctx->pfx), ctx->gagg, ctx->ntiles, ctx->nc, seq);
   FinalizeArgs fa;
   fa.st = ctx->st;
   fa.totd = ctx->totd;
@@ -409,8 +407,9 @@ template <class T> void enqueue_mid(imrp_ctx* ctx, LaunchSeq& seq, bool record) 
     fa.canti[l] = ctx->canti[l];
     fa.cdrive[l] = ctx->canti[l] * 4.0 * kPi * ctx->n_tilde;
   }
-  launch_group_scan<T>(ctx->gagg, ctx->gswork, ctx->gsticket, static_cast<T*>(ctx->gbase),
-                       static_cast<T*>(ctx->tot), ctx->totd, ctx->ngroups, ctx->nc, ctx->gseg, &fa, seq);
+  launch_scans<T>(static_cast<T*>(ctx->agg), static_cast<T*>(ctx->pfx), ctx->gagg, ctx->gswork, ctx->gsticket,
+                  static_cast<T*>(ctx->gbase), static_cast<T*>(ctx->tot), ctx->totd, ctx->ntiles, ctx->nc, ctx->gseg,
+                  &fa, seq);
 }
 
 // Launches one step (record = 1) or the field evaluation without push (record = 0).

@@ -1066,7 +1066,8 @@ constexpr int kTsTiles = 128;  // tiles per CTA
 
 template <class T>
 __global__ void __launch_bounds__(256) k_tile_scan(const T* __restrict__ agg, T* __restrict__ pfx,
-                                                   double* __restrict__ gagg, int64_t tw, int64_t ts, int nc) {
+                                                   double* __restrict__ gagg, double* __restrict__ csum, int64_t tw,
+                                                   int64_t ts, int nc) {
   chain_wait();
   using V4 = typename Vec4<T>::type;
   using C = CSum<T>;
@@ -1126,19 +1127,17 @@ __global__ void __launch_bounds__(256) k_tile_scan(const T* __restrict__ agg, T*
   const int u = u0 + lane;
   if (u < nc) {
     if (warp < kTsTiles / 32 && tile0 + 32 * warp < tw) gagg[(tile0 / 32 + warp) * nc + u] = cs_double(gt[warp][lane]);
+    if (csum && warp == kTsTiles / 32) {  // the sum of this CTA's groups
+      double sum = 0.0;
+      for (int k = 0; k < kTsTiles / 32 && tile0 + 32 * k < tw; ++k) sum += cs_double(gt[k][lane]);
+      csum[int64_t(blockIdx.x) * nc + u] = sum;
+    }
     const int tend = tw - tile0 < kTsTiles ? int(tw - tile0) : kTsTiles;
     T* dst = pfx + (tile0 + warp) * nc + u;
     const int64_t step = 8 * int64_t(nc);
 #pragma unroll 4
     for (int t = warp; t < tend; t += 8, dst += step) *dst = buf[lane][t];
   }
-}
-
-template <class T>
-void launch_tile_scan(const T* agg, T* pfx, double* gagg, int64_t ntiles, int nc, LaunchSeq& seq) {
-  const int64_t tw = tiles_whole(ntiles), ts = tile_stride(ntiles);
-  const dim3 grid(unsigned((tw + kTsTiles - 1) / kTsTiles), unsigned((nc + kTsRows - 1) / kTsRows));
-  if (tw > 0) seq(k_tile_scan<T>, grid, 256, 0, agg, pfx, gagg, tw, ts, nc);
 }
 
 // ============================================================================
@@ -1152,8 +1151,8 @@ void launch_tile_scan(const T* agg, T* pfx, double* gagg, int64_t ntiles, int nc
 // the last CTA of a column block to finish (an atomic ticket, no waiting)
 // scans the segment sums of that block in a fixed order, so the result is
 // the same whichever CTA finishes last. k_group_bases then walks each warp's
-// groups once more and writes the bases. With one segment (up to kGsOne
-// groups) k_group_sums writes the bases itself.
+// groups once more and writes the bases. Up to kGsOne groups one kernel
+// (k_group_scan) does all of it.
 // The CTA that completes the last column block (a second ticket) runs the
 // step's finalize, which needs the totals alone.
 // Work space w (FP64): [nseg][8][nc] warp sums, then [nseg][nc] segment sums,
@@ -1207,10 +1206,89 @@ __device__ __forceinline__ void finalize_step(const FinalizeArgs& a, int lane) {
   }
 }
 
+// After the totals of a block of components are written (by warp 0 of the calling CTA): the last of
+// the `blocks` blocks finalizes the step.
+__device__ __forceinline__ void group_finalize(const FinalizeArgs& fin, unsigned* ticket, unsigned blocks, unsigned warp,
+                                               unsigned lane) {
+  if (!fin.st || warp != 0) return;
+  __threadfence();
+  __syncwarp();
+  unsigned t = 0;
+  if (lane == 0) t = atomicAdd(&ticket[blocks], 1u);
+  if (__shfl_sync(0xffffffffu, t, 0) == blocks - 1) {
+    __threadfence();
+    if (lane == 0) ticket[blocks] = 0u;
+    finalize_step(fin, int(lane));
+  }
+}
+
+// Up to kGsOne groups: the bases and the totals in one kernel. csum holds the sums of runs of
+// kGsRun groups (of one CTA of the tile scan each; with one segment they are formed here); CTA
+// (column block b, segment s) has kGsWarps runs, one per warp. The CTA adds up the runs of the other segments before it (Rs) or after it
+// (Is), its warps taking them in turn; then each warp adds the segment's own runs on that side and
+// walks its groups. The CTAs of the first segment form the totals. Every CTA sums up to
+// kGsOne / kGsRun runs again, in FP64 (1/64 of the FP32 rate): that sets kGsOne. A step
+// against sums, segment scan and bases in two kernels: N = 1e5, l_max = 16 84.6 -> 82.2 us, N = 3e5,
+// l_max = 8 86.2 -> 84.1; 489 groups (N = 5e5, l_max = 1) 71.7 and 71.6, 684 (N = 7e5) 229 and 231.
+constexpr int kGsRun = kTsTiles / 32;
+template <class T>
+__global__ void __launch_bounds__(kGsWarps * 32) k_group_scan(const double* __restrict__ gagg,
+                                                              const double* __restrict__ csum, unsigned* ticket,
+                                                              T* __restrict__ gbase, T* __restrict__ tot, double* totd,
+                                                              int ngroups, int nc, FinalizeArgs fin) {
+  chain_wait();
+  __shared__ double others[kGsWarps][32], own[kGsWarps][32];
+  const unsigned lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int c = int(blockIdx.x) * 32 + int(lane);
+  const bool okc = c < nc, suffix = (c & 1) != 0, first = blockIdx.y == 0;
+  const int nrun = (ngroups + kGsRun - 1) / kGsRun, r0 = int(blockIdx.y) * kGsWarps, r = r0 + int(warp);
+  const int64_t g0 = int64_t(r) * kGsRun;
+  double v[kGsRun];
+#pragma unroll
+  for (int k = 0; k < kGsRun; ++k) v[k] = okc && g0 + k < ngroups ? gagg[(g0 + k) * nc + c] : 0.0;
+  double rest = 0.0;
+  if (gridDim.y > 1) {
+    own[warp][lane] = okc && r < nrun ? csum[int64_t(r) * nc + c] : 0.0;
+    double sum = 0.0;
+    // in the first segment both kinds of component take the runs after it (its bases or the totals)
+#pragma unroll 4
+    for (int k = int(warp); k < nrun; k += kGsWarps)
+      if (okc && (suffix || first ? k >= r0 + kGsWarps : k < r0)) sum += csum[int64_t(k) * nc + c];
+    others[warp][lane] = sum;
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < kGsWarps; ++k) rest += others[k][lane];
+  } else {  // one segment: the runs summed here
+    double sum = v[0];
+#pragma unroll
+    for (int k = 1; k < kGsRun; ++k) sum += v[k];
+    own[warp][lane] = sum;
+    __syncthreads();
+  }
+  double run = first && !suffix ? 0.0 : rest;
+#pragma unroll
+  for (int k = 0; k < kGsWarps; ++k)
+    if (suffix ? k > int(warp) : k < int(warp)) run += own[k][lane];
+#pragma unroll
+  for (int q = 0; q < kGsRun; ++q) {
+    const int64_t g = g0 + (suffix ? kGsRun - 1 - q : q);
+    if (okc && g < ngroups) gbase[g * nc + c] = T(run);
+    run += suffix ? v[kGsRun - 1 - q] : v[q];
+  }
+  if (!first) return;
+  if (warp == 0 && okc) {
+#pragma unroll
+    for (int k = 0; k < kGsWarps; ++k) rest += own[k][lane];
+    tot[c] = T(rest);
+    totd[c] = rest;
+  }
+  group_finalize(fin, ticket, gridDim.x, warp, lane);
+}
+
 template <class T>
 __global__ void __launch_bounds__(kGsWarps * 32) k_group_sums(const double* __restrict__ gagg,
                                                               double* __restrict__ w, unsigned* __restrict__ ticket,
-                                                              T* __restrict__ gbase, T* __restrict__ tot, double* totd,
+                                                              T* __restrict__ tot, double* totd,
                                                               int64_t ngroups, int nc, int64_t G, int nseg,
                                                               FinalizeArgs fin) {
   chain_wait();
@@ -1231,72 +1309,38 @@ __global__ void __launch_bounds__(kGsWarps * 32) k_group_sums(const double* __re
   if (okc) {
 #pragma unroll 4
     for (int64_t g = g0; g < g1; ++g) run += gagg[g * nc + c];
-    if (nseg > 1) wsum[(int64_t(seg) * kGsWarps + warp) * nc + c] = run;
+    wsum[(int64_t(seg) * kGsWarps + warp) * nc + c] = run;
   }
   ws[warp][lane] = run;
   __syncthreads();
-  if (nseg == 1) {
-    double base = 0.0, all = 0.0;
+  if (warp == 0 && okc) {
+    double sum = 0.0;
 #pragma unroll
-    for (int k = 0; k < kGsWarps; ++k) {
-      const double v = ws[suffix ? kGsWarps - 1 - k : k][lane];
-      if (suffix ? kGsWarps - 1 - k > int(warp) : k < int(warp)) base += v;
-      all += v;
-    }
-    if (okc) {
-#pragma unroll 4
-      for (int64_t k = 0; k < g1 - g0; ++k) {
-        const int64_t g = suffix ? g1 - 1 - k : g0 + k;
-        gbase[g * nc + c] = T(base);
-        base += gagg[g * nc + c];
-      }
-      if (warp == 0) {
-        tot[c] = T(all);
-        totd[c] = all;
-      }
-    }
-  } else {
-    if (warp == 0 && okc) {
-      double sum = 0.0;
-#pragma unroll
-      for (int k = 0; k < kGsWarps; ++k) sum += ws[k][lane];
-      ssum[int64_t(seg) * nc + c] = sum;
-    }
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0) last = atomicAdd(&ticket[blockIdx.x], 1u) == unsigned(nseg - 1);
-    __syncthreads();
-    if (!last) return;
-    __threadfence();
-    // all warps stage the segment sums (independent loads in flight together),
-    // then warp 0 scans them from shared memory in a fixed order
-    for (int k = int(warp); k < nseg; k += kGsWarps) sst[k][lane] = okc ? __ldcg(ssum + int64_t(k) * nc + c) : 0.0;
-    __syncthreads();
-    if (warp == 0 && okc) {
-      double all = 0.0;
-      for (int k = 0; k < nseg; ++k) {
-        const int s2 = suffix ? nseg - 1 - k : k;
-        sbase[int64_t(s2) * nc + c] = all;
-        all += sst[s2][lane];
-      }
-      tot[c] = T(all);
-      totd[c] = all;
-    }
-    if (threadIdx.x == 0) ticket[blockIdx.x] = 0u;  // ready for the next step
+    for (int k = 0; k < kGsWarps; ++k) sum += ws[k][lane];
+    ssum[int64_t(seg) * nc + c] = sum;
   }
-  if (!fin.st) return;
-  // the totals of this column block are written (by warp 0): the last block finalizes
-  if (warp == 0) {
-    __threadfence();
-    __syncwarp();
-    unsigned t = 0;
-    if (lane == 0) t = atomicAdd(&ticket[gridDim.x], 1u);
-    if (__shfl_sync(0xffffffffu, t, 0) == gridDim.x - 1) {
-      __threadfence();
-      if (lane == 0) ticket[gridDim.x] = 0u;
-      finalize_step(fin, int(lane));
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) last = atomicAdd(&ticket[blockIdx.x], 1u) == unsigned(nseg - 1);
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  // all warps stage the segment sums (independent loads in flight together),
+  // then warp 0 scans them from shared memory in a fixed order
+  for (int k = int(warp); k < nseg; k += kGsWarps) sst[k][lane] = okc ? __ldcg(ssum + int64_t(k) * nc + c) : 0.0;
+  __syncthreads();
+  if (warp == 0 && okc) {
+    double all = 0.0;
+    for (int k = 0; k < nseg; ++k) {
+      const int s2 = suffix ? nseg - 1 - k : k;
+      sbase[int64_t(s2) * nc + c] = all;
+      all += sst[s2][lane];
     }
+    tot[c] = T(all);
+    totd[c] = all;
   }
+  if (threadIdx.x == 0) ticket[blockIdx.x] = 0u;  // ready for the next step
+  group_finalize(fin, ticket, gridDim.x, warp, lane);
 }
 
 template <class T>
@@ -1327,15 +1371,24 @@ __global__ void __launch_bounds__(kGsWarps * 32) k_group_bases(const double* __r
 }
 
 template <class T>
-void launch_group_scan(const double* gagg, double* work, unsigned* ticket, T* gbase, T* tot, double* totd,
-                       int64_t ngroups, int nc, int gseg, const FinalizeArgs* fin, LaunchSeq& seq) {
-  if (ngroups <= 0) return;
+void launch_scans(const T* agg, T* pfx, double* gagg, double* work, unsigned* ticket, T* gbase, T* tot, double* totd,
+                  int64_t ntiles, int nc, int gseg, const FinalizeArgs* fin, LaunchSeq& seq) {
+  const int64_t tw = tiles_whole(ntiles), ts = tile_stride(ntiles), ngroups = tw / kTilesPerGroup;
+  if (tw <= 0) return;
+  const bool one = ngroups <= kGsOne;
+  const dim3 grid(unsigned((tw + kTsTiles - 1) / kTsTiles), unsigned((nc + kTsRows - 1) / kTsRows));
+  const FinalizeArgs fa = fin ? *fin : FinalizeArgs{};
+  const dim3 cols1(unsigned(gs_col_blocks(nc)), unsigned((grid.x + kGsWarps - 1) / kGsWarps));
+  seq(k_tile_scan<T>, grid, 256, 0, agg, pfx, gagg, one && cols1.y > 1 ? work : nullptr, tw, ts, nc);
+  if (one) {
+    seq(k_group_scan<T>, cols1, kGsWarps * 32, 0, gagg, work, ticket, gbase, tot, totd, int(ngroups), nc, fa);
+    return;
+  }
   const int64_t G = gs_seg_len(ngroups, gseg);
   const int nseg = int(gs_nseg(ngroups, gseg));
-  const dim3 grid(unsigned(gs_col_blocks(nc)), unsigned(nseg));
-  seq(k_group_sums<T>, grid, kGsWarps * 32, 0, gagg, work, ticket, gbase, tot, totd, ngroups, nc, G, nseg,
-      fin ? *fin : FinalizeArgs{});
-  if (nseg > 1) seq(k_group_bases<T>, grid, kGsWarps * 32, 0, gagg, work, gbase, ngroups, nc, G);
+  const dim3 cols(unsigned(gs_col_blocks(nc)), unsigned(nseg));
+  seq(k_group_sums<T>, cols, kGsWarps * 32, 0, gagg, work, ticket, tot, totd, ngroups, nc, G, nseg, fa);
+  seq(k_group_bases<T>, cols, kGsWarps * 32, 0, gagg, work, gbase, ngroups, nc, G);
 }
 
 // Step state after a load: step 0, nothing recorded, the first kick is a half kick.
@@ -1497,7 +1550,7 @@ template <class T> cudaError_t preload_core_kernels_t() {
       reinterpret_cast<const void*>(&k_load<T>),        reinterpret_cast<const void*>(&k_state_dump<T>),
       reinterpret_cast<const void*>(&k_scatter_by_id<T>), reinterpret_cast<const void*>(&k_state_out<T>),
       reinterpret_cast<const void*>(&k_tile_scan<T>),   reinterpret_cast<const void*>(&k_group_sums<T>),
-      reinterpret_cast<const void*>(&k_group_bases<T>)};
+      reinterpret_cast<const void*>(&k_group_bases<T>), reinterpret_cast<const void*>(&k_group_scan<T>)};
   for (const void* f : fns) {
     const cudaError_t e = cudaFuncGetAttributes(&fa, f);
     if (e != cudaSuccess) return e;
@@ -1540,9 +1593,8 @@ cudaError_t preload_core_kernels() {
   template void launch_scatter_by_id<T>(const T* const*, int, const uint32_t*, double*, int64_t,   \
                                         LaunchSeq&);                                               \
   template void launch_state_out<T>(const Part<T>*, double*, double*, uint32_t*, int64_t, cudaStream_t); \
-  template void launch_tile_scan<T>(const T*, T*, double*, int64_t, int, LaunchSeq&);                \
-  template void launch_group_scan<T>(const double*, double*, unsigned*, T*, T*, double*, int64_t, int, \
-                                     int, const FinalizeArgs*, LaunchSeq&);
+  template void launch_scans<T>(const T*, T*, double*, double*, unsigned*, T*, T*, double*, int64_t, int, int, \
+                                const FinalizeArgs*, LaunchSeq&);
 IMRP_INST_CORE(float)
 IMRP_INST_CORE(double)
 

@@ -265,11 +265,9 @@ __host__ __device__ constexpr int64_t tile_stride(int64_t ntiles) { return tiles
 // kGsWarps warps (32 components per CTA, one per lane).
 constexpr int kGsWarps = 8;
 constexpr int kGsMaxSeg = 64;
-// Up to kGsOne groups (4 per warp) one CTA per 32 components does it all: the
-// sums, the bases and no second kernel.
-constexpr int64_t kGsOne = 32;
+// Up to kGsOne groups one kernel does it all (k_group_scan).
+constexpr int64_t kGsOne = 320;
 __host__ __device__ inline int64_t gs_seg_len(int64_t ngroups, int gseg) {
-  if (ngroups <= kGsOne) return (ngroups + kGsWarps - 1) / kGsWarps * kGsWarps;
   int64_t G = (ngroups + kGsMaxSeg - 1) / kGsMaxSeg;
   if (G < gseg) G = gseg;
   return (G + kGsWarps - 1) / kGsWarps * kGsWarps;
@@ -281,7 +279,8 @@ __host__ __device__ inline int64_t gs_nseg(int64_t ngroups, int gseg) {
 // tickets of the group scan: one per column block, one for the finalize
 __host__ __device__ constexpr int gs_tickets(int nc) { return (nc + 31) / 32 + 1; }
 // FP64 work space of the group scan for nc components: per segment the
-// kGsWarps warp sums, the segment sum and the segment's base.
+// kGsWarps warp sums, the segment sum and the segment's base; or the sums of the
+// runs of 4 groups that k_group_scan takes.
 __host__ __device__ constexpr int64_t gs_work_doubles(int nc) { return int64_t(kGsMaxSeg) * (kGsWarps + 2) * nc; }
 __host__ __device__ constexpr int gs_col_blocks(int nc) { return (nc + 31) / 32; }
 

@@ -122,11 +122,6 @@ template <class T>
 void launch_state_out(const Part<T>* st, double* x, double* v, uint32_t* inv, int64_t n, cudaStream_t s);
 
 // ---- scans (imrp_core.cu) ---------------------------------------------------
-// in-group scans of agg[u][tile] (row stride tile_stride(ntiles)) into
-// pfx[tile][u] (tile-major: one tile's nc carries contiguous), group totals
-// into gagg[g][u] (FP64)
-template <class T>
-void launch_tile_scan(const T* agg, T* pfx, double* gagg, int64_t ntiles, int nc, LaunchSeq& seq);
 struct FinalizeArgs {
   StepState* st;
   const double* totd;
@@ -156,15 +151,17 @@ template <class T> inline void derive_field_args(FieldArgs<T>& a) {
   a.ion_coef_h = float(a.ion_coef);
   a.ion_coef_l = float(a.ion_coef - double(a.ion_coef_h));
 }
-// group scan over gagg:
-// gseg: least number of groups per segment (16, 32 or 64; chosen by the
+// In-group scans of agg[u][tile] (row stride tile_stride(ntiles)) into
+// pfx[tile][u] (tile-major: one tile's nc carries contiguous), the group totals
+// gagg[g][u] (FP64), and the scan over the groups into gbase and the totals tot
+// and totd. gseg: least number of groups per segment (16, 32 or 64; chosen by the
 // autotuner). work: gs_work_doubles(nc) doubles; ticket: gs_tickets(nc)
 // counters, zero before the first call (each call leaves them zero). fin (or
 // null): the step's finalize (drive, kick weight, Q_diff tally), run once the
 // totals are complete.
 template <class T>
-void launch_group_scan(const double* gagg, double* work, unsigned* ticket, T* gbase, T* tot, double* totd,
-                       int64_t ngroups, int nc, int gseg, const FinalizeArgs* fin, LaunchSeq& seq);
+void launch_scans(const T* agg, T* pfx, double* gagg, double* work, unsigned* ticket, T* gbase, T* tot, double* totd,
+                  int64_t ntiles, int nc, int gseg, const FinalizeArgs* fin, LaunchSeq& seq);
 // Loads the device code of every degree-independent kernel of both precisions
 // (CUDA loads modules lazily, at a kernel's first launch or query, and the
 // load reserves device memory): the allocation-free entry point calls it at

@@ -181,8 +181,6 @@ int run(const imrp_params* p, const double* x, int64_t n, int64_t step, double* 
   ma.agg = static_cast<T*>(P(o.agg));
   ma.parts = mom_parts(sizeof(T), L, n, mom_ppt(sizeof(T), n));
   ks->moments(ma, seq);
-  launch_tile_scan<T>(static_cast<T*>(P(o.agg)), static_cast<T*>(P(o.pfx)), static_cast<double*>(P(o.gagg)),
-                      ntiles, nc, seq);
   double canti[kTabL] = {0}, f[kTabL] = {0};
   for (int l = 1; l <= L; ++l) {
     f[l] = coef_f(l, d, p->eps_D);
@@ -205,9 +203,10 @@ int run(const imrp_params* p, const double* x, int64_t n, int64_t step, double* 
     fa.canti[l] = canti[l];
     fa.cdrive[l] = canti[l] * 4.0 * kPi * n_tilde;
   }
-  launch_group_scan<T>(static_cast<double*>(P(o.gagg)), static_cast<double*>(P(o.gswork)),
-                       static_cast<unsigned*>(P(o.gsticket)), static_cast<T*>(P(o.gbase)),
-                       static_cast<T*>(P(o.tot)), static_cast<double*>(P(o.totd)), ngroups, nc, 32, &fa, seq);
+  launch_scans<T>(static_cast<T*>(P(o.agg)), static_cast<T*>(P(o.pfx)), static_cast<double*>(P(o.gagg)),
+                  static_cast<double*>(P(o.gswork)), static_cast<unsigned*>(P(o.gsticket)),
+                  static_cast<T*>(P(o.gbase)), static_cast<T*>(P(o.tot)), static_cast<double*>(P(o.totd)), ntiles, nc,
+                  32, &fa, seq);
   FieldArgs<T> a;
   memset(&a, 0, sizeof(a));
   a.x = st1[0]; a.y = st1[1]; a.z = st1[2]; a.vx = st1[3]; a.vy = st1[4]; a.vz = st1[5];
