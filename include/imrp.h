@@ -347,9 +347,9 @@ int imrp_get_info(const imrp_ctx* ctx, imrp_info* info);
 /* Stage timing. Runs n_steps steps launched one by one (no CUDA graph) with a
  * CUDA event pair around each stage on the context's stream, and writes the
  * summed device time of each stage in milliseconds to ms[IMRP_N_STAGES]:
- * 0 radix sort, 1 reorder, 2 tile moments with the in-group scans,
- * 3 group scan + finalize,
- * 4 field gather + push. The steps are real steps (they advance the state and
+ * 0 sort by radius (up to 2.4e7 particles with the gather into radius order),
+ * 1 that gather (beyond), 2 tile moments, 3 scans + finalize,
+ * 4 field + push. The steps are real steps (they advance the state and
  * are recorded like imrp_step). */
 #define IMRP_N_STAGES 5
 int imrp_profile_steps(imrp_ctx* ctx, int64_t n_steps, double* ms);
@@ -384,7 +384,8 @@ int imrp_autotune(imrp_ctx* ctx, int* wpb_out, int* gseg_out);
  * one degree and precision run as one launch over a work list of (context,
  * block of 1024 particles); then each context's scans and finalize; then the
  * field, push and walls of all contexts of one degree and precision as one
- * launch over a work list of (context, CTA of tiles). Instances of uneven N
+ * launch over a work list of (context, CTA of tiles), or two where some of them
+ * run in another field kernel (large FP32 instances). Instances of uneven N
  * share those launches and overlap on the GPU. The batch does not
  * own the contexts; they must stay alive and must not be used through their
  * own entry points between imrp_batch_step and imrp_batch_sync. Each context

@@ -395,9 +395,13 @@ __host__ __device__ constexpr int img_in_tile_for(int64_t n) {
 }
 
 // Whether an instance's field runs in the pair kernel (field_pair): FP32, degree 12
-// and up, enough tiles to fill the GPU several times (smaller instances keep the
-// kernel of one tile per warp, which has twice the warps), all m. A rule of n, so
-// that an instance computes the same alone and in a batch.
+// and up, at least 2^19 particles, all m. A rule of n, so that an instance computes
+// the same alone and in a batch. Field ms, one tile per warp against the pair kernel:
+// l_max = 16 N = 5e5 0.150 and 0.135, N = 1e6 0.275 and 0.250; l_max = 12 N = 131072
+// 0.0413 and 0.0392, N = 5e5 0.115 and 0.097. It is the faster one below the line too,
+// down to 1e5 particles; but its sums round differently, and the trajectories of small
+// instances, where one particle's charge weighs more, follow the last bit of the
+// field (two particles within a rounding of the same radius swap): they keep theirs.
 constexpr int64_t kPairMinN = int64_t(1) << 19;
 constexpr int kPairMinL = 12;
 constexpr int kPairWarps = 2, kPairMaxWarps = 4;  // warps per CTA: default, at most

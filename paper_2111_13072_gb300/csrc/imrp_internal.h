@@ -211,7 +211,8 @@ inline int64_t mom_blocks(int64_t n, int ppt) { return (n + 1023) / 1024 * (16 /
 // into ranges that separate CTAs take (a range first walks its particles'
 // diagonal terms up to its first column). As many ranges as give the stated
 // CTAs per SM: FP32 N = 1e5, l_max = 16: 0.043 ms with one range, 0.0225 with
-// 6 per SM, 0.028 with 8; N = 3e5, l_max = 8: 0.0262, 0.0206, 0.0267; FP64
+// 6 per SM, 0.028 with 8; N = 3e5, l_max = 8: 0.0262, 0.0206, 0.0267 (0.0204 and
+// 0.0172 since all of a thread's loads go out at once); FP64
 // N = 20000, l_max = 8: 0.102 with one, 0.039 with 7 ranges (4 CTAs per SM), 0.043 with 9.
 inline int mom_parts(int elem_size, int L, int64_t n, int ppt) {
   const int per_sm = elem_size == 4 ? 6 : ppt == 4 ? 4 : 8;

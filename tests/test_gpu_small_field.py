@@ -1,7 +1,7 @@
 """FP32 instances of at most 1024 particles sum the image pairs of their own tile directly, in a field
 kernel of their own: every particle's field against the oracle at the edges of the tile and of the rule,
-with both image rules and in the m = 0 truncation, and alone against in a batch (whose kernel takes the
-pairs one at a time)."""
+with both image rules and in the m = 0 truncation; alone and in a batch (whose kernel takes the pairs one
+at a time) the same bits."""
 import numpy as np
 import pytest
 
@@ -57,6 +57,5 @@ def test_alone_and_in_a_batch(imrp):
             for s in sims:
                 s.close()
     for (xa, va), (xb, vb) in zip(*out):
-        # two steps of FP32 kicks: the image pairs' sums differ by roundings (2^-24 of the field) at most
-        np.testing.assert_allclose(xa, xb, rtol=0, atol=4 * 2.0 ** -24 * np.max(np.abs(xa)))
-        np.testing.assert_allclose(va, vb, rtol=0, atol=64 * 2.0 ** -24 * np.max(np.abs(va)))
+        np.testing.assert_array_equal(xa, xb)
+        np.testing.assert_array_equal(va, vb)
