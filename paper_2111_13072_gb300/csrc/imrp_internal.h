@@ -77,13 +77,14 @@ constexpr int64_t sort_blocks(int64_t n) { return (n + kSortTile - 1) / kSortTil
 // Scratch of the bucket sort's first pass: the digits' totals and the ticket of its CTAs, zero
 // between sorts (zeroed at allocation), and the digits' cursors. Behind it stand, for the global
 // passes, the block counts of 256 digits per block and the digit totals.
-constexpr int kSortDigits = 4096;
+constexpr int kSortDigits = 8192;
 struct alignas(64) SortState {
   uint32_t tot[kSortDigits], cur[kSortDigits], ticket;
 };
 constexpr size_t sort_scratch_bytes(int64_t n) {
   return sizeof(SortState) + sizeof(uint32_t) * size_t(256 * sort_blocks(n) + 256);
 }
+int sort_digits(int64_t n);  // digits of the first pass for n keys alone on the GPU
 // Sorts the particles src[0 .. n) by the key bytes first_byte..3 (stable: keys equal in those
 // bytes keep their order). k0/v0 hold the keys and slots 0 .. n-1; k1/v1 are scratch of n;
 // scratch: sort_scratch_bytes(n). Either gathers the particles into the component arrays dst and

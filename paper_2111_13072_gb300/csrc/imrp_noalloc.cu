@@ -85,7 +85,7 @@ constexpr double kEps0 = 8.8541878128e-12;
 // Per-call set-up of what must start at zero or at the given step: the step
 // state, the group scan's tickets and the sort's digit totals (the scratch keeps the
 // previous call's contents, and another n or degree lays it out differently).
-struct NaInit { StepState* st; int64_t step; unsigned* ticket; int nticket; SortState* sort; };
+struct NaInit { StepState* st; int64_t step; unsigned* ticket; int nticket; SortState* sort; int ndigit; };
 
 // FP64 [n][3] positions -> particle records, ids 0..n-1, zero velocities, and their radius keys;
 // flags positions outside 1 < r < r_out or non-finite. The first block does the set-up too. (As
@@ -97,7 +97,7 @@ __global__ void __launch_bounds__(256) k_na_load(const double* __restrict__ x, P
   chain_wait();
   if (blockIdx.x == 0) {
     for (int k = threadIdx.x; k < in.nticket; k += 256) in.ticket[k] = 0u;
-    for (int k = threadIdx.x; k < kSortDigits; k += 256) in.sort->tot[k] = 0u;
+    for (int k = threadIdx.x; k < in.ndigit; k += 256) in.sort->tot[k] = 0u;
     if (threadIdx.x == 0) {
       in.sort->ticket = 0u;
       in.st->step = in.step;
@@ -166,7 +166,8 @@ int run(const imrp_params* p, const double* x, int64_t n, int64_t step, double* 
   int* err = g_derr[dev];
   *g_err[dev] = 0;
   LaunchSeq seq(s);
-  const NaInit init{st, step, static_cast<unsigned*>(P(o.gsticket)), gs_tickets(nc), static_cast<SortState*>(P(o.sort))};
+  const NaInit init{st, step, static_cast<unsigned*>(P(o.gsticket)), gs_tickets(nc), static_cast<SortState*>(P(o.sort)),
+                    sort_digits(n)};
   seq(k_na_load<T>, unsigned((n + 255) / 256), 256, 0, x, st0, key0, idx0, n, r_out, make_radius_key(r_out), err, init);
   const uint32_t* perm =
       launch_radix_sort<T>(key0, idx0, static_cast<uint32_t*>(P(o.key1)), static_cast<uint32_t*>(P(o.idx1)), P(o.sort),
