@@ -251,6 +251,10 @@ int check_err(imrp_ctx* ctx) {
   const int h = ctx->host->err;
   if (h) {
     ctx->host->err = 0;
+    if (h & kErrSort) {  // no order of the particles: what follows from it is void
+      ctx->loaded = false;
+      return ctx->fail(IMRP_E_CUDA, "the sort's work area was overwritten");
+    }
     if (h & kErrNaN) return ctx->fail(IMRP_E_NAN, "non-finite value in the particle state");
     if (h & kErrRange) return ctx->fail(IMRP_E_INVAL, "a particle lies outside 1 < r < r_out");
   }
@@ -376,7 +380,7 @@ template <class T> void enqueue_pre(imrp_ctx* ctx, LaunchSeq& seq, cudaEvent_t* 
   stage_event(seq, ev, 0);
   const uint32_t* perm =
       launch_radix_sort<T>(ctx->key0, ctx->idx0, ctx->key1, ctx->idx1, ctx->sort_scratch, n, sort_first_byte(ctx->prec),
-                           st, sorted_ptrs<T>(ctx), ctx->srt_id, seq, shared_gpu);
+                           st, sorted_ptrs<T>(ctx), ctx->srt_id, ctx->derr, seq, shared_gpu);
   stage_event(seq, ev, 1);
   if (perm) launch_reorder<T>(st, sorted_ptrs<T>(ctx), ctx->srt_id, perm, n, seq);
 }
@@ -505,6 +509,10 @@ size_t footprint_bytes(int64_t N, int L, int prec) {
   return b;
 }
 
+// What must start at zero (the sort's totals and ticket, the scans' tickets) is zeroed on the
+// context's own stream and waited for by imrp_create: a plain cudaMemset runs on the legacy
+// stream, which that non-blocking stream does not wait for, and beside other contexts' queued
+// steps it can run as late as in the middle of the new context's sorts.
 int alloc_ctx(imrp_ctx* ctx) {
   const int64_t N = ctx->p.N;
   const size_t es = ctx->prec == 1 ? sizeof(float) : sizeof(double);
@@ -519,7 +527,7 @@ int alloc_ctx(imrp_ctx* ctx) {
   CK(cudaMalloc(&ctx->key1, N * sizeof(uint32_t)));
   CK(cudaMalloc(&ctx->idx1, N * sizeof(uint32_t)));
   CK(cudaMalloc(&ctx->sort_scratch, sort_scratch_bytes(N)));
-  CK(cudaMemset(ctx->sort_scratch, 0, sizeof(SortState)));
+  CK(cudaMemsetAsync(ctx->sort_scratch, 0, sizeof(SortState), ctx->own_stream));
   CK(cudaMalloc(&ctx->agg, tile_stride(ntiles) * nc * es));
   CK(cudaMalloc(&ctx->pfx, tile_stride(ntiles) * nc * es));
   CK(cudaMalloc(&ctx->gbase, ngroups * nc * es));
@@ -528,7 +536,7 @@ int alloc_ctx(imrp_ctx* ctx) {
   CK(cudaMalloc(&ctx->totd, nc * sizeof(double)));
   CK(cudaMalloc(&ctx->gswork, gs_work_doubles(nc) * sizeof(double)));
   CK(cudaMalloc(&ctx->gsticket, gs_tickets(nc) * sizeof(unsigned)));
-  CK(cudaMemset(ctx->gsticket, 0, gs_tickets(nc) * sizeof(unsigned)));
+  CK(cudaMemsetAsync(ctx->gsticket, 0, gs_tickets(nc) * sizeof(unsigned), ctx->own_stream));
   CK(cudaMalloc(&ctx->eout, 3 * N * es));
   CK(cudaMalloc(&ctx->stage, 6 * N * sizeof(double)));
   CK(cudaMalloc(&ctx->st, sizeof(StepState)));
@@ -653,6 +661,7 @@ int imrp_create(const imrp_params* p, imrp_ctx** out) {
     delete ctx;
     return rc == IMRP_E_CUDA ? IMRP_E_NOMEM : rc;
   }
+  if (cudaStreamSynchronize(ctx->own_stream) != cudaSuccess) { free_all(ctx); delete ctx; return IMRP_E_CUDA; }
   ctx->cap = p->N;
   *out = ctx;
   return IMRP_OK;
@@ -699,7 +708,7 @@ int imrp_set_species(imrp_ctx* ctx, int64_t n_electrons, double ion_charge, doub
       CK(cudaMalloc(&ctx->qtotd, sizeof(double)));
       CK(cudaMalloc(&ctx->qwork, gs_work_doubles(1) * sizeof(double)));
       CK(cudaMalloc(&ctx->qticket, gs_tickets(1) * sizeof(unsigned)));
-      CK(cudaMemset(ctx->qticket, 0, gs_tickets(1) * sizeof(unsigned)));
+      CK(cudaMemsetAsync(ctx->qticket, 0, gs_tickets(1) * sizeof(unsigned), ctx->stream));
     }
     ctx->species = 1;
     ctx->sp_ne = n_electrons;

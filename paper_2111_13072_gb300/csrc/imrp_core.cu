@@ -359,7 +359,10 @@ __device__ __forceinline__ void count_byte(const uint32_t* keys, int64_t len, in
 // into the buckets' starts; k_sort_spread reserves each digit's keys of a CTA with one atomic on
 // the bucket's cursor and writes them there, in any order: the order within a bucket is settled
 // by the comparisons of k_bucket_sort, so the result does not depend on the order of the atomics.
-// In its scratch (SortState) the totals and the ticket are zero between sorts.
+// In its scratch (SortState) the totals and the ticket are zero between sorts: whoever allocates it
+// zeroes it in the order of the stream that sorts. Were they not, the cursors would lead out of the
+// arrays: a place past the end is skipped, and a bucket that is no part of the array left out, with
+// an error status that the next synchronising call returns.
 // The stable pass (histogram matrix, row scan, ranked scatter; it serves the four global passes of
 // very large arrays) took 7 + 6 + 20 us at N = 2e6; these two take 10 + 16, bound by latency.
 constexpr int kSpreadThreads = 512;
@@ -436,7 +439,7 @@ __global__ void __launch_bounds__(kSpreadThreads) k_sort_count(const uint32_t* _
 
 __global__ void __launch_bounds__(kSpreadThreads) k_sort_spread(const uint32_t* __restrict__ keys, int64_t n, int shift,
                                                                 int nd, SortState* st, uint32_t* __restrict__ kout,
-                                                                uint32_t* __restrict__ vout) {
+                                                                uint32_t* __restrict__ vout, int* err) {
   chain_wait();
   extern __shared__ __align__(16) uint32_t sbuf[];
   uint32_t* const cnt = sbuf;  // [nd]: counts, then the place of the CTA's first key of the digit
@@ -473,8 +476,12 @@ __global__ void __launch_bounds__(kSpreadThreads) k_sort_spread(const uint32_t* 
     const int64_t o = base + i * kSpreadThreads + int64_t(t);
     if (o < n) {
       const uint32_t p = cnt[k[i] >> shift] + r[i];
-      kout[p] = k[i];
-      vout[p] = uint32_t(o);
+      if (p < n) {
+        kout[p] = k[i];
+        vout[p] = uint32_t(o);
+      } else {
+        atomicOr(err, kErrSort);
+      }
     }
   }
 }
@@ -516,7 +523,7 @@ template <class T, int NT, int MINB>
 __global__ void __launch_bounds__(NT, MINB) k_bucket_sort(uint32_t* k1, uint32_t* v1, uint32_t* k0, uint32_t* v0,
                                                           const SortState* __restrict__ st, int64_t n_all, int cap,
                                                           int tb, int sb, const Part<T>* __restrict__ src,
-                                                          SoA<T> dst) {
+                                                          SoA<T> dst, int* err) {
   chain_wait();
   extern __shared__ __align__(16) uint32_t sbuf[];
   __shared__ uint32_t s_w[NT / 32];
@@ -528,8 +535,17 @@ __global__ void __launch_bounds__(NT, MINB) k_bucket_sort(uint32_t* k1, uint32_t
   if (st) {  // the cursors are the buckets' ends now
     start = blockIdx.x ? st->cur[blockIdx.x - 1] : 0u;
     len = int64_t(st->cur[blockIdx.x]) - start;
+    if (len < 0 || start + len > n_all) {  // never with a sort state in order; uniform over the CTA
+      if (t == 0) atomicOr(err, kErrSort);
+      return;
+    }
   }
   if (len == 0) return;  // uniform over the CTA
+  const auto slot = [&](uint32_t v) {  // a slot that the spread did not write is no particle
+    if (v < n_all) return v;
+    atomicOr(err, kErrSort);
+    return 0u;
+  };
   const uint32_t* const sk = k1 + start;
   const uint32_t* const sv = v1 + start;
   {
@@ -640,6 +656,7 @@ __global__ void __launch_bounds__(NT, MINB) k_bucket_sort(uint32_t* k1, uint32_t
               const uint32_t kq = ks[q];
               at[u] += kq < key || (kq == key && vs[q] < from[u]) ? 1u : 0u;
             }
+            from[u] = slot(from[u]);
           }
           Part<T> x[G];
 #pragma unroll
@@ -676,7 +693,7 @@ __global__ void __launch_bounds__(NT, MINB) k_bucket_sort(uint32_t* k1, uint32_t
     uint32_t* x = ak; ak = dk; dk = x;
     x = av; av = dv; dv = x;
   }
-  for (int64_t i = t; i < len; i += NT) put_part<T>(dst, start + i, src[av[i]]);
+  for (int64_t i = t; i < len; i += NT) put_part<T>(dst, start + i, src[slot(av[i])]);
 }
 
 // Largest N for the bucket sort (2930 keys a bucket on average); larger arrays take the four global
@@ -736,8 +753,8 @@ cudaError_t set_sort_attributes() {
 
 template <class T>
 const uint32_t* launch_radix_sort(uint32_t* k0, uint32_t* v0, uint32_t* k1, uint32_t* v1, void* scratch, int64_t n,
-                                  int first_byte, const Part<T>* src, T* const* dst, uint32_t* id_dst, LaunchSeq& seq,
-                                  bool shared_gpu) {
+                                  int first_byte, const Part<T>* src, T* const* dst, uint32_t* id_dst, int* err,
+                                  LaunchSeq& seq, bool shared_gpu) {
   if (n <= 1) return v0;
   SoA<T> d;
   for (int c = 0; c < 6; ++c) d.d[c] = dst[c];
@@ -746,7 +763,7 @@ const uint32_t* launch_radix_sort(uint32_t* k0, uint32_t* v0, uint32_t* k1, uint
   if (first_byte == 0 && n <= kBsSingleN) {
     const int cap = int((n + 255) / 256 * 256), sb = bucket_bits(n, kBsOneThreads);
     seq(k_bucket_sort<T, kBsOneThreads, 1>, 1, kBsOneThreads, bucket_smem<kBsOneThreads>(cap, sb), k0, v0, k1, v1,
-        nullptr, n, cap, 0, sb, src, d);
+        nullptr, n, cap, 0, sb, src, d, err);
     return nullptr;
   }
   if (first_byte == 0 && n <= kBucketSortMaxN) {
@@ -755,9 +772,9 @@ const uint32_t* launch_radix_sort(uint32_t* k0, uint32_t* v0, uint32_t* k1, uint
     const int cap = bucket_cap(mean), sb = bucket_bits(mean, kBsThreads);
     const unsigned blocks = unsigned((n + kSpreadTile - 1) / kSpreadTile);
     seq(k_sort_count, blocks, kSpreadThreads, sizeof(uint32_t) * nd, k0, n, shift, nd, st);
-    seq(k_sort_spread, blocks, kSpreadThreads, sizeof(uint32_t) * nd, k0, n, shift, nd, st, k1, v1);
+    seq(k_sort_spread, blocks, kSpreadThreads, sizeof(uint32_t) * nd, k0, n, shift, nd, st, k1, v1, err);
     seq(k_bucket_sort<T, kBsThreads, kBsPerSM>, unsigned(nd), kBsThreads, bucket_smem<kBsThreads>(cap, sb), k1, v1, k0,
-        v0, st, n, cap, tb, sb, src, d);
+        v0, st, n, cap, tb, sb, src, d, err);
     return nullptr;
   }
   const int64_t nblk = sort_blocks(n);
@@ -953,6 +970,7 @@ __global__ void k_scatter_by_id(Ptr6<T> p, int nc, const uint32_t* __restrict__ 
   const int64_t j = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   if (j >= n) return;
   const int64_t k = id[j];
+  if (k >= n) return;  // only after a sort that ended with kErrSort
   for (int c = 0; c < nc; ++c) out[k * nc + c] = double(p.d[c][j]);
 }
 
@@ -979,13 +997,14 @@ __global__ void k_state_out(const Part<T>* __restrict__ st, double* __restrict__
   if (j >= n) return;
   const Part<T> p = st[j];
   const int64_t k = p.id;
+  if (k >= n) return;  // only after a sort that ended with kErrSort; so below
   x[3 * k] = p.x; x[3 * k + 1] = p.y; x[3 * k + 2] = p.z;
   v[3 * k] = p.vx; v[3 * k + 1] = p.vy; v[3 * k + 2] = p.vz;
 }
 template <class T>
 __global__ void k_inverse_ids(const Part<T>* __restrict__ st, uint32_t* __restrict__ inv, int64_t n) {
   const int64_t j = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (j < n) inv[st[j].id] = uint32_t(j);
+  if (j < n && st[j].id < n) inv[st[j].id] = uint32_t(j);
 }
 template <class T>
 __global__ void k_state_gather(const Part<T>* __restrict__ st, const uint32_t* __restrict__ inv,
@@ -993,7 +1012,9 @@ __global__ void k_state_gather(const Part<T>* __restrict__ st, const uint32_t* _
   chain_wait();
   const int64_t k = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   if (k >= n) return;
-  const Part<T> p = st[inv[k]];
+  const int64_t j = inv[k];
+  if (j >= n) return;
+  const Part<T> p = st[j];
   x[3 * k] = p.x; x[3 * k + 1] = p.y; x[3 * k + 2] = p.z;
   v[3 * k] = p.vx; v[3 * k + 1] = p.vy; v[3 * k + 2] = p.vz;
 }
@@ -1585,7 +1606,7 @@ cudaError_t preload_core_kernels() {
 // explicit instantiations
 #define IMRP_INST_CORE(T)                                                                          \
   template const uint32_t* launch_radix_sort<T>(uint32_t*, uint32_t*, uint32_t*, uint32_t*, void*, int64_t, int,      \
-                                                const Part<T>*, T* const*, uint32_t*, LaunchSeq&, bool);             \
+                                                const Part<T>*, T* const*, uint32_t*, int*, LaunchSeq&, bool);       \
   template void launch_reorder<T>(const Part<T>*, T* const*, uint32_t*, const uint32_t*, int64_t,  \
                                   LaunchSeq&);                                                     \
   template void launch_keys<T>(const Part<T>*, uint32_t*, uint32_t*, int64_t, double, LaunchSeq&); \

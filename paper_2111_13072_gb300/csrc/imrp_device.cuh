@@ -134,7 +134,7 @@ template <class T> __device__ __forceinline__ uint32_t radius_key(T x, T y, T z,
 }
 
 // Device error flags (bitwise or).
-enum : int { kErrNaN = 1, kErrRange = 4 };
+enum : int { kErrNaN = 1, kErrSort = 2, kErrRange = 4 };
 
 template <class T> struct Vec4;
 template <> struct Vec4<float> { using type = float4; };

@@ -75,7 +75,7 @@ constexpr int kSortItems = 8;
 constexpr int kSortTile = kSortThreads * kSortItems;  // keys per CTA
 constexpr int64_t sort_blocks(int64_t n) { return (n + kSortTile - 1) / kSortTile; }
 // Scratch of the bucket sort's first pass: the digits' totals and the ticket of its CTAs, zero
-// between sorts (zeroed at allocation), and the digits' cursors. Behind it stand, for the global
+// between sorts (zeroed before the first, in the order of its stream), and the digits' cursors. Behind it stand, for the global
 // passes, the block counts of 256 digits per block and the digit totals.
 constexpr int kSortDigits = 8192;
 struct alignas(64) SortState {
@@ -88,7 +88,8 @@ int sort_digits(int64_t n);  // digits of the first pass for n keys alone on the
 // Sorts the particles src[0 .. n) by the key bytes first_byte..3 (stable: keys equal in those
 // bytes keep their order). k0/v0 hold the keys and slots 0 .. n-1; k1/v1 are scratch of n;
 // scratch: sort_scratch_bytes(n). Either gathers the particles into the component arrays dst and
-// id_dst itself and returns null, or returns the buffer that holds the slots in key order.
+// id_dst itself and returns null, or returns the buffer that holds the slots in key order. err
+// receives kErrSort if the sort state was not in order (then the order is not to be used).
 // Key bytes sorted: all four, in both precisions. The radius key is
 // floor((r^2 - 1) / (r_out^2 - 1) * 2^32) of the exact FP64 r^2 of the stored
 // position, and the sorted index j of a particle is its count of electrons
@@ -97,8 +98,8 @@ int sort_digits(int64_t n);  // digits of the first pass for n keys alone on the
 inline int sort_first_byte(int) { return 0; }
 template <class T>
 const uint32_t* launch_radix_sort(uint32_t* k0, uint32_t* v0, uint32_t* k1, uint32_t* v1, void* scratch, int64_t n,
-                                  int first_byte, const Part<T>* src, T* const* dst, uint32_t* id_dst, LaunchSeq& seq,
-                                  bool shared_gpu = false);
+                                  int first_byte, const Part<T>* src, T* const* dst, uint32_t* id_dst, int* err,
+                                  LaunchSeq& seq, bool shared_gpu = false);
 
 // ---- state movement and keys (imrp_core.cu) ---------------------------------
 // The state is an array of Part<T> records in the order of the last push (or

@@ -171,7 +171,7 @@ int run(const imrp_params* p, const double* x, int64_t n, int64_t step, double* 
   seq(k_na_load<T>, unsigned((n + 255) / 256), 256, 0, x, st0, key0, idx0, n, r_out, make_radius_key(r_out), err, init);
   const uint32_t* perm =
       launch_radix_sort<T>(key0, idx0, static_cast<uint32_t*>(P(o.key1)), static_cast<uint32_t*>(P(o.idx1)), P(o.sort),
-                           n, sort_first_byte(sizeof(T) == 4 ? 1 : 0), st0, st1, id1, seq);
+                           n, sort_first_byte(sizeof(T) == 4 ? 1 : 0), st0, st1, id1, err, seq);
   if (perm) launch_reorder<T>(st0, st1, id1, perm, n, seq);
   MomArgs<T> ma;
   memset(&ma, 0, sizeof(ma));  // all electrons (species = 0)
@@ -254,6 +254,7 @@ int run(const imrp_params* p, const double* x, int64_t n, int64_t step, double* 
   if (cudaGetLastError() != cudaSuccess) return IMRP_E_CUDA;
   if (cudaStreamSynchronize(s) != cudaSuccess) return IMRP_E_CUDA;
   const int h = *g_err[dev];
+  if (h & kErrSort) return IMRP_E_CUDA;
   if (h & kErrNaN) return IMRP_E_NAN;
   if (h & kErrRange) return IMRP_E_INVAL;
   return IMRP_OK;
