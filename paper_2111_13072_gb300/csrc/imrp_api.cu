@@ -752,7 +752,7 @@ int imrp_set_ion_profile(imrp_ctx* ctx, const double* q_ion, int64_t n_tab, doub
       }
       ctx->ion_cap = n_tab;
     }
-    CK(cudaMemcpy(ctx->ion_q, q_ion, n_tab * sizeof(double), cudaMemcpyHostToDevice));
+    CK(upload(ctx->ion_q, q_ion, n_tab * sizeof(double)));
     ctx->ion_n = n_tab;
     ctx->ion_qe = q_elec_total;
     ctx->ion_qs = q_s;
@@ -1249,10 +1249,10 @@ template <class T> int fill_group(imrp_batch* b, BatchGroup& g) {
       cudaMalloc(&g.dmom_items, mi.size() * sizeof(int2)) != cudaSuccess ||
       cudaMalloc(&g.dfield_items, fi.size() * sizeof(int2)) != cudaSuccess)
     return IMRP_E_NOMEM;
-  if (cudaMemcpy(g.dmom, ma.data(), ma.size() * sizeof(MomArgs<T>), cudaMemcpyHostToDevice) != cudaSuccess ||
-      cudaMemcpy(g.dfield, fa.data(), fa.size() * sizeof(FieldArgs<T>), cudaMemcpyHostToDevice) != cudaSuccess ||
-      cudaMemcpy(g.dmom_items, mi.data(), mi.size() * sizeof(int2), cudaMemcpyHostToDevice) != cudaSuccess ||
-      cudaMemcpy(g.dfield_items, fi.data(), fi.size() * sizeof(int2), cudaMemcpyHostToDevice) != cudaSuccess)
+  if (upload(g.dmom, ma.data(), ma.size() * sizeof(MomArgs<T>)) != cudaSuccess ||
+      upload(g.dfield, fa.data(), fa.size() * sizeof(FieldArgs<T>)) != cudaSuccess ||
+      upload(g.dmom_items, mi.data(), mi.size() * sizeof(int2)) != cudaSuccess ||
+      upload(g.dfield_items, fi.data(), fi.size() * sizeof(int2)) != cudaSuccess)
     return IMRP_E_CUDA;
   return IMRP_OK;
 }
@@ -1464,8 +1464,8 @@ template <class T> int time_group_field(imrp_batch* b, const BatchGroup& g, int 
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   if (cudaMalloc(&dfa, fa.size() * sizeof(FieldArgs<T>)) != cudaSuccess ||
       cudaMalloc(&dfi, fi.size() * sizeof(int2)) != cudaSuccess ||
-      cudaMemcpy(dfa, fa.data(), fa.size() * sizeof(FieldArgs<T>), cudaMemcpyHostToDevice) != cudaSuccess ||
-      cudaMemcpy(dfi, fi.data(), fi.size() * sizeof(int2), cudaMemcpyHostToDevice) != cudaSuccess ||
+      upload(dfa, fa.data(), fa.size() * sizeof(FieldArgs<T>)) != cudaSuccess ||
+      upload(dfi, fi.data(), fi.size() * sizeof(int2)) != cudaSuccess ||
       cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess) {
     rc = IMRP_E_CUDA;
   } else {

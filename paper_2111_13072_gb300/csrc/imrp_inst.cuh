@@ -279,6 +279,9 @@ template <class T, int L> cudaError_t set_attr() {
       if (e == cudaSuccess) e = cudaMemcpyToSymbol(c_an2, h_an2, sizeof(h_an2));             \
       if (e != cudaSuccess) return int(e);                                                   \
     }                                                                                        \
+    /* kernels on non-blocking streams read the tables (see upload) */                       \
+    e = cudaStreamSynchronize(cudaStreamLegacy);                                             \
+    if (e != cudaSuccess) return int(e);                                                     \
     cudaError_t es[] = {set_attr<T, Ls>()...};                                               \
     for (cudaError_t x : es)                                                                 \
       if (x != cudaSuccess) return int(x);                                                   \

@@ -39,6 +39,14 @@ inline double coef_canti(int l, double d, double eps) {
   return (l % 2 == 1) ? coef_cprime((l + 1) / 2) * coef_bP(l, d, eps) : 0.0;
 }
 
+// Copies host memory to device memory that kernels on any stream may read: the data is there when
+// this returns. A plain cudaMemcpy of pageable memory may return before its last transfer to the
+// device, and non-blocking streams do not wait for the legacy stream that it runs on.
+inline cudaError_t upload(void* dst, const void* src, size_t bytes) {
+  const cudaError_t e = cudaMemcpy(dst, src, bytes, cudaMemcpyHostToDevice);
+  return e != cudaSuccess ? e : cudaStreamSynchronize(cudaStreamLegacy);
+}
+
 // ---- launches ---------------------------------------------------------------
 // A sequence of dependent kernel launches on one stream. A launch whose
 // predecessor on the stream is a kernel of the same sequence gets the

@@ -16,3 +16,12 @@ def _sources():
 def test_memory_is_zeroed_on_a_stream():
     found = [name for name, text in _sources() if re.search(r"\bcudaMemset\s*\(", text)]
     assert not found
+
+
+def test_uploads_are_done_before_kernels_on_other_streams():
+    text = dict(_sources())
+    # the one other user copies and reads on the legacy stream
+    before, own = text["imrp_api.cu"].split("int imrp_admittance(", 1)
+    assert not re.search(r"\bcudaMemcpy\s*\(", before + own.split("\n}\n", 1)[1])
+    init = text["imrp_inst.cuh"].rpartition("cudaMemcpyToSymbol")[2]
+    assert "cudaStreamSynchronize(cudaStreamLegacy)" in init.split("done[dev] = true")[0]
