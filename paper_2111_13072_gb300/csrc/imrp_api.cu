@@ -99,6 +99,7 @@ struct imrp_ctx {
   unsigned* gsticket = nullptr;
   double *qhist = nullptr, *uhist = nullptr;
   int64_t hcap = 0;
+  int64_t pitch_cap = 0;  // largest hcap that a 2D copy takes as its pitch
   double* stage = nullptr;  // [cap][6] FP64 staging for load / readback
   // streamed loads: two staging buffers filled on the copy stream (allocated on first use)
   double* astage[2] = {nullptr, nullptr};
@@ -624,6 +625,9 @@ int imrp_create(const imrp_params* p, imrp_ctx** out) {
   }
   ctx->nc = 2 * ncomp(ctx->L);
   cudaGetDevice(&ctx->device);
+  int pitch = 0;
+  cudaDeviceGetAttribute(&pitch, cudaDevAttrMaxPitch, ctx->device);
+  ctx->pitch_cap = pitch / int64_t(sizeof(double));
   cudaError_t e = cudaStreamCreateWithFlags(&ctx->own_stream, cudaStreamNonBlocking);
   if (e != cudaSuccess) { delete ctx; return IMRP_E_CUDA; }
   ctx->stream = ctx->own_stream;
@@ -830,9 +834,10 @@ int imrp_get_qdiff(imrp_ctx* ctx, int64_t first, int64_t count, double* qd, doub
                      (long long)ctx->host_step);
   if (count == 0) return IMRP_OK;
   const int64_t h = first - ctx->hist_first;
-  if (count <= kHostSamples && (qd || ua)) {
+  if (count <= kHostSamples && ctx->hcap <= ctx->pitch_cap && (qd || ua)) {
     // both series in one copy through the page-locked block: two copies to pageable
-    // memory and one of the error flag took 37 us a call, this and the wait 17
+    // memory and one of the error flag took 37 us a call, this and the wait 17. The
+    // series are rows hcap apart: a longer history passes the device's largest pitch
     double* s = ctx->host->samples;
     CK(cudaMemcpy2DAsync(s, count * sizeof(double), ctx->qhist + h, ctx->hcap * sizeof(double), count * sizeof(double),
                          2, cudaMemcpyDeviceToHost, ctx->stream));
