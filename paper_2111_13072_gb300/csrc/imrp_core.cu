@@ -347,8 +347,15 @@ __device__ __forceinline__ void count_byte(const uint32_t* keys, int64_t len, in
       k[i] = idx < len ? keys[idx] : 0u;
     }
 #pragma unroll
-    for (int i = 0; i < kBsItems; ++i)
-      if (i0 + int64_t(i) * NT + threadIdx.x < len) atomicAdd(&cnt[(k[i] >> shift) & 255u], 1u);
+    for (int i = 0; i < kBsItems; ++i) {
+      const bool ok = i0 + int64_t(i) * NT + threadIdx.x < len;
+      const unsigned d = (k[i] >> shift) & 255u, d0 = __shfl_sync(0xffffffffu, d, 0);
+      if (__all_sync(0xffffffffu, ok && d == d0)) {  // 32 keys of one digit: one atomic
+        if (threadIdx.x % 32 == 0) atomicAdd(&cnt[d0], 32u);
+      } else if (ok) {
+        atomicAdd(&cnt[d], 1u);
+      }
+    }
   }
 }
 
@@ -501,9 +508,15 @@ template <class T> __device__ __forceinline__ void put_part(const SoA<T>& dst, i
 // sort: the CTA counts the digits (shared atomics), scans the counts, places (key, slot) by
 // digit in any order, and each placed key finds its rank among the few of its digit by comparing
 // (key, slot): the order of a stable sort of the input slots by key, whatever the order of the
-// atomics. A bucket of more than cap keys takes several rounds, each over a range of the digits. A
-// digit of more than kBsMaxRun keys (many ties, very narrow shells) sends the bucket through
-// stable byte passes in L2 instead (by slot, then by key).
+// atomics. A bucket of more than cap keys is placed by digit in global memory and ranked in ranges
+// of digits that fit: its work grows with its keys. A comparison costs some 0.08 ns of the CTA's
+// time, a byte pass of eight ballots 1 ns per key: beyond kBsMeanRun keys in a key's digit on average
+// (or kBsMaxRun in one: one thread's share) the bucket goes through stable byte passes in L2
+// instead. Sort and gather of uneven sets (us; rounds that each read the whole bucket and a line
+// at kBsMaxRun alone -> this; byte passes by slot and by key for every bucket): N = 3e5 with nine
+// tenths of the particles in 0.03 of the range of r^2 351 -> 232 (569), in 0.01 2037 -> 955 (1611), in
+// 0.003 8104 -> 1756 (3001); N = 2e6 with 0.03 445 -> 362 (563), 0.01 2585 -> 1234 (1488), 0.001 13770
+// -> 8120 (13860); 30 discrete radii 1488 -> 1096 (1472). One CTA still takes all of a bucket.
 // k1 (v1): keys and input slots of the buckets (without st the keys in input order, v1 scratch);
 // k0, v0: scratch for the byte passes. tb: leading key bits the same in all of a bucket;
 // sb <= 32 - tb, 2^sb >= NT.
@@ -513,7 +526,8 @@ template <class T> __device__ __forceinline__ void put_part(const SoA<T>& dst, i
 // ballots per 32 keys took 0.067 ms of the 0.111 ms sort of 2e6 keys and the gather a kernel of
 // 0.024 ms; this kernel 0.040 with the gather, sort and gather 0.138 -> 0.069. N = 3001 0.032 ->
 // 0.012, N = 20000 0.027 -> 0.0175, N = 5e5 0.051 -> 0.027.
-constexpr int kBsMaxRun = 256;
+constexpr int kBsMaxRun = 256, kBsMeanRun = 32;
+constexpr int kBsTies = 32;  // ties of one key ordered by counting; more by three passes over the slots
 constexpr size_t kBsRankBytes = 8;  // shared memory per key: key and slot
 constexpr int kBsThreads = 512, kBsPerSM = 3;  // CTA of a bucket, resident per SM
 constexpr int kBsOneThreads = 1024;  // the one CTA of a small array
@@ -588,7 +602,20 @@ __global__ void __launch_bounds__(NT, MINB) k_bucket_sort(uint32_t* k1, uint32_t
       sum += c;
       big = c > big ? c : big;
     }
-    if (!__syncthreads_or(big > unsigned(kBsMaxRun))) {
+    bool rank = true;
+    if (__syncthreads_or(big > unsigned(kBsMeanRun))) {  // a crowded digit: what the comparisons would be
+      if (t == 0) s_w[0] = 0u;
+      rank = !__syncthreads_or(big > unsigned(kBsMaxRun));
+      if (rank) {
+        uint32_t pairs = 0;
+        for (int d = 0; d < per; ++d) pairs += mine[d] * mine[d];
+        atomicAdd(s_w, pairs);
+        __syncthreads();
+        rank = s_w[0] <= uint32_t(kBsMeanRun) * uint32_t(n);
+        __syncthreads();
+      }
+    }
+    if (rank) {
       uint32_t inc = sum;
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {
@@ -605,42 +632,48 @@ __global__ void __launch_bounds__(NT, MINB) k_bucket_sort(uint32_t* k1, uint32_t
         off = end;
       }
       __syncthreads();
-      // rounds over ranges [d0, d1) of digits with at most cap keys each: one, but for overfull buckets
+      // One range of digits for all of a bucket, but for an overfull one: that is placed in global
+      // memory (k0, v0) and comes back in ranges [d0, d1) of at most cap keys each.
       const uint32_t digits = 1u << sb;
+      const bool over = n > cap;
+      auto place = [&](int i0, uint32_t* kd, uint32_t* vd) {
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const uint32_t s = (k[u] << tb) >> shift;
+          if (i0 + u * NT + int(t) < n) {
+            const uint32_t p = once ? cnt[s] + r[u] : atomicAdd(&cnt[s + 1], 1u);
+            kd[p] = k[u];
+            vd[p] = v[u];
+          }
+        }
+      };
+      if (once) {
+        place(0, ks, vs);
+      } else {
+        for (int i0 = 0; i0 < n; i0 += NT * U) {
+          load(i0);
+          place(i0, over ? k0 + start : ks, over ? v0 + start : vs);
+        }
+      }
+      __syncthreads();  // the cursors stand at the digits' ends: cnt[s] is the start of s
       for (uint32_t d0 = 0; d0 < digits;) {
         uint32_t base = 0, d1 = digits, m = n;
-        if (n > cap) {  // the cursors from d0 on still stand at the digits' starts
-          base = cnt[d0 + 1];
+        if (over) {
+          base = cnt[d0];
           uint32_t lo = d0 + 1, hi = digits;  // the last d1 with start(d1) - base <= cap
           while (lo < hi) {
             const uint32_t mid = (lo + hi + 1) / 2;
-            if ((mid < digits ? cnt[mid + 1] : uint32_t(n)) - base <= uint32_t(cap)) lo = mid;
+            if (cnt[mid] - base <= uint32_t(cap)) lo = mid;
             else hi = mid - 1;
           }
           d1 = lo;
-          m = (d1 < digits ? cnt[d1 + 1] : uint32_t(n)) - base;
-          __syncthreads();  // the cursors have been read
-        }
-        auto place = [&](int i0) {
-#pragma unroll
-          for (int u = 0; u < U; ++u) {
-            const uint32_t s = (k[u] << tb) >> shift;
-            if (i0 + u * NT + int(t) < n && s >= d0 && s < d1) {
-              const uint32_t p = (once ? cnt[s] + r[u] : atomicAdd(&cnt[s + 1], 1u)) - base;
-              ks[p] = k[u];
-              vs[p] = v[u];
-            }
+          m = cnt[d1] - base;
+          for (uint32_t i = t; i < m; i += NT) {
+            ks[i] = k0[start + base + i];
+            vs[i] = v0[start + base + i];
           }
-        };
-        if (once) {
-          place(0);
-        } else {
-          for (int i0 = 0; i0 < n; i0 += NT * U) {
-            load(i0);
-            place(i0);
-          }
+          __syncthreads();
         }
-        __syncthreads();
         constexpr int G = MINB == 1 ? 4 : 2;  // gathers in flight per thread
         for (uint32_t p0 = 0; p0 < m; p0 += NT * G) {
           uint32_t at[G], from[G];
@@ -671,19 +704,28 @@ __global__ void __launch_bounds__(NT, MINB) k_bucket_sort(uint32_t* k1, uint32_t
       return;
     }
   }
-  // stable byte passes: by input slot (the bytes that n_all has; the whole array is in that
-  // order already), then by the key bits below the bucket's
+  // Stable byte passes by the key bits in which the bucket's keys differ. The whole array is in the
+  // order of its slots already. In a bucket ties are then ordered by counting the slots among them,
+  // or by passes over the slots (the bytes that n_all has) before those over the keys: at once where
+  // more than kBsTies keys share a value on average, afterwards where a run of ties is longer.
   __syncthreads();  // the counts have been read
   BsShared<NT>& sh = *reinterpret_cast<BsShared<NT>*>(sbuf);
   uint32_t *ak = k1 + start, *av = v1 + start, *dk = k0 + start, *dv = v0 + start;
-  if (!st) {
-    for (int64_t i = t; i < len; i += NT) av[i] = uint32_t(i);
-    __syncthreads();
+  if (t == 0) s_w[0] = 0u;
+  uint32_t diff = 0;
+  {
+    const uint32_t first = ak[0];
+#pragma unroll 4
+    for (int64_t i = t; i < len; i += NT) diff |= ak[i] ^ first;
   }
-  for (int pass = st ? 0 : 4; pass < 8; ++pass) {
-    const bool by_slot = pass < 4;
-    const int shift = 8 * (pass & 3);
-    if (by_slot ? ((n_all - 1) >> shift) == 0 : shift >= 32 - tb) continue;
+  if (!st)
+    for (int64_t i = t; i < len; i += NT) av[i] = uint32_t(i);
+  __syncthreads();
+  diff = __reduce_or_sync(0xffffffffu, diff);
+  if (lane == 0) atomicOr(s_w, diff);
+  __syncthreads();
+  diff = s_w[0];
+  auto pass = [&](bool by_slot, int shift) {
     if (t < 256) sh.cnt[t] = 0u;
     __syncthreads();
     count_byte<NT>(by_slot ? av : ak, len, shift, sh.cnt);
@@ -692,8 +734,48 @@ __global__ void __launch_bounds__(NT, MINB) k_bucket_sort(uint32_t* k1, uint32_t
     else bucket_pass<NT>(ak, av, dk, dv, int(len), shift, sh);
     uint32_t* x = ak; ak = dk; dk = x;
     x = av; av = dv; dv = x;
+  };
+  auto by_slot = [&]() {
+    for (int shift = 0; shift < 32 && ((n_all - 1) >> shift) != 0; shift += 8) pass(true, shift);
+  };
+  auto by_key = [&]() {
+    for (int shift = 0; shift < 32; shift += 8)
+      if ((diff >> shift) & 255u) pass(false, shift);
+  };
+  bool in_order = !st || int64_t(diff) * kBsTies < len;  // ties come out in the order of their slots
+  if (st && in_order) by_slot();
+  by_key();
+  if (!in_order) {
+    bool ties = false;
+    for (int64_t i = t; i + kBsTies < len; i += NT) ties = ties || ak[i] == ak[i + kBsTies];
+    if (__syncthreads_or(ties)) {
+      by_slot();
+      by_key();
+      in_order = true;
+    }
   }
-  for (int64_t i = t; i < len; i += NT) put_part<T>(dst, start + i, src[slot(av[i])]);
+  constexpr int G = 4;  // gathers in flight per thread
+  const int m = int(len);
+  for (int i0 = 0; i0 < m; i0 += NT * G) {
+    int at[G];
+    uint32_t from[G];
+#pragma unroll
+    for (int u = 0; u < G; ++u) {
+      const int i = at[u] = i0 + u * NT + int(t);
+      from[u] = 0u;
+      if (i >= m) continue;
+      const uint32_t key = ak[i], v = av[i];
+      for (int q = i - 1; !in_order && q >= 0 && ak[q] == key; --q) at[u] -= av[q] > v;
+      for (int q = i + 1; !in_order && q < m && ak[q] == key; ++q) at[u] += av[q] < v;
+      from[u] = slot(v);
+    }
+    Part<T> x[G];
+#pragma unroll
+    for (int u = 0; u < G; ++u) x[u] = src[from[u]];
+#pragma unroll
+    for (int u = 0; u < G; ++u)
+      if (i0 + u * NT + int(t) < m) put_part<T>(dst, start + at[u], x[u]);
+  }
 }
 
 // Largest N for the bucket sort (2930 keys a bucket on average); larger arrays take the four global
@@ -718,7 +800,7 @@ inline int sort_digit_bits(int64_t n, bool shared_gpu) {
   return b;
 }
 int sort_digits(int64_t n) { return 1 << sort_digit_bits(n, false); }
-// Shared-memory capacity for buckets of `mean` keys on average (a larger one takes more rounds)
+// Shared-memory capacity for buckets of `mean` keys on average (a larger one takes several ranges)
 inline int bucket_cap(int64_t mean) {
   int64_t c = (mean + mean / 4 * 3 + 255) / 256 * 256;
   if (c < 2048) c = 2048;
