@@ -216,11 +216,18 @@ __device__ __forceinline__ void moments_block(const MomArgs<T>& a, int64_t item,
     const T X = PX[i], Y = PY[i], Z = PZ[i];
     const int o = (k % PPT) * S + k / PPT;
     const T r2 = fma_t(Z, Z, fma_t(Y, Y, X * X));
-    // FP64: from the reciprocal root, which is needed anyway (a division costs some 20
-    // FP64 operations, and every column range stages its particles)
+    // FP64: from the reciprocal root, which is needed anyway, with one correction by the
+    // remainder (a division costs some 20 FP64 operations, and every column range stages its
+    // particles). q enters to the power of the degree: without the correction the sums of a
+    // particle near the equator are 2.4 times as far off at l_max = 24 as with a division, with it
+    // they are as near.
     T ir = rsqrt_t(r2), q;
-    if constexpr (sizeof(T) == 8) q = a.rho * (ir * ir);
-    else q = a.rho / r2;
+    if constexpr (sizeof(T) == 8) {
+      q = a.rho * (ir * ir);
+      q = fma(fma(-q, r2, a.rho), ir * ir, q);
+    } else {
+      q = a.rho / r2;
+    }
     sx[o] = X * ri; sy[o] = Y * ri; sz[o] = Z * ri;
     sq[o] = q;
     // the particle's charge seeds its harmonics: -1 for an electron, q_ion
