@@ -371,9 +371,11 @@ int imrp_fp32_peak(double* tflops, int* sm_count);
  *
  * imrp_autotune times, on the loaded particles and with field evaluations only
  * (the state does not advance), the field kernel at 8, 4, 2 and 1 warps per
- * CTA and the group scan (the FP64 scan over the 1024-particle scan groups)
+ * CTA (FP64 with all m has one shape, 4) and the group scan (the FP64 scan over the 1024-particle scan groups)
  * at 16, 32 and 64 groups per segment at least, and keeps the fastest of each
- * for the context. wpb_out / gseg_out (may be NULL) receive the choices.
+ * for the context; a later load of a number of particles that another field
+ * kernel or launch shape serves takes that one's default instead of the tuned
+ * warps per CTA. wpb_out / gseg_out (may be NULL) receive the choices.
  * Errors: IMRP_E_STATE (nothing loaded), IMRP_E_CUDA. */
 int imrp_autotune(imrp_ctx* ctx, int* wpb_out, int* gseg_out);
 

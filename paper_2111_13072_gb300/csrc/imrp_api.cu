@@ -80,7 +80,9 @@ struct imrp_ctx {
   int wpb = 8;                 // warps per CTA of the field kernel for the loaded n
   int wpb_full = 8;            // its choice when the tiles fill the GPU several times
   int resident[4] = {0};       // resident warps per SM at 8, 4, 2, 1 warps per CTA
-  bool tuned = false;          // wpb was chosen by the autotuner
+  int tuned_wpb = 0;           // the autotuner's choice (0: none), the field kernel it was measured
+  int tuned_kernel = 0;        // with (FieldKernel) and what field_wpb gives for that load
+  int tuned_rule = 0;
   int gseg = 32;  // least groups per segment of the group scan
   // streams / graphs
   cudaStream_t own_stream = nullptr, stream = nullptr;
@@ -194,6 +196,19 @@ int field_wpb(const imrp_ctx* c, int64_t ntiles) {
   return best;
 }
 
+// The kernel that runs the field of n particles (field_launch's order).
+enum FieldKernel { kFieldTile, kFieldSmall, kFieldPair, kFieldTeam };
+FieldKernel field_kernel_of(const imrp_ctx* c, int64_t n) {
+  if (uses_pairs(c, n)) return kFieldPair;
+  if (uses_team(c)) return kFieldTeam;
+  return c->prec == 1 && img_in_tile_for<float>(n) ? kFieldSmall : kFieldTile;
+}
+// Whether the autotuner's shape is the loaded particles': it was measured for one kernel and one
+// number of tiles, and stands in for field_wpb while the kernel and field_wpb's answer are those.
+bool shape_tuned(const imrp_ctx* c) {
+  return c->tuned_wpb > 0 && c->tuned_kernel == field_kernel_of(c, c->n) && c->tuned_rule == field_wpb(c, c->ntiles);
+}
+
 // What depends on the number of particles of a load or restore.
 void set_count(imrp_ctx* c, int64_t n) {
   c->n = n;
@@ -201,7 +216,7 @@ void set_count(imrp_ctx* c, int64_t n) {
   c->n_ion = n_ion_of(c, n);
   c->ntiles = (n + 31) / 32;
   c->ngroups = (c->ntiles + kTilesPerGroup - 1) / kTilesPerGroup;
-  if (!c->tuned) c->wpb = field_wpb(c, c->ntiles);
+  c->wpb = shape_tuned(c) ? c->tuned_wpb : field_wpb(c, c->ntiles);
 }
 
 void free_all(imrp_ctx* c) {
@@ -1115,8 +1130,9 @@ extern "C" int imrp_autotune(imrp_ctx* ctx, int* wpb_out, int* gseg_out) {
   if (!ctx) return IMRP_E_INVAL;
   if (!ctx->loaded) return ctx->fail(IMRP_E_STATE, "autotune before load");
   const int reps = 3;
-  // field kernel: warps per CTA
-  {
+  // field kernel: warps per CTA (the FP64 kernel of four warps per tile has one shape)
+  if (!uses_team(ctx)) {
+    const int rule = field_wpb(ctx, ctx->ntiles);
     int best_w = ctx->wpb;
     float best = 1e30f;
     for (int w : {8, 4, 2, 1}) {
@@ -1129,8 +1145,9 @@ extern "C" int imrp_autotune(imrp_ctx* ctx, int* wpb_out, int* gseg_out) {
       if (rc) return rc;
       if (ms < best) { best = ms; best_w = w; }
     }
-    ctx->wpb = best_w;
-    ctx->tuned = true;
+    ctx->wpb = ctx->tuned_wpb = best_w;
+    ctx->tuned_kernel = field_kernel_of(ctx, ctx->n);
+    ctx->tuned_rule = rule;
   }
   // group scan: least groups per segment
   {
@@ -1146,7 +1163,7 @@ extern "C" int imrp_autotune(imrp_ctx* ctx, int* wpb_out, int* gseg_out) {
     ctx->gseg = best_c;
   }
   drop_graphs(ctx);
-  if (wpb_out) *wpb_out = ctx->wpb;
+  if (wpb_out) *wpb_out = uses_team(ctx) ? kTeam : ctx->wpb;
   if (gseg_out) *gseg_out = ctx->gseg;
   return check_err(ctx);
 }
@@ -1274,10 +1291,12 @@ int build_groups(imrp_batch* b) {
       g = &b->groups.back();
       g->prec = ctx->prec;
       g->L = ctx->L;
-      g->wpb = ctx->tuned ? ctx->wpb : ctx->wpb_full;  // of the group's first context, unless tuned
       for (const int3& t : b->tuned)
         if (t.x == g->prec && t.y == g->L) g->wpb = t.z;
     }
+    // of the group's first context in k_field_batch, unless the batch is tuned
+    const FieldKernel k = field_kernel_of(ctx, ctx->n);
+    if (g->wpb == 0 && (k == kFieldTile || k == kFieldSmall)) g->wpb = shape_tuned(ctx) ? ctx->wpb : ctx->wpb_full;
     g->members.push_back(int(i));
   }
   for (auto& g : b->groups) {
@@ -1462,7 +1481,6 @@ template <class T> int time_group_field(imrp_batch* b, const BatchGroup& g, int 
     for (int64_t t = 0; t < ctx->ntiles; t += wpb) fi.push_back(make_int2(int(k), int(t)));
   }
   *ms = 0.f;
-  if (fi.empty()) return IMRP_OK;
   void* dfa = nullptr;
   int2* dfi = nullptr;
   int rc = IMRP_OK;
@@ -1521,6 +1539,7 @@ extern "C" int imrp_batch_autotune(imrp_batch* b) {
   if (rc) { b->err = "batch work lists"; return rc; }
   b->tuned.clear();
   for (auto& g : b->groups) {
+    if (g.nfield == 0) continue;  // nothing runs in k_field_batch: no shape to choose
     int best_w = g.wpb;
     float best = 1e30f;
     for (int w : {8, 4, 2, 1}) {

@@ -412,6 +412,7 @@ template <class T> __host__ __device__ constexpr bool field_pair_rule(int L, int
 
 // Whether an instance's field runs in the FP64 kernel of four warps per tile
 // (field_team): all FP64 instances with all m.
+constexpr int kTeam = 4;
 template <class T> __host__ __device__ constexpr bool field_team_rule(int m0_only) { return sizeof(T) == 8 && !m0_only; }
 
 // Column chunks of the far field: chunk q of the multipole (Is) part covers

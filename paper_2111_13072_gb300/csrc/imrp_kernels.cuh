@@ -1719,7 +1719,6 @@ __global__ void __launch_bounds__(kPairMaxWarps * 32, 4) k_field_pair_batch(cons
 // average), N = 40000: 0.266 -> 0.194; l_max = 12, N = 60000: 0.486 -> 0.415; l_max = 16,
 // N = 250001: 2.49 -> 2.28; l_max = 2, N = 1e6: 1.79 -> 1.54.
 // ----------------------------------------------------------------------------
-constexpr int kTeam = 4;
 __host__ __device__ constexpr size_t team_smem(int L) {
   return sizeof(double) * (size_t(12) * nP(L) + 32 * (2 * L + 2) + 32 * 6 + kTeam * 3 * 32 + 2 * (2 * pair_run(L) + 1));
 }
