@@ -980,8 +980,8 @@ template <class T>
 __global__ void k_load(const double* __restrict__ xs, const double* __restrict__ vs,
                        const uint32_t* __restrict__ ids, Part<T>* __restrict__ st, uint32_t* __restrict__ key,
                        uint32_t* __restrict__ kidx, int64_t n, double r_out2, RadiusKey rk, int* err) {
-  const int64_t j = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (j >= n) return;
+  const int64_t j0 = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+  const int64_t j = j0 < n ? j0 : n - 1;  // (every thread votes below)
   double v[6];
   bool fin = true;
 #pragma unroll
@@ -998,7 +998,6 @@ __global__ void k_load(const double* __restrict__ xs, const double* __restrict__
   p.x = narrow<T>(v[0]); p.y = narrow<T>(v[1]); p.z = narrow<T>(v[2]);
   p.vx = narrow<T>(v[3]); p.vy = narrow<T>(v[4]); p.vz = narrow<T>(v[5]);
   p.id = ids ? ids[j] : uint32_t(j);
-  st[j] = p;
   // range test and radius key (radius_key's two forms, with r^2 shared)
   bool inside;
   uint32_t k;
@@ -1014,8 +1013,12 @@ __global__ void k_load(const double* __restrict__ xs, const double* __restrict__
     inside = r2 > 1.0 && r2 < r_out2;
     k = key_of_r2(r2, rk);
   }
-  if (!fin) atomicOr(err, kErrNaN);
-  else if (!inside) atomicOr(err, kErrRange);
+  // one atomic per CTA: the flags stand in host memory, where atomics are done one after the other
+  // (8e6 bad particles with one per warp 4.9 ms, a good load 2.2)
+  const bool nan = __syncthreads_or(!fin), out = __syncthreads_or(fin && !inside);
+  if (threadIdx.x == 0 && (nan || out)) atomicOr(err, (nan ? kErrNaN : 0) | (out ? kErrRange : 0));
+  if (j0 >= n) return;
+  st[j] = p;
   key[j] = k;
   kidx[j] = uint32_t(j);
 }
