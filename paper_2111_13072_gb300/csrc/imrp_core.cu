@@ -533,11 +533,93 @@ constexpr int kBsThreads = 512, kBsPerSM = 3;  // CTA of a bucket, resident per 
 constexpr int kBsOneThreads = 1024;  // the one CTA of a small array
 static_assert(kBsThreads >= 256 && kBsOneThreads >= 256, "256 threads scan the byte counts");
 
+// Stable byte passes over the bucket start .. start + len by the key bits in which its keys differ, and
+// the gather. The whole array (in_slots) is in the order of its slots already. In a bucket ties are then
+// ordered by counting the slots among them, or by passes over the slots (the bytes that n_all has) before
+// those over the keys: at once where more than kBsTies keys share a value on average, afterwards where a
+// run of ties is longer. A function of its own: inlined, it makes the kernel spill for all its buckets
+// (52 bytes with 512 threads, so none; sort of N = 1e5: 20.5 us, so 19.8; 2e6: 73.0 and 71.5).
+template <class T, int NT>
+__device__ __noinline__ void bucket_bytes(uint32_t* k1, uint32_t* v1, uint32_t* k0, uint32_t* v0, int64_t start, int64_t len,
+                                          int64_t n_all, bool in_slots, const Part<T>* src, const SoA<T>& dst, int* err) {
+  extern __shared__ __align__(16) uint32_t sbuf[];
+  __shared__ uint32_t s_diff;
+  const unsigned t = threadIdx.x, lane = t & 31;
+  BsShared<NT>& sh = *reinterpret_cast<BsShared<NT>*>(sbuf);
+  uint32_t *ak = k1, *av = v1, *dk = k0, *dv = v0;
+  if (t == 0) s_diff = 0u;
+  uint32_t diff = 0;
+  {
+    const uint32_t first = ak[0];
+#pragma unroll 4
+    for (int64_t i = t; i < len; i += NT) diff |= ak[i] ^ first;
+  }
+  if (in_slots)
+    for (int64_t i = t; i < len; i += NT) av[i] = uint32_t(i);
+  __syncthreads();
+  diff = __reduce_or_sync(0xffffffffu, diff);
+  if (lane == 0) atomicOr(&s_diff, diff);
+  __syncthreads();
+  diff = s_diff;
+  auto pass = [&](bool by_slot, int shift) {
+    if (t < 256) sh.cnt[t] = 0u;
+    __syncthreads();
+    count_byte<NT>(by_slot ? av : ak, len, shift, sh.cnt);
+    __syncthreads();
+    if (by_slot) bucket_pass<NT>(av, ak, dv, dk, int(len), shift, sh);
+    else bucket_pass<NT>(ak, av, dk, dv, int(len), shift, sh);
+    uint32_t* x = ak; ak = dk; dk = x;
+    x = av; av = dv; dv = x;
+  };
+  auto by_slot = [&]() {
+    for (int shift = 0; shift < 32 && ((n_all - 1) >> shift) != 0; shift += 8) pass(true, shift);
+  };
+  auto by_key = [&]() {
+    for (int shift = 0; shift < 32; shift += 8)
+      if ((diff >> shift) & 255u) pass(false, shift);
+  };
+  bool in_order = in_slots || int64_t(diff) * kBsTies < len;  // ties come out in the order of their slots
+  if (!in_slots && in_order) by_slot();
+  by_key();
+  if (!in_order) {
+    bool ties = false;
+    for (int64_t i = t; i + kBsTies < len; i += NT) ties = ties || ak[i] == ak[i + kBsTies];
+    if (__syncthreads_or(ties)) {
+      by_slot();
+      by_key();
+      in_order = true;
+    }
+  }
+  constexpr int G = 4;  // gathers in flight per thread
+  const int m = int(len);
+  for (int i0 = 0; i0 < m; i0 += NT * G) {
+    int at[G];
+    uint32_t from[G];
+#pragma unroll
+    for (int u = 0; u < G; ++u) {
+      const int i = at[u] = i0 + u * NT + int(t);
+      from[u] = 0u;
+      if (i >= m) continue;
+      const uint32_t key = ak[i], v = av[i];
+      for (int q = i - 1; !in_order && q >= 0 && ak[q] == key; --q) at[u] -= av[q] > v;
+      for (int q = i + 1; !in_order && q < m && ak[q] == key; ++q) at[u] += av[q] < v;
+      from[u] = v < n_all ? v : 0u;
+      if (v >= n_all) atomicOr(err, kErrSort);
+    }
+    Part<T> x[G];
+#pragma unroll
+    for (int u = 0; u < G; ++u) x[u] = src[from[u]];
+#pragma unroll
+    for (int u = 0; u < G; ++u)
+      if (i0 + u * NT + int(t) < m) put_part<T>(dst, start + at[u], x[u]);
+  }
+}
+
 template <class T, int NT, int MINB>
 __global__ void __launch_bounds__(NT, MINB) k_bucket_sort(uint32_t* k1, uint32_t* v1, uint32_t* k0, uint32_t* v0,
                                                           const SortState* __restrict__ st, int64_t n_all, int cap,
                                                           int tb, int sb, const Part<T>* __restrict__ src,
-                                                          SoA<T> dst, int* err) {
+                                                          const __grid_constant__ SoA<T> dst, int* err) {
   chain_wait();
   extern __shared__ __align__(16) uint32_t sbuf[];
   __shared__ uint32_t s_w[NT / 32];
@@ -685,6 +767,7 @@ __global__ void __launch_bounds__(NT, MINB) k_bucket_sort(uint32_t* k1, uint32_t
             const uint32_t key = ks[p], s = (key << tb) >> shift, b = cnt[s] - base, e = cnt[s + 1] - base;
             from[u] = vs[p];
             at[u] = b;
+#pragma unroll 1  // a digit has few keys (sort of N = 5e5: 33.6 us, unrolled 34.2; 2e6: 71.1 and 71.5)
             for (uint32_t q = b; q < e; ++q) {
               const uint32_t kq = ks[q];
               at[u] += kq < key || (kq == key && vs[q] < from[u]) ? 1u : 0u;
@@ -704,78 +787,8 @@ __global__ void __launch_bounds__(NT, MINB) k_bucket_sort(uint32_t* k1, uint32_t
       return;
     }
   }
-  // Stable byte passes by the key bits in which the bucket's keys differ. The whole array is in the
-  // order of its slots already. In a bucket ties are then ordered by counting the slots among them,
-  // or by passes over the slots (the bytes that n_all has) before those over the keys: at once where
-  // more than kBsTies keys share a value on average, afterwards where a run of ties is longer.
   __syncthreads();  // the counts have been read
-  BsShared<NT>& sh = *reinterpret_cast<BsShared<NT>*>(sbuf);
-  uint32_t *ak = k1 + start, *av = v1 + start, *dk = k0 + start, *dv = v0 + start;
-  if (t == 0) s_w[0] = 0u;
-  uint32_t diff = 0;
-  {
-    const uint32_t first = ak[0];
-#pragma unroll 4
-    for (int64_t i = t; i < len; i += NT) diff |= ak[i] ^ first;
-  }
-  if (!st)
-    for (int64_t i = t; i < len; i += NT) av[i] = uint32_t(i);
-  __syncthreads();
-  diff = __reduce_or_sync(0xffffffffu, diff);
-  if (lane == 0) atomicOr(s_w, diff);
-  __syncthreads();
-  diff = s_w[0];
-  auto pass = [&](bool by_slot, int shift) {
-    if (t < 256) sh.cnt[t] = 0u;
-    __syncthreads();
-    count_byte<NT>(by_slot ? av : ak, len, shift, sh.cnt);
-    __syncthreads();
-    if (by_slot) bucket_pass<NT>(av, ak, dv, dk, int(len), shift, sh);
-    else bucket_pass<NT>(ak, av, dk, dv, int(len), shift, sh);
-    uint32_t* x = ak; ak = dk; dk = x;
-    x = av; av = dv; dv = x;
-  };
-  auto by_slot = [&]() {
-    for (int shift = 0; shift < 32 && ((n_all - 1) >> shift) != 0; shift += 8) pass(true, shift);
-  };
-  auto by_key = [&]() {
-    for (int shift = 0; shift < 32; shift += 8)
-      if ((diff >> shift) & 255u) pass(false, shift);
-  };
-  bool in_order = !st || int64_t(diff) * kBsTies < len;  // ties come out in the order of their slots
-  if (st && in_order) by_slot();
-  by_key();
-  if (!in_order) {
-    bool ties = false;
-    for (int64_t i = t; i + kBsTies < len; i += NT) ties = ties || ak[i] == ak[i + kBsTies];
-    if (__syncthreads_or(ties)) {
-      by_slot();
-      by_key();
-      in_order = true;
-    }
-  }
-  constexpr int G = 4;  // gathers in flight per thread
-  const int m = int(len);
-  for (int i0 = 0; i0 < m; i0 += NT * G) {
-    int at[G];
-    uint32_t from[G];
-#pragma unroll
-    for (int u = 0; u < G; ++u) {
-      const int i = at[u] = i0 + u * NT + int(t);
-      from[u] = 0u;
-      if (i >= m) continue;
-      const uint32_t key = ak[i], v = av[i];
-      for (int q = i - 1; !in_order && q >= 0 && ak[q] == key; --q) at[u] -= av[q] > v;
-      for (int q = i + 1; !in_order && q < m && ak[q] == key; ++q) at[u] += av[q] < v;
-      from[u] = slot(v);
-    }
-    Part<T> x[G];
-#pragma unroll
-    for (int u = 0; u < G; ++u) x[u] = src[from[u]];
-#pragma unroll
-    for (int u = 0; u < G; ++u)
-      if (i0 + u * NT + int(t) < m) put_part<T>(dst, start + at[u], x[u]);
-  }
+  bucket_bytes<T, NT>(k1 + start, v1 + start, k0 + start, v0 + start, start, len, n_all, !st, src, dst, err);
 }
 
 // Largest N for the bucket sort (2930 keys a bucket on average); larger arrays take the four global
