@@ -35,6 +35,9 @@ METRIC = "particle-steps/s at N=2e6,l_max=16 (mixed vs FP64); served spectra p50
 UNIT = "particle-steps/s"
 BUCKET_SORT_SINGLE_N = 4096   # the library sorts up to this many keys in 1 launch,
 BUCKET_SORT_MAX_N = 24000000  # up to this many in 4 stages, more in 12
+PAIR_MIN_N, PAIR_MIN_L = 1 << 19, 12  # FP32 instances of the field's pair kernel: from here on
+IMG_IN_TILE_MAX_N = 1024      # FP32 instances of k_field_small: up to here
+FP64_SMALL_MOMENTS_MAX_N = 99 * 1024  # FP64 instances with 4 particles per thread in the moments: up to here
 
 
 def sort_launches(n):
@@ -93,10 +96,24 @@ def field_flops_per_particle(L):
 
 
 def field_kernel(w, n):
-    """The field kernel that a workload of n particles runs (the library's rule)."""
-    if w.precision == 1 and w.l_max >= 12 and n >= 1 << 19 and not w.m0_only:
+    """The field kernel that a workload of n particles runs alone (the library's rules, in its order)."""
+    if w.precision == 1 and w.l_max >= PAIR_MIN_L and n >= PAIR_MIN_N and not w.m0_only:
         return "k_field_pair (field + push, two tiles per warp)"
-    return "k_field (field + push)" if w.precision == 1 else "k_field_team (field + push, FP64)"
+    if w.precision == 0 and not w.m0_only:
+        return "k_field_team (field + push, FP64)"
+    if w.precision == 1 and n <= IMG_IN_TILE_MAX_N:
+        return "k_field_small (field + push, image pairs of the tile summed directly)"
+    return "k_field (field + push)"
+
+
+def batched_launches(ws):
+    """Launches of the moments and field stages of one batched step: per degree and
+    precision one for the moments (FP64: one more where both of the moments' shapes
+    occur) and one for the field (one more where some members run in a kernel of
+    their own, the pair or the FP64 kernel, and some in k_field_batch)."""
+    moments = {(w.precision, w.l_max, w.precision == 0 and w.N <= FP64_SMALL_MOMENTS_MAX_N) for w in ws}
+    field = {(w.precision, w.l_max, field_kernel(w, w.N).split()[0] in ("k_field_pair", "k_field_team")) for w in ws}
+    return len(moments) + len(field)
 
 
 def kernel_hash():
@@ -323,15 +340,14 @@ def ensemble_measure(steps, warmup, autotune=True, n_instances=64, stream=None):
     ntot = sum(w.N for w in ws)
     for s in sims:
         s.close()
-    # per context: all stages but moments and field; per degree and precision:
-    # one moments and one field launch
-    launches = sum(step_launches(w.N) - 2 - fused_stages(w.N) for w in ws) + 2 * len({(w.precision, w.l_max) for w in ws})
+    # per context: all stages but moments and field
+    launches = sum(step_launches(w.N) - 2 - fused_stages(w.N) for w in ws) + batched_launches(ws)
     return {"value": ntot * steps / (ms / 1e3), "unit": UNIT, "instances": n_instances,
             "gpu_launches_per_step": launches,
             "particles": ntot, "steps": steps, "ms_per_step": ms / steps, "autotuned": autotune,
             "workload": "64 instances, N log-uniform [1e4,1e6], T_e U[0.5,5] eV, n_e log-U[1e14,1e17], "
                         "l_max in {8,12,16}, mixed precision, one captured graph per step pair, "
-                        "one moments and one field launch per degree"}
+                        "one moments launch and one or two field launches per degree"}
 
 
 def ensemble_compare(steps, warmup):
