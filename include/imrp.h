@@ -447,8 +447,10 @@ int imrp_batch_failed(const imrp_batch* b);
  * current: CUDA loads device code lazily, and loading reserves device memory
  * (the code, its tables and the static array itself), so the set-up loads
  * every kernel this entry point can launch (both precisions, every degree up
- * to IMRP_NOALLOC_MAX_L), fills their constant tables and looks up the device
- * address of the static array with cudaGetSymbolAddress. Make that first call
+ * to IMRP_NOALLOC_MAX_L), fills their constant tables, looks up the device
+ * address of the static array with cudaGetSymbolAddress and reserves one
+ * page-locked word of host memory (cudaHostAlloc, mapped) for the device's error
+ * flag, which is held until the process exits. Make that first call
  * at start-up, where reserving memory is allowed, and before any stream
  * capture; later calls load and reserve nothing. The set-up does not survive
  * a cudaDeviceReset of the device (nor does anything else of this library):

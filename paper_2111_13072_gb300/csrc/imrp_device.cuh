@@ -398,10 +398,13 @@ __host__ __device__ constexpr int img_in_tile_for(int64_t n) {
 // and up, at least 2^19 particles, all m. A rule of n, so that an instance computes
 // the same alone and in a batch. Field ms, one tile per warp against the pair kernel:
 // l_max = 16 N = 5e5 0.150 and 0.135, N = 1e6 0.275 and 0.250; l_max = 12 N = 131072
-// 0.0413 and 0.0392, N = 5e5 0.115 and 0.097. It is the faster one below the line too,
-// down to 1e5 particles; but its sums round differently, and the trajectories of small
-// instances, where one particle's charge weighs more, follow the last bit of the
-// field (two particles within a rounding of the same radius swap): they keep theirs.
+// 0.0413 and 0.0392, N = 5e5 0.115 and 0.097. It is the faster one below the line too:
+// N = 100003, l_max = 12, 16, 24 0.0357, 0.0433, 0.0888 and 0.0331, 0.0415, 0.0826; N = 300001
+// 0.0759, 0.0968, 0.2158 and 0.0638, 0.0887, 0.1726. Its error against the FP64 field is 0.2 to
+// 0.7 % larger there (N = 100003, l_max = 16, three seeds: 1.037, 0.983, 1.026e-6 and 1.044, 0.990,
+// 1.034e-6 of the rms), and the trajectories of small instances, where one particle's
+// charge weighs more, follow the last bit of the field (two particles within a rounding of
+// the same radius swap): they keep theirs.
 constexpr int64_t kPairMinN = int64_t(1) << 19;
 constexpr int kPairMinL = 12;
 constexpr int kPairWarps = 2, kPairMaxWarps = 4;  // warps per CTA: default, at most

@@ -172,10 +172,11 @@ template <class T> inline void derive_field_args(FieldArgs<T>& a) {
 template <class T>
 void launch_scans(const T* agg, T* pfx, double* gagg, double* work, unsigned* ticket, T* gbase, T* tot, double* totd,
                   int64_t ntiles, int nc, int gseg, const FinalizeArgs* fin, LaunchSeq& seq);
-// Loads the device code of every degree-independent kernel of both precisions
-// (CUDA loads modules lazily, at a kernel's first launch or query, and the
-// load reserves device memory): the allocation-free entry point calls it at
-// its set-up so that later calls load nothing.
+// Loads the device code of the degree-independent kernels of both precisions that
+// the allocation-free entry point can launch, and of some others (CUDA loads
+// device code lazily, at a kernel's first launch or query, and the load reserves
+// device memory): that entry point calls it at its set-up so that its later
+// calls load nothing. (The read-back by ids and the transform are not among them.)
 cudaError_t preload_core_kernels();
 // opt-in shared memory of the sort's bucket kernel (once per device, before
 // the first sort)

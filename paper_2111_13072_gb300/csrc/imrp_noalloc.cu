@@ -1,7 +1,8 @@
 // imrp_field_noalloc: the field evaluation of imrp_get_field for callers that
 // cannot allocate device memory (see include/imrp.h). All intermediate
-// buffers live in one file-scope device array of fixed size; nothing here
-// calls cudaMalloc, cudaFree or any other allocating routine.
+// buffers live in one file-scope device array of fixed size; no call allocates
+// or frees device memory. The first call on a device also takes one page-locked
+// mapped word of host memory for its error flag, which is kept until exit.
 #include <cuda_runtime.h>
 #include <math.h>
 #include <string.h>
@@ -66,7 +67,7 @@ void* g_addr[64] = {nullptr};  // device address of g_scratch, per device
 volatile int* g_err[64] = {nullptr};
 int* g_derr[64] = {nullptr};
 // The table of per-degree kernels is built when the library is loaded, so
-// that the entry point itself never allocates (not even host memory).
+// that no call allocates host memory for it.
 std::vector<KernelSet<float>> g_f;
 std::vector<KernelSet<double>> g_d;
 struct Registry {
